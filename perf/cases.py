@@ -189,6 +189,13 @@ def _select_preds(case):
     return [("rating", aiq.GE, 3)] if case["shape"] == "tiny" else [("rating", aiq.GE, 4), ("year", aiq.GE, 2000)]
 
 
+def _selected(case, cols):
+    keep = np.ones(case["rows"], bool)
+    for c, _, v in _select_preds(case):
+        keep &= cols[c] >= v
+    return np.nonzero(keep)[0]
+
+
 def _weight_specs(s):
     specs = [("embed", (s.vocab, s.d_model), 0.0)]
     for l in range(s.n_layers):
@@ -428,12 +435,13 @@ def work(case):
         return {"bytes": case["build"] * 12 + case["rows"] * (8 + 0.2 * 8), "flops": 0}
     if op == "select":
         s = Shape(case["shape"])
-        p = 0.6 if case["shape"] == "tiny" else 2 / 15
-        mean = 32 if case["median"] == 0 else case["median"] * 1.12
-        S = max(1.0, case["rows"] * p)
-        T = S * mean + case["prefix"]
-        flops = 2.0 * s.layer_weights() * s.n_layers * T
-        flops += 4.0 * s.qd * s.n_layers * S * (mean * case["prefix"] + mean * mean * 0.6)
+        cols, offsets, _, _ = _select_table(case, _rng(case, 0))
+        n = (offsets[1:] - offsets[:-1])[_selected(case, cols)].astype(np.float64)
+        P, T = case["prefix"], float(n.sum()) + case["prefix"]
+        pairs = float((n * P + n * (n + 1) / 2).sum()) + P * (P + 1) / 2
+        # the last layer's O and MLP are needed at each row's last token only
+        tail = 2.0 * s.d_model * (s.qd + 3 * s.d_ffn) * (T - len(n))
+        flops = 2.0 * s.layer_weights() * s.n_layers * T - tail + 4.0 * s.qd * s.n_layers * pairs
         return {"bytes": 2.0 * s.layer_weights() * s.n_layers + T * 2 * s.d_model + case["rows"] * 8, "flops": flops}
     decode = op.startswith("decode")
     if op in ("attention", "decode_attention"):
@@ -547,10 +555,7 @@ def _layer64(st):
 
 def _select64(case, rng):
     cols, offsets, tokens, prefix = _select_table(case, rng)
-    keep = np.ones(case["rows"], bool)
-    for c, _, v in _select_preds(case):
-        keep &= cols[c] >= v
-    rows = np.nonzero(keep)[0]
+    rows = _selected(case, cols)
     if not len(rows):
         return {"rows": rows.astype(np.int32), "logits": np.zeros((0, 2))}
     s = Shape(case["shape"])
