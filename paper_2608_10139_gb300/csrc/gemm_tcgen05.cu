@@ -20,6 +20,8 @@
 //             already fills the other accumulator.
 #include <cudaTypedefs.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 #include "kernels.h"
 
@@ -150,13 +152,29 @@ __device__ __forceinline__ void add_store_f32x32(float* dst, const float* v, flo
   }
 }
 
+// Sum of squares of 16 consecutive columns.  A row's sum over 128 columns is
+// always these eight sums added in order, whichever tile width formed them, so
+// that a row's norm does not depend on how many rows its GEMM had.
+__device__ __forceinline__ float sum_sq16(const float* v) {
+  float s = 0.f;
+#pragma unroll
+  for (int j = 0; j < 16; ++j) s = __fmaf_rn(v[j], v[j], s);
+  return s;
+}
+
 // 1 / RMS of an accumulator row from its partial sums of squares (fixed
 // summation order), or 1 when the GEMM's input is already normalised.
 __device__ __forceinline__ float row_inv_rms(const GemmEpilogue& ep, int row, bool live) {
   if (!ep.row_ss || !live) return 1.f;
   const float* p = ep.row_ss + static_cast<int64_t>(row) * ep.ss_parts;
   float s = 0.f;
-  if ((ep.ss_parts & 3) == 0) {
+  if (ep.ss_split == 8) {  // eight 16-column sums per 128 columns (ss_parts is a multiple of 8)
+    const float4* p4 = reinterpret_cast<const float4*>(p);
+    for (int i = 0; i < ep.ss_parts / 8; ++i) {
+      const float4 a = __ldg(p4 + 2 * i), b = __ldg(p4 + 2 * i + 1);
+      s += ((((((a.x + a.y) + a.z) + a.w) + b.x) + b.y) + b.z) + b.w;
+    }
+  } else if ((ep.ss_parts & 3) == 0) {
     const float4* p4 = reinterpret_cast<const float4*>(p);
     for (int i = 0; i < ep.ss_parts / 4; ++i) {
       const float4 v = __ldg(p4 + i);
@@ -202,7 +220,7 @@ __device__ __forceinline__ void epilogue_tile(const KArgs& a, uint32_t trow, int
   bool bad = false;
   if constexpr (EPI == EPI_RESID_F32) {
     float* o = static_cast<float*>(ep.out) + static_cast<int64_t>(row) * ep.ldo + n0;
-    float part = 0.f;  // sum of squares of the new residual over 128 columns
+    float part = 0.f;  // sum of squares of the new residual over 128 columns (sum_sq16 groups, in order)
 #pragma unroll 1
     for (int c = 0; c < BN; c += 64) {
       float v0[32], v1[32];
@@ -212,8 +230,9 @@ __device__ __forceinline__ void epilogue_tile(const KArgs& a, uint32_t trow, int
         add_store_f32x32(o + c + 32, v1, v1);
         if (ep.xh_out) {
           __half* xh = ep.xh_out + static_cast<int64_t>(row) * ep.ldo + n0 + c;
-#pragma unroll
-          for (int j = 0; j < 32; ++j) part += v0[j] * v0[j] + v1[j] * v1[j];
+          const float s0 = sum_sq16(v0), s1 = sum_sq16(v0 + 16), s2 = sum_sq16(v1), s3 = sum_sq16(v1 + 16);
+          part = (c & 64) ? part + s0 : s0;
+          part = ((part + s1) + s2) + s3;
           if (ep.xh_gain) {
             // the next attention norm's gain goes on the activation (the QKV
             // weights stay exact): one fp16 rounding of x * g per element
@@ -232,10 +251,7 @@ __device__ __forceinline__ void epilogue_tile(const KArgs& a, uint32_t trow, int
           }
           store_f16x32(xh, v0, bad);
           store_f16x32(xh + 32, v1, bad);
-          if ((c & 127) == 64) {
-            ep.ss_out[static_cast<int64_t>(row) * ep.ss_parts + (n0 + c) / 128] = part;
-            part = 0.f;
-          }
+          if ((c & 127) == 64) ep.ss_out[static_cast<int64_t>(row) * ep.ss_parts + (n0 + c) / 128] = part;
         }
       }
     }
@@ -281,12 +297,14 @@ __device__ __forceinline__ void epilogue_tile(const KArgs& a, uint32_t trow, int
     for (int c = 0; c < BN / 2; c += 32) {
       float g[32], u[32];
       load2x32(trow + c, trow + BN / 2 + c, g, u);
-#pragma unroll
-      for (int j = 0; j < 32; ++j) {
-        const float gj = g[j] * inv;
-        g[j] = gj / (1.0f + expf(-gj)) * (u[j] * inv);
-      }
+      // rows past M hold zeros, and a division of zero leaves the fast path:
+      // skipping them takes a 128-row tile with dead rows from 21 to 6 us
       if (live) {
+#pragma unroll
+        for (int j = 0; j < 32; ++j) {
+          const float gj = g[j] * inv;
+          g[j] = gj / (1.0f + expf(-gj)) * (u[j] * inv);
+        }
         store_f16x32(o + c, g, bad);
         if (ep.lo_off > 0) {
 #pragma unroll
@@ -786,6 +804,357 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 }
 
+// ------------------------------------------------------------- few rows ---
+// Products with few rows (a generation step, the shared prefix's own pass, a
+// small chunk, the final layer's last tokens): MT x BN tiles of one CTA with
+// MT = 64 or 128 and BN = 16 .. 128, so that even N = 2048 gives every SM a slice of the weights
+// to stream.  Bound by the weights' read from DRAM; what each CTA moves per
+// 64-deep k-block is (rows of A + BN) x 128 bytes, so A's box holds only the
+// rows that exist (rounded up to 8; the MMA's other rows read whatever follows
+// in shared memory and are never stored).  One TMA per operand fills a stage
+// of `sub` 64-deep blocks: A as {64, rows, sub}, B as {64, BN / 2, 2, sub}
+// whose two halves lie `half` weight rows apart.  The halves hold what the
+// epilogue combines: the gate and up columns (half = bn / 2, the interleave
+// the caller laid the weights out with), the two halves of a head (half =
+// head_dim / 2), or the tile's own halves (half = BN / 2, contiguous).
+// Every element's products are summed in the order of the large-tile kernels
+// and every epilogue step is the same operation, so a row's results do not
+// depend on which kernel computed it.
+constexpr int kFewSmem = 200 * 1024;  // operand ring
+constexpr int kFewStages = 16;
+constexpr int kFewSlack = 128 * 128;  // an A tile's MMA reads MT rows from its slot's start
+
+struct FewArgs {
+  int a_rows;  // rows of A's box
+  int sub;     // 64-deep blocks per stage
+  int stages;
+  int half;    // weight rows between the two halves of a tile
+};
+
+__device__ __forceinline__ void store_f16x8(__half* dst, const float* v, bool& bad) {
+  uint32_t w[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const float a = v[2 * j], b = v[2 * j + 1];
+    bad |= !(fabsf(a) <= 65504.f) || !(fabsf(b) <= 65504.f);
+    __half2 h = __floats2half2_rn(a, b);
+    w[j] = *reinterpret_cast<uint32_t*>(&h);
+  }
+  *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// First weight row of tile nt's two halves: tiles walk the `half` rows of a
+// block in steps of BN / 2, then go to the next block of 2 * half rows.
+template <int BN>
+__device__ __forceinline__ int few_n0(int nt, int half) {
+  const int per = half / (BN / 2);
+  return (nt / per) * 2 * half + (nt % per) * (BN / 2);
+}
+
+template <int BN, int EPI>
+__device__ __forceinline__ void epilogue_few(const KArgs& a, uint32_t trow, int row, bool live, int n0, int half,
+                                             float inv) {
+  const GemmEpilogue& ep = a.ep;
+  constexpr int HB = BN / 2;
+  constexpr int W = HB < 16 ? HB : 16;  // columns of each half per step
+  bool bad = false;
+  const int64_t r = row;
+#pragma unroll 1
+  for (int c = 0; c < HB; c += W) {
+    uint32_t ru[W], rv[W];
+#pragma unroll
+    for (int j = 0; j < W; j += 8) {
+      tmem_ld_32x32b_x8(trow + c + j, ru + j);
+      tmem_ld_32x32b_x8(trow + HB + c + j, rv + j);
+    }
+    tmem_ld_wait();
+    if (live) {
+      float x[W], y[W];
+#pragma unroll
+      for (int j = 0; j < W; ++j) {
+        x[j] = u2f(ru[j]) * inv;
+        y[j] = u2f(rv[j]) * inv;
+      }
+      if constexpr (EPI == EPI_SWIGLU_F16) {
+        __half* o = static_cast<__half*>(ep.out) + r * ep.ldo + (n0 / (2 * half)) * half + n0 % (2 * half) + c;
+#pragma unroll
+        for (int j = 0; j < W; ++j) x[j] = x[j] / (1.0f + expf(-x[j])) * y[j];
+#pragma unroll
+        for (int j = 0; j < W; j += 8) store_f16x8(o + j, x + j, bad);
+        if (ep.lo_off > 0) {
+#pragma unroll
+          for (int j = 0; j < W; ++j) y[j] = x[j] - __half2float(__float2half_rn(x[j]));
+#pragma unroll
+          for (int j = 0; j < W; j += 8) store_f16x8(o + ep.lo_off + j, y + j, bad);
+        }
+      } else if constexpr (EPI == EPI_RESID_F32) {
+        float* o = static_cast<float*>(ep.out) + r * ep.ldo + n0 + c;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          float* v = h ? y : x;
+          float4* o4 = reinterpret_cast<float4*>(o + h * HB);
+#pragma unroll
+          for (int j = 0; j < W / 4; ++j) {
+            float4 t = o4[j];
+            t.x += v[4 * j];
+            t.y += v[4 * j + 1];
+            t.z += v[4 * j + 2];
+            t.w += v[4 * j + 3];
+            o4[j] = t;
+            v[4 * j] = t.x;
+            v[4 * j + 1] = t.y;
+            v[4 * j + 2] = t.z;
+            v[4 * j + 3] = t.w;
+          }
+        }
+        if (ep.xh_out) {
+          float* ss = ep.ss_out + r * ep.ss_parts + (n0 + c) / 16;  // ss_split == 8: one slot per 16 columns
+          if constexpr (BN == 16) {
+            float s = 0.f;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) s = __fmaf_rn(x[j], x[j], s);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) s = __fmaf_rn(y[j], y[j], s);
+            ss[0] = s;
+          } else {
+            ss[0] = sum_sq16(x);
+            ss[HB / 16] = sum_sq16(y);
+          }
+          __half* xh = ep.xh_out + r * ep.ldo + n0 + c;
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            float* v = h ? y : x;
+#pragma unroll
+            for (int j = 0; j < W; j += 8) {
+              if (ep.xh_gain) {
+                const uint4 gv = __ldg(reinterpret_cast<const uint4*>(ep.xh_gain + n0 + c + h * HB + j));
+                const uint32_t gw[4] = {gv.x, gv.y, gv.z, gv.w};
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                  v[j + 2 * i] *= __uint_as_float(gw[i] << 16);
+                  v[j + 2 * i + 1] *= __uint_as_float(gw[i] & 0xFFFF0000u);
+                }
+              }
+              store_f16x8(xh + h * HB + j, v + j, bad);
+            }
+          }
+        }
+      } else {
+        __half* o = static_cast<__half*>(ep.out) + r * ep.ldo + n0 + c;
+        if (EPI == EPI_ROPE_F16 && n0 < ep.rope_cols) {
+          // column n0 + c + j of the head's first half and its partner `half` columns on
+          const int64_t toff = static_cast<int64_t>(ep.positions[row]) * half + n0 % (2 * half) + c;
+#pragma unroll
+          for (int j = 0; j < W; j += 4) {
+            const float4 cs4 = __ldg(reinterpret_cast<const float4*>(ep.rope_cos + toff + j));
+            const float4 sn4 = __ldg(reinterpret_cast<const float4*>(ep.rope_sin + toff + j));
+            const float cs[4] = {cs4.x, cs4.y, cs4.z, cs4.w}, sn[4] = {sn4.x, sn4.y, sn4.z, sn4.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const float a1 = x[j + i], a2 = y[j + i];
+              x[j + i] = a1 * cs[i] - a2 * sn[i];
+              y[j + i] = a2 * cs[i] + a1 * sn[i];
+            }
+          }
+        }
+#pragma unroll
+        for (int j = 0; j < W; j += 8) {
+          store_f16x8(o + j, x + j, bad);
+          store_f16x8(o + half + j, y + j, bad);
+        }
+      }
+    }
+    __syncwarp();
+  }
+  if (bad) set_dev_error(ep.err, DEVERR_FP16_RANGE);
+}
+
+// One stage's MMAs: SUB 64-deep blocks of A (a_blk bytes apart) and B.
+template <int SUB, int BN>
+__device__ __forceinline__ void few_issue(uint32_t d, uint64_t da, uint64_t db, uint32_t a_blk, uint32_t idesc,
+                                          bool first) {
+#pragma unroll
+  for (int sb = 0; sb < SUB; ++sb)
+#pragma unroll
+    for (int k = 0; k < BK / UMMA_K; ++k) {
+      // descriptors count 16-byte units; UMMA_K fp16 = 32 bytes
+      const uint64_t a = da + sb * (a_blk >> 4) + 2 * k, b = db + sb * (BN * 128 >> 4) + 2 * k;
+      if (sb == 0 && k == 0)
+        umma_f16_ss(d, a, b, idesc, !first);
+      else
+        umma_f16_ss_acc(d, a, b, idesc);
+    }
+}
+
+template <int MT, int BN, int EPI>
+__global__ void __launch_bounds__(kThreads, 1)
+    k_gemm_few(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ CUtensorMap tma_b, KArgs args,
+               FewArgs fa) {
+  constexpr int TMEM_COLS = 2 * BN < 32 ? 32 : 2 * BN;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  __shared__ uint64_t full[kFewStages], empty[kFewStages], tfull[2], tempty[2], mma_done;
+  __shared__ uint32_t tmem_slot;
+  __shared__ int abort_word;
+  volatile int* abort_flag = &abort_word;
+
+  const int warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31;
+  int* err = args.ep.err;
+  const uint32_t stages = fa.stages, sub = fa.sub;
+  const uint32_t a_blk = fa.a_rows * 128, a_bytes = sub * a_blk;  // one 64-deep block / one stage of A
+  constexpr uint32_t b_blk = BN * 128;
+  const uint32_t b_bytes = sub * b_blk;
+  uint8_t* sA = smem;
+  uint8_t* sB = smem + stages * a_bytes;
+
+  if (threadIdx.x == 0) {
+    for (uint32_t s = 0; s < stages; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&tfull[i], 1);
+      mbar_init(&tempty[i], 4);
+    }
+    mbar_init(&mma_done, 1);
+    *abort_flag = 0;
+    fence_mbar_init();
+    tma_prefetch_desc(&tma_a);
+    tma_prefetch_desc(&tma_b);
+  }
+  if (warp == 1) {
+    tmem_alloc(&tmem_slot, TMEM_COLS);
+    tmem_relinquish();
+    tc_fence_before();
+  }
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = tmem_slot;
+
+  const int num_m = (args.M + MT - 1) / MT;
+  const int num_tiles = num_m * (args.N / BN);
+  const int kblocks = args.K / (BK * sub);
+  // row tiles fastest: the CTAs that share a weight slice run together
+
+  if (warp == 0) {
+    if (lane == 0) {
+      // ---------------------------------------------------- TMA producer
+      uint32_t issued = 0, s = 0, ph = 1;
+      bool ok = true;
+      for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
+        const int m0 = (tile % num_m) * MT;
+        const int n0 = few_n0<BN>(tile / num_m, fa.half);
+        for (int kb = 0; kb < kblocks; ++kb) {
+          if (!mbar_wait_bounded(&empty[s], ph, abort_flag, err)) {
+            ok = false;
+            break;
+          }
+          mbar_arrive_expect_tx(&full[s], a_bytes + b_bytes);
+          tma_load_4d(sB + s * b_bytes, &tma_b, &full[s], 0, n0, 0, kb * sub);
+          tma_load_3d(sA + s * a_bytes, &tma_a, &full[s], 0, m0, kb * sub);
+          ++issued;
+          if (++s == stages) {
+            s = 0;
+            ph ^= 1;
+          }
+        }
+      }
+      if (!ok) {
+        // drain this thread's copies still in flight before the CTA can exit
+        volatile int never = 0;
+        for (uint32_t i = issued > stages ? issued - stages : 0; i < issued; ++i)
+          mbar_wait_bounded(&full[i % stages], (i / stages) & 1, &never, nullptr, 200000000ull);
+      }
+    }
+  } else if (warp == 1) {
+    // -------------------------------------------------------- MMA issuer
+    // The whole warp walks the stages and one elected lane issues: the
+    // descriptors then stay in uniform registers.  Issue is what a short MMA
+    // waits for: 90 clocks each when formed per MMA in one lane, against the
+    // tensor core's own 39 (128 x 16 x 16) or 23 (64 x 16 x 16).
+    constexpr uint32_t idesc = idesc_f16_f32(MT, BN);
+    const uint64_t da0 = smem_desc_k_sw128(smem_u32(sA)), db0 = smem_desc_k_sw128(smem_u32(sB));
+    const uint32_t tb = __shfl_sync(0xffffffffu, tmem_base, 0);
+    uint32_t s = 0, ph = 0;
+    int acc = 0;
+    uint32_t acc_ph = 0;
+    bool ok = true;
+    for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
+      if (!__all_sync(0xffffffffu, mbar_wait_bounded(&tempty[acc], acc_ph ^ 1, abort_flag, err))) break;
+      tc_fence_after();
+      const uint32_t d_tmem = tb + acc * BN;
+      for (int kb = 0; kb < kblocks; ++kb) {
+        if (!__all_sync(0xffffffffu, mbar_wait_bounded(&full[s], ph, abort_flag, err))) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        const uint64_t da = da0 + s * (a_bytes >> 4), db = db0 + s * (b_bytes >> 4);
+        if (elect_one()) {
+          if (sub == 8)
+            few_issue<8, BN>(d_tmem, da, db, a_blk, idesc, kb == 0);
+          else if (sub == 4)
+            few_issue<4, BN>(d_tmem, da, db, a_blk, idesc, kb == 0);
+          else if (sub == 2)
+            few_issue<2, BN>(d_tmem, da, db, a_blk, idesc, kb == 0);
+          else
+            few_issue<1, BN>(d_tmem, da, db, a_blk, idesc, kb == 0);
+          umma_commit(&empty[s]);
+        }
+        __syncwarp();
+        if (++s == stages) {
+          s = 0;
+          ph ^= 1;
+        }
+      }
+      if (!ok) break;
+      if (elect_one()) umma_commit(&tfull[acc]);
+      __syncwarp();
+      acc ^= 1;
+      if (acc == 0) acc_ph ^= 1;
+    }
+    // every MMA issued above has completed once this arrives
+    if (elect_one()) umma_commit(&mma_done);
+    __syncwarp();
+    volatile int never = 0;
+    mbar_wait_bounded(&mma_done, 0, &never, err);
+  } else {
+    // ------------------------------------------------------------ epilogue
+    const int quarter = warp & 3;  // TMEM lanes this warp may access
+    int acc = 0;
+    uint32_t acc_ph = 0;
+    for (int tile = blockIdx.x; tile < num_tiles; tile += gridDim.x) {
+      const int m0 = (tile % num_m) * MT;
+      const int n0 = few_n0<BN>(tile / num_m, fa.half);
+      // a 64-row accumulator takes the first 16 TMEM lanes of each quarter
+      const int row = m0 + quarter * (MT / 4) + lane;
+      const bool live = (MT == 128 || lane < 16) && row < args.M;
+      if (EPI == EPI_RESID_F32) {
+        if (live)
+          prefetch_l2(static_cast<const float*>(args.ep.out) + static_cast<int64_t>(row) * args.ep.ldo + n0, BN * 4);
+      }
+      const float inv = EPI == EPI_ROPE_F16 || EPI == EPI_SWIGLU_F16 ? row_inv_rms(args.ep, row, live) : 1.f;
+      if (!__all_sync(0xffffffffu, mbar_wait_bounded(&tfull[acc], acc_ph, abort_flag, err))) break;
+      tc_fence_after();
+      if (m0 + quarter * (MT / 4) < args.M)  // warp-uniform: this warp holds at least one live row
+        epilogue_few<BN, EPI>(args, tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + acc * BN, row, live,
+                              n0, fa.half, inv);
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&tempty[acc]);
+      acc ^= 1;
+      if (acc == 0) acc_ph ^= 1;
+    }
+  }
+
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc(tmem_base, TMEM_COLS);
+  }
+}
+
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
   if (!fn) {
@@ -906,7 +1275,133 @@ int dispatch_epi(const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap
   return cudaErrorInvalidValue;
 }
 
+// A of k_gemm_few, [rows, K] as {64, rows, K / 64}: box 64 x box_rows x sub.
+bool make_map_few_a(CUtensorMap* m, const __half* base, int64_t rows, int64_t K, int64_t ld, int box_rows, int sub) {
+  auto fn = encode_fn();
+  if (!fn) return false;
+  cuuint64_t dims[3] = {BK, static_cast<cuuint64_t>(rows), static_cast<cuuint64_t>(K / BK)};
+  cuuint64_t strides[2] = {static_cast<cuuint64_t>(ld * 2), BK * 2};
+  cuuint32_t box[3] = {BK, static_cast<cuuint32_t>(box_rows), static_cast<cuuint32_t>(sub)};
+  cuuint32_t estr[3] = {1, 1, 1};
+  return fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<__half*>(base), dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// B of k_gemm_few, [N, K] as {64, row, half, K / 64}: box 64 x BN / 2 x 2 x sub,
+// the second half `half` rows after the first.
+bool make_map_few_b(CUtensorMap* m, const __half* base, int64_t N, int64_t K, int64_t ld, int bn, int half, int sub) {
+  auto fn = encode_fn();
+  if (!fn) return false;
+  cuuint64_t dims[4] = {BK, static_cast<cuuint64_t>(N - half), 2, static_cast<cuuint64_t>(K / BK)};
+  cuuint64_t strides[3] = {static_cast<cuuint64_t>(ld * 2), static_cast<cuuint64_t>(half * ld * 2), BK * 2};
+  cuuint32_t box[4] = {BK, static_cast<cuuint32_t>(bn / 2), 2, static_cast<cuuint32_t>(sub)};
+  cuuint32_t estr[4] = {1, 1, 1, 1};
+  return fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 4, const_cast<__half*>(base), dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// Weight rows between the two halves of a tile (see k_gemm_few).
+int few_half(int tile, int bn, const GemmEpilogue& ep) {
+  if (ep.kind == EPI_SWIGLU_F16) return bn / 2;
+  if (ep.kind == EPI_ROPE_F16) return ep.head_dim / 2;
+  return tile / 2;
+}
+
+template <int MT, int BN, int EPI>
+int launch_few(const __half* A, int64_t lda, const __half* B, int64_t ldb, const KArgs& a, int bn, int num_sms,
+               cudaStream_t stream) {
+  FewArgs fa;
+  fa.a_rows = a.M < MT ? (a.M + 7) / 8 * 8 : MT;
+  fa.half = few_half(BN, bn, a.ep);
+  // the deepest stage (one TMA per operand) that leaves four of them in the ring
+  const int block = (fa.a_rows + BN) * 128;
+  fa.sub = 1;
+  for (int s = 8; s > 1; s /= 2)
+    if (a.K % (BK * s) == 0 && 4 * s * block <= kFewSmem) {
+      fa.sub = s;
+      break;
+    }
+  fa.stages = kFewSmem / (fa.sub * block);
+  if (fa.stages > kFewStages) fa.stages = kFewStages;
+  CUtensorMap ma, mb;
+  if (!make_map_few_a(&ma, A, a.M, a.K, lda, fa.a_rows, fa.sub) ||
+      !make_map_few_b(&mb, B, a.N, a.K, ldb, BN, fa.half, fa.sub))
+    return cudaErrorInvalidValue;
+  constexpr int SM = 1024 + kFewSmem + kFewSlack;
+  static_assert(SM + 1024 <= 232448, "shared memory per block");
+  cudaError_t e = cudaFuncSetAttribute(k_gemm_few<MT, BN, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, SM);
+  if (e != cudaSuccess) return e;
+  const int tiles = ((a.M + MT - 1) / MT) * (a.N / BN);
+  k_gemm_few<MT, BN, EPI><<<tiles < num_sms ? tiles : num_sms, kThreads, SM, stream>>>(ma, mb, a, fa);
+  return cudaGetLastError();
+}
+
+template <int BN>
+int dispatch_few(const __half* A, int64_t lda, const __half* B, int64_t ldb, const KArgs& a, int bn, int num_sms,
+                 cudaStream_t s) {
+  const bool m64 = a.M <= 64;
+  switch (a.ep.kind) {
+    case EPI_ROPE_F16:
+      return m64 ? launch_few<64, BN, EPI_ROPE_F16>(A, lda, B, ldb, a, bn, num_sms, s)
+                 : launch_few<128, BN, EPI_ROPE_F16>(A, lda, B, ldb, a, bn, num_sms, s);
+    case EPI_SWIGLU_F16:
+      return m64 ? launch_few<64, BN, EPI_SWIGLU_F16>(A, lda, B, ldb, a, bn, num_sms, s)
+                 : launch_few<128, BN, EPI_SWIGLU_F16>(A, lda, B, ldb, a, bn, num_sms, s);
+    case EPI_RESID_F32:
+    case EPI_RESID_ADD:  // the same sum, added by the epilogue threads
+      return m64 ? launch_few<64, BN, EPI_RESID_F32>(A, lda, B, ldb, a, bn, num_sms, s)
+                 : launch_few<128, BN, EPI_RESID_F32>(A, lda, B, ldb, a, bn, num_sms, s);
+  }
+  return cudaErrorInvalidValue;
+}
+
 }  // namespace
+
+// The kernels' times are estimated from what bounds them, in SM clocks, and the
+// smallest wins.  Per 64-deep k-block a CTA takes the larger of its MMAs (45
+// clocks each at 64 rows, where issue bounds them; 45 to 64 at 128 rows) and of
+// its operands' arrival (60 bytes per clock); the large tiles measure 720
+// (128 x 256), 540 (128 x 128) and 660 (CTA pair).  An epilogue column costs 100
+// clocks where the threads add to the residual, 50 for SwiGLU, 40 for RoPE and 22 for the
+// TMA add; a tile's epilogue runs beside the next tile's main loop.  Measured
+// (us, weights from DRAM; with about 7 us of launch and event overhead):
+//   M     N      K      large   16     32     64     128
+//   24    2048   8192   55.6    18.5   21.3   23.0   32.1
+//   300   2048   8192   59.3    71.9   52.1   34.2   46.3
+//   1000  2048   8192   55.3    157    95.2   56.6   48.8
+//   24    28672  4096   53.3    67.1   48.5   44.7   48.9
+//   500   28672  4096   96.5    516    266    146    113
+int gemm_few_tile(int M, int N, int K, int bn, bool pair, const GemmEpilogue& ep, int num_sms) {
+  if (M > kFewRowsMax) return 0;
+  int epi = 0, epi_large = 0;  // clocks per column
+  switch (ep.kind) {
+    case EPI_ROPE_F16: epi = epi_large = 40; break;
+    case EPI_SWIGLU_F16: epi = epi_large = 50; break;
+    case EPI_RESID_F32: epi = epi_large = 100; break;
+    case EPI_RESID_ADD: epi = 100, epi_large = 22; break;
+    default: return 0;  // the plain and argmax epilogues
+  }
+  const int64_t kblocks = K / BK;
+  auto cost = [&](int64_t tiles, int64_t units, int64_t per_kblock, int64_t epilogue) {
+    const int64_t waves = (tiles + units - 1) / units, main = kblocks * per_kblock;
+    return main + (waves - 1) * std::max(main, epilogue) + epilogue;
+  };
+  const int64_t m128 = (M + 127) / 128;
+  int64_t best = pair && K % (BK * CfgPair::SUB) == 0
+                     ? cost((M + 255) / 256 * (N / 256), num_sms / 2, 660, 256 * epi_large)
+                     : cost(m128 * (N / bn), num_sms, bn == 256 ? 720 : 540, bn * epi_large);
+  int tile = 0;
+  const int a_rows = M < 128 ? (M + 7) / 8 * 8 : 128;
+  for (int t = 16; t <= 128; t *= 2) {
+    if (t / 2 > few_half(t, bn, ep)) break;  // a tile's halves lie within a gate / up block or a head
+    const int64_t mma = M <= 64 ? std::max(180, 2 * t) : 160 + t * 3 / 4;
+    const int64_t c = cost(m128 * (N / t), num_sms, std::max<int64_t>(mma, (a_rows + t) * 128 / 60), t * epi);
+    if (c < best) best = c, tile = t;
+  }
+  return tile;
+}
 
 int gemm_f16_tcgen05(const __half* A, int64_t lda, const __half* B, int64_t ldb, int M, int N, int K, int bn,
                      bool pair, const GemmEpilogue& ep, int num_sms, cudaStream_t stream) {
@@ -924,6 +1419,13 @@ int gemm_f16_tcgen05(const __half* A, int64_t lda, const __half* B, int64_t ldb,
   if (ep.kind == EPI_RESID_ADD &&
       (!ep.out || (reinterpret_cast<uintptr_t>(ep.out) & 15) || (ep.ldo * 4) % 16 != 0 || ep.xh_out))
     return cudaErrorInvalidValue;
+  KArgs a{M, N, K, ep};
+  switch (gemm_few_tile(M, N, K, bn, pair, ep, num_sms)) {
+    case 16: return dispatch_few<16>(A, lda, B, ldb, a, bn, num_sms, stream);
+    case 32: return dispatch_few<32>(A, lda, B, ldb, a, bn, num_sms, stream);
+    case 64: return dispatch_few<64>(A, lda, B, ldb, a, bn, num_sms, stream);
+    case 128: return dispatch_few<128>(A, lda, B, ldb, a, bn, num_sms, stream);
+  }
   CUtensorMap ma, mb, mc;
   if (!make_map(&ma, A, M, K, lda, BM) || !make_map(&mb, B, N, K, ldb, pair ? 128 : bn)) return cudaErrorInvalidValue;
   if (ep.kind == EPI_RESID_ADD) {
@@ -931,7 +1433,6 @@ int gemm_f16_tcgen05(const __half* A, int64_t lda, const __half* B, int64_t ldb,
   } else {
     mc = ma;  // unused by the other epilogues
   }
-  KArgs a{M, N, K, ep};
   if (pair) return dispatch_pair(ma, mb, mc, a, num_sms, stream);
   return bn == 256 ? dispatch_epi<256>(ma, mb, mc, a, num_sms, stream)
                    : dispatch_epi<128>(ma, mb, mc, a, num_sms, stream);

@@ -34,9 +34,11 @@ struct GemmEpilogue {
   //    rsqrt(sum(row_ss[row][0..ss_parts)) / d_norm + eps) before the epilogue;
   //  - producer (RESID): also write the new residual as fp16 (xh_out), times
   //    the next norm's gain (xh_gain, bf16 [N]) when given, and the unscaled
-  //    residual's per-128-column sums of squares (ss_out [row][n / 128]).
+  //    residual's per-128-column sums of squares (ss_out [row][n / 128]), or
+  //    with ss_split == 8 their eight 16-column terms (ss_out [row][n / 16]).
   const float* row_ss = nullptr;
-  int ss_parts = 0;
+  int ss_parts = 0;                    // slots per row
+  int ss_split = 1;                    // slots per 128 columns: 1, or 8 where gemm_few_tile says so
   float d_norm = 1.f;
   float eps = 0.f;
   __half* xh_out = nullptr;
@@ -54,6 +56,11 @@ struct GemmEpilogue {
 // Requires K % 64 == 0, N % bn == 0, bn in {128, 256}, 16-byte aligned rows.
 // pair: 256 x 256 tiles on clusters of two CTAs (cta_group::2); needs bn == 256.
 // Returns 0 or a cudaError_t value.
+constexpr int kFewRowsMax = 16384;  // rows that the few-rows kernel takes at most
+// Tile width of the few-rows kernel that gemm_f16_tcgen05 takes for this product
+// (16, 32, 64 or 128), or 0 for the large-tile kernels.  A product with ss_out
+// needs ss_split = 8 where this is not 0, and 1 where it is.
+int gemm_few_tile(int M, int N, int K, int bn, bool pair, const GemmEpilogue& ep, int num_sms);
 int gemm_f16_tcgen05(const __half* A, int64_t lda, const __half* B, int64_t ldb, int M, int N, int K, int bn,
                      bool pair, const GemmEpilogue& ep, int num_sms, cudaStream_t stream);
 

@@ -248,6 +248,55 @@ def test_gemm_cta_pair_rope(ctx):
     _close(_np64(out), ref, 2e-3, 2e-3 * np.sqrt(K) * 0.05, "pair rope")
 
 
+@pytest.mark.parametrize("epi,N,K,bn,hd", [(1, 768, 192, 256, 64), (1, 512, 512, 256, 128), (1, 384, 128, 128, 32),
+                                           (2, 256, 1024, 256, 0), (2, 384, 64, 128, 0), (5, 256, 512, 256, 0),
+                                           (3, 512, 256, 256, 0), (3, 1024, 128, 128, 0)])
+def test_gemm_few_rows_matches_large_tiles(ctx, epi, N, K, bn, hd):
+    """Products with few rows take narrow tiles: the oracle's product within the
+    output's rounding, and bit for bit the rows that a product with more rows than
+    the narrow tiles are ever used for gives."""
+    rng = np.random.default_rng(N + K + epi)
+    big = 16384 + 40
+    A = rng.standard_normal((big, K)).astype(np.float16)
+    B = (rng.standard_normal((N, K)) * 0.05).astype(np.float16)
+    width = N // 2 if epi == 3 else N
+    R = rng.standard_normal((big, width)).astype(np.float32)
+    pos = rng.integers(0, 300, big).astype(np.int32)
+    cs = torch.zeros((300, max(hd, 32) // 2), dtype=torch.float32, device="cuda")
+    sn = torch.zeros_like(cs)
+    ctx.op_rope_table(cs.data_ptr(), sn.data_ptr(), 300, max(hd, 32), 1.0e4)
+    rope_cols = 2 * N // 3 // max(hd, 1) * hd
+    dA, dB, dP = _h(A), _h(B), _h(pos)
+
+    def run(M):
+        out = _h(R) if epi in (2, 5) else torch.zeros((big, width), dtype=torch.float16, device="cuda")
+        ctx.op_gemm(dA.data_ptr(), K, dB.data_ptr(), K, M, N, K, bn, epi, out.data_ptr(), width, dP.data_ptr(),
+                    cs.data_ptr(), sn.data_ptr(), rope_cols, hd)
+        torch.cuda.synchronize()
+        return out
+
+    large = run(big)
+    rows = [1, 8, 63, 64, 65, 127, 128, 129, 300, 1000]
+    y = A[:rows[-1]].astype(np.float64) @ B.astype(np.float64).T
+    if epi == 1:
+        qk = tf.rope(y[:, :rope_cols].reshape(len(y), -1, hd), pos[:len(y)], 1.0e4).reshape(len(y), rope_cols)
+        ref = np.concatenate([qk, y[:, rope_cols:]], axis=1)
+    elif epi == 3:
+        t = y.reshape(len(y), -1, 2, bn // 2)
+        ref = (tf.silu(t[:, :, 0]) * t[:, :, 1]).reshape(len(y), -1)
+    else:
+        ref = R[:len(y)].astype(np.float64) + y
+    before = _h(R) if epi in (2, 5) else torch.zeros_like(large)
+    for M in rows:
+        out = run(M)
+        assert torch.equal(out[:M], large[:M]), f"epilogue {epi}, {M} rows"
+        assert torch.equal(out[M:], before[M:]), f"epilogue {epi}, {M} rows: a row past the product was written"
+    if epi in (2, 5):   # fp32: the bounds of test_gemm_residual_add
+        _close(_np64(out[:rows[-1]]), ref, 1e-5, 2e-6 * np.sqrt(K), f"few rows epilogue {epi}")
+    else:               # fp16: the bounds of test_gemm_swiglu and test_gemm_qkv_rope
+        _close(_np64(out[:rows[-1]]), ref, 3e-3, 3e-3 * max(np.sqrt(K) * 0.05, K * 0.0025), f"few rows epilogue {epi}")
+
+
 def test_attention_tcgen05_matches_mma_sync_kernel(ctx):
     """The tcgen05 and the mma.sync attention kernels agree on a GQA batch with a
     shared prefix (both also match the oracle above)."""
