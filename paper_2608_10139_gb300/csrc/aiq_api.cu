@@ -870,7 +870,8 @@ aiq_status prefill_phase(aiq_ctx* c, const TableD& t, ModelD& m, const aiq_selec
   }
   AIQ_TRY(ensure_rope(c, m, static_cast<int>(P + max_len + (gp ? gp->max_new : 0))));
   PrefillBufs pb;
-  AIQ_TRY(prefill_bufs(c, m, std::max<int64_t>(Bmax, 64), Rmax, &pb));
+  // a chunk of rows with empty text has more rows than tokens
+  AIQ_TRY(prefill_bufs(c, m, std::max<int64_t>({Bmax, Rmax, 64}), Rmax, &pb));
   const aiq_model_config& g = m.cfg;
   const int64_t ldkv = 2 * static_cast<int64_t>(g.n_kv_heads) * g.head_dim;
   DecodeBufs db{};

@@ -231,6 +231,32 @@ def test_rows_with_empty_text(ctx):
     ctx.free_model(mh)
 
 
+def test_more_rows_than_tokens():
+    """A chunk whose rows are all but a few without text has more rows than
+    tokens: the per-row buffers are sized for the rows."""
+    from helpers import gpu_ctx
+    w = synth.C1_TINY
+    q = synth.make_inputs(w)
+    n = q.table.n_rows
+    lens = np.zeros(n, np.int64)
+    lens[[3, 200, 311]] = [2, 5, 1]
+    offsets = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    table = synth.Table(n, q.table.cols, offsets, np.arange(8, dtype=np.int32))
+    c = gpu_ctx()   # a context of its own: no workspace left by larger queries
+    try:
+        mh, W = _model(c, w.model, w.weight_seed)
+        t = _load(c, table)
+        r = c.run_select(t, mh, [], q.prefix, w.label_ids, agg=w.agg, flags=aiq.FLAG_LOGITS)
+        o = oq.run_select(table, q.prefix, [], w.label_ids, w.agg, tf.Model(w.model, W, True))
+        assert np.array_equal(r.cand_row_ids, o.cand_rows) and r.n_candidates == n
+        compare_logits(r.label_logits, o.logits, "more rows than tokens")
+        assert np.all(r.label_logits[lens == 0] == r.label_logits[0])
+        g = c.run_transform(t, mh, [], q.prefix, 3)
+        assert np.all(g.gen_tokens[lens == 0] == g.gen_tokens[0])
+    finally:
+        c.close()
+
+
 def test_degenerate_queries(ctx):
     w = synth.C1_TINY
     q = synth.make_inputs(w)
