@@ -173,7 +173,8 @@ struct aiq_ctx {
   int device = 0;
   int num_sms = 0;
   cudaStream_t stream = nullptr;
-  int* d_err = nullptr;
+  volatile int* h_err = nullptr;  // the kernels' error word, in mapped pinned host memory
+  int* d_err = nullptr;           // its device address
   int64_t* h_pin = nullptr;  // pinned staging for control scalars
   size_t bytes_max = SIZE_MAX;
   size_t bytes_used = 0;
@@ -254,11 +255,11 @@ aiq_status sync_and_check(aiq_ctx* c) {
   }
   CUDA_TRY(cudaGetLastError());
   CUDA_TRY(cudaStreamSynchronize(c->stream));
-  int err = 0;
-  CUDA_TRY(cudaMemcpy(&err, c->d_err, sizeof(int), cudaMemcpyDeviceToHost));
+  // The stream has finished, so the word is final.  Reading it back with a
+  // blocking copy cost 12 us a call, more than most step-level kernels.
+  const int err = *c->h_err;
   if (err) {
-    // cleared on the context's stream, ordered before the next call's kernels
-    CUDA_TRY(cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream));
+    *c->h_err = 0;  // no kernel is in flight
     if (err & (DEVERR_DUP_BUILD_KEY | DEVERR_SENTINEL_KEY))
       return fail(AIQ_ERR_INVALID_ARG, "join build keys must be unique and differ from INT64_MIN");
     if (err & DEVERR_HASH_FULL) return fail(AIQ_ERR_CAPACITY, "hash table probe sequence exhausted");
@@ -352,16 +353,27 @@ aiq_status gemm(aiq_ctx* c, const char* name, const __half* A, int64_t lda, cons
   return AIQ_OK;
 }
 
-// Causal GQA attention over a packed chunk: the work list, then the tcgen05
-// kernel (head_dim 64/128) or the mma.sync kernel.
+// Query tokens per attention work item: the tcgen05 kernel's (head_dim 64/128)
+// or the mma.sync kernel's.
+int attention_tile_tokens(const aiq_ctx* c, int Hq, int Hkv, int hd) {
+  return c->attention_tc && attention_tc_supported(hd, Hq, Hkv) ? attention_tc_tile_tokens(Hq, Hkv) : 64;
+}
+
+// The work list of a packed chunk, the same for each of its layers.
+void attention_tiles(aiq_ctx* c, int64_t n_seqs, const int32_t* seq_start, int32_t* tile_seq, int32_t* tile_q0,
+                     int32_t* n_tiles, int Hq, int Hkv, int hd) {
+  launch_attn_tiles(seq_start, static_cast<int32_t>(n_seqs), attention_tile_tokens(c, Hq, Hkv, hd), tile_seq, tile_q0,
+                    n_tiles, c->stream);
+  counted(c, 1);
+}
+
+// Causal GQA attention over a packed chunk whose work list attention_tiles made.
 aiq_status attention(aiq_ctx* c, const __half* qkv, int64_t T, int64_t n_seqs, const int32_t* seq_start,
-                     int32_t* tile_seq, int32_t* tile_q0, int32_t* n_tiles, int Hq, int Hkv, int hd,
+                     const int32_t* tile_seq, const int32_t* tile_q0, const int32_t* n_tiles, int Hq, int Hkv, int hd,
                      const __half* pkv, int P, __half* out) {
   const bool tc = c->attention_tc && attention_tc_supported(hd, Hq, Hkv);
-  const int tq = tc ? attention_tc_tile_tokens(Hq, Hkv) : 64;
+  const int tq = attention_tile_tokens(c, Hq, Hkv, hd);
   const int n_tiles_max = static_cast<int>((T + tq - 1) / tq + n_seqs);
-  launch_attn_tiles(seq_start, static_cast<int32_t>(n_seqs), tq, tile_seq, tile_q0, n_tiles, c->stream);
-  counted(c, 1);
   ProfScope p(c, "attention", 0, 0);
   if (tc) {
     const int e = launch_attention_tc(qkv, T, seq_start, tile_seq, tile_q0, n_tiles_max, n_tiles, Hq, Hkv, hd, pkv, P,
@@ -532,6 +544,7 @@ aiq_status run_layers(aiq_ctx* c, ModelD& m, const PrefillBufs& b, int64_t T, in
     launch_embed(b.tok, T, m.embed, d, b.resid, b.xn, b.ss_attn, m.layers[0].attn_norm, c->d_err, c->stream);
     counted(c, T > 0);
   }
+  attention_tiles(c, n_seqs, b.seq_start, b.tile_seq, b.tile_q0, b.n_tiles, Hq, Hkv, hd);
   for (int l = 0; l < g.n_layers; ++l) {
     const LayerD& L = m.layers[l];
     GemmEpilogue e1;
@@ -1505,14 +1518,18 @@ aiq_status aiq_init(int device, aiq_ctx** out) {
   c->num_sms = prop.multiProcessorCount;
   if (const char* cap = std::getenv("AIQ_DEVICE_BYTES_MAX")) c->bytes_max = std::strtoull(cap, nullptr, 10);
   cudaError_t e = cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking);
-  if (e == cudaSuccess) e = cudaMalloc(&c->d_err, sizeof(int));
-  if (e == cudaSuccess) e = cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+  void* word = nullptr;
+  if (e == cudaSuccess) e = cudaHostAlloc(&word, sizeof(int), cudaHostAllocMapped);
+  if (e == cudaSuccess) {
+    c->h_err = static_cast<volatile int*>(word);
+    *c->h_err = 0;
+    e = cudaHostGetDevicePointer(reinterpret_cast<void**>(&c->d_err), word, 0);
+  }
   if (e == cudaSuccess) e = cudaMallocHost(&c->h_pin, 64 * sizeof(int64_t));
   if (e != cudaSuccess) {
     cudaGetLastError();
     if (c->h_pin) cudaFreeHost(c->h_pin);
-    if (c->d_err) cudaFree(c->d_err);
+    if (c->h_err) cudaFreeHost(const_cast<int*>(c->h_err));
     if (c->stream) cudaStreamDestroy(c->stream);
     delete c;
     return fail(AIQ_ERR_CUDA, std::string("context setup: ") + cudaGetErrorString(e));
@@ -1534,7 +1551,7 @@ void aiq_shutdown(aiq_ctx* c) {
     cudaEventDestroy(r.b);
   }
   for (auto e : c->ev_pool) cudaEventDestroy(e);
-  cudaFree(c->d_err);
+  cudaFreeHost(const_cast<int*>(c->h_err));
   cudaFreeHost(c->h_pin);
   cudaStreamDestroy(c->stream);
   delete c;
@@ -1746,10 +1763,8 @@ aiq_status aiq_load_model(aiq_ctx* c, const aiq_model_config* cfg, const void* c
   cudaError_t e = cudaStreamSynchronize(c->stream);
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) return fail_model(fail(AIQ_ERR_CUDA, std::string("model upload: ") + cudaGetErrorString(e)));
-  int err = 0;
-  cudaMemcpy(&err, c->d_err, sizeof(int), cudaMemcpyDeviceToHost);
-  if (err) {
-    cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream);
+  if (*c->h_err) {
+    *c->h_err = 0;
     return fail_model(fail(AIQ_ERR_UNSUPPORTED, "a linear weight is outside the fp16 range"));
   }
 #undef M_TRY
@@ -1960,6 +1975,7 @@ aiq_status aiq_op_attention(aiq_ctx* c, const void* qkv, int64_t T, const int32_
   AIQ_TRY(ws(c, "op.tile_q0", cap, &tile_q0));
   AIQ_TRY(ws(c, "op.n_tiles", 1, &n_tiles));
   if (P < 0 || (P > 0 && !prefix_kv)) return fail(AIQ_ERR_INVALID_ARG, "bad prefix");
+  attention_tiles(c, n_seqs, seq_start, tile_seq, tile_q0, n_tiles, Hq, Hkv, hd);
   AIQ_TRY(attention(c, static_cast<const __half*>(qkv), T, n_seqs, seq_start, tile_seq, tile_q0, n_tiles, Hq, Hkv, hd,
                     static_cast<const __half*>(prefix_kv), P, static_cast<__half*>(out)));
   const aiq_status st = sync_and_check(c);

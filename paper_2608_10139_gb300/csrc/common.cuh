@@ -21,8 +21,10 @@ enum : int {
   DEVERR_BOUNDS = 1 << 5,        // an index failed its bounds check
 };
 
+// The word is host memory that the device maps (read by the host once the
+// stream has finished, with no copy), hence the system scope.
 __device__ __forceinline__ void set_dev_error(int* err, int bits) {
-  if (err) atomicOr(err, bits);
+  if (err) atomicOr_system(err, bits);
 }
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
