@@ -6,39 +6,41 @@
 // keys of the shared prompt prefix (computed once per query, in prefix_kv)
 // come first, then the sequence's own keys up to the tile's last token.
 //
-//   warp 0    TMA: the Q tile (3-D box hd x heads x tokens) into one of two
-//             slots, then K and V blocks of 64 keys into two separate rings of
-//             NKV slots (128-byte swizzle).  A K slot is free once the S MMA
-//             that read it has completed, a V slot once the PV MMA that read
-//             it has, so a block's loads are issued NKV blocks ahead.  The
-//             same thread publishes each item's bounds (sequence start and
-//             length, first token, key/value head) in a four-slot shared
-//             ring, so the softmax warps never wait on global loads between
-//             items.
-//   warp 1    tcgen05.mma: S = Q K^T into one of two 64-column TMEM score
-//             buffers, and O += P V into the item's TMEM output accumulator,
-//             with P read from TMEM (it overwrites its own scores) and V read
-//             as an MN-major operand straight from its TMA tile.
-//   warps 2-5 one query row per thread: read its 64 scores with tcgen05.ld,
-//             apply the causal / prefix / length mask, keep the running max
-//             (the output is rescaled only when the max grows by more than
-//             2^8, so P never exceeds 256), and write exp2(s - max) as fp16
-//             pairs back over the first 32 columns of the same score buffer
-//             with tcgen05.st; an item's output is divided by the row sum and
-//             stored after the next item's first block: through a shared
-//             staging tile and one TMA store when all the tile's tokens
-//             belong to its sequence, row by row otherwise.
+//   warp 0    TMA: the Q tile (3-D box hd x heads x tokens), then K and V blocks
+//             of 64 keys into two rings (128-byte swizzle).  A K slot is free
+//             once the S MMA that read it has completed, a V slot once the PV MMA
+//             that read it has.  The same thread publishes each item's bounds in a
+//             four-slot shared ring, an item ahead of its loads, so that no role
+//             waits on global loads between items.
+//   warp 1    tcgen05.mma: S = Q K^T into a 64-column TMEM score buffer, and
+//             O += P V into the output accumulator, with P read from TMEM (it
+//             overwrites its own scores) and V read as an MN-major operand
+//             straight from its TMA tile.
+//   warps 2-5 one query row per thread: read its 64 scores with tcgen05.ld, 32
+//             at a time, apply the causal / prefix / length mask, and write
+//             exp2(s - max) as fp16 pairs back over the first 32 columns of the
+//             same score buffer with tcgen05.st.  The running max is raised
+//             (and the output rescaled) only when it grows by more than 2^8, so
+//             P never exceeds 256: the exponents are formed with the old max
+//             while the new one is found, and formed again in the rare block
+//             that raises it.  An item's output is divided by the row sum and
+//             stored by its threads in 32-byte pieces, live rows only.
 //
-// Ordering without extra waits: the MMA warp issues S(g+1) before PV(g), and
-// tcgen05 MMAs of one thread run in issue order, so S(g+2), which reuses the
-// score buffer of block g, only starts after PV(g) has read P(g).  The commit
-// that signals S(g) tracks every earlier MMA of the thread, so a softmax
-// thread that has seen S(g) complete knows PV(g-2) has too: its parity waits
-// on the two PV barriers can never be a full phase behind.  The softmax warps
-// signal P on one barrier per score buffer: S(g+1) is ready before PV(g) is
-// issued, so one warp may finish block g+1 while another still writes P(g),
-// and on a single barrier its second arrival would complete block g's phase
-// early; a warp cannot reach block g+2 before PV(g), so two barriers suffice.
+// Latency bounds it: a block costs a softmax warp some 500 issue clocks, and the
+// way from its P to its next scores (two barriers, PV and S) takes as long.  So
+// several CTAs share an SM, each SM sub-partition switching between their softmax
+// warps, and every wait that can be taken before P arrives is: the MMA warp has
+// the next block's K, V and Q in hand when P comes, and issues PV(g) and S(g+1)
+// together.
+//
+// Ordering: tcgen05 MMAs of one thread run in issue order.  With one score
+// buffer S(g+1) is issued after PV(g), which reads P(g) from that buffer; a
+// softmax thread that has seen S(g) complete therefore knows that PV(g-1) has,
+// too.  With two buffers S(g+1) is issued before PV(g) inside an item, S(g+2)
+// after it, and seeing S(g) implies PV(g-2); the thread waits for PV(g-1) before
+// it rescales the output.  Either way its parity waits on the two PV barriers
+// can never be a full phase behind.  P is signalled on one barrier per score
+// buffer: a warp cannot signal P(g + NS) before PV(g) has been issued.
 // Work items are persistent per CTA; every wait is bounded.
 #include <cudaTypedefs.h>
 
@@ -51,29 +53,39 @@ namespace {
 constexpr int kThreadsTC = 192;
 constexpr int kKeys = 64;  // keys per block
 
+// Three CTAs per SM at head_dim 64, two at 128 (TMEM holds 512 columns).  Measured
+// at 970 rows of the select workload's text (128,867 tokens, 64 prefix keys, 32/8
+// heads, head_dim 64): 387 us, four CTAs with one Q slot and two K slots 399,
+// two with four K and V slots 455, and 445 for two CTAs of 192 threads that double
+// the score buffers and accumulators and store through shared memory; at head_dim
+// 128 (150 rows, 34,972 tokens, 128 prefix keys): 222 us, 226 with three K slots,
+// and 353 for one such CTA per SM.  A CTA of two tiles that share K and V took 427
+// and 346 us: its one MMA warp then serves both tiles' hand-offs in turn.
 template <int HD>
 struct ACfg {
   static constexpr int NC = HD / 64;             // 64-column sub-tiles of one head
-  static constexpr int NKV = 3;                  // slots of the K ring and of the V ring
+  static constexpr int CTAS = HD == 64 ? 3 : 2;  // per SM
+  static constexpr int NQ = HD == 64 ? 2 : 1;    // Q slots
+  static constexpr int NK = HD == 64 ? 3 : 2;    // slots of the K ring
+  static constexpr int NV = 2;                   // slots of the V ring
+  static constexpr int NS = HD == 64 ? 1 : 2;    // score buffers
   static constexpr int Q_BYTES = 128 * HD * 2;   // 128 rows
   static constexpr int SUB = 64 * 128;           // one [64 x 64] fp16 sub-tile
   static constexpr int K_BYTES = NC * SUB;
-  static constexpr int OFF_Q = 0;                // two slots
-  static constexpr int OFF_K = OFF_Q + 2 * Q_BYTES;
-  static constexpr int OFF_V = OFF_K + NKV * K_BYTES;
-  static constexpr int OFF_OUT = OFF_V + NKV * K_BYTES;  // output staging tile (TMA store source)
-  static constexpr int OFF_INFO = OFF_OUT + Q_BYTES;     // item bounds ring, 4 x int4
+  static constexpr int OFF_Q = 0;
+  static constexpr int OFF_K = OFF_Q + NQ * Q_BYTES;
+  static constexpr int OFF_V = OFF_K + NK * K_BYTES;
+  static constexpr int OFF_INFO = OFF_V + NV * K_BYTES;  // item bounds ring, 4 x int4
   static constexpr int OFF_BAR = OFF_INFO + 4 * 16;
-  static constexpr int N_BARS = 4 + 4 * NKV + 2 + 2 + 2 + 2 + 1 + 4 + 4 + 2;
-  static constexpr int SMEM = 1024 + OFF_BAR + N_BARS * 8 + 16;
-  // two 64-column score buffers, then two HD-column output accumulators (one
-  // per alternating work item), rounded up to a power of two
-  static constexpr int TMEM_COLS = HD == 64 ? 256 : 512;
-  static constexpr int O_COL = 128;
+  static constexpr int N_BARS = 2 * NQ + 2 * NK + 2 * NV + 2 + 2 + 2 + 1 + 1 + 8;
+  static constexpr int SMEM = OFF_BAR + N_BARS * 8 + 16;
+  // the score buffers, then the output accumulator
+  static constexpr int TMEM_COLS = HD == 64 ? 128 : 256;
+  static constexpr int O_COL = NS * kKeys;
+  static_assert(O_COL + HD <= TMEM_COLS && CTAS * TMEM_COLS <= 512, "TMEM columns");
+  // each CTA also keeps 1 KB of the SM's shared memory
+  static_assert(CTAS * (SMEM + 1024) <= 233472, "shared memory per SM");
 };
-// two CTAs per SM at HD = 64 (each also keeps 1 KB of the SM's shared memory)
-static_assert(2 * (ACfg<64>::SMEM + 1024) <= 233472, "HD = 64 tiles must fit two CTAs per SM");
-static_assert(ACfg<128>::SMEM <= 232448, "HD = 128 tiles must fit one CTA");
 
 struct AttnArgs {
   const int32_t* seq_start;
@@ -85,18 +97,6 @@ struct AttnArgs {
   __half* out;
   int* err;
 };
-
-__device__ __forceinline__ void load2x32_f(uint32_t ta, uint32_t tb, float* va, float* vb) {
-  uint32_t ra[32], rb[32];
-  tmem_ld_32x32b_x32(ta, ra);
-  tmem_ld_32x32b_x32(tb, rb);
-  tmem_ld_wait();
-#pragma unroll
-  for (int j = 0; j < 32; ++j) {
-    va[j] = __uint_as_float(ra[j]);
-    vb[j] = __uint_as_float(rb[j]);
-  }
-}
 
 // 2^x with the SFU's approximation (relative error ~2^-22, flushes
 // subnormals): plenty for probabilities that are rounded to fp16 next.
@@ -125,11 +125,10 @@ __device__ __forceinline__ float2 fadd2(float2 a, float2 b) {
   return bits_f2(r);
 }
 
-// Shared -> global tile copy by the TMA unit (3-D box), in a bulk async-group.
-__device__ __forceinline__ void tma_store_3d(const CUtensorMap* map, const void* smem_src, int x, int y, int z) {
-  asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.tile.bulk_group [%0, {%1, %2, %3}], [%4];" ::"l"(
-                   reinterpret_cast<uint64_t>(map)),
-               "r"(x), "r"(y), "r"(z), "r"(smem_u32(smem_src))
+// 32 bytes to global memory in one instruction (32-byte aligned).
+__device__ __forceinline__ void st_global_v8(void* p, const uint32_t* r) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(r[0]), "r"(r[1]), "r"(r[2]),
+               "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
                : "memory");
 }
 
@@ -156,68 +155,105 @@ __device__ __forceinline__ void umma_f16_ts(uint32_t d_tmem, uint32_t a_tmem, ui
       : "memory");
 }
 
+// 32 scores of this thread's row from TMEM, those of keys >= lim masked.
+__device__ __forceinline__ void load_scores(uint32_t taddr, float* v, bool mask, int lim) {
+  uint32_t r[32];
+  tmem_ld_32x32b_x32(taddr, r);
+  tmem_ld_wait();
+#pragma unroll
+  for (int c = 0; c < 32; ++c) v[c] = __uint_as_float(r[c]);
+  if (mask) {
+    const uint32_t visible = lim >= 32 ? ~0u : (lim <= 0 ? 0u : (1u << lim) - 1u);
+#pragma unroll
+    for (int c = 0; c < 32; ++c) v[c] = (visible >> c) & 1u ? v[c] : -INFINITY;
+  }
+}
+
+// Eight independent partial maxima keep the chain short.
+__device__ __forceinline__ float max32(const float* v) {
+  float pm[8];
+#pragma unroll
+  for (int c = 0; c < 8; ++c) pm[c] = v[c];
+#pragma unroll
+  for (int c = 8; c < 32; ++c) pm[c & 7] = fmaxf(pm[c & 7], v[c]);
+  return fmaxf(fmaxf(fmaxf(pm[0], pm[1]), fmaxf(pm[2], pm[3])), fmaxf(fmaxf(pm[4], pm[5]), fmaxf(pm[6], pm[7])));
+}
+
+// P of 32 scores: exp2(scale v - m) as fp16 pairs, added (in fp32) to ps.
+__device__ __forceinline__ void exp32(const float* v, float scale_log2, float m, uint32_t* pk, float2* ps) {
+  const float2 sc2 = make_float2(scale_log2, scale_log2), nm2 = make_float2(-m, -m);
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    const float2 x = ffma2(make_float2(v[2 * i], v[2 * i + 1]), sc2, nm2);
+    const float2 p = make_float2(ex2_approx(x.x), ex2_approx(x.y));
+    ps[i & 3] = fadd2(ps[i & 3], p);
+    __half2 h = __floats2half2_rn(p.x, p.y);
+    pk[i] = *reinterpret_cast<uint32_t*>(&h);
+  }
+}
+
 template <int HD>
-__global__ void __launch_bounds__(kThreadsTC, HD == 64 ? 2 : 1)
+__global__ void __launch_bounds__(kThreadsTC, ACfg<HD>::CTAS)
     k_attention_tc(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_kv,
-                   const __grid_constant__ CUtensorMap tm_pre, const __grid_constant__ CUtensorMap tm_out, AttnArgs a) {
+                   const __grid_constant__ CUtensorMap tm_pre, AttnArgs a) {
   using C = ACfg<HD>;
-  constexpr int NKV = C::NKV;
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::OFF_BAR);
-  uint64_t* q_full = bars + 0;             // [2]
-  uint64_t* q_empty = bars + 2;            // [2]: the item's S MMAs have completed
-  uint64_t* k_full = bars + 4;             // [NKV]
-  uint64_t* k_empty = k_full + NKV;        // [NKV]: the S MMA of the block has completed
-  uint64_t* v_full = k_empty + NKV;        // [NKV]
-  uint64_t* v_empty = v_full + NKV;        // [NKV]: the PV MMA of the block has completed
-  uint64_t* s_full = v_empty + NKV;        // [2]
-  uint64_t* p_full = s_full + 2;           // [2]: P of block g written over its scores (score buffer g & 1)
+  constexpr int NQ = C::NQ, NK = C::NK, NV = C::NV, NS = C::NS;
+  extern __shared__ __align__(1024) uint8_t smem[];  // swizzled tiles want 1024-byte alignment
+  uint64_t* q_full = reinterpret_cast<uint64_t*>(smem + C::OFF_BAR);  // [NQ]
+  uint64_t* q_empty = q_full + C::NQ;      // [NQ]: the item's S MMAs have completed
+  uint64_t* k_full = q_empty + C::NQ;      // [NK]
+  uint64_t* k_empty = k_full + NK;         // [NK]: the S MMA of the block has completed
+  uint64_t* v_full = k_empty + NK;         // [NV]
+  uint64_t* v_empty = v_full + NV;         // [NV]: the PV MMA of the block has completed
+  uint64_t* s_full = v_empty + NV;         // [NS]: block g's scores, g % NS
+  uint64_t* p_full = s_full + 2;           // [NS]: P of block g written over its scores
   uint64_t* o_done = p_full + 2;           // [2]: PV of block g commits o_done[g & 1]
-  uint64_t* o_free = o_done + 2;           // [2]: output accumulator it & 1 read out
-  uint64_t* mma_done = o_free + 2;
+  uint64_t* o_free = o_done + 2;           // the item's output has been read out
+  uint64_t* mma_done = o_free + 1;
   uint64_t* info_full = mma_done + 1;      // [4]: item bounds published by the TMA thread
-  uint64_t* info_empty = info_full + 4;    // [4]: read by the four softmax warps
-  uint64_t* out_full = info_empty + 4;     // the staging tile holds an item's output (4 warps)
-  uint64_t* out_free = out_full + 1;       // the previous TMA store has read the staging tile
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(out_free + 1);
+  uint64_t* info_empty = info_full + 4;    // [4]: read by the MMA warp and the four softmax warps
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(info_empty + 4);
   int4* info = reinterpret_cast<int4*>(smem + C::OFF_INFO);
-  uint8_t* sOut = smem + C::OFF_OUT;
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   auto sQ = [&](int b) { return smem + C::OFF_Q + b * C::Q_BYTES; };
   auto sK = [&](int b) { return smem + C::OFF_K + b * C::K_BYTES; };
   auto sV = [&](int b) { return smem + C::OFF_V + b * C::K_BYTES; };
+  if (smem_u32(smem) & 1023) {  // no tile is touched then
+    if (threadIdx.x == 0) set_dev_error(a.err, DEVERR_BOUNDS);
+    return;
+  }
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int* err = a.err;
   if (threadIdx.x == 0) {
-    for (int b = 0; b < 2; ++b) {
+    for (int b = 0; b < NQ; ++b) {
       mbar_init(&q_full[b], 1);
       mbar_init(&q_empty[b], 1);
-      mbar_init(&s_full[b], 1);
-      mbar_init(&p_full[b], 4);
-      mbar_init(&o_done[b], 1);
-      mbar_init(&o_free[b], 4);
     }
-    for (int b = 0; b < NKV; ++b) {
+    for (int b = 0; b < NK; ++b) {
       mbar_init(&k_full[b], 1);
       mbar_init(&k_empty[b], 1);
+    }
+    for (int b = 0; b < NV; ++b) {
       mbar_init(&v_full[b], 1);
       mbar_init(&v_empty[b], 1);
     }
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(&s_full[b], 1);
+      mbar_init(&p_full[b], 4);
+      mbar_init(&o_done[b], 1);
+    }
+    mbar_init(o_free, 4);
     mbar_init(mma_done, 1);
     for (int b = 0; b < 4; ++b) {
       mbar_init(&info_full[b], 1);
-      mbar_init(&info_empty[b], 4);
+      mbar_init(&info_empty[b], 5);
     }
-    mbar_init(out_full, 4);
-    mbar_init(out_free, 1);
     *abort_flag = 0;
     fence_mbar_init();
     tma_prefetch_desc(&tm_q);
     tma_prefetch_desc(&tm_kv);
     tma_prefetch_desc(&tm_pre);
-    tma_prefetch_desc(&tm_out);
   }
   if (warp == 1) {
     tmem_alloc(tmem_slot, C::TMEM_COLS);
@@ -230,6 +266,14 @@ __global__ void __launch_bounds__(kThreadsTC, HD == 64 ? 2 : 1)
 
   const int n_work = *a.n_tiles * a.Hkv;
   const int n_pre = (a.P + kKeys - 1) / kKeys;
+  // key blocks of an item: the shared prefix's, then the row's own up to the tile's last token
+  auto blocks_of = [&](int4 inf) -> int { return n_pre + (min(inf.z + a.TQ, inf.y) + kKeys - 1) / kKeys; };
+  // Every wait of the MMA and softmax warps is taken warp-uniformly: a lane that
+  // gives up (timeout or abort) makes the whole warp give up, so no lane is left
+  // alone in the warp-synchronous instructions that follow.
+  auto wait_all = [&](uint64_t* bar, uint32_t parity) -> bool {
+    return __all_sync(0xffffffffu, mbar_wait_bounded(bar, parity, abort_flag, err));
+  };
 
   if (warp == 0) {
     if (lane == 0) {
@@ -238,377 +282,319 @@ __global__ void __launch_bounds__(kThreadsTC, HD == 64 ? 2 : 1)
       uint32_t gv = 0;  // key blocks whose V load was issued
       int it = 0;       // Q loads issued
       bool ok = true;
-      for (int w = blockIdx.x; w < n_work && ok; w += gridDim.x) {
-        const int tidx = w / a.Hkv, kvh = w % a.Hkv;
-        const int s = a.tile_seq[tidx], q0 = a.tile_q0[tidx];
-        const int st = a.seq_start[s], len = a.seq_start[s + 1] - st;
-        const int q_end = min(q0 + a.TQ, len);
-        const int n_kv = n_pre + (q_end + kKeys - 1) / kKeys;
-        // the softmax warps take the item's bounds from this ring instead of
-        // reading them from global memory at every item start
-        const int is = it & 3;
-        if (!mbar_wait_bounded(&info_empty[is], ((it >> 2) & 1) ^ 1, abort_flag, err)) break;
-        info[is] = make_int4(st, len, q0, kvh);
+      // an item's bounds hang on two dependent loads: the work list is read three
+      // items ahead, the sequence's bounds two ahead, and published one ahead
+      auto list = [&](int w) -> int2 {
+        if (w >= n_work) return make_int2(0, 0);
+        const int i = w / a.Hkv;
+        return make_int2(__ldg(a.tile_seq + i), __ldg(a.tile_q0 + i));
+      };
+      auto bounds = [&](int2 l, int w) -> int4 {
+        const int st = __ldg(a.seq_start + l.x);
+        return make_int4(st, __ldg(a.seq_start + l.x + 1) - st, l.y, w % a.Hkv);
+      };
+      auto publish = [&](int item, const int4& inf) -> bool {
+        const int is = item & 3;
+        if (!mbar_wait_bounded(&info_empty[is], ((item >> 2) & 1) ^ 1, abort_flag, err)) return false;
+        info[is] = inf;
         mbar_arrive(&info_full[is]);
-        const int qb = it & 1;
-        if (!mbar_wait_bounded(&q_empty[qb], ((it >> 1) & 1) ^ 1, abort_flag, err)) break;
+        return true;
+      };
+      const int step = gridDim.x;
+      int w = blockIdx.x;
+      int4 cur = bounds(list(w), w), nxt = bounds(list(w + step), w + step);
+      int2 ahead = list(w + 2 * step);
+      if (w < n_work) ok = publish(0, cur);
+      for (; w < n_work && ok; w += step) {
+        const int4 after = bounds(ahead, w + 2 * step);
+        ahead = list(w + 3 * step);
+        const int st = cur.x, kvh = cur.w;
+        const int n_kv = blocks_of(cur);
+        const int qb = it % NQ;
+        if (!mbar_wait_bounded(&q_empty[qb], ((it / NQ) & 1) ^ 1, abort_flag, err)) break;
         mbar_arrive_expect_tx(&q_full[qb], C::Q_BYTES);
         ++it;
         for (int c = 0; c < C::NC; ++c)
-          tma_load_3d(sQ(qb) + c * (128 * 128), &tm_q, &q_full[qb], c * 64, kvh * a.G, st + q0);
+          tma_load_3d(sQ(qb) + c * (128 * 128), &tm_q, &q_full[qb], c * 64, kvh * a.G, st + cur.z);
+        if (w + step < n_work && !publish(it, nxt)) break;
         for (int j = 0; j < n_kv; ++j, ++g) {
-          const int b = g % NKV;
-          const uint32_t ph = ((g / NKV) & 1) ^ 1;
           const bool pre = j < n_pre;
           const CUtensorMap* map = pre ? &tm_pre : &tm_kv;
           const int kcol = pre ? kvh * HD : (a.Hq + kvh) * HD;
           const int vcol = pre ? (a.Hkv + kvh) * HD : (a.Hq + a.Hkv + kvh) * HD;
           const int row = pre ? j * kKeys : st + (j - n_pre) * kKeys;
-          if (!mbar_wait_bounded(&k_empty[b], ph, abort_flag, err)) {
+          const int kb = g % NK, vb = g % NV;
+          if (!mbar_wait_bounded(&k_empty[kb], ((g / NK) & 1) ^ 1, abort_flag, err)) {
             ok = false;
             break;
           }
-          mbar_arrive_expect_tx(&k_full[b], C::K_BYTES);
-          for (int c = 0; c < C::NC; ++c) tma_load_2d(sK(b) + c * C::SUB, map, &k_full[b], kcol + c * 64, row);
-          if (!mbar_wait_bounded(&v_empty[b], ph, abort_flag, err)) {
+          mbar_arrive_expect_tx(&k_full[kb], C::K_BYTES);
+          for (int c = 0; c < C::NC; ++c) tma_load_2d(sK(kb) + c * C::SUB, map, &k_full[kb], kcol + c * 64, row);
+          if (!mbar_wait_bounded(&v_empty[vb], ((g / NV) & 1) ^ 1, abort_flag, err)) {
             ok = false;
             ++g;  // this block's K load is in flight, its V load is not
             break;
           }
-          mbar_arrive_expect_tx(&v_full[b], C::K_BYTES);
-          for (int c = 0; c < C::NC; ++c) tma_load_2d(sV(b) + c * C::SUB, map, &v_full[b], vcol + c * 64, row);
+          mbar_arrive_expect_tx(&v_full[vb], C::K_BYTES);
+          for (int c = 0; c < C::NC; ++c) tma_load_2d(sV(vb) + c * C::SUB, map, &v_full[vb], vcol + c * 64, row);
           ++gv;
         }
+        cur = nxt;
+        nxt = after;
       }
       if (!ok || *abort_flag) {
         // let this thread's copies still in flight land before the CTA can exit
         // (the last use of each slot is the only one that can be outstanding)
         volatile int never = 0;
-        for (uint32_t i = g > NKV ? g - NKV : 0; i < g; ++i)
-          mbar_wait_bounded(&k_full[i % NKV], (i / NKV) & 1, &never, nullptr, 200000000ull);
-        for (uint32_t i = gv > NKV ? gv - NKV : 0; i < gv; ++i)
-          mbar_wait_bounded(&v_full[i % NKV], (i / NKV) & 1, &never, nullptr, 200000000ull);
-        for (int i = it > 2 ? it - 2 : 0; i < it; ++i)
-          mbar_wait_bounded(&q_full[i & 1], (i >> 1) & 1, &never, nullptr, 200000000ull);
+        for (uint32_t i = g > NK ? g - NK : 0; i < g; ++i)
+          mbar_wait_bounded(&k_full[i % NK], (i / NK) & 1, &never, nullptr, 200000000ull);
+        for (uint32_t i = gv > NV ? gv - NV : 0; i < gv; ++i)
+          mbar_wait_bounded(&v_full[i % NV], (i / NV) & 1, &never, nullptr, 200000000ull);
+        for (int i = it > NQ ? it - NQ : 0; i < it; ++i)
+          mbar_wait_bounded(&q_full[i % NQ], (i / NQ) & 1, &never, nullptr, 200000000ull);
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ------------------------------------------------------------ MMA
-      constexpr uint32_t idesc_s = idesc_f16_f32(128, kKeys);
-      constexpr uint32_t idesc_o = idesc_f16_f32(128, HD) | (1u << 16);  // B (= V) MN-major
-      uint32_t g = 0;
-      int it = 0;
-      bool ok = true;
-      auto issue_s = [&](uint32_t gg, int qb) -> bool {
-        const int kb = gg % NKV;
-        if (!mbar_wait_bounded(&k_full[kb], (gg / NKV) & 1, abort_flag, err)) return false;
-        tc_fence_after();
-        const uint32_t d = tmem_base + (gg & 1) * kKeys;
+    // -------------------------------------------------------------- MMA
+    // the whole warp walks the blocks and one elected lane issues, so that the
+    // descriptors stay in uniform registers
+    constexpr uint32_t idesc_s = idesc_f16_f32(128, kKeys);
+    constexpr uint32_t idesc_o = idesc_f16_f32(128, HD) | (1u << 16);  // B (= V) MN-major
+    const uint32_t tb = __shfl_sync(0xffffffffu, tmem_base, 0);
+    const uint64_t dq0 = smem_desc_k_sw128(smem_u32(sQ(0))), dk0 = smem_desc_k_sw128(smem_u32(sK(0)));
+    const uint64_t dv0 = smem_desc_mn_sw128(smem_u32(sV(0)), HD == 64 ? 1024u : 8192u, 1024u);
+    // (one lane) S of block gg, its K and Q landed; `last`: its item's last block,
+    // after which Q's slot is free
+    auto issue_s = [&](uint32_t gg, int qb, bool last) {
+      const uint32_t kb = gg % NK;
+      const uint32_t d = tb + (gg % NS) * kKeys;
+      const uint64_t dq = dq0 + qb * (C::Q_BYTES >> 4), dk = dk0 + kb * (C::K_BYTES >> 4);
 #pragma unroll
-        for (int c = 0; c < C::NC; ++c)
+      for (int c = 0; c < C::NC; ++c)
 #pragma unroll
-          for (int k = 0; k < 4; ++k)
-            umma_f16_ss(d, smem_desc_k_sw128(smem_u32(sQ(qb) + c * (128 * 128)) + k * 32),
-                        smem_desc_k_sw128(smem_u32(sK(kb) + c * C::SUB) + k * 32), idesc_s, (c | k) != 0);
-        umma_commit(&k_empty[kb]);
-        umma_commit(&s_full[gg & 1]);
-        return true;
-      };
-      // key blocks of an item (the shared prefix's, then the row's own up to
-      // the tile's last token)
-      auto blocks_of = [&](int w) -> int {
-        const int tidx = w / a.Hkv;
-        const int s = a.tile_seq[tidx], q0 = a.tile_q0[tidx];
-        const int len = a.seq_start[s + 1] - a.seq_start[s];
-        return n_pre + (min(q0 + a.TQ, len) + kKeys - 1) / kKeys;
-      };
+        for (int k = 0; k < 4; ++k) {
+          const uint64_t qa = dq + c * (128 * 128 >> 4) + 2 * k, ka = dk + c * (C::SUB >> 4) + 2 * k;
+          if (c == 0 && k == 0)
+            umma_f16_ss(d, qa, ka, idesc_s, 0);
+          else
+            umma_f16_ss_acc(d, qa, ka, idesc_s);
+        }
+      umma_commit(&s_full[gg % NS]);
+      umma_commit(&k_empty[kb]);
+      if (last) umma_commit(&q_empty[qb]);
+    };
+    // the blocks of item `item` (ring slot item & 3), once its Q and first K have landed
+    auto take_item = [&](int item, uint32_t gg, int* n) -> bool {
+      const int is = item & 3;
+      if (!wait_all(&info_full[is], (item >> 2) & 1)) return false;
+      *n = blocks_of(info[is]);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&info_empty[is]);
+      return wait_all(&q_full[item % NQ], (item / NQ) & 1) && wait_all(&k_full[gg % NK], (gg / NK) & 1);
+    };
+    uint32_t g = 0;
+    int it = 0, n_kv = 0;
+    bool ok = true;
+    int w = blockIdx.x;
+    if (w < n_work) {
       // The blocks of all this CTA's items form one stream: the scores of the
-      // next block, also the first block of the next item, are issued before
-      // this block's PV, so an item boundary costs no extra hand-off.
-      int w = blockIdx.x;
-      if (w < n_work) {
-        int n_kv = blocks_of(w);
-        if (!mbar_wait_bounded(&q_full[0], 0, abort_flag, err) || (tc_fence_after(), !issue_s(g, 0))) ok = false;
-        while (ok) {
-          const int qb = it & 1;
-          const int w_next = w + gridDim.x;
-          const int n_next = w_next < n_work ? blocks_of(w_next) : 0;
-          for (int j = 0; j < n_kv; ++j, ++g) {
-            if (j + 1 < n_kv) {
-              if (!issue_s(g + 1, qb)) {
-                ok = false;
-                break;
-              }
-            } else {
-              umma_commit(&q_empty[qb]);  // all S MMAs of this item issued
-              if (n_next > 0) {
-                const int it1 = it + 1;
-                if (!mbar_wait_bounded(&q_full[it1 & 1], (it1 >> 1) & 1, abort_flag, err)) {
-                  ok = false;
-                  break;
-                }
-                tc_fence_after();
-                if (!issue_s(g + 1, it1 & 1)) {
-                  ok = false;
-                  break;
-                }
-              }
-            }
-            if (!mbar_wait_bounded(&p_full[g & 1], (g >> 1) & 1, abort_flag, err)) {
+      // next block, also the first block of the next item, are issued as soon
+      // as their buffer allows, so an item boundary costs no extra hand-off.
+      ok = take_item(0, 0, &n_kv);
+      if (ok) {
+        tc_fence_after();
+        if (elect_one()) issue_s(0, 0, n_kv == 1);
+        __syncwarp();
+      }
+      while (ok) {
+        const bool more = w + static_cast<int>(gridDim.x) < n_work;
+        int n_next = 0;
+        for (int j = 0; j < n_kv; ++j, ++g) {
+          const bool inside = j + 1 < n_kv;
+          // With two score buffers the next scores of this item come before this
+          // block's PV; the next item's come after it, as its Q may have to wait
+          // for this item's last S.
+          const bool early = NS == 2 && inside;
+          if (inside) {
+            if (!wait_all(&k_full[(g + 1) % NK], ((g + 1) / NK) & 1)) {
               ok = false;
               break;
             }
-            // the first PV overwrites this item's accumulator: the softmax warps
-            // must have read out the output of the item two back
-            if (j == 0 && !mbar_wait_bounded(&o_free[qb], ((it >> 1) & 1) ^ 1, abort_flag, err)) {
-              ok = false;
-              break;
+            if (early) {
+              tc_fence_after();
+              if (elect_one()) issue_s(g + 1, it % NQ, j + 2 == n_kv);
+              __syncwarp();
             }
-            const int vb = g % NKV;
-            if (!mbar_wait_bounded(&v_full[vb], (g / NKV) & 1, abort_flag, err)) {
+          } else if (more && NQ > 1 && !take_item(it + 1, g + 1, &n_next)) {
+            ok = false;
+            break;
+          }
+          // the first PV overwrites the accumulator: the softmax warps must have
+          // read out the previous item's output
+          const uint32_t vb = g % NV;
+          if (!wait_all(&v_full[vb], (g / NV) & 1) || (j == 0 && !wait_all(o_free, (it & 1) ^ 1)) ||
+              !wait_all(&p_full[g % NS], (g / NS) & 1)) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          const uint64_t dv = dv0 + vb * (C::K_BYTES >> 4);
+          if (elect_one()) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+              umma_f16_ts(tb + C::O_COL, tb + (g % NS) * kKeys + k * 8, dv + k * (2048 >> 4), idesc_o, (j | k) != 0);
+            umma_commit(&o_done[g & 1]);
+            umma_commit(&v_empty[vb]);
+            if (!early && inside) issue_s(g + 1, it % NQ, j + 2 == n_kv);
+            if (!inside && more && NQ > 1) issue_s(g + 1, (it + 1) % NQ, n_next == 1);
+          }
+          __syncwarp();
+          if (!inside && more && NQ == 1) {
+            if (!take_item(it + 1, g + 1, &n_next)) {
               ok = false;
               break;
             }
             tc_fence_after();
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-              umma_f16_ts(tmem_base + C::O_COL + qb * HD, tmem_base + (g & 1) * kKeys + k * 8,
-                          smem_desc_mn_sw128(smem_u32(sV(vb)) + k * 2048, HD == 64 ? 1024u : 8192u, 1024u),
-                          idesc_o, (j | k) != 0);
-            umma_commit(&v_empty[vb]);
-            umma_commit(&o_done[g & 1]);
+            if (elect_one()) issue_s(g + 1, (it + 1) % NQ, n_next == 1);
+            __syncwarp();
           }
-          if (!ok || n_next == 0) break;
-          w = w_next;
-          n_kv = n_next;
-          ++it;
         }
+        if (!ok || !more) break;
+        w += gridDim.x;
+        n_kv = n_next;
+        ++it;
       }
-      umma_commit(mma_done);
-      volatile int never = 0;
-      mbar_wait_bounded(mma_done, 0, &never, err);
     }
+    if (elect_one()) umma_commit(mma_done);
+    __syncwarp();
+    volatile int never = 0;
+    mbar_wait_bounded(mma_done, 0, &never, err);
   } else {
     // ------------------------------------------------- softmax / epilogue
     const int quarter = warp & 3;
     const int r = quarter * 32 + lane;  // TMEM lane = query row of the tile
     const int t = r / a.G, gq = r % a.G;
     const uint32_t trow = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16);
+    const uint32_t ocol = trow + C::O_COL;
+    const bool wide = (reinterpret_cast<uintptr_t>(a.out) & 31) == 0;  // 32-byte stores
     uint32_t g = 0;
     int it = 0;
     bool ok = true;
-    // PV of block gg done (o_done completes once per block on slot gg & 1;
-    // this thread has already seen PV of block gg - 2 complete, and PV of
-    // block gg + 2 needs a P that it has not yet written, so parity is exact)
-    // Every wait of these warps is taken warp-uniformly: a lane that gives up
-    // (timeout or abort) makes the whole warp give up, so no lane is left
-    // alone in the warp-synchronous tcgen05 loads and stores that follow.
-    auto wait_all = [&](uint64_t* bar, uint32_t parity) -> bool {
-      return __all_sync(0xffffffffu, mbar_wait_bounded(bar, parity, abort_flag, err));
-    };
+    // PV of block gg done (see the ordering note above: the parity is exact)
     auto wait_pv = [&](uint32_t gg) -> bool { return wait_all(&o_done[gg & 1], (gg >> 1) & 1); };
-    // The output of an item is read out after the next item's first block
-    // (its last PV may still be running meanwhile): O / l, stored for the
-    // tile's real tokens, then the accumulator is handed back to the MMA warp.
-    // A tile whose tokens all belong to its sequence is written by one TMA
-    // store of the CTA's staging tile (rows in TMEM-lane order = the box's
-    // token-major, head-minor order, 128-byte swizzle); a ragged last tile is
-    // written row by row, live rows only, since its box would reach into the
-    // next sequence's tokens.  nf counts the full-tile read-outs: the k-th
-    // waits for out_free phase k - 1 (the store of read-out k - 1 has read
-    // the staging tile) and its four warps complete out_full phase k.
-    struct Pending {
-      bool on, live, full;
-      int buf, kvh, tok;
-      uint32_t g_last;
-      float inv;
-      __half* dst;
-    } pend{false, false, false, 0, 0, 0, 0, 0.f, nullptr};
-    uint32_t nf = 0;
-    const bool issuer = threadIdx.x == 64;
-    auto flush = [&]() -> bool {
-      if (!wait_pv(pend.g_last)) return false;
-      tc_fence_after();
-      if (pend.full) {
-        if (nf > 0) {
-          if (issuer) {
-            bulk_wait_group_read<0>();
-            mbar_arrive(out_free);
-          }
-          if (!wait_all(out_free, (nf - 1) & 1)) return false;
-        }
-      }
-      const uint32_t ocol = trow + C::O_COL + pend.buf * HD;
-#pragma unroll 1
-      for (int c = 0; c < HD; c += 32) {
-        uint32_t o[32];
-        tmem_ld_32x32b_x32(ocol + c, o);
-        tmem_ld_wait();
-        if (pend.full) {
-          uint8_t* row = sOut + (c >> 6) * (128 * 128) + r * 128;
-#pragma unroll
-          for (int q4 = 0; q4 < 4; ++q4) {
-            uint32_t pk[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              __half2 h = __floats2half2_rn(__uint_as_float(o[q4 * 8 + 2 * i]) * pend.inv,
-                                            __uint_as_float(o[q4 * 8 + 2 * i + 1]) * pend.inv);
-              pk[i] = *reinterpret_cast<uint32_t*>(&h);
-            }
-            const int chunk = ((c & 63) >> 3) + q4;
-            *reinterpret_cast<uint4*>(row + ((chunk ^ (r & 7)) << 4)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-          }
-        } else if (pend.live) {
-          uint4* d4 = reinterpret_cast<uint4*>(pend.dst + c);
-#pragma unroll
-          for (int q4 = 0; q4 < 4; ++q4) {
-            uint32_t pk[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              __half2 h = __floats2half2_rn(__uint_as_float(o[q4 * 8 + 2 * i]) * pend.inv,
-                                            __uint_as_float(o[q4 * 8 + 2 * i + 1]) * pend.inv);
-              pk[i] = *reinterpret_cast<uint32_t*>(&h);
-            }
-            d4[q4] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-          }
-        }
-      }
-      tc_fence_before();
-      if (pend.full) fence_proxy_async_smem();
-      __syncwarp();
-      if (lane == 0) {
-        mbar_arrive(&o_free[pend.buf]);
-        if (pend.full) mbar_arrive(out_full);
-      }
-      if (pend.full) {
-        // the storing thread's wait decides for its whole warp
-        bool stored = true;
-        if (issuer) {
-          stored = mbar_wait_bounded(out_full, nf & 1, abort_flag, err);
-          if (stored) {
-#pragma unroll
-            for (int cc = 0; cc < C::NC; ++cc)
-              tma_store_3d(&tm_out, sOut + cc * (128 * 128), cc * 64, pend.kvh * a.G, pend.tok);
-            bulk_commit_group();
-          }
-        }
-        if (!__shfl_sync(0xffffffffu, stored, 0)) return false;
-        ++nf;
-      }
-      pend.on = false;
-      return true;
-    };
     for (int w = blockIdx.x; w < n_work && ok; w += gridDim.x, ++it) {
       const int is = it & 3;
-      if (!wait_all(&info_full[is], (it >> 2) & 1)) {
-        ok = false;
-        break;
-      }
+      if (!wait_all(&info_full[is], (it >> 2) & 1)) break;
       const int4 inf = info[is];
       __syncwarp();
       if (lane == 0) mbar_arrive(&info_empty[is]);
       const int st = inf.x, len = inf.y, q0 = inf.z, kvh = inf.w;
-      const int q_end = min(q0 + a.TQ, len);
-      const int n_kv = n_pre + (q_end + kKeys - 1) / kKeys;
+      const int n_kv = blocks_of(inf);
       const int qpos = q0 + t;
-      const uint32_t ocol = trow + C::O_COL + (it & 1) * HD;
       float m_used = 0.f, l = 0.f;
       for (int j = 0; j < n_kv; ++j, ++g) {
-        const int b = g & 1;
-        if (!wait_all(&s_full[b], (g >> 1) & 1)) {
+        const uint32_t sb = g % NS;
+        if (!wait_all(&s_full[sb], (g / NS) & 1)) {
           ok = false;
           break;
         }
         tc_fence_after();
-        float v[64];
-        load2x32_f(trow + b * kKeys, trow + b * kKeys + 32, v, v + 32);
+        const uint32_t scol = trow + sb * kKeys;
         const bool pre = j < n_pre;
         const int key0 = (pre ? j : j - n_pre) * kKeys;
         // warp-uniform: only the prefix's last block and the causal diagonal /
         // sequence end need a mask; then key c is visible iff c < lim
-        const bool need_mask = pre ? (key0 + kKeys > a.P) : (key0 + kKeys - 1 > q0 || key0 + kKeys > len);
-        if (need_mask) {
-          const int lim = pre ? a.P - key0 : min(qpos + 1, len) - key0;
-#pragma unroll
-          for (int c = 0; c < 64; ++c) v[c] = c < lim ? v[c] : -INFINITY;
-        }
-        // running max on the raw scores; the softmax scale (with log2 e) is
-        // folded into one FFMA inside the exponent below
-        // (eight independent partial maxima keep the FMNMX chain short)
-        float pm[8];
-#pragma unroll
-        for (int c = 0; c < 8; ++c) pm[c] = v[c];
-#pragma unroll
-        for (int c = 8; c < 64; ++c) pm[c & 7] = fmaxf(pm[c & 7], v[c]);
-        const float mr = fmaxf(fmaxf(fmaxf(pm[0], pm[1]), fmaxf(pm[2], pm[3])),
-                               fmaxf(fmaxf(pm[4], pm[5]), fmaxf(pm[6], pm[7])));
-        const float mx = mr * a.scale_log2;
+        const bool mask = pre ? (key0 + kKeys > a.P) : (key0 + kKeys - 1 > q0 || key0 + kKeys > len);
+        const int lim = pre ? a.P - key0 : min(qpos + 1, len) - key0;
+        float v[32];
         if (j == 0) {
-          m_used = mx == -INFINITY ? 0.f : mx;
-        } else {
-          const bool grow = mx > m_used + 8.f;
-          if (__any_sync(0xffffffffu, grow)) {
-            // rescale this warp's output rows once the previous block's PV is done
+          // running max on the raw scores; the softmax scale (with log2 e) is
+          // folded into one FMA inside the exponent
+          load_scores(scol, v, mask, lim);
+          float mr = max32(v);
+          load_scores(scol + 32, v, mask, lim - 32);
+          mr = fmaxf(mr, max32(v));
+          m_used = mr == -INFINITY ? 0.f : mr * a.scale_log2;
+        }
+        uint32_t pk[32];
+        float2 ps[4];
+        for (;;) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) ps[i] = make_float2(0.f, 0.f);
+          load_scores(scol, v, mask, lim);
+          float mr = max32(v);
+          exp32(v, a.scale_log2, m_used, pk, ps);
+          load_scores(scol + 32, v, mask, lim - 32);
+          mr = fmaxf(mr, max32(v));
+          exp32(v, a.scale_log2, m_used, pk + 16, ps);
+          const float mx = mr * a.scale_log2;
+          const bool grow = j > 0 && mx > m_used + 8.f;
+          if (!__any_sync(0xffffffffu, grow)) break;
+          // rescale this warp's output rows once the previous block's PV is done,
+          // and form this block's P again from its scores, still in place
+          if (NS == 2) {
             if (!wait_pv(g - 1)) {
               ok = false;
               break;
             }
             tc_fence_after();
-            const float f = grow ? ex2_approx(m_used - mx) : 1.f;
-            if (grow) {
-              l *= f;
-              m_used = mx;
-            }
-#pragma unroll 1
-            for (int c = 0; c < HD; c += 32) {
-              uint32_t o[32];
-              tmem_ld_32x32b_x32(ocol + c, o);
-              tmem_ld_wait();
-#pragma unroll
-              for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * f);
-              tmem_st_32x32b_x32(ocol + c, o);
-            }
-            tmem_st_wait();
           }
-        }
-        float2 ps[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-        const float2 sc2 = make_float2(a.scale_log2, a.scale_log2), nm2 = make_float2(-m_used, -m_used);
-        uint32_t pk[32];
+          const float f = grow ? ex2_approx(m_used - mx) : 1.f;
+          if (grow) {
+            l *= f;
+            m_used = mx;
+          }
+#pragma unroll 1
+          for (int c = 0; c < HD; c += 32) {
+            uint32_t o[32];
+            tmem_ld_32x32b_x32(ocol + c, o);
+            tmem_ld_wait();
 #pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          const float2 x = ffma2(make_float2(v[2 * i], v[2 * i + 1]), sc2, nm2);
-          const float2 p = make_float2(ex2_approx(x.x), ex2_approx(x.y));
-          ps[i & 3] = fadd2(ps[i & 3], p);
-          __half2 h = __floats2half2_rn(p.x, p.y);
-          pk[i] = *reinterpret_cast<uint32_t*>(&h);
+            for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * f);
+            tmem_st_32x32b_x32(ocol + c, o);
+          }
+          tmem_st_wait();
         }
+        if (!ok) break;
         l += ((ps[0].x + ps[0].y) + (ps[1].x + ps[1].y)) + ((ps[2].x + ps[2].y) + (ps[3].x + ps[3].y));
         // P (fp16 pairs) over the first 32 columns of this block's score buffer
-        tmem_st_32x32b_x32(trow + b * kKeys, pk);
+        tmem_st_32x32b_x32(scol, pk);
         tmem_st_wait();
         tc_fence_before();  // this block's score reads and P writes are complete
         __syncwarp();
-        if (lane == 0) mbar_arrive(&p_full[b]);
-        if (j == 0 && pend.on && !flush()) {
-          ok = false;
-          break;
-        }
+        if (lane == 0) mbar_arrive(&p_full[sb]);
       }
       if (!ok) break;
-      pend.on = true;
-      pend.live = qpos < len;
-      pend.full = q0 + a.TQ <= len;
-      pend.kvh = kvh;
-      pend.tok = st + q0;
-      pend.buf = it & 1;
-      pend.g_last = g - 1;
-      pend.inv = l > 0.f ? 1.f / l : 0.f;
-      pend.dst = a.out + static_cast<int64_t>(st + qpos) * (a.Hq * HD) + (kvh * a.G + gq) * HD;
+      // O / l of the tile's real tokens, once the item's last PV is done
+      if (!wait_pv(g - 1)) break;
+      tc_fence_after();
+      const float inv = l > 0.f ? 1.f / l : 0.f;
+      __half* dst = a.out + static_cast<int64_t>(st + qpos) * (a.Hq * HD) + (kvh * a.G + gq) * HD;
+#pragma unroll 1
+      for (int c = 0; c < HD; c += 32) {
+        uint32_t o[32], pk[16];
+        tmem_ld_32x32b_x32(ocol + c, o);
+        tmem_ld_wait();
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+          __half2 h = __floats2half2_rn(__uint_as_float(o[2 * i]) * inv, __uint_as_float(o[2 * i + 1]) * inv);
+          pk[i] = *reinterpret_cast<uint32_t*>(&h);
+        }
+        if (qpos < len) {
+          if (wide) {
+            st_global_v8(dst + c, pk);
+            st_global_v8(dst + c + 16, pk + 8);
+          } else {
+#pragma unroll
+            for (int q4 = 0; q4 < 4; ++q4)
+              reinterpret_cast<uint4*>(dst + c)[q4] = make_uint4(pk[4 * q4], pk[4 * q4 + 1], pk[4 * q4 + 2], pk[4 * q4 + 3]);
+          }
+        }
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(o_free);
     }
-    if (ok && pend.on) flush();
-    // the CTA's shared memory must outlive the TMA stores that read it
-    if (issuer) bulk_wait_group_all();
   }
 
   __syncthreads();
@@ -656,16 +642,14 @@ bool map3d_q(CUtensorMap* m, const __half* base, int64_t T, int heads, int hd, i
 }
 
 template <int HD>
-int launch_tc(const CUtensorMap& mq, const CUtensorMap& mkv, const CUtensorMap& mpre, const CUtensorMap& mout,
-              const AttnArgs& a,
+int launch_tc(const CUtensorMap& mq, const CUtensorMap& mkv, const CUtensorMap& mpre, const AttnArgs& a,
               int n_work_max, int num_sms, cudaStream_t s) {
   using C = ACfg<HD>;
   cudaError_t e = cudaFuncSetAttribute(k_attention_tc<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
   if (e != cudaSuccess) return e;
-  const int per_sm = C::SMEM <= 113 * 1024 ? 2 : 1;
-  const int grid = n_work_max < num_sms * per_sm ? n_work_max : num_sms * per_sm;
+  const int grid = n_work_max < num_sms * C::CTAS ? n_work_max : num_sms * C::CTAS;
   if (grid <= 0) return 0;
-  k_attention_tc<HD><<<grid, kThreadsTC, C::SMEM, s>>>(mq, mkv, mpre, mout, a);
+  k_attention_tc<HD><<<grid, kThreadsTC, C::SMEM, s>>>(mq, mkv, mpre, a);
   return cudaGetLastError();
 }
 
@@ -685,10 +669,11 @@ int launch_attention_tc(const __half* qkv, int64_t T, const int32_t* seq_start, 
   if (n_tiles_max <= 0 || T <= 0) return 0;
   const int G = Hq / Hkv, TQ = 128 / G;
   const int heads = Hq + 2 * Hkv;
-  CUtensorMap mq, mkv, mpre, mout;
-  if (!map3d_q(&mq, qkv, T, heads, hd, G, TQ) || !map2d(&mkv, qkv, T, int64_t(heads) * hd) ||
-      !map3d_q(&mout, out, T, Hq, hd, G, TQ))
+  CUtensorMap mq, mkv, mpre;
+  if (!map3d_q(&mq, qkv, T, heads, hd, G, TQ) || !map2d(&mkv, qkv, T, int64_t(heads) * hd))
     return cudaErrorInvalidValue;
+  // the output's rows are written in 16- or 32-byte pieces
+  if (reinterpret_cast<uintptr_t>(out) & 15) return cudaErrorInvalidValue;
   if (prefix_kv && P > 0) {
     if (!map2d(&mpre, prefix_kv, P, int64_t(2) * Hkv * hd)) return cudaErrorInvalidValue;
   } else {
@@ -698,8 +683,8 @@ int launch_attention_tc(const __half* qkv, int64_t T, const int32_t* seq_start, 
   AttnArgs a{seq_start, tile_seq, tile_q0, n_tiles_dev, Hq, Hkv, G, TQ, P,
              1.4426950408889634f / sqrtf(static_cast<float>(hd)), out, err};
   const int n_work_max = n_tiles_max * Hkv;
-  return hd == 64 ? launch_tc<64>(mq, mkv, mpre, mout, a, n_work_max, num_sms, s)
-                  : launch_tc<128>(mq, mkv, mpre, mout, a, n_work_max, num_sms, s);
+  return hd == 64 ? launch_tc<64>(mq, mkv, mpre, a, n_work_max, num_sms, s)
+                  : launch_tc<128>(mq, mkv, mpre, a, n_work_max, num_sms, s);
 }
 
 }  // namespace aiq

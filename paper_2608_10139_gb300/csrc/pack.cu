@@ -95,29 +95,38 @@ __global__ void k_pack_chunk(const int64_t* cu, const int32_t* ids, const int32_
   }
 }
 
-// Attention work list: one entry per (sequence, block of `tq` query tokens), one block.
+// Attention work list: one entry per (sequence, block of `tq` query tokens), one
+// block.  A launch is a chain of barriers, so each 1024 sequences take one: a
+// shuffle scan within the warps, then every warp scans the 32 warp totals.
 __global__ void __launch_bounds__(1024) k_attn_tiles(const int32_t* seq_start, int32_t n, int32_t tq,
                                                      int32_t* tile_seq, int32_t* tile_q0, int32_t* n_tiles) {
-  __shared__ int32_t sh[1024];
+  __shared__ int32_t sh[2][32];  // alternate, so that one barrier a round is enough
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int32_t carry = 0;
-  for (int32_t b = 0; b < n; b += 1024) {
+  for (int32_t b = 0, k = 0; b < n; b += 1024, k ^= 1) {
     const int32_t i = b + threadIdx.x;
     const int32_t cnt = i < n ? (seq_start[i + 1] - seq_start[i] + tq - 1) / tq : 0;
-    sh[threadIdx.x] = cnt;
-    __syncthreads();
-    for (int o = 1; o < 1024; o <<= 1) {
-      int32_t y = threadIdx.x >= o ? sh[threadIdx.x - o] : 0;
-      __syncthreads();
-      sh[threadIdx.x] += y;
-      __syncthreads();
+    int32_t incl = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += y;
     }
-    int32_t at = carry + sh[threadIdx.x] - cnt;
+    if (lane == 31) sh[k][warp] = incl;
+    __syncthreads();
+    int32_t tot = sh[k][lane];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int32_t y = __shfl_up_sync(0xffffffffu, tot, o);
+      if (lane >= o) tot += y;
+    }
+    const int32_t before = warp ? __shfl_sync(0xffffffffu, tot, (warp - 1) & 31) : 0;
+    const int32_t at = carry + before + incl - cnt;
     for (int32_t q = 0; q < cnt; ++q) {
       tile_seq[at + q] = i;
       tile_q0[at + q] = q * tq;
     }
-    carry += sh[1023];
-    __syncthreads();
+    carry += __shfl_sync(0xffffffffu, tot, 31);
   }
   if (threadIdx.x == 0) *n_tiles = carry;
 }
