@@ -739,7 +739,7 @@ aiq_status decode_layers(aiq_ctx* c, ModelD& m, const PrefillBufs& b, const Deco
       const int e = launch_decode_attention(b.qkv, nqkv, R, Hq, Hkv, hd, pkv ? pkv + l * P * ldkv : nullptr, P,
                                             d.kvc + l * Tc * ldkv, b.seq_start,
                                             d.gkv + static_cast<int64_t>(l) * R * d.gcap * ldkv, d.gcap, slot, b.att,
-                                            c->d_err, c->stream);
+                                            c->d_err, c->num_sms, c->stream);
       counted(c, 1);
       if (e != 0)
         return fail(AIQ_ERR_CUDA, std::string("decode attention launch: ") +
@@ -1996,7 +1996,7 @@ aiq_status aiq_op_decode_attention(aiq_ctx* c, const void* qkv, int32_t R, int32
   const int e = launch_decode_attention(static_cast<const __half*>(qkv), static_cast<int64_t>(Hq + 2 * Hkv) * hd, R,
                                         Hq, Hkv, hd, static_cast<const __half*>(prefix_kv), P,
                                         static_cast<const __half*>(own_kv), seq_start, static_cast<__half*>(gen_kv),
-                                        gen_cap, slot, static_cast<__half*>(out), c->d_err, c->stream);
+                                        gen_cap, slot, static_cast<__half*>(out), c->d_err, c->num_sms, c->stream);
   if (e != 0) return fail(AIQ_ERR_CUDA, std::string("decode attention launch: ") +
                                             cudaGetErrorString(static_cast<cudaError_t>(e)));
   return sync_and_check(c);

@@ -255,6 +255,225 @@ __global__ void __launch_bounds__(kDecThreads, HD == 128 ? 2 : 3) k_decode_atten
   }
 }
 
+// ------------------------------------------------- many rows: a warp per task
+// The same attention for batches with enough (row, KV head) tasks to fill the
+// GPU: a warp takes a whole task, so no partial states are merged and no block
+// waits for its slowest warp, and a persistent warp walks the key blocks of all
+// its tasks as one stream, the next block's cp.async in flight while this one's
+// MMAs run.  Bound by the cached keys' and values' read from HBM: a decode batch
+// of the select workload (3263 rows of about 216 keys, 32/8 heads, head_dim 64,
+// 1.07 GB) takes 225 us against 388 with a block per task, 0.7 of the measured
+// copy bandwidth.  Half-sized blocks with five CTAs take 247, two CTAs 279, and a
+// 256-byte L2 prefetch on the copies 242.
+template <int HD>
+struct DecStream {
+  static constexpr int NW = 4;                          // warps per CTA
+  static constexpr int KB = HD == 128 ? 16 : 32;        // keys per block
+  static constexpr int STAGES = 2;
+  static constexpr int LDS = HD + 8;                    // padded smem row (halves): conflict-free ldmatrix
+  static constexpr int STAGE_HALVES = 2 * KB * LDS;     // K block then V block
+  static constexpr int SMEM = NW * STAGES * STAGE_HALVES * 2;
+  static constexpr int CTAS = HD == 32 ? 4 : 3;           // per SM
+  static_assert(CTAS * (SMEM + 1024) <= 233472, "shared memory per SM");
+};
+
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+template <int HD>
+__global__ void __launch_bounds__(DecStream<HD>::NW * 32, DecStream<HD>::CTAS)
+    k_decode_attention_stream(DecArgs a, int n_tasks) {
+  using C = DecStream<HD>;
+  constexpr int KB = C::KB, LDS = C::LDS;
+  constexpr int KS = HD / 16;  // k-steps of Q K^T
+  constexpr int DN = HD / 8;   // 8-wide output column tiles
+  constexpr int CH = HD / 8;   // 16-byte chunks per row
+  extern __shared__ __align__(16) uint8_t smem_raw[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int G = a.G;
+  const int kd = a.Hkv * HD;
+  const int64_t ld = 2 * static_cast<int64_t>(kd);
+  __half* ring = reinterpret_cast<__half*>(smem_raw) + warp * C::STAGES * C::STAGE_HALVES;
+  const int gq = lane >> 2, tq = lane & 3;
+  const int step = gridDim.x * C::NW;
+
+  // a task's rows: prompt start and length; the task after it is looked up a task ahead
+  struct Task {
+    int r, h, st, len;
+  };
+  auto task = [&](int i) -> Task {
+    Task t{0, 0, 0, 0};
+    if (i < n_tasks) {
+      t.r = i / a.Hkv;
+      t.h = i % a.Hkv;
+      t.st = __ldg(a.seq_start + t.r);
+      t.len = __ldg(a.seq_start + t.r + 1) - t.st;
+    }
+    return t;
+  };
+  // K and V of keys key0 .. key0 + KB - 1 of a task: shared prefix, the row's
+  // prompt, its generated tokens, this step's own; rows past the last are zeros
+  auto stage = [&](const Task& t, int key0, int slot) {
+    __half* sK = ring + slot * C::STAGE_HALVES;
+    __half* sV = sK + KB * LDS;
+    const int n_keys = a.P + t.len + a.slot + 1;
+    const __half* qrow = a.qkv + static_cast<int64_t>(t.r) * a.ldq;
+    const __half* gen = a.gkv + static_cast<int64_t>(t.r) * a.gcap * ld;
+#pragma unroll
+    for (int i = 0; i < KB * CH / 32; ++i) {
+      const int c = lane + 32 * i;
+      const int kr = c / CH, part = c % CH;
+      const int j = key0 + kr;
+      const bool valid = j < n_keys;
+      const int o = j - a.P;  // token of the row
+      const __half* k;
+      if (o < 0)
+        k = a.pkv + j * ld;
+      else if (o < t.len)
+        k = a.kvc + (t.st + o) * ld;
+      else if (j < n_keys - 1)
+        k = gen + (o - t.len) * ld;
+      else
+        k = qrow + a.Hq * HD;  // this step's token (and, unread, the rows past it)
+      k += t.h * HD + part * 8;
+      cp_async16(smem_u32(sK + kr * LDS + part * 8), k, valid);
+      cp_async16(smem_u32(sV + kr * LDS + part * 8), k + kd, valid);
+    }
+    cp_async_commit();
+  };
+
+  int i = blockIdx.x * C::NW + warp;
+  Task cur = task(i), nxt = task(i + step);
+  if (i < n_tasks) stage(cur, 0, 0);
+  int slot = 0;
+  for (; i < n_tasks; i += step) {
+    const int n_keys = a.P + cur.len + a.slot + 1;
+    const __half* qrow = a.qkv + static_cast<int64_t>(cur.r) * a.ldq;
+    const Task after = task(i + 2 * step);
+    // A fragments of the query tile: row gq is query head h G + gq (rows >= G and 8..15 are zero padding)
+    uint32_t qf[KS][2];
+    {
+      const uint32_t* q32 = reinterpret_cast<const uint32_t*>(qrow + (cur.h * G + gq) * HD);
+#pragma unroll
+      for (int kk = 0; kk < KS; ++kk) {
+        qf[kk][0] = gq < G ? q32[(kk * 16 + 2 * tq) / 2] : 0u;
+        qf[kk][1] = gq < G ? q32[(kk * 16 + 8 + 2 * tq) / 2] : 0u;
+      }
+    }
+    // this token's key and value into its cache slot, for the later steps
+    for (int c = lane; c < 2 * CH; c += 32) {
+      const int v = c / CH, part = c % CH;
+      __half* dst = a.gkv + (static_cast<int64_t>(cur.r) * a.gcap + a.slot) * ld + v * kd + cur.h * HD;
+      reinterpret_cast<uint4*>(dst)[part] = reinterpret_cast<const uint4*>(qrow + (a.Hq + v * a.Hkv + cur.h) * HD)[part];
+    }
+    float o[DN][2];
+#pragma unroll
+    for (int d = 0; d < DN; ++d) o[d][0] = o[d][1] = 0.f;
+    float m0 = -INFINITY, l0 = 0.f;
+    for (int key0 = 0; key0 < n_keys; key0 += KB, slot ^= 1) {
+      // the next block, of this task or the next one, into the other slot
+      if (key0 + KB < n_keys)
+        stage(cur, key0 + KB, slot ^ 1);
+      else if (i + step < n_tasks)
+        stage(nxt, 0, slot ^ 1);
+      else
+        cp_async_commit();  // an empty group, so that the wait below means the same
+      cp_async_wait<1>();
+      __syncwarp();
+      const __half* sK = ring + slot * C::STAGE_HALVES;
+      const __half* sV = sK + KB * LDS;
+      float sc[KB / 8][4];
+#pragma unroll
+      for (int n = 0; n < KB / 8; ++n) sc[n][0] = sc[n][1] = sc[n][2] = sc[n][3] = 0.f;
+#pragma unroll
+      for (int kk = 0; kk < KS; ++kk) {
+        const uint32_t qa[4] = {qf[kk][0], 0u, qf[kk][1], 0u};
+#pragma unroll
+        for (int np = 0; np < KB / 16; ++np) {
+          const int mat = lane >> 3;
+          const int key = np * 16 + (lane & 7) + 8 * (mat >> 1);
+          const int dim = kk * 16 + 8 * (mat & 1);
+          uint32_t bb[4];
+          ldsm_x4(bb, smem_u32(sK + key * LDS + dim));
+          mma16816(sc[2 * np], qa, bb[0], bb[1]);
+          mma16816(sc[2 * np + 1], qa, bb[2], bb[3]);
+        }
+      }
+      // log2 units, keys past the end masked; row gq uses elements 0 and 1
+      float mx = -INFINITY;
+#pragma unroll
+      for (int n = 0; n < KB / 8; ++n) {
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const int key = key0 + n * 8 + 2 * tq + e;
+          const float v = key < n_keys ? sc[n][e] * a.scale_log2 : -INFINITY;
+          sc[n][e] = v;
+          mx = fmaxf(mx, v);
+        }
+      }
+      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+      // P is relative to the block's own maximum, so that its largest value is
+      // exactly 1 in fp16, and the block's output joins the running one in fp32
+      // (P relative to the running maximum has a 4 % larger error)
+      const float mn = fmaxf(m0, mx);  // finite: key0 < n_keys
+      const float c0 = exp2f(m0 - mn), c1 = exp2f(mx - mn);
+      const float mb = mx == -INFINITY ? 0.f : mx;  // a block of infinitely low scores adds nothing
+      m0 = mn;
+      float rs = 0.f;
+#pragma unroll
+      for (int n = 0; n < KB / 8; ++n) {
+        sc[n][0] = exp2f(sc[n][0] - mb);
+        sc[n][1] = exp2f(sc[n][1] - mb);
+        rs += sc[n][0] + sc[n][1];
+      }
+      // a lane's sums cover its own keys only; the quad adds them at the end
+      l0 = l0 * c0 + rs * c1;
+      uint32_t pa[KB / 16][4];
+#pragma unroll
+      for (int k2 = 0; k2 < KB / 16; ++k2) {
+        pa[k2][0] = pack_h2(sc[2 * k2][0], sc[2 * k2][1]);
+        pa[k2][2] = pack_h2(sc[2 * k2 + 1][0], sc[2 * k2 + 1][1]);
+        pa[k2][1] = pa[k2][3] = 0u;
+      }
+#pragma unroll
+      for (int dp = 0; dp < DN / 2; ++dp) {
+        float t0[4] = {0.f, 0.f, 0.f, 0.f}, t1[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int k2 = 0; k2 < KB / 16; ++k2) {
+          const int mat = lane >> 3;
+          const int key = k2 * 16 + (lane & 7) + 8 * (mat & 1);
+          const int dim = dp * 16 + 8 * (mat >> 1);
+          uint32_t bb[4];
+          ldsm_x4_t(bb, smem_u32(sV + key * LDS + dim));
+          mma16816(t0, pa[k2], bb[0], bb[1]);
+          mma16816(t1, pa[k2], bb[2], bb[3]);
+        }
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          o[2 * dp][e] = o[2 * dp][e] * c0 + t0[e] * c1;
+          o[2 * dp + 1][e] = o[2 * dp + 1][e] * c0 + t1[e] * c1;
+        }
+      }
+      __syncwarp();  // every lane is done with this slot before it is refilled
+    }
+    l0 += __shfl_xor_sync(0xffffffffu, l0, 1);
+    l0 += __shfl_xor_sync(0xffffffffu, l0, 2);
+    if (gq < G) {
+      __half* orow = a.out + static_cast<int64_t>(cur.r) * a.Hq * HD + (cur.h * G + gq) * HD;
+#pragma unroll
+      for (int d = 0; d < DN; ++d)
+        *reinterpret_cast<__half2*>(orow + d * 8 + 2 * tq) = __floats2half2_rn(o[d][0] / l0, o[d][1] / l0);
+    }
+    cur = nxt;
+    nxt = after;
+  }
+  cp_async_wait_all();
+}
+
 // Next token of each row from the LM head's packed (max, first index), the
 // pad mask after an eos, and the position the token takes when fed back.
 __global__ void k_decode_select(unsigned long long* best, int R, int t, int max_new, int eos, int pad, int V,
@@ -318,7 +537,25 @@ __global__ void k_gather_rows_i32(const int32_t* src, int width, const int32_t* 
 }
 
 template <int HD>
-int launch_dec(const DecArgs& a, int R, cudaStream_t s) {
+int launch_dec_stream(const DecArgs& a, int R, int num_sms, cudaStream_t s) {
+  using C = DecStream<HD>;
+  cudaError_t e =
+      cudaFuncSetAttribute(k_decode_attention_stream<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
+  if (e != cudaSuccess) return e;
+  const int64_t tasks = static_cast<int64_t>(R) * a.Hkv, full = static_cast<int64_t>(num_sms) * C::CTAS;
+  const int64_t need = (tasks + C::NW - 1) / C::NW;
+  k_decode_attention_stream<HD><<<static_cast<unsigned>(need < full ? need : full), C::NW * 32, C::SMEM, s>>>(
+      a, static_cast<int>(tasks));
+  return cudaGetLastError();
+}
+
+template <int HD>
+int launch_dec(const DecArgs& a, int R, int num_sms, cudaStream_t s) {
+  // A warp per task once every warp has four: fewer leave the last ones running
+  // alone (measured: 32/8 heads, head_dim 64, 500 rows of about 200 keys 80 -> 65
+  // us, but of about 500 keys 133 either way; head_dim 128, 500 long rows 213 -> 265).
+  using W = DecStream<HD>;
+  if (static_cast<int64_t>(R) * a.Hkv >= int64_t(4) * num_sms * W::CTAS * W::NW) return launch_dec_stream<HD>(a, R, num_sms, s);
   using C = DecCfg<HD>;
   cudaError_t e = cudaFuncSetAttribute(k_decode_attention<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
   if (e != cudaSuccess) return e;
@@ -330,7 +567,7 @@ int launch_dec(const DecArgs& a, int R, cudaStream_t s) {
 
 int launch_decode_attention(const __half* qkv, int64_t ldq, int R, int Hq, int Hkv, int hd, const __half* pkv, int P,
                             const __half* kvc, const int32_t* seq_start, __half* gkv, int gcap, int slot, __half* out,
-                            int* err, cudaStream_t s) {
+                            int* err, int num_sms, cudaStream_t s) {
   if (R <= 0) return 0;
   const int G = Hkv > 0 ? Hq / Hkv : 0;
   if (Hkv <= 0 || Hq % Hkv || !(G == 1 || G == 2 || G == 4 || G == 8) || !(hd == 32 || hd == 64 || hd == 128) ||
@@ -339,9 +576,9 @@ int launch_decode_attention(const __half* qkv, int64_t ldq, int R, int Hq, int H
   DecArgs a{qkv, ldq, Hq, Hkv, Hq / Hkv, pkv, P, kvc, seq_start, gkv, gcap, slot,
             1.4426950408889634f / sqrtf(static_cast<float>(hd)), out, err};
   switch (hd) {
-    case 32: return launch_dec<32>(a, R, s);
-    case 64: return launch_dec<64>(a, R, s);
-    default: return launch_dec<128>(a, R, s);
+    case 32: return launch_dec<32>(a, R, num_sms, s);
+    case 64: return launch_dec<64>(a, R, num_sms, s);
+    default: return launch_dec<128>(a, R, num_sms, s);
   }
 }
 

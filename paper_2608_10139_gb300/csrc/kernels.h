@@ -199,7 +199,7 @@ int launch_wait_expiry(uint64_t limit_ns, int* err, cudaStream_t s);
 // (keys then values).  Returns 0 or a cudaError_t value.
 int launch_decode_attention(const __half* qkv, int64_t ldq, int R, int Hq, int Hkv, int hd, const __half* pkv, int P,
                             const __half* kvc, const int32_t* seq_start, __half* gkv, int gcap, int slot, __half* out,
-                            int* err, cudaStream_t s);
+                            int* err, int num_sms, cudaStream_t s);
 // Token of step t for every row from the packed LM-head argmax (best[] is reset
 // to 0), pad after an eos, and the fed-back position P + len + t.
 void launch_decode_select(unsigned long long* best, int R, int t, int max_new, int eos, int pad, int V, int32_t* done,

@@ -213,3 +213,36 @@ def test_op_decode_attention_matches_fp32_reference(ctx, hd, hq, hkv):
             ref[r, h * hd:(h + 1) * hd] = p @ v
     got = out.float().cpu()
     assert torch.allclose(got, ref, rtol=2e-3, atol=2e-3), (got - ref).abs().max()
+
+
+@pytest.mark.parametrize("hd,hq,hkv", [(32, 4, 4), (64, 16, 8), (64, 8, 1), (128, 16, 4)])
+def test_op_decode_attention_many_rows(ctx, hd, hq, hkv):
+    """Batches large enough for a warp per (row, KV head): rows around the edges of a
+    key block (no prompt, one key short of a block, a full one, one over), against
+    fp64 and, slot for slot, the cache that the call appends to."""
+    torch = pytest.importorskip("torch")
+    g = torch.Generator(device="cuda").manual_seed(hd + hkv)
+    R, P, cap, slot = 10000 // hkv + 7, 3, 4, 2
+    lens = torch.tensor([0, 1, 9, 10, 11, 12, 25, 26, 27, 28, 58, 59, 90]).repeat(R // 13 + 1)[:R]
+    ss = torch.zeros(R + 1, dtype=torch.int32)
+    ss[1:] = torch.cumsum(lens, 0)
+    kd, T = hkv * hd, int(lens.sum())
+    rnd = lambda *n: torch.randn(*n, generator=g, device="cuda").half()  # noqa: E731
+    qkv, pkv, own, gen = rnd(R, (hq + 2 * hkv) * hd), rnd(P, 2 * kd), rnd(T, 2 * kd), rnd(R, cap, 2 * kd)
+    gen[:, slot + 1:] = float("nan")   # slots past this step's are never read
+    before, dss = gen.clone(), ss.cuda()
+    out = torch.empty(R, hq * hd, dtype=torch.float16, device="cuda")
+    torch.cuda.synchronize()
+    ctx.op_decode_attention(qkv.data_ptr(), R, hq, hkv, hd, own.data_ptr(), dss.data_ptr(), gen.data_ptr(), cap, slot,
+                            out.data_ptr(), pkv.data_ptr(), P)
+    torch.cuda.synchronize()
+    before[:, slot] = qkv[:, hq * hd:]
+    assert torch.equal(gen[:, :slot + 1], before[:, :slot + 1])
+    for r in list(range(26)) + list(range(R - 26, R)):
+        kv = torch.cat([pkv, own[ss[r]:ss[r + 1]], before[r, :slot + 1]]).double().view(-1, 2, hkv, hd)
+        k, v = (kv[:, i].repeat_interleave(hq // hkv, 1) for i in (0, 1))
+        q = qkv[r, :hq * hd].double().view(hq, hd)
+        p = (torch.einsum("hd,nhd->hn", q, k) / hd ** 0.5).softmax(-1)
+        ref = torch.einsum("hn,nhd->hd", p, v).flatten()
+        # fp16 probabilities and output: 2^-11 relative each, sums of |p v| at most max |v| (about 4.5)
+        assert (out[r].double() - ref).abs().max() <= 2 ** -11 * (ref.abs().max() + 2 * 4.5), r
