@@ -176,6 +176,8 @@ struct aiq_ctx {
   volatile int* h_err = nullptr;  // the kernels' error word, in mapped pinned host memory
   int* d_err = nullptr;           // its device address
   int64_t* h_pin = nullptr;  // pinned staging for control scalars
+  int64_t* d_pin = nullptr;  // its device address
+  unsigned int* d_arrived = nullptr;  // arrival counter of the tile-count scans (zero between launches)
   size_t bytes_max = SIZE_MAX;
   size_t bytes_used = 0;
   int64_t next_handle = 1;
@@ -415,12 +417,29 @@ ResultH& new_result(aiq_ctx* c, aiq_result_h* out) {
 
 // ----------------------------------------------------- relational phase ---
 
+constexpr int64_t kDirectBuildRows = int64_t(1) << 22;  // join: build rows hashed without compacting them first
+
 // Predicate (+ probe) over `t`, compaction into ids (and payload).  Returns S.
 aiq_status filter_compact(aiq_ctx* c, const TableD& t, const PredSet& ps, const ProbeSpec& probe, const char* tag,
                           int64_t* S_out, int32_t** ids_out, int32_t** payload_out) {
   const int64_t n = t.n_rows;
   const int64_t nb = (n + kRowsPerBlock - 1) / kRowsPerBlock;
   std::string b = tag;
+  ProbeSpec pr = probe;
+  int32_t* ids;
+  // a small table: one launch, where there is room for every row's id
+  if (!pr.keys && filter_is_small(n) && ws(c, (b + ".ids").c_str(), n, &ids) == AIQ_OK) {
+    {
+      ProfScope p(c, "predicate_mask", 0, 0);
+      launch_filter_small(ps, n, ids, c->d_pin, nullptr, c->stream);
+      counted(c, 1);
+    }
+    AIQ_TRY(sync_and_check(c));
+    *S_out = c->h_pin[0];
+    *ids_out = ids;
+    if (payload_out) *payload_out = nullptr;
+    return AIQ_OK;
+  }
   uint32_t* bits;
   int32_t* bcnt;
   int64_t* boff;
@@ -429,29 +448,21 @@ aiq_status filter_compact(aiq_ctx* c, const TableD& t, const PredSet& ps, const 
   AIQ_TRY(ws(c, (b + ".boff").c_str(), nb + 1, &boff));
   int64_t* scan_tmp;
   AIQ_TRY(ws(c, (b + ".scan").c_str(), 2 * (nb / kRowsPerBlock + 2), &scan_tmp));
-  ProbeSpec pr = probe;
   if (pr.keys) {
     AIQ_TRY(ws(c, (b + ".match").c_str(), std::max<int64_t>(n, 1), &pr.match_out));
   }
   {
     ProfScope p(c, "predicate_mask", 0, 0);
-    launch_predicate_mask(ps, pr, n, bits, bcnt, c->d_err, c->stream);
-    counted(c, n > 0);
+    counted(c, launch_predicate_scan(ps, pr, n, bits, bcnt, boff, c->d_arrived, c->d_pin, scan_tmp, c->stream));
   }
-  {
-    ProfScope p(c, "scan_tiles", 0, 0);
-    launch_scan_lengths(bcnt, nb, boff, scan_tmp, c->stream);
-    counted(c, nb > 0 ? 3 : 0);
-  }
-  AIQ_TRY(read_i64(c, boff + nb, 1, c->h_pin));
+  AIQ_TRY(sync_and_check(c));
   const int64_t S = c->h_pin[0];
-  int32_t* ids;
   AIQ_TRY(ws(c, (b + ".ids").c_str(), std::max<int64_t>(S, 1), &ids));
   int32_t* pay = nullptr;
   if (pr.keys) AIQ_TRY(ws(c, (b + ".payload").c_str(), std::max<int64_t>(S, 1), &pay));
   {
     ProfScope p(c, "compact", 0, 0);
-    launch_compact(bits, boff, n, ids, pr.match_out, pay, c->stream);
+    launch_compact(bits, boff, n, ids, pr.match_out, pay, c->stream, c->d_arrived);
     counted(c, n > 0);
   }
   *S_out = S;
@@ -1144,20 +1155,31 @@ aiq_status run_query(aiq_ctx* c, const TableD* build, int32_t build_key, const a
   if (build) {
     PredSet bps{};
     AIQ_TRY(make_pred_set(*build, build_preds, n_bp, &bps));
-    int64_t Sb = 0;
-    int32_t* bids;
-    AIQ_TRY(filter_compact(c, *build, bps, ProbeSpec{}, "jb", &Sb, &bids, nullptr));
+    const int64_t* bkeys = static_cast<const int64_t*>(build->cols[build_key].data);
     int64_t cap = 64;
-    while (cap < 2 * Sb) cap <<= 1;
-    unsigned long long* tk;
-    int32_t* tv;
-    AIQ_TRY(ws(c, "j.keys", cap, &tk));
-    AIQ_TRY(ws(c, "j.vals", cap, &tv));
-    {
+    while (cap < 2 * build->n_rows) cap <<= 1;
+    unsigned long long* tk = nullptr;
+    int32_t* tv = nullptr;
+    // Up to kDirectBuildRows build rows (100 MB of table) the rows that pass the
+    // terms go straight into a table sized for all rows; above, and where that
+    // table does not fit, they are compacted first and the table sized for them.
+    if (build->n_rows <= kDirectBuildRows && ws(c, "j.keys", cap, &tk) == AIQ_OK &&
+        ws(c, "j.vals", cap, &tv) == AIQ_OK) {
       ProfScope p(c, "hash_build", 0, 0);
       launch_fill_u64(tk, cap, 0x8000000000000000ull, c->stream);
-      launch_hash_build(static_cast<const int64_t*>(build->cols[build_key].data), bids, Sb, tk, tv, cap, c->d_err,
-                        c->stream);
+      launch_hash_build_where(bkeys, bps, build->n_rows, tk, tv, cap, c->d_err, c->stream);
+      counted(c, 1 + (build->n_rows > 0));
+    } else {
+      int64_t Sb = 0;
+      int32_t* bids;
+      AIQ_TRY(filter_compact(c, *build, bps, ProbeSpec{}, "jb", &Sb, &bids, nullptr));
+      cap = 64;
+      while (cap < 2 * Sb) cap <<= 1;
+      AIQ_TRY(ws(c, "j.keys", cap, &tk));
+      AIQ_TRY(ws(c, "j.vals", cap, &tv));
+      ProfScope p(c, "hash_build", 0, 0);
+      launch_fill_u64(tk, cap, 0x8000000000000000ull, c->stream);
+      launch_hash_build(bkeys, bids, Sb, tk, tv, cap, c->d_err, c->stream);
       counted(c, 1 + (Sb > 0));
     }
     pr.keys = static_cast<const int64_t*>(probe.cols[probe_key].data);
@@ -1525,9 +1547,14 @@ aiq_status aiq_init(int device, aiq_ctx** out) {
     *c->h_err = 0;
     e = cudaHostGetDevicePointer(reinterpret_cast<void**>(&c->d_err), word, 0);
   }
-  if (e == cudaSuccess) e = cudaMallocHost(&c->h_pin, 64 * sizeof(int64_t));
+  if (e == cudaSuccess) e = cudaHostAlloc(&c->h_pin, 64 * sizeof(int64_t), cudaHostAllocMapped);
+  if (e == cudaSuccess) e = cudaHostGetDevicePointer(&c->d_pin, c->h_pin, 0);
+  if (e == cudaSuccess) e = cudaMalloc(&c->d_arrived, sizeof(unsigned int));
+  if (e == cudaSuccess) e = cudaMemsetAsync(c->d_arrived, 0, sizeof(unsigned int), c->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) {
     cudaGetLastError();
+    if (c->d_arrived) cudaFree(c->d_arrived);
     if (c->h_pin) cudaFreeHost(c->h_pin);
     if (c->h_err) cudaFreeHost(const_cast<int*>(c->h_err));
     if (c->stream) cudaStreamDestroy(c->stream);
@@ -1552,6 +1579,7 @@ void aiq_shutdown(aiq_ctx* c) {
   }
   for (auto e : c->ev_pool) cudaEventDestroy(e);
   cudaFreeHost(const_cast<int*>(c->h_err));
+  cudaFree(c->d_arrived);
   cudaFreeHost(c->h_pin);
   cudaStreamDestroy(c->stream);
   delete c;

@@ -7,7 +7,7 @@
 // cudaMalloc's implicit device-wide synchronisation or its failure under
 // memory pressure.  aiq_filter_compact_static gives them the same kernels as
 // the query path (predicate bitmask, tile-count scan, compaction), with their
-// scratch (bitmask, tile counts, tile offsets) held in one file-scope device
+// scratch (bitmask, tile counts, tile offsets, arrival counter) held in one file-scope device
 // array instead of a context's workspace.
 //
 // The array is a global of this shared library: every GPU that loads the
@@ -37,7 +37,9 @@ constexpr size_t kBitsBytes = kStaticMaxRows / 8;                        // 2 Mi
 constexpr size_t kCountBytes = kStaticTiles * sizeof(int32_t);          // 32 KiB tile counts
 constexpr size_t kOffsetBytes = (kStaticTiles + 1) * sizeof(int64_t);   // 64 KiB + 8 tile offsets
 constexpr size_t kOffsetAt = kBitsBytes + kCountBytes;
-constexpr size_t kStaticScratchBytes = ((kOffsetAt + kOffsetBytes + 255) / 256) * 256;
+constexpr size_t kArrivedAt = ((kOffsetAt + kOffsetBytes + 255) / 256) * 256;  // arrival counter, zero between calls
+constexpr size_t kStaticScratchBytes = kArrivedAt + 256;
+static_assert(kStaticTiles <= kScanTilesMax, "the last block scans the tile counts");
 
 static __device__ __align__(256) unsigned char g_filter_scratch[kStaticScratchBytes];
 
@@ -73,8 +75,6 @@ aiq_status scratch_for_current_device(unsigned char** out) {
   return AIQ_OK;
 }
 
-__global__ void k_copy_count(const int64_t* src, int64_t* dst) { *dst = *src; }
-
 }  // namespace
 
 extern "C" {
@@ -103,15 +103,19 @@ aiq_status aiq_filter_compact_static(const aiq_term* terms, int32_t n_terms, int
   uint32_t* bits = reinterpret_cast<uint32_t*>(scratch);
   int32_t* counts = reinterpret_cast<int32_t*>(scratch + kBitsBytes);
   int64_t* offsets = reinterpret_cast<int64_t*>(scratch + kOffsetAt);
+  unsigned int* arrived = reinterpret_cast<unsigned int*>(scratch + kArrivedAt);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  const int64_t tiles = (n_rows + kRowsPerBlock - 1) / kRowsPerBlock;
-  // Every scratch word the compaction reads is written earlier in this call
-  // (each tile writes its whole bitmask slice and its count; the scan writes
-  // offsets[0..tiles]), so nothing is carried over from the previous call.
-  launch_predicate_mask(ps, ProbeSpec{}, n_rows, bits, counts, nullptr, s);
-  launch_scan_counts(counts, tiles, offsets, s);
-  launch_compact(bits, offsets, n_rows, ids_out, nullptr, nullptr, s);
-  k_copy_count<<<1, 1, 0, s>>>(offsets + tiles, count_out);
+  if (filter_is_small(n_rows)) {
+    launch_filter_small(ps, n_rows, ids_out, count_out, nullptr, s);
+  } else {
+    // Every scratch word the compaction reads is written earlier in this call
+    // (each tile writes its whole bitmask slice and its count; the scan writes
+    // offsets[0..tiles]), so nothing is carried over from the previous call but
+    // the arrival counter, which every scan leaves at zero.
+    launch_predicate_scan(ps, ProbeSpec{}, n_rows, bits, counts, offsets,
+                          arrived, count_out, nullptr, s);
+    launch_compact(bits, offsets, n_rows, ids_out, nullptr, nullptr, s, arrived);
+  }
   // A failed predicate launch is recorded (and its CUDA error consumed) by its
   // launcher; take that record here so that it is reported by this call and
   // not left behind for the next call on this host thread.

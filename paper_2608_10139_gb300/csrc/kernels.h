@@ -89,18 +89,41 @@ struct ProbeSpec {
   int32_t* match_out = nullptr;   // build row per probe row (valid where the bit is set)
 };
 
-// mask bits + per-block survivor counts.
-void launch_predicate_mask(const PredSet& ps, const ProbeSpec& probe, int64_t n_rows, uint32_t* bits,
-                           int32_t* block_counts, int* err, cudaStream_t s);
+// How the block that finishes last scans the tile counts (arrived == nullptr: it does not).
+struct TileScan {
+  const int32_t* counts;  // [tiles]
+  int64_t* offsets;       // [tiles + 1]
+  unsigned int* arrived;  // zero between launches
+  int64_t* total;         // optional: a second place for the total (host memory that the device maps)
+};
+constexpr int64_t kSmallRows = 16384;      // rows that one block filters on its own
+constexpr unsigned kScanTilesMax = 8192;   // tiles whose counts the last block scans
+
+// Filter of 1 .. kSmallRows rows (16-byte aligned columns) in one launch: the
+// survivors' ids and their number, in *count and, when given, *count2.
+bool filter_is_small(int64_t n_rows);
+void launch_filter_small(const PredSet& ps, int64_t n_rows, int32_t* ids, int64_t* count, int64_t* count2,
+                         cudaStream_t s);
+// Mask bits, per-tile survivor counts and their exclusive scan offsets[tiles + 1].
+// arrived: a counter that is zero before the first call; total (optional) also
+// receives the number of survivors; scan_tmp (optional): >= 2 * (ceil(tiles /
+// 2048) + 1) int64 for the multi-block scan.  Returns the number of kernels.
+int launch_predicate_scan(const PredSet& ps, const ProbeSpec& probe, int64_t n_rows, uint32_t* bits,
+                          int32_t* block_counts, int64_t* offsets, unsigned int* arrived, int64_t* total,
+                          int64_t* scan_tmp, cudaStream_t s);
 // Exclusive scan of n int32 counts into int64 offsets[n+1] (one block).
 void launch_scan_counts(const int32_t* counts, int64_t n, int64_t* offsets, cudaStream_t s);
 // Order-preserving compaction of set bits: ids_out[k] = row of the k-th set bit;
-// optionally gathers `payload[row]` into payload_out[k].
+// optionally gathers `payload[row]` into payload_out[k], and sets *arrived (a
+// scan's counter) to zero.
 void launch_compact(const uint32_t* bits, const int64_t* block_offsets, int64_t n_rows, int32_t* ids_out,
-                    const int32_t* payload, int32_t* payload_out, cudaStream_t s);
+                    const int32_t* payload, int32_t* payload_out, cudaStream_t s, unsigned int* arrived = nullptr);
 
 void launch_hash_build(const int64_t* keys, const int32_t* rows, int64_t n, unsigned long long* table_keys,
                        int32_t* table_vals, int64_t capacity, int* err, cudaStream_t s);
+// As launch_hash_build, for the rows 0 .. n - 1 that satisfy the terms.
+void launch_hash_build_where(const int64_t* keys, const PredSet& ps, int64_t n, unsigned long long* table_keys,
+                             int32_t* table_vals, int64_t capacity, int* err, cudaStream_t s);
 void launch_fill_u64(unsigned long long* p, int64_t n, unsigned long long v, cudaStream_t s);
 
 // ------------------------------------------------------------------ pack ---

@@ -7,7 +7,9 @@
 //    movies on movie id) runs in the same pass for rows that pass the terms.
 //  * order-preserving stream compaction: tile counts -> exclusive scan ->
 //    each tile re-reads only its 256-byte bitmask slice and writes the ids of
-//    its set bits at its offset (reduce-then-scan; no inter-block waits).
+//    its set bits at its offset (reduce-then-scan; no inter-block waits).  Up to
+//    kScanTilesMax tiles the block that finishes last scans the counts itself;
+//    up to kSmallRows rows one block does the whole filter.
 //  * open-addressing hash table (int64 key -> build row), linear probing with
 //    a bounded probe sequence.
 //  * decision (Fig. 2: strict yes > no, or first argmax) and the masked
@@ -93,8 +95,8 @@ __device__ __forceinline__ uint32_t cmp8(const T* v, int op, T c) {
   return bits;
 }
 
-__device__ __forceinline__ uint32_t eval_term(const PredDev& p, const TermRows& t) {
-  if (p.type == 1) return cmp8<int64_t>(reinterpret_cast<const int64_t*>(t.w), p.op, p.ivalue);
+// A term on a 4-byte column.
+__device__ __forceinline__ uint32_t eval_term4(const PredDev& p, const TermRows& t) {
   if (p.type == 2) return cmp8<float>(reinterpret_cast<const float*>(t.w), p.op, static_cast<float>(p.fvalue));
   // int32: a constant outside the int32 range decides every row alike (as the
   // SQL comparison in int64 would); inside it, compare in 32 bits
@@ -107,17 +109,9 @@ __device__ __forceinline__ uint32_t eval_term(const PredDev& p, const TermRows& 
   return cmp8<int32_t>(v, p.op, static_cast<int32_t>(p.ivalue));
 }
 
-__device__ __forceinline__ int probe_lookup(const ProbeSpec& pr, unsigned long long key) {
-  if (key == kEmptyKey) return -1;
-  const unsigned long long mask = static_cast<unsigned long long>(pr.capacity - 1);
-  unsigned long long slot = hash64(key) & mask;
-  for (int64_t i = 0; i < pr.capacity; ++i) {
-    const unsigned long long k = pr.table_keys[slot];
-    if (k == key) return pr.table_vals[slot];
-    if (k == kEmptyKey) return -1;
-    slot = (slot + 1) & mask;
-  }
-  return -1;
+__device__ __forceinline__ uint32_t eval_term(const PredDev& p, const TermRows& t) {
+  if (p.type == 1) return cmp8<int64_t>(reinterpret_cast<const int64_t*>(t.w), p.op, p.ivalue);
+  return eval_term4(p, t);
 }
 
 // Each thread holds one byte of row bits (rows 8*t .. 8*t+7 of the tile);
@@ -140,52 +134,13 @@ __device__ __forceinline__ int write_words_and_count(uint32_t byte, uint32_t* bi
   return total;
 }
 
-// Evaluates the terms (and the join probe) on one 2048-row tile; thread t
-// covers rows 8t .. 8t+7.  `stage` holds the tile's column chunks when the
-// tile is full; the ragged last tile reads global memory directly.
-__device__ __forceinline__ void predicate_tile(const PredSet& ps, const ProbeSpec& probe, int64_t n, int64_t tile,
-                                               const uint8_t* stage, const int* s_off, uint32_t* bits,
-                                               int32_t* block_counts, int* red) {
-  const int64_t r0 = tile * kRowsPerBlock + threadIdx.x * 8;
-  uint32_t byte = 0;
-  if (r0 < n) {
-    byte = r0 + 8 <= n ? 0xFFu : ((1u << (n - r0)) - 1u);
-    for (int i = 0; i < ps.n; ++i) {
-      TermRows t;
-      if (stage) {
-        const int4* src = reinterpret_cast<const int4*>(stage + s_off[i]) + threadIdx.x * (ps.p[i].type == 1 ? 4 : 2);
-        t.w[0] = src[0];
-        t.w[1] = src[1];
-        if (ps.p[i].type == 1) {
-          t.w[2] = src[2];
-          t.w[3] = src[3];
-        }
-      } else {
-        load_term(ps.p[i], r0, n, t);
-      }
-      byte &= eval_term(ps.p[i], t);
-    }
-    if (probe.keys) {
-#pragma unroll 1
-      for (int j = 0; j < 8; ++j) {
-        if (byte & (1u << j)) {
-          const int m = probe_lookup(probe, static_cast<unsigned long long>(probe.keys[r0 + j]));
-          if (m < 0) byte &= ~(1u << j);
-          else probe.match_out[r0 + j] = m;
-        }
-      }
-    }
-  }
-  const int total = write_words_and_count(byte, bits + tile * (kRowsPerBlock / 32), red);
-  if (threadIdx.x == 0) block_counts[tile] = total;
-}
-
-// One 2048-row tile per block.  Thread 0 first asks the bulk-copy engine to
-// pull every term's column chunk of the tile (2048 x 4 or 8 bytes) into L2,
+// Any number of terms (also none, or more than four): one 2048-row tile per
+// block, thread t on rows 8t .. 8t+7.  Thread 0 first asks the bulk-copy engine to
+// pull every later term's column chunk of the tile (2048 x 4 or 8 bytes) into L2,
 // so all columns stream from DRAM at once while each thread's own 16-byte
 // loads of successive terms follow one after the other.
-__global__ void __launch_bounds__(kThreads) k_predicate_mask(PredSet ps, ProbeSpec probe, int64_t n, uint32_t* bits,
-                                                             int32_t* block_counts, int* err) {
+__global__ void __launch_bounds__(kThreads) k_predicate_mask(PredSet ps, int64_t n, uint32_t* bits,
+                                                             int32_t* block_counts) {
   __shared__ int red[kThreads / 32];
   const int64_t tile = blockIdx.x;
   if (threadIdx.x == 0 && (tile + 1) * kRowsPerBlock <= n) {
@@ -197,52 +152,155 @@ __global__ void __launch_bounds__(kThreads) k_predicate_mask(PredSet ps, ProbeSp
                    : "memory");
     }
   }
-  predicate_tile(ps, probe, n, tile, nullptr, nullptr, bits, block_counts, red);
-  (void)err;
+  const int64_t r0 = tile * kRowsPerBlock + threadIdx.x * 8;
+  uint32_t byte = 0;
+  if (r0 < n) {
+    byte = r0 + 8 <= n ? 0xFFu : ((1u << (n - r0)) - 1u);
+    for (int i = 0; i < ps.n; ++i) {
+      TermRows t;
+      load_term(ps.p[i], r0, n, t);
+      byte &= eval_term(ps.p[i], t);
+    }
+  }
+  const int total = write_words_and_count(byte, bits + tile * (kRowsPerBlock / 32), red);
+  if (threadIdx.x == 0) block_counts[tile] = total;
 }
 
-// The common case, 1..4 terms on 4-byte columns and no join probe: every
-// term's loads are issued before the first compare, in a coalesced layout
-// (lane l of warp w takes rows 4l..4l+3 and 128+4l..128+4l+3 of the warp's
-// 256 rows, so one 16-byte load instruction covers 512 contiguous bytes),
-// and eight lanes' nibbles form one bitmask word.  Same bitmask and tile
-// counts as k_predicate_mask.
+// Block-wide exclusive scan of one int per thread (NT threads).
 template <int NT>
-__global__ void __launch_bounds__(kThreads) k_predicate_mask4(PredSet ps, int64_t n, uint32_t* bits,
-                                                              int32_t* block_counts) {
+__device__ __forceinline__ int block_excl_scan(int v, int* sh, int* total) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int x = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    int y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) sh[warp] = x;
+  __syncthreads();
+  if (warp == 0) {
+    int s = lane < NT / 32 ? sh[lane] : 0;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      int y = __shfl_up_sync(0xffffffffu, s, o);
+      if (lane >= o) s += y;
+    }
+    if (lane < NT / 32) sh[lane] = s;
+  }
+  __syncthreads();
+  const int before = warp ? sh[warp - 1] : 0;
+  *total = sh[NT / 32 - 1];
+  return before + x - v;
+}
+
+// Called by every thread of every block once its tile's count is written (by
+// thread 0): the block that arrives last scans all counts into offsets, writes
+// the total wherever it is wanted and leaves the arrival counter at zero for the
+// next launch.  No block waits for another.
+template <int NT>
+__device__ __forceinline__ void scan_in_last_block(const TileScan& ts) {
+  __shared__ int sh[NT / 32];
+  __shared__ int last;
+  if (threadIdx.x == 0) {
+    __threadfence();  // the count before the arrival
+    last = atomicAdd(ts.arrived, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();  // the arrivals before the other blocks' counts
+  constexpr int kPer = 16;
+  const int64_t n = gridDim.x;
+  int64_t carry = 0;
+  for (int64_t base = 0; base < n; base += NT * kPer) {
+    const int64_t i0 = base + threadIdx.x * kPer;
+    int v[kPer];
+    int s = 0;
+#pragma unroll
+    for (int j = 0; j < kPer; j += 4) {
+      if (i0 + j + 4 <= n) {
+        *reinterpret_cast<int4*>(v + j) = __ldcg(reinterpret_cast<const int4*>(ts.counts + i0 + j));
+      } else {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[j + k] = i0 + j + k < n ? __ldcg(ts.counts + i0 + j + k) : 0;
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) s += v[j];
+    int total;
+    int64_t run = carry + block_excl_scan<NT>(s, sh, &total);
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+      if (i0 + j < n) ts.offsets[i0 + j] = run;
+      run += v[j];
+    }
+    carry += total;
+    __syncthreads();  // sh is reused
+  }
+  if (threadIdx.x == 0) {
+    ts.offsets[n] = carry;
+    if (ts.total) *ts.total = carry;
+    *ts.arrived = 0;
+  }
+}
+
+// 1..4 terms and no join probe (every workload's filter): N8 terms on int64
+// columns, then N4 on 4-byte ones.  Every term's loads are issued before the
+// first compare, in a coalesced layout (lane l of warp w takes rows 4l..4l+3 and
+// 128+4l..128+4l+3 of the warp's 256 rows, so one 16-byte load instruction covers
+// 512 contiguous bytes), and eight lanes' nibbles form one bitmask word.  Same
+// bitmask and tile counts as k_predicate_mask, whose terms load one after the
+// other.  4,195,081 rows of an int32, an int64 and a float32 term (67 MB) take 18.7
+// us from a cold cache with the counts' scan in the last block, against 15.5 us for
+// k_predicate_mask plus 7.4 for a scan and a copy of the count in launches of their own.
+template <int N8, int N4>
+__global__ void __launch_bounds__(kThreads) k_predicate_cols(PredSet ps, int64_t n, uint32_t* bits,
+                                                             int32_t* block_counts, TileScan ts) {
   __shared__ int red[kThreads / 32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t ra = static_cast<int64_t>(blockIdx.x) * kRowsPerBlock + warp * 256 + lane * 4;
   const int64_t rb = ra + 128;
-  int4 va[NT], vb[NT];
+  TermRows t[N8 + N4];
   const bool full = rb + 4 <= n;
 #pragma unroll
-  for (int i = 0; i < NT; ++i) {
-    const int32_t* c = static_cast<const int32_t*>(ps.p[i].col);
-    if (full) {
-      va[i] = __ldg(reinterpret_cast<const int4*>(c + ra));
-      vb[i] = __ldg(reinterpret_cast<const int4*>(c + rb));
-    } else {
-      int32_t* x = reinterpret_cast<int32_t*>(&va[i]);
-      int32_t* y = reinterpret_cast<int32_t*>(&vb[i]);
+  for (int i = 0; i < N8 + N4; ++i) {
+    if (i < N8) {
+      const int64_t* c = static_cast<const int64_t*>(ps.p[i].col);
+      if (full) {
+        t[i].w[0] = __ldg(reinterpret_cast<const int4*>(c + ra));
+        t[i].w[1] = __ldg(reinterpret_cast<const int4*>(c + ra) + 1);
+        t[i].w[2] = __ldg(reinterpret_cast<const int4*>(c + rb));
+        t[i].w[3] = __ldg(reinterpret_cast<const int4*>(c + rb) + 1);
+      } else {
+        int64_t* v = reinterpret_cast<int64_t*>(t[i].w);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        x[j] = ra + j < n ? c[ra + j] : 0;
-        y[j] = rb + j < n ? c[rb + j] : 0;
+        for (int j = 0; j < 4; ++j) {
+          v[j] = ra + j < n ? c[ra + j] : 0;
+          v[4 + j] = rb + j < n ? c[rb + j] : 0;
+        }
+      }
+    } else {
+      const int32_t* c = static_cast<const int32_t*>(ps.p[i].col);
+      if (full) {
+        t[i].w[0] = __ldg(reinterpret_cast<const int4*>(c + ra));
+        t[i].w[1] = __ldg(reinterpret_cast<const int4*>(c + rb));
+      } else {
+        int32_t* v = reinterpret_cast<int32_t*>(t[i].w);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          v[j] = ra + j < n ? c[ra + j] : 0;
+          v[4 + j] = rb + j < n ? c[rb + j] : 0;
+        }
       }
     }
   }
   uint32_t byte = 0;
 #pragma unroll
   for (int j = 0; j < 4; ++j) byte |= (static_cast<uint32_t>(ra + j < n) << j) | (static_cast<uint32_t>(rb + j < n) << (4 + j));
+  // value j < 4 of a term is row ra + j, value 4 + j is row rb + j
 #pragma unroll
-  for (int i = 0; i < NT; ++i) {
-    TermRows t;
-    t.w[0] = va[i];
-    t.w[1] = vb[i];
-    // eval_term's value j < 4 is row ra + j, value 4 + j is row rb + j
-    byte &= eval_term(ps.p[i], t);
-  }
+  for (int i = 0; i < N8 + N4; ++i)
+    byte &= i < N8 ? cmp8<int64_t>(reinterpret_cast<const int64_t*>(t[i].w), ps.p[i].op, ps.p[i].ivalue)
+                   : eval_term4(ps.p[i], t[i]);
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     uint32_t w = ((byte >> (4 * h)) & 0xFu) << (4 * (lane & 7));
@@ -261,34 +319,154 @@ __global__ void __launch_bounds__(kThreads) k_predicate_mask4(PredSet ps, int64_
     for (int i = 0; i < kThreads / 32; ++i) total += red[i];
     block_counts[blockIdx.x] = total;
   }
+  if (ts.arrived) scan_in_last_block<kThreads>(ts);
 }
 
-// Block-wide exclusive scan of one int per thread (kThreads threads).
-__device__ __forceinline__ int block_excl_scan(int v, int* sh, int* total) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int x = v;
+// A term's 4 result bits for rows r0 .. r0 + 3 (r0 a multiple of 4).
+__device__ __forceinline__ uint32_t eval_rows4(const PredDev& p, int64_t r0, int64_t n) {
+  TermRows t;
+  const bool full = r0 + 4 <= n;
+  if (p.type == 1) {
+    const int64_t* c = static_cast<const int64_t*>(p.col) + r0;
+    int64_t* v = reinterpret_cast<int64_t*>(t.w);
+    if (full) {
+      t.w[0] = __ldg(reinterpret_cast<const int4*>(c));
+      t.w[1] = __ldg(reinterpret_cast<const int4*>(c) + 1);
+    } else {
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    int y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
-  }
-  if (lane == 31) sh[warp] = x;
-  __syncthreads();
-  if (warp == 0) {
-    int s = lane < kThreads / 32 ? sh[lane] : 0;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      int y = __shfl_up_sync(0xffffffffu, s, o);
-      if (lane >= o) s += y;
+      for (int j = 0; j < 4; ++j) v[j] = r0 + j < n ? c[j] : 0;
     }
-    if (lane < kThreads / 32) sh[lane] = s;
+#pragma unroll
+    for (int j = 4; j < 8; ++j) v[j] = 0;
+    return cmp8<int64_t>(v, p.op, p.ivalue) & 0xFu;
   }
-  __syncthreads();
-  const int before = warp ? sh[warp - 1] : 0;
-  *total = sh[kThreads / 32 - 1];
-  return before + x - v;
+  const int32_t* c = static_cast<const int32_t*>(p.col) + r0;
+  int32_t* v = reinterpret_cast<int32_t*>(t.w);
+  if (full) {
+    t.w[0] = __ldg(reinterpret_cast<const int4*>(c));
+  } else {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v[j] = r0 + j < n ? c[j] : 0;
+  }
+#pragma unroll
+  for (int j = 4; j < 8; ++j) v[j] = 0;
+  return eval_term4(p, t) & 0xFu;
 }
 
+constexpr int kProbeThreads = 512;  // x 4 rows = kRowsPerBlock
+
+// The terms and the join probe of one 2048-row tile.  A thread's four keys are
+// hashed together and their table slots read together (a probe is a chain of
+// dependent reads: 500,000 rows took 14.7 us with eight in turn and 9.6 for the
+// scan's three launches, 12.5 now with the scan); collisions walk on for the keys
+// that are left.
+__global__ void __launch_bounds__(kProbeThreads) k_probe_mask(PredSet ps, ProbeSpec probe, int64_t n, uint32_t* bits,
+                                                              int32_t* block_counts, TileScan ts) {
+  __shared__ int red[kProbeThreads / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t r0 = static_cast<int64_t>(blockIdx.x) * kRowsPerBlock + threadIdx.x * 4;
+  uint32_t nib = 0;
+  if (r0 < n) {
+    nib = r0 + 4 <= n ? 0xFu : ((1u << (n - r0)) - 1u);
+    unsigned long long key[4];
+    if (r0 + 4 <= n) {
+      const ulonglong2 a = __ldg(reinterpret_cast<const ulonglong2*>(probe.keys + r0));
+      const ulonglong2 b = __ldg(reinterpret_cast<const ulonglong2*>(probe.keys + r0) + 1);
+      key[0] = a.x, key[1] = a.y, key[2] = b.x, key[3] = b.y;
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) key[j] = r0 + j < n ? static_cast<unsigned long long>(probe.keys[r0 + j]) : kEmptyKey;
+    }
+    for (int i = 0; i < ps.n; ++i) nib &= eval_rows4(ps.p[i], r0, n);
+    const unsigned long long mask = static_cast<unsigned long long>(probe.capacity - 1);
+    unsigned long long slot[4];
+    uint32_t open = 0;  // keys still looked for
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      slot[j] = hash64(key[j]) & mask;
+      open |= static_cast<uint32_t>(((nib >> j) & 1u) && key[j] != kEmptyKey) << j;
+    }
+    nib &= open;
+    for (int64_t step = 0; open && step < probe.capacity; ++step) {
+      unsigned long long k[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if ((open >> j) & 1u) k[j] = probe.table_keys[slot[j]];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if (!((open >> j) & 1u)) continue;
+        if (k[j] == key[j]) {
+          open &= ~(1u << j);  // found; slot[j] is its slot
+        } else if (k[j] == kEmptyKey) {
+          open &= ~(1u << j);
+          nib &= ~(1u << j);
+        } else {
+          slot[j] = (slot[j] + 1) & mask;
+        }
+      }
+    }
+    nib &= ~open;  // a table without an empty slot: every slot has been looked at
+    int m[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) m[j] = (nib >> j) & 1u ? probe.table_vals[slot[j]] : -1;
+    if (r0 + 4 <= n)
+      *reinterpret_cast<int4*>(probe.match_out + r0) = make_int4(m[0], m[1], m[2], m[3]);
+    else
+      for (int j = 0; r0 + j < n; ++j) probe.match_out[r0 + j] = m[j];
+  }
+  uint32_t w = nib << (4 * (lane & 7));
+  w |= __shfl_xor_sync(0xffffffffu, w, 1);
+  w |= __shfl_xor_sync(0xffffffffu, w, 2);
+  w |= __shfl_xor_sync(0xffffffffu, w, 4);
+  if ((lane & 7) == 0) bits[blockIdx.x * int64_t(kRowsPerBlock / 32) + warp * 4 + (lane >> 3)] = w;
+  int c = __popc(nib);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+  if (lane == 0) red[warp] = c;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int total = 0;
+    for (int i = 0; i < kProbeThreads / 32; ++i) total += red[i];
+    block_counts[blockIdx.x] = total;
+  }
+  if (ts.arrived) scan_in_last_block<kProbeThreads>(ts);
+}
+
+constexpr int kSmallThreads = 1024;
+
+// The whole filter of a small table in one block: each pass evaluates 8 rows a
+// thread, scans the survivor counts and writes the ids.  At these sizes a launch
+// costs more than the rows: a call on 10,007 rows takes 8.0 us in one launch,
+// against 14.7 in four.
+__global__ void __launch_bounds__(kSmallThreads) k_filter_small(PredSet ps, int64_t n, int32_t* ids, int64_t* count,
+                                                                int64_t* count2) {
+  __shared__ int sh[kSmallThreads / 32];
+  int base = 0;
+  for (int64_t p0 = 0; p0 < n; p0 += kSmallThreads * 8) {
+    const int64_t r0 = p0 + threadIdx.x * 8;
+    uint32_t byte = 0;
+    if (r0 < n) {
+      byte = r0 + 8 <= n ? 0xFFu : ((1u << (n - r0)) - 1u);
+      for (int i = 0; i < ps.n; ++i) {
+        TermRows t;
+        load_term(ps.p[i], r0, n, t);
+        byte &= eval_term(ps.p[i], t);
+      }
+    }
+    int total;
+    int at = base + block_excl_scan<kSmallThreads>(__popc(byte), sh, &total);
+    for (uint32_t b = byte; b; b &= b - 1) ids[at++] = static_cast<int32_t>(r0) + __ffs(b) - 1;
+    base += total;
+    __syncthreads();  // sh is reused
+  }
+  if (threadIdx.x == 0) {
+    *count = base;
+    if (count2) *count2 = base;
+  }
+}
+
+constexpr unsigned kWideTilesMax = 488;          // k_compact_wide without a payload
+constexpr unsigned kWidePayloadTilesMax = 2432;  // and with one: 16 blocks per SM
 constexpr int kCompactWarps = 4;  // warps (= 2048-row tiles at a time) per compaction block
 
 // One warp per 2048-row tile: lane l owns bitmask words l and 32 + l of the
@@ -297,11 +475,14 @@ constexpr int kCompactWarps = 4;  // warps (= 2048-row tiles at a time) per comp
 // row offsets of its word's set bits, in order, into the warp's own 16-bit
 // shared-memory slice; the slice is then written out as one coalesced run of
 // ids.  No block-wide barrier is involved.  A payload (the join's build row
-// per probe row) is gathered straight to its output position (PAYLOAD).
+// per probe row) is gathered in that last loop (PAYLOAD): in the set-bit loop each
+// gather stalled its lane (8.5 us for 500,000 probe rows).
 template <bool PAYLOAD>
 __global__ void __launch_bounds__(kCompactWarps * 32) k_compact(const uint32_t* bits, const int64_t* block_offsets,
                                                                 int64_t n, int32_t* ids, const int32_t* payload,
-                                                                int32_t* payload_out) {
+                                                                int32_t* payload_out, unsigned int* arrived) {
+  // calls that overlap against the rules may leave the scan's counter behind: the next ones start from zero
+  if (arrived && blockIdx.x == 0 && threadIdx.x == 0) *arrived = 0;
   __shared__ uint16_t s_ids[kCompactWarps][kRowsPerBlock];  // row offsets within the tile
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t n_tiles = (n + kRowsPerBlock - 1) / kRowsPerBlock;
@@ -328,13 +509,48 @@ __global__ void __launch_bounds__(kCompactWarps * 32) k_compact(const uint32_t* 
         const int j = __ffs(b) - 1;
         b &= b - 1;
         s_ids[warp][at] = static_cast<uint16_t>(base + j);
-        if (PAYLOAD) payload_out[out + at] = payload[tile0 + base + j];  // joins: a gather, written in place
         ++at;
       }
       at0 += __shfl_sync(0xffffffffu, incl, 31);
     }
     __syncwarp();
-    for (int i = lane; i < at0; i += 32) ids[out + i] = static_cast<int32_t>(tile0 + s_ids[warp][i]);
+    for (int i = lane; i < at0; i += 32) {
+      const int64_t row = tile0 + s_ids[warp][i];
+      ids[out + i] = static_cast<int32_t>(row);
+      if (PAYLOAD) payload_out[out + i] = payload[row];
+    }
+  }
+}
+
+// The same for few tiles: a block per tile, 8 rows a thread, so that a tile's ids
+// and payload gathers are all in flight together (a warp per tile leaves most of
+// the GPU idle and walks them in turn: 500,000 rows with a payload 11.5 us, here
+// 3.8).  Without a payload the two are even at 489 tiles (3.6 us) and a warp per
+// tile is the faster above (2049 tiles: 4.4 us against 5.1).
+template <bool PAYLOAD>
+__global__ void __launch_bounds__(kThreads) k_compact_wide(const uint32_t* bits, const int64_t* block_offsets,
+                                                           int32_t* ids, const int32_t* payload, int32_t* payload_out,
+                                                           unsigned int* arrived) {
+  __shared__ int sh[kThreads / 32];
+  if (arrived && blockIdx.x == 0 && threadIdx.x == 0) *arrived = 0;  // as k_compact
+  const int64_t tile = blockIdx.x;
+  const uint32_t byte = reinterpret_cast<const uint8_t*>(bits + tile * (kRowsPerBlock / 32))[threadIdx.x];
+  const int64_t out = block_offsets[tile];
+  const int64_t r0 = tile * kRowsPerBlock + threadIdx.x * 8;
+  int m[8];
+  if (PAYLOAD) {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) m[j] = (byte >> j) & 1u ? __ldg(payload + r0 + j) : 0;
+  }
+  int total;
+  int64_t at = out + block_excl_scan<kThreads>(__popc(byte), sh, &total);
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    if ((byte >> j) & 1u) {
+      ids[at] = static_cast<int32_t>(r0 + j);
+      if (PAYLOAD) payload_out[at] = m[j];
+      ++at;
+    }
   }
 }
 
@@ -396,7 +612,7 @@ __global__ void __launch_bounds__(kThreads) k_tile_scan(const int32_t* in, int64
     s += v[j];
   }
   int total;
-  int pre = block_excl_scan(s, sh, &total);
+  int pre = block_excl_scan<kThreads>(s, sh, &total);
   int64_t run = tile_off[blockIdx.x] + pre;
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
@@ -408,12 +624,8 @@ __global__ void __launch_bounds__(kThreads) k_tile_scan(const int32_t* in, int64
 
 // ----------------------------------------------------------- hash build ---
 
-__global__ void k_hash_build(const int64_t* keys, const int32_t* rows, int64_t n, unsigned long long* tk,
-                             int32_t* tv, int64_t cap, int* err) {
-  const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const int32_t row = rows[i];
-  const unsigned long long key = static_cast<unsigned long long>(keys[row]);
+__device__ __forceinline__ void hash_insert(unsigned long long key, int32_t row, unsigned long long* tk, int32_t* tv,
+                                            int64_t cap, int* err) {
   if (key == kEmptyKey) {
     set_dev_error(err, DEVERR_SENTINEL_KEY);
     return;
@@ -433,6 +645,33 @@ __global__ void k_hash_build(const int64_t* keys, const int32_t* rows, int64_t n
     slot = (slot + 1) & mask;
   }
   set_dev_error(err, DEVERR_HASH_FULL);
+}
+
+// The build rows given by id.
+__global__ void k_hash_build(const int64_t* keys, const int32_t* rows, int64_t n, unsigned long long* tk,
+                             int32_t* tv, int64_t cap, int* err) {
+  const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  hash_insert(static_cast<unsigned long long>(keys[rows[i]]), rows[i], tk, tv, cap, err);
+}
+
+// The build rows that satisfy the terms, straight from the columns: the table is
+// sized for all rows, so that neither their ids nor their number is needed first.
+__global__ void k_hash_build_where(const int64_t* keys, PredSet ps, int64_t n, unsigned long long* tk, int32_t* tv,
+                                   int64_t cap, int* err) {
+  const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const unsigned long long key = static_cast<unsigned long long>(keys[i]);
+  uint32_t pass = 1;
+  for (int t = 0; t < ps.n; ++t) {
+    TermRows v{};
+    if (ps.p[t].type == 1)
+      reinterpret_cast<int64_t*>(v.w)[0] = static_cast<const int64_t*>(ps.p[t].col)[i];
+    else
+      v.w[0].x = static_cast<const int32_t*>(ps.p[t].col)[i];
+    pass &= eval_term(ps.p[t], v);
+  }
+  if (pass & 1u) hash_insert(key, static_cast<int32_t>(i), tk, tv, cap, err);
 }
 
 __global__ void k_fill_u64(unsigned long long* p, int64_t n, unsigned long long v) {
@@ -562,22 +801,81 @@ inline unsigned blocks_for(int64_t n, int64_t per) { return static_cast<unsigned
 
 }  // namespace
 
-void launch_predicate_mask(const PredSet& ps, const ProbeSpec& probe, int64_t n_rows, uint32_t* bits,
-                           int32_t* block_counts, int* err, cudaStream_t s) {
-  if (n_rows <= 0) return;
+namespace {
+
+template <int N8>
+void launch_cols(int n4, unsigned grid, const PredSet& ps, int64_t n, uint32_t* bits, int32_t* counts,
+                 const TileScan& ts, cudaStream_t s) {
+  switch (n4) {
+    case 0:
+      if constexpr (N8 > 0) k_predicate_cols<N8, 0><<<grid, kThreads, 0, s>>>(ps, n, bits, counts, ts);
+      break;
+    case 1:
+      if constexpr (N8 < 4) k_predicate_cols<N8, 1><<<grid, kThreads, 0, s>>>(ps, n, bits, counts, ts);
+      break;
+    case 2:
+      if constexpr (N8 < 3) k_predicate_cols<N8, 2><<<grid, kThreads, 0, s>>>(ps, n, bits, counts, ts);
+      break;
+    case 3:
+      if constexpr (N8 < 2) k_predicate_cols<N8, 3><<<grid, kThreads, 0, s>>>(ps, n, bits, counts, ts);
+      break;
+    default:
+      if constexpr (N8 < 1) k_predicate_cols<N8, 4><<<grid, kThreads, 0, s>>>(ps, n, bits, counts, ts);
+      break;
+  }
+}
+
+// The terms on int64 columns first (k_predicate_cols); a conjunction has no order.
+PredSet wide_first(const PredSet& ps, int* n8) {
+  PredSet o = ps;
+  int at = 0;
+  for (int wide = 1; wide >= 0; --wide)
+    for (int i = 0; i < ps.n; ++i)
+      if ((ps.p[i].type == 1) == (wide == 1)) o.p[at++] = ps.p[i];
+  *n8 = 0;
+  while (*n8 < ps.n && o.p[*n8].type == 1) ++*n8;
+  return o;
+}
+
+}  // namespace
+
+bool filter_is_small(int64_t n_rows) { return n_rows > 0 && n_rows <= kSmallRows; }
+
+void launch_filter_small(const PredSet& ps, int64_t n_rows, int32_t* ids, int64_t* count, int64_t* count2,
+                         cudaStream_t s) {
+  k_filter_small<<<1, kSmallThreads, 0, s>>>(ps, n_rows, ids, count, count2);
+}
+
+int launch_predicate_scan(const PredSet& ps, const ProbeSpec& probe, int64_t n_rows, uint32_t* bits,
+                          int32_t* block_counts, int64_t* offsets, unsigned int* arrived, int64_t* total,
+                          int64_t* scan_tmp, cudaStream_t s) {
+  if (n_rows <= 0) {
+    cudaMemsetAsync(offsets, 0, sizeof(int64_t), s);
+    if (total) cudaMemcpyAsync(total, offsets, sizeof(int64_t), cudaMemcpyDefault, s);
+    return 0;
+  }
   const unsigned grid = blocks_for(n_rows, kRowsPerBlock);
-  bool four = ps.n >= 1 && ps.n <= 4 && !probe.keys;
-  for (int i = 0; i < ps.n; ++i)
-    four = four && ps.p[i].type != 1 && (reinterpret_cast<uintptr_t>(ps.p[i].col) & 15) == 0;
-  if (four) {
-    switch (ps.n) {
-      case 1: k_predicate_mask4<1><<<grid, kThreads, 0, s>>>(ps, n_rows, bits, block_counts); break;
-      case 2: k_predicate_mask4<2><<<grid, kThreads, 0, s>>>(ps, n_rows, bits, block_counts); break;
-      case 3: k_predicate_mask4<3><<<grid, kThreads, 0, s>>>(ps, n_rows, bits, block_counts); break;
-      default: k_predicate_mask4<4><<<grid, kThreads, 0, s>>>(ps, n_rows, bits, block_counts); break;
+  bool aligned = true;
+  for (int i = 0; i < ps.n; ++i) aligned = aligned && (reinterpret_cast<uintptr_t>(ps.p[i].col) & 15) == 0;
+  // One block scans 2048 counts a microsecond: past kScanTilesMax tiles the
+  // three-kernel scan, whose blocks share the counts, is the faster.
+  TileScan ts{block_counts, offsets, grid <= kScanTilesMax ? arrived : nullptr, total};
+  bool fused = ts.arrived != nullptr;
+  if (probe.keys) {
+    k_probe_mask<<<grid, kProbeThreads, 0, s>>>(ps, probe, n_rows, bits, block_counts, ts);
+  } else if (ps.n >= 1 && ps.n <= 4 && aligned) {
+    int n8 = 0;
+    const PredSet o = wide_first(ps, &n8);
+    switch (n8) {
+      case 0: launch_cols<0>(o.n, grid, o, n_rows, bits, block_counts, ts, s); break;
+      case 1: launch_cols<1>(o.n - 1, grid, o, n_rows, bits, block_counts, ts, s); break;
+      case 2: launch_cols<2>(o.n - 2, grid, o, n_rows, bits, block_counts, ts, s); break;
+      case 3: launch_cols<3>(o.n - 3, grid, o, n_rows, bits, block_counts, ts, s); break;
+      default: launch_cols<4>(0, grid, o, n_rows, bits, block_counts, ts, s); break;
     }
   } else {
-    k_predicate_mask<<<grid, kThreads, 0, s>>>(ps, probe, n_rows, bits, block_counts, err);
+    k_predicate_mask<<<grid, kThreads, 0, s>>>(ps, n_rows, bits, block_counts);
+    fused = false;
   }
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
@@ -585,6 +883,16 @@ void launch_predicate_mask(const PredSet& ps, const ProbeSpec& probe, int64_t n_
     snprintf(buf, sizeof(buf), "predicate mask launch (grid %u, terms %d)", grid, ps.n);
     set_launch_error(buf, e);
   }
+  if (fused) return 1;
+  int launches = 4;
+  if (scan_tmp) {
+    launch_scan_lengths(block_counts, grid, offsets, scan_tmp, s);
+  } else {
+    launch_scan_counts(block_counts, grid, offsets, s);
+    launches = 2;
+  }
+  if (total) cudaMemcpyAsync(total, offsets + grid, sizeof(int64_t), cudaMemcpyDefault, s);
+  return launches;
 }
 
 void launch_scan_counts(const int32_t* counts, int64_t n, int64_t* offsets, cudaStream_t s) {
@@ -592,19 +900,35 @@ void launch_scan_counts(const int32_t* counts, int64_t n, int64_t* offsets, cuda
 }
 
 void launch_compact(const uint32_t* bits, const int64_t* block_offsets, int64_t n_rows, int32_t* ids_out,
-                    const int32_t* payload, int32_t* payload_out, cudaStream_t s) {
+                    const int32_t* payload, int32_t* payload_out, cudaStream_t s, unsigned int* arrived) {
   if (n_rows <= 0) return;
-  const unsigned grid = blocks_for(n_rows, int64_t(kRowsPerBlock) * kCompactWarps);  // one tile per warp
+  const unsigned tiles = blocks_for(n_rows, kRowsPerBlock);
+  if (tiles <= (payload_out ? kWidePayloadTilesMax : kWideTilesMax)) {
+    if (payload_out)
+      k_compact_wide<true><<<tiles, kThreads, 0, s>>>(bits, block_offsets, ids_out, payload, payload_out, arrived);
+    else
+      k_compact_wide<false><<<tiles, kThreads, 0, s>>>(bits, block_offsets, ids_out, payload, payload_out, arrived);
+    return;
+  }
+  const unsigned grid = (tiles + kCompactWarps - 1) / kCompactWarps;  // one tile per warp
   if (payload_out)
-    k_compact<true><<<grid, kCompactWarps * 32, 0, s>>>(bits, block_offsets, n_rows, ids_out, payload, payload_out);
+    k_compact<true><<<grid, kCompactWarps * 32, 0, s>>>(bits, block_offsets, n_rows, ids_out, payload, payload_out,
+                                                        arrived);
   else
-    k_compact<false><<<grid, kCompactWarps * 32, 0, s>>>(bits, block_offsets, n_rows, ids_out, payload, payload_out);
+    k_compact<false><<<grid, kCompactWarps * 32, 0, s>>>(bits, block_offsets, n_rows, ids_out, payload, payload_out,
+                                                         arrived);
 }
 
 void launch_hash_build(const int64_t* keys, const int32_t* rows, int64_t n, unsigned long long* table_keys,
                        int32_t* table_vals, int64_t capacity, int* err, cudaStream_t s) {
   if (n <= 0) return;
   k_hash_build<<<blocks_for(n, 256), 256, 0, s>>>(keys, rows, n, table_keys, table_vals, capacity, err);
+}
+
+void launch_hash_build_where(const int64_t* keys, const PredSet& ps, int64_t n, unsigned long long* table_keys,
+                             int32_t* table_vals, int64_t capacity, int* err, cudaStream_t s) {
+  if (n <= 0) return;
+  k_hash_build_where<<<blocks_for(n, 256), 256, 0, s>>>(keys, ps, n, table_keys, table_vals, capacity, err);
 }
 
 void launch_fill_u64(unsigned long long* p, int64_t n, unsigned long long v, cudaStream_t s) {

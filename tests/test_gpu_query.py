@@ -64,6 +64,67 @@ def test_filter_compaction_bit_exact(ctx, n):
         ctx.free_table(ref_t)
 
 
+MIXES = [  # every count of int64 and 4-byte terms that has a kernel of its own, and five terms
+    "b", "bb", "bbb", "bbbb", "ab", "abb", "babb", "abc", "cabb", "aabc", "ac", "aca", "acca", "abcab",
+]
+
+
+@pytest.mark.parametrize("n", [1, 8191, 8193, 16384, 16385, 70_001, (1 << 24) + 1])
+def test_filter_term_mixes(ctx, n):
+    """Conjunctions over columns of every type in any order, at the sizes where the
+    filter changes kernels: one block (16,384 rows), the last block's scan (2^24),
+    and the allocation-free call on the same columns."""
+    torch = pytest.importorskip("torch")
+    t = _random_table(n, n + 5)
+    ref_t = ctx.load_table(t.cols, n_rows=n)
+    dev = {k: torch.from_numpy(v).cuda() for k, v in t.cols.items()}
+    code = {"a": aiq.INT32, "b": aiq.INT64, "c": aiq.FLOAT32}
+    ids = torch.empty(n, dtype=torch.int32, device="cuda")
+    count = torch.empty(1, dtype=torch.int64, device="cuda")
+    consts = {"a": [(rel.GE, 2), (rel.NE, 7)], "b": [(rel.GT, -2**39), (rel.LE, 2**39), (rel.NE, 3), (rel.LT, 2**40)],
+              "c": [(rel.LE, 0.75), (rel.GT, -1.5)]}
+    try:
+        for mix in MIXES if n < 1 << 24 else MIXES[::4]:
+            preds = [(k, *consts[k][mix[:i].count(k)]) for i, k in enumerate(mix)]
+            want = rel.compact(rel.predicate_mask(t.cols, preds, n))
+            r = ctx.run_select(ref_t, 0, preds, [], [0, 1], flags=aiq.FLAG_RELATIONAL_ONLY)
+            assert np.array_equal(r.cand_row_ids, want), mix
+            if n <= 1 << 24:
+                torch.cuda.synchronize()
+                aiq.filter_compact_static([(dev[k].data_ptr(), code[k], o, v) for k, o, v in preds], n,
+                                          ids.data_ptr(), count.data_ptr(), 0)
+                torch.cuda.synchronize()
+                assert int(count) == len(want) and np.array_equal(ids[:len(want)].cpu().numpy(), want), mix
+    finally:
+        ctx.free_table(ref_t)
+
+
+@pytest.mark.parametrize("m,n", [(1, 3), (40, 2047), (3000, 70_001), ((1 << 22) + 3, 20_000)])
+def test_join_probe_sizes(ctx, m, n):
+    """Build sides hashed straight from their columns and (the largest) compacted
+    first; crowded tables, absent keys and the empty-slot sentinel among the probes."""
+    rng = np.random.default_rng(m)
+    keys = rng.permutation(np.arange(-(m // 2), m - m // 2, dtype=np.int64)) * 3
+    build = {"k": keys, "y": rng.integers(0, 4, m).astype(np.int32)}
+    probe = {"k": rng.integers(-2 * m - 2, 2 * m + 2, n).astype(np.int64), "a": rng.integers(0, 10, n).astype(np.int32)}
+    probe["k"][::97] = -2**63
+    tb, tp = ctx.load_table(build), ctx.load_table(probe)
+    try:
+        for bp, pp in [([], []), ([("y", rel.GE, 1)], [("a", rel.LT, 8)])]:
+            r = ctx.run_join_select(tb, "k", bp, tp, "k", 0, pp, [], [0, 1], agg=aiq.AGG_COUNT,
+                                    flags=aiq.FLAG_RELATIONAL_ONLY)
+            ok_b = rel.predicate_mask(build, bp, m)
+            order = np.argsort(keys)
+            at = np.searchsorted(keys[order], probe["k"]).clip(0, m - 1)
+            hit = order[at]
+            sel = (keys[hit] == probe["k"]) & ok_b[hit] & rel.predicate_mask(probe, pp, n)
+            assert np.array_equal(r.cand_row_ids, np.nonzero(sel)[0])
+            assert np.array_equal(r.cand_build_rows, hit[sel])
+    finally:
+        ctx.free_table(tb)
+        ctx.free_table(tp)
+
+
 def test_join_small_with_orphans_and_repeats(ctx):
     rng = np.random.default_rng(3)
     m, n = 300, 5000
