@@ -1365,7 +1365,7 @@ int dispatch_few(const __half* A, int64_t lda, const __half* B, int64_t ldb, con
 // its operands' arrival (60 bytes per clock); the large tiles measure 720
 // (128 x 256), 540 (128 x 128) and 660 (CTA pair).  An epilogue column costs 100
 // clocks where the threads add to the residual, 50 for SwiGLU, 40 for RoPE and 22 for the
-// TMA add; a tile's epilogue runs beside the next tile's main loop.  Measured
+// TMA add, and each epilogue 1200 more for its hand-offs; a tile's epilogue runs beside the next tile's main loop.  Measured
 // (us, weights from DRAM; with about 7 us of launch and event overhead):
 //   M     N      K      large   16     32     64     128
 //   24    2048   8192   55.6    18.5   21.3   23.0   32.1
@@ -1386,6 +1386,7 @@ int gemm_few_tile(int M, int N, int K, int bn, bool pair, const GemmEpilogue& ep
   const int64_t kblocks = K / BK;
   auto cost = [&](int64_t tiles, int64_t units, int64_t per_kblock, int64_t epilogue) {
     const int64_t waves = (tiles + units - 1) / units, main = kblocks * per_kblock;
+    epilogue += 1200;
     return main + (waves - 1) * std::max(main, epilogue) + epilogue;
   };
   const int64_t m128 = (M + 127) / 128;
