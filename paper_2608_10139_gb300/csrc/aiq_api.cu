@@ -372,19 +372,19 @@ void attention_tiles(aiq_ctx* c, int64_t n_seqs, const int32_t* seq_start, int32
 // Causal GQA attention over a packed chunk whose work list attention_tiles made.
 aiq_status attention(aiq_ctx* c, const __half* qkv, int64_t T, int64_t n_seqs, const int32_t* seq_start,
                      const int32_t* tile_seq, const int32_t* tile_q0, const int32_t* n_tiles, int Hq, int Hkv, int hd,
-                     const __half* pkv, int P, __half* out) {
+                     const PrefixKV& prefix, __half* out) {
   const bool tc = c->attention_tc && attention_tc_supported(hd, Hq, Hkv);
   const int tq = attention_tile_tokens(c, Hq, Hkv, hd);
   const int n_tiles_max = static_cast<int>((T + tq - 1) / tq + n_seqs);
   ProfScope p(c, "attention", 0, 0);
   if (tc) {
-    const int e = launch_attention_tc(qkv, T, seq_start, tile_seq, tile_q0, n_tiles_max, n_tiles, Hq, Hkv, hd, pkv, P,
+    const int e = launch_attention_tc(qkv, T, seq_start, tile_seq, tile_q0, n_tiles_max, n_tiles, Hq, Hkv, hd, prefix,
                                       out, c->d_err, c->num_sms, c->stream);
     if (e != 0)
       return fail(AIQ_ERR_CUDA, std::string("tcgen05 attention launch: ") +
                                     cudaGetErrorString(static_cast<cudaError_t>(e)));
   } else {
-    launch_attention(qkv, T, seq_start, tile_seq, tile_q0, n_tiles_max, n_tiles, Hq, Hkv, hd, pkv, P, out, c->d_err,
+    launch_attention(qkv, T, seq_start, tile_seq, tile_q0, n_tiles_max, n_tiles, Hq, Hkv, hd, prefix, out, c->d_err,
                      c->stream);
   }
   counted(c, T > 0 && n_seqs > 0);
@@ -495,6 +495,8 @@ aiq_status ensure_rope(aiq_ctx* c, ModelD& m, int max_pos) {
   return AIQ_OK;
 }
 
+constexpr int32_t kMergedPrefixMax = 1024;  // prefix tokens that run with the first chunk
+
 struct PrefillBufs {
   int32_t *tok, *pos, *seq_start, *last_idx, *tile_seq, *tile_q0, *n_tiles, *last_compact;
   float *resid, *resid_last;
@@ -525,14 +527,15 @@ aiq_status prefill_bufs(aiq_ctx* c, const ModelD& m, int64_t B, int64_t max_rows
 }
 
 // Decoder forward over one packed chunk of n_seqs sequences / T tokens.
-// pkv_in (optional): per-layer keys/values [L][P][2 Hkv hd] of the shared
-// prefix that every sequence attends; pkv_out (optional): where this pass
-// stores its own keys/values per layer (the prefix pass).
+// The shared prefix that every sequence attends: its per-layer keys/values
+// pkv_in [L][P_in][2 Hkv hd], or, with prefix_first, the chunk's own first
+// sequence of P_in tokens.  kv_out (optional): where this pass stores the
+// keys/values of its first kv_rows tokens per layer.
 // rows_only_last: the final layer's O-projection and MLP run only on each
 // sequence's last token (the only position whose output reaches the label
 // head); the result lands in b.resid_last, rows in sequence order.
 aiq_status run_layers(aiq_ctx* c, ModelD& m, const PrefillBufs& b, int64_t T, int64_t n_seqs, const __half* pkv_in,
-                      int P_in, __half* pkv_out, bool rows_only_last) {
+                      int P_in, bool prefix_first, __half* kv_out, int64_t kv_rows, bool rows_only_last) {
   const aiq_model_config& g = m.cfg;
   const int d = g.d_model, hd = g.head_dim, Hq = g.n_heads, Hkv = g.n_kv_heads, f = g.d_ffn;
   const int nqkv = (Hq + 2 * Hkv) * hd;
@@ -574,11 +577,16 @@ aiq_status run_layers(aiq_ctx* c, ModelD& m, const PrefillBufs& b, int64_t T, in
     e1.d_norm = static_cast<float>(d);
     e1.eps = g.rms_eps;
     AIQ_TRY(gemm(c, "gemm_qkv_rope", b.xn, d, L.wqkv, d, M, nqkv, d, m.bn_qkv, e1));
-    if (pkv_out && T > 0)
-      CUDA_TRY(cudaMemcpy2DAsync(pkv_out + l * T * ldkv, ldkv * sizeof(__half), b.qkv + Hq * hd,
-                                 nqkv * sizeof(__half), ldkv * sizeof(__half), T, cudaMemcpyDeviceToDevice, c->stream));
-    AIQ_TRY(attention(c, b.qkv, T, n_seqs, b.seq_start, b.tile_seq, b.tile_q0, b.n_tiles, Hq, Hkv, hd,
-                      pkv_in ? pkv_in + l * P_in * ldkv : nullptr, P_in, b.att));
+    if (kv_out && kv_rows > 0)
+      CUDA_TRY(cudaMemcpy2DAsync(kv_out + l * kv_rows * ldkv, ldkv * sizeof(__half), b.qkv + Hq * hd,
+                                 nqkv * sizeof(__half), ldkv * sizeof(__half), kv_rows, cudaMemcpyDeviceToDevice,
+                                 c->stream));
+    PrefixKV prefix;
+    if (prefix_first)
+      prefix = PrefixKV{b.qkv + Hq * hd, nqkv, P_in, true};
+    else if (pkv_in)
+      prefix = PrefixKV{pkv_in + l * P_in * ldkv, ldkv, P_in, false};
+    AIQ_TRY(attention(c, b.qkv, T, n_seqs, b.seq_start, b.tile_seq, b.tile_q0, b.n_tiles, Hq, Hkv, hd, prefix, b.att));
     const bool prune = rows_only_last && l == g.n_layers - 1;
     GemmEpilogue e2;
     e2.kind = EPI_RESID_F32;
@@ -648,6 +656,7 @@ struct QueryState {
   float* logits = nullptr;       // [S, K]
   int64_t T = 0, n_chunks = 0, pairs = 0;  // T: row tokens (prefix excluded)
   int64_t P = 0;                            // prefix tokens, run once
+  bool merged_prefix = false;               // ... as the first chunk's first sequence
 };
 
 // Generation state of an AI_TRANSFORM query (Table 1): greedy decoding of
@@ -887,15 +896,30 @@ aiq_status prefill_phase(aiq_ctx* c, const TableD& t, ModelD& m, const aiq_selec
   std::vector<int64_t> chunks(2 * (n_chunks + 1));
   CUDA_TRY(cudaMemcpyAsync(chunks.data(), chunk_d, chunks.size() * sizeof(int64_t), cudaMemcpyDeviceToHost, c->stream));
   AIQ_TRY(sync_and_check(c));
-  int64_t Bmax = P, Rmax = 1;
-  for (int64_t i = 0; i < n_chunks; ++i) {
-    Bmax = std::max(Bmax, chunks[2 * (i + 1) + 1] - chunks[2 * i + 1]);
-    Rmax = std::max(Rmax, chunks[2 * (i + 1)] - chunks[2 * i]);
-  }
   AIQ_TRY(ensure_rope(c, m, static_cast<int>(P + max_len + (gp ? gp->max_new : 0))));
+  // The shared prefix runs through the decoder once.  As the first sequence of the
+  // first chunk it costs no pass over the weights and no launches of its own (the
+  // 1B shape, 58 rows behind 64 tokens: 11.5 -> 10.9 ms; the tiny query 467 -> 376
+  // us); a pass of its own, before the chunks, is left for generation, for a long
+  // prefix and where the larger chunk's buffers do not fit.
+  bool merged = P > 0 && P <= kMergedPrefixMax && !gp;
+  int64_t Bmax, Rmax;
   PrefillBufs pb;
-  // a chunk of rows with empty text has more rows than tokens
-  AIQ_TRY(prefill_bufs(c, m, std::max<int64_t>({Bmax, Rmax, 64}), Rmax, &pb));
+  for (;;) {
+    Bmax = P;
+    Rmax = 1;
+    for (int64_t i = 0; i < n_chunks; ++i) {
+      const bool with_prefix = merged && i == 0;
+      Bmax = std::max(Bmax, chunks[2 * (i + 1) + 1] - chunks[2 * i + 1] + (with_prefix ? P : 0));
+      Rmax = std::max(Rmax, chunks[2 * (i + 1)] - chunks[2 * i] + (with_prefix ? 1 : 0));
+    }
+    // a chunk of rows with empty text has more rows than tokens
+    const aiq_status s = prefill_bufs(c, m, std::max<int64_t>({Bmax, Rmax, 64}), Rmax, &pb);
+    if (s == AIQ_OK) break;
+    if (!merged) return s;
+    merged = false;
+  }
+  st->merged_prefix = merged;
   const aiq_model_config& g = m.cfg;
   const int64_t ldkv = 2 * static_cast<int64_t>(g.n_kv_heads) * g.head_dim;
   DecodeBufs db{};
@@ -913,13 +937,14 @@ aiq_status prefill_phase(aiq_ctx* c, const TableD& t, ModelD& m, const aiq_selec
   __half* pkv = nullptr;
   float* prefix_last;
   AIQ_TRY(ws(c, "pf.prefix_last", g.d_model, &prefix_last));
-  if (P > 0) {
-    // the shared prefix once: its per-layer keys/values and its last hidden state
+  if (P > 0 && (!merged || n_chunks > 1))
     AIQ_TRY(ws(c, "pf.prefix_kv", static_cast<int64_t>(g.n_layers) * P * ldkv, &pkv));
+  if (P > 0 && !merged) {
+    // the shared prefix once: its per-layer keys/values and its last hidden state
     NvtxPhase pr("prefix");
-    launch_pack_prefix(prefix_d, P, pb.tok, pb.pos, pb.seq_start, c->stream);
+    launch_pack_prefix(prefix_d, P, pb.tok, pb.pos, pb.seq_start, pb.last_idx, c->stream);
     counted(c, 1);
-    AIQ_TRY(run_layers(c, m, pb, P, 1, nullptr, 0, pkv, false));
+    AIQ_TRY(run_layers(c, m, pb, P, 1, nullptr, 0, false, pkv, P, false));
     CUDA_TRY(cudaMemcpyAsync(prefix_last, pb.resid + static_cast<int64_t>(P - 1) * g.d_model, g.d_model * sizeof(float),
                              cudaMemcpyDeviceToDevice, c->stream));
   }
@@ -928,14 +953,21 @@ aiq_status prefill_phase(aiq_ctx* c, const TableD& t, ModelD& m, const aiq_selec
     const int64_t Tc = chunks[2 * (i + 1) + 1] - chunks[2 * i + 1];
     if (r1 <= r0) continue;
     NvtxPhase chunk_range("chunk");
+    const bool first = merged && i == 0;  // sequence 0 is the prefix, the rows follow
+    const int64_t tok0 = first ? P : 0, seq0 = first ? 1 : 0;
     {
       ProfScope p(c, "pack_chunk", 0, 0);
+      if (first) launch_pack_prefix(prefix_d, P, pb.tok, pb.pos, pb.seq_start, pb.last_idx, c->stream);
       launch_pack_chunk(cu, st->ids, col.offsets, static_cast<const int32_t*>(col.data), P, r0, r1, pb.tok, pb.pos,
-                        pb.seq_start, pb.last_idx, c->stream, st->ids2);
-      counted(c, 1);
+                        pb.seq_start + seq0, pb.last_idx + seq0, c->stream, st->ids2, tok0);
+      counted(c, 1 + seq0);
     }
-    // generation keeps every layer's prompt keys/values of the chunk for the decode steps
-    AIQ_TRY(run_layers(c, m, pb, Tc, r1 - r0, pkv, static_cast<int>(P), gp ? db.kvc : nullptr, true));
+    // generation keeps every layer's prompt keys/values of the chunk for the decode
+    // steps; a first chunk keeps the prefix's for the chunks after it
+    AIQ_TRY(run_layers(c, m, pb, tok0 + Tc, seq0 + r1 - r0, first ? nullptr : pkv, static_cast<int>(P), first,
+                       gp ? db.kvc : (first ? pkv : nullptr), gp ? Tc : P, true));
+    if (first)  // the final hidden state of the prefix's last token, for rows without text
+      CUDA_TRY(cudaMemcpyAsync(prefix_last, pb.resid_last, g.d_model * sizeof(float), cudaMemcpyDeviceToDevice, c->stream));
     if (gp) {
       cudaEvent_t e0 = take_event(c), e1 = take_event(c);
       CUDA_TRY(cudaEventRecord(e0, c->stream));
@@ -944,7 +976,7 @@ aiq_status prefill_phase(aiq_ctx* c, const TableD& t, ModelD& m, const aiq_selec
       gp->spans.push_back({e0, e1});
     } else {
       ProfScope p(c, "label_head", 0, 0);
-      launch_label_head(pb.resid_last, pb.last_compact, prefix_last, r1 - r0, g.d_model, m.final_norm, g.rms_eps,
+      launch_label_head(pb.resid_last, pb.last_compact + seq0, prefix_last, r1 - r0, g.d_model, m.final_norm, g.rms_eps,
                         m.lm_head, m.lm_bias, labels_d, K, logits + r0 * K, c->stream);
       counted(c, 1);
     }
@@ -1229,12 +1261,13 @@ aiq_status run_query(aiq_ctx* c, const TableD* build, int32_t build_key, const a
     const aiq_model_config& g = m->cfg;
     const double pre = st.S > 0 ? static_cast<double>(st.P) : 0.0;
     // final layer: Q/K/V for every token, O-projection and MLP for each row's last token only
+    // (and for the prefix's, when it runs with the first chunk; for all its tokens otherwise)
     const double d = g.d_model, qd = double(g.n_heads) * g.head_dim, kd = double(g.n_kv_heads) * g.head_dim;
     const double per_layer = m->linear_flops_per_token / g.n_layers;
     const double tail = 2.0 * (qd * d + 3.0 * d * g.d_ffn);
     R.v.prefill_flops = per_layer * (g.n_layers - 1) * (static_cast<double>(st.T) + pre) +
                         2.0 * d * (qd + 2 * kd) * static_cast<double>(st.T) + tail * static_cast<double>(st.S) +
-                        per_layer * pre +
+                        (st.merged_prefix ? 2.0 * d * (qd + 2 * kd) * pre + tail : per_layer * pre) +
                         4.0 * g.n_heads * g.head_dim * g.n_layers * (static_cast<double>(st.pairs) + pre * (pre + 1) / 2) +
                         2.0 * g.d_model * K * static_cast<double>(st.S);
   }
@@ -1483,7 +1516,7 @@ aiq_status run_pair_select(aiq_ctx* c, const TableD& t, int32_t key_col, ModelD*
     const double tail = 2.0 * (qd * d + 3.0 * d * g.d_ffn);
     dst.v.prefill_flops = per_layer * (g.n_layers - 1) * (static_cast<double>(st.T) + pre) +
                           2.0 * d * (qd + 2 * kd) * static_cast<double>(st.T) + tail * static_cast<double>(st.S) +
-                          per_layer * pre +
+                          (st.merged_prefix ? 2.0 * d * (qd + 2 * kd) * pre + tail : per_layer * pre) +
                           4.0 * g.n_heads * g.head_dim * g.n_layers * (static_cast<double>(st.pairs) + pre * (pre + 1) / 2) +
                           2.0 * g.d_model * 2 * static_cast<double>(st.S);
   }
@@ -2004,8 +2037,9 @@ aiq_status aiq_op_attention(aiq_ctx* c, const void* qkv, int64_t T, const int32_
   AIQ_TRY(ws(c, "op.n_tiles", 1, &n_tiles));
   if (P < 0 || (P > 0 && !prefix_kv)) return fail(AIQ_ERR_INVALID_ARG, "bad prefix");
   attention_tiles(c, n_seqs, seq_start, tile_seq, tile_q0, n_tiles, Hq, Hkv, hd);
+  const PrefixKV prefix{static_cast<const __half*>(prefix_kv), 2 * static_cast<int64_t>(Hkv) * hd, P, false};
   AIQ_TRY(attention(c, static_cast<const __half*>(qkv), T, n_seqs, seq_start, tile_seq, tile_q0, n_tiles, Hq, Hkv, hd,
-                    static_cast<const __half*>(prefix_kv), P, static_cast<__half*>(out)));
+                    prefix, static_cast<__half*>(out)));
   const aiq_status st = sync_and_check(c);
   collect_profile(c);
   return st;

@@ -67,7 +67,7 @@ template <int HD>
 __global__ void __launch_bounds__(kThreads) k_attention(const __half* __restrict__ qkv, const int32_t* seq_start,
                                                         const int32_t* tile_seq, const int32_t* tile_q0,
                                                         const int32_t* n_tiles, int Hq, int Hkv,
-                                                        const __half* __restrict__ prefix_kv, int P, float scale_log2,
+                                                        PrefixKV prefix, float scale_log2,
                                                         __half* __restrict__ out) {
   constexpr int LDS = HD + 8;
   constexpr int KS = HD / 16;  // k-steps of QK^T
@@ -90,11 +90,12 @@ __global__ void __launch_bounds__(kThreads) k_attention(const __half* __restrict
   const __half* Kg = qkv + static_cast<int64_t>(st) * ld + (Hq + kvh) * HD;
   const __half* Vg = qkv + static_cast<int64_t>(st) * ld + (Hq + Hkv + kvh) * HD;
   const int q_end = min(q0 + BQ, len);
+  const int P = prefix.is_seq0 && s == 0 ? 0 : prefix.P;
   const int n_pre = (P + BKV - 1) / BKV;  // blocks of prefix keys (positions 0..P-1)
   const int n_kv = n_pre + (q_end + BKV - 1) / BKV;
-  const int64_t ldp = static_cast<int64_t>(2 * Hkv) * HD;
-  const __half* Kp = prefix_kv + kvh * HD;
-  const __half* Vp = prefix_kv + (Hkv + kvh) * HD;
+  const int64_t ldp = prefix.ld;
+  const __half* Kp = prefix.kv + kvh * HD;
+  const __half* Vp = prefix.kv + (Hkv + kvh) * HD;
   auto load_kv = [&](int j, int buf) {
     if (j < n_pre) {
       load_rows<HD>(sK + buf * BKV * LDS, Kp, j * BKV, P, ldp);
@@ -268,14 +269,14 @@ __global__ void __launch_bounds__(kThreads) k_attention(const __half* __restrict
 
 template <int HD>
 void launch_hd(const __half* qkv, const int32_t* seq_start, const int32_t* tile_seq, const int32_t* tile_q0,
-               int n_tiles_max, const int32_t* n_tiles_dev, int Hq, int Hkv, const __half* pkv, int P, __half* out,
-               cudaStream_t s) {
+               int n_tiles_max, const int32_t* n_tiles_dev, int Hq, int Hkv, const PrefixKV& prefix,
+               __half* out, cudaStream_t s) {
   constexpr int LDS = HD + 8;
   const int smem = (BQ + 4 * BKV) * LDS * 2;
   cudaFuncSetAttribute(k_attention<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   const float scale_log2 = 1.4426950408889634f / sqrtf(static_cast<float>(HD));
   dim3 grid(n_tiles_max, Hq);
-  k_attention<HD><<<grid, kThreads, smem, s>>>(qkv, seq_start, tile_seq, tile_q0, n_tiles_dev, Hq, Hkv, pkv, P,
+  k_attention<HD><<<grid, kThreads, smem, s>>>(qkv, seq_start, tile_seq, tile_q0, n_tiles_dev, Hq, Hkv, prefix,
                                                scale_log2, out);
 }
 
@@ -283,13 +284,14 @@ void launch_hd(const __half* qkv, const int32_t* seq_start, const int32_t* tile_
 
 void launch_attention(const __half* qkv, int64_t /*T*/, const int32_t* seq_start, const int32_t* tile_seq,
                       const int32_t* tile_q0, int n_tiles_max, const int32_t* n_tiles_dev, int Hq, int Hkv, int hd,
-                      const __half* prefix_kv, int P, __half* out, int* /*err*/, cudaStream_t s) {
+                      const PrefixKV& prefix, __half* out, int* /*err*/, cudaStream_t s) {
   if (n_tiles_max <= 0) return;
-  if (!prefix_kv) P = 0;
+  PrefixKV p = prefix;
+  if (!p.kv) p.P = 0;
   switch (hd) {
-    case 32: launch_hd<32>(qkv, seq_start, tile_seq, tile_q0, n_tiles_max, n_tiles_dev, Hq, Hkv, prefix_kv, P, out, s); break;
-    case 64: launch_hd<64>(qkv, seq_start, tile_seq, tile_q0, n_tiles_max, n_tiles_dev, Hq, Hkv, prefix_kv, P, out, s); break;
-    case 128: launch_hd<128>(qkv, seq_start, tile_seq, tile_q0, n_tiles_max, n_tiles_dev, Hq, Hkv, prefix_kv, P, out, s); break;
+    case 32: launch_hd<32>(qkv, seq_start, tile_seq, tile_q0, n_tiles_max, n_tiles_dev, Hq, Hkv, p, out, s); break;
+    case 64: launch_hd<64>(qkv, seq_start, tile_seq, tile_q0, n_tiles_max, n_tiles_dev, Hq, Hkv, p, out, s); break;
+    case 128: launch_hd<128>(qkv, seq_start, tile_seq, tile_q0, n_tiles_max, n_tiles_dev, Hq, Hkv, p, out, s); break;
   }
 }
 

@@ -93,6 +93,7 @@ struct AttnArgs {
   const int32_t* tile_q0;
   const int32_t* n_tiles;
   int Hq, Hkv, G, TQ, P;
+  bool prefix_is_seq0;  // the first sequence is the prefix: its items have no prefix keys
   float scale_log2;
   __half* out;
   int* err;
@@ -265,9 +266,15 @@ __global__ void __launch_bounds__(kThreadsTC, ACfg<HD>::CTAS)
   const uint32_t tmem_base = *tmem_slot;
 
   const int n_work = *a.n_tiles * a.Hkv;
-  const int n_pre = (a.P + kKeys - 1) / kKeys;
+  // An item's bounds {start, length, first token, key/value head}; kNoPrefix is
+  // added to the head of an item without prefix keys.
+  constexpr int kNoPrefix = 1 << 24;
+  const int n_prefix = (a.P + kKeys - 1) / kKeys;
+  auto prefix_blocks = [&](const int4& inf) -> int { return inf.w < kNoPrefix ? n_prefix : 0; };
   // key blocks of an item: the shared prefix's, then the row's own up to the tile's last token
-  auto blocks_of = [&](int4 inf) -> int { return n_pre + (min(inf.z + a.TQ, inf.y) + kKeys - 1) / kKeys; };
+  auto blocks_of = [&](const int4& inf) -> int {
+    return prefix_blocks(inf) + (min(inf.z + a.TQ, inf.y) + kKeys - 1) / kKeys;
+  };
   // Every wait of the MMA and softmax warps is taken warp-uniformly: a lane that
   // gives up (timeout or abort) makes the whole warp give up, so no lane is left
   // alone in the warp-synchronous instructions that follow.
@@ -291,7 +298,8 @@ __global__ void __launch_bounds__(kThreadsTC, ACfg<HD>::CTAS)
       };
       auto bounds = [&](int2 l, int w) -> int4 {
         const int st = __ldg(a.seq_start + l.x);
-        return make_int4(st, __ldg(a.seq_start + l.x + 1) - st, l.y, w % a.Hkv);
+        return make_int4(st, __ldg(a.seq_start + l.x + 1) - st, l.y,
+                         w % a.Hkv + (a.prefix_is_seq0 && l.x == 0 ? kNoPrefix : 0));
       };
       auto publish = [&](int item, const int4& inf) -> bool {
         const int is = item & 3;
@@ -308,7 +316,7 @@ __global__ void __launch_bounds__(kThreadsTC, ACfg<HD>::CTAS)
       for (; w < n_work && ok; w += step) {
         const int4 after = bounds(ahead, w + 2 * step);
         ahead = list(w + 3 * step);
-        const int st = cur.x, kvh = cur.w;
+        const int st = cur.x, kvh = cur.w % kNoPrefix, n_pre = prefix_blocks(cur);
         const int n_kv = blocks_of(cur);
         const int qb = it % NQ;
         if (!mbar_wait_bounded(&q_empty[qb], ((it / NQ) & 1) ^ 1, abort_flag, err)) break;
@@ -488,8 +496,8 @@ __global__ void __launch_bounds__(kThreadsTC, ACfg<HD>::CTAS)
       const int4 inf = info[is];
       __syncwarp();
       if (lane == 0) mbar_arrive(&info_empty[is]);
-      const int st = inf.x, len = inf.y, q0 = inf.z, kvh = inf.w;
-      const int n_kv = blocks_of(inf);
+      const int st = inf.x, len = inf.y, q0 = inf.z, kvh = inf.w % kNoPrefix;
+      const int n_pre = prefix_blocks(inf), n_kv = blocks_of(inf);
       const int qpos = q0 + t;
       float m_used = 0.f, l = 0.f;
       for (int j = 0; j < n_kv; ++j, ++g) {
@@ -616,11 +624,11 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn_attn() {
   return fn;
 }
 
-bool map2d(CUtensorMap* m, const __half* base, int64_t rows, int64_t cols) {
+bool map2d(CUtensorMap* m, const __half* base, int64_t rows, int64_t cols, int64_t ld) {
   auto fn = encode_fn_attn();
   if (!fn) return false;
   cuuint64_t dims[2] = {static_cast<cuuint64_t>(cols), static_cast<cuuint64_t>(rows)};
-  cuuint64_t strides[1] = {static_cast<cuuint64_t>(cols * 2)};
+  cuuint64_t strides[1] = {static_cast<cuuint64_t>(ld * 2)};
   cuuint32_t box[2] = {64, 64};
   cuuint32_t estr[2] = {1, 1};
   return fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<__half*>(base), dims, strides, box, estr,
@@ -665,22 +673,23 @@ int attention_tc_tile_tokens(int Hq, int Hkv) { return 128 / (Hq / Hkv); }
 
 int launch_attention_tc(const __half* qkv, int64_t T, const int32_t* seq_start, const int32_t* tile_seq,
                         const int32_t* tile_q0, int n_tiles_max, const int32_t* n_tiles_dev, int Hq, int Hkv, int hd,
-                        const __half* prefix_kv, int P, __half* out, int* err, int num_sms, cudaStream_t s) {
+                        const PrefixKV& prefix, __half* out, int* err, int num_sms, cudaStream_t s) {
   if (n_tiles_max <= 0 || T <= 0) return 0;
   const int G = Hq / Hkv, TQ = 128 / G;
   const int heads = Hq + 2 * Hkv;
   CUtensorMap mq, mkv, mpre;
-  if (!map3d_q(&mq, qkv, T, heads, hd, G, TQ) || !map2d(&mkv, qkv, T, int64_t(heads) * hd))
+  if (!map3d_q(&mq, qkv, T, heads, hd, G, TQ) || !map2d(&mkv, qkv, T, int64_t(heads) * hd, int64_t(heads) * hd))
     return cudaErrorInvalidValue;
   // the output's rows are written in 16- or 32-byte pieces
   if (reinterpret_cast<uintptr_t>(out) & 15) return cudaErrorInvalidValue;
-  if (prefix_kv && P > 0) {
-    if (!map2d(&mpre, prefix_kv, P, int64_t(2) * Hkv * hd)) return cudaErrorInvalidValue;
+  int P = prefix.P;
+  if (prefix.kv && P > 0) {
+    if (!map2d(&mpre, prefix.kv, P, int64_t(2) * Hkv * hd, prefix.ld)) return cudaErrorInvalidValue;
   } else {
     mpre = mkv;
     P = 0;
   }
-  AttnArgs a{seq_start, tile_seq, tile_q0, n_tiles_dev, Hq, Hkv, G, TQ, P,
+  AttnArgs a{seq_start, tile_seq, tile_q0, n_tiles_dev, Hq, Hkv, G, TQ, P, prefix.is_seq0,
              1.4426950408889634f / sqrtf(static_cast<float>(hd)), out, err};
   const int n_work_max = n_tiles_max * Hkv;
   return hd == 64 ? launch_tc<64>(mq, mkv, mpre, a, n_work_max, num_sms, s)

@@ -144,10 +144,11 @@ void launch_chunk_bounds_rows(const int64_t* cu, int64_t S, int64_t rows_per_chu
 // chunk-local sequence starts and last-token index (-1 for a row without tokens).
 void launch_pack_chunk(const int64_t* cu, const int32_t* ids, const int64_t* offsets, const int32_t* text,
                        int32_t prefix_len, int64_t r0, int64_t r1, int32_t* tok, int32_t* pos, int32_t* seq_start,
-                       int32_t* last_idx, cudaStream_t s, const int32_t* ids2 = nullptr);
-// The shared prefix as a single sequence at positions 0..P-1.
+                       int32_t* last_idx, cudaStream_t s, const int32_t* ids2 = nullptr, int64_t tok0 = 0);
+// The shared prefix as a single sequence at positions 0..P-1.  Rows packed behind
+// it take seq_start + 1, last_idx + 1 and tok0 = P.
 void launch_pack_prefix(const int32_t* prefix, int32_t P, int32_t* tok, int32_t* pos, int32_t* seq_start,
-                        cudaStream_t s);
+                        int32_t* last_idx, cudaStream_t s);
 // Attention work list of a chunk: one entry per (sequence, block of tile_tokens query tokens).
 void launch_attn_tiles(const int32_t* seq_start, int32_t n_seqs, int32_t tile_tokens, int32_t* tile_seq,
                        int32_t* tile_q0, int32_t* n_tiles_dev, cudaStream_t s);
@@ -167,11 +168,17 @@ void launch_embed(const int32_t* tok, int64_t T, const uint16_t* emb, int d, flo
 // fp16(v - fp16(v)) (a two-term operand for a K-doubled GEMM).
 void launch_rmsnorm(const float* x, int64_t T, int d, const uint16_t* g, float eps, __half* out, int* err,
                     cudaStream_t s, bool split = false);
-// prefix_kv (optional): [P, 2 Hkv hd] fp16 keys then values of a shared prefix that
+// prefix.kv (optional): [P, 2 Hkv hd] fp16 keys then values of a shared prefix that
 // every sequence's queries also attend (prefix positions precede the sequence).
+struct PrefixKV {
+  const __half* kv = nullptr;
+  int64_t ld = 0;         // elements between rows
+  int P = 0;
+  bool is_seq0 = false;   // the first sequence is the prefix itself: it attends only its own keys
+};
 void launch_attention(const __half* qkv, int64_t T, const int32_t* seq_start, const int32_t* tile_seq,
                       const int32_t* tile_q0, int n_tiles_max, const int32_t* n_tiles_dev, int Hq, int Hkv,
-                      int hd, const __half* prefix_kv, int P, __half* out, int* err, cudaStream_t s);
+                      int hd, const PrefixKV& prefix, __half* out, int* err, cudaStream_t s);
 // Gathers each row's last-token attention output and residual into dense [n, .]
 // buffers for the final layer's row-only O-projection and MLP.
 void launch_gather_last(const __half* att, int ld_att, const float* resid, int d, const int32_t* last_idx, int64_t n,
@@ -182,7 +189,7 @@ bool attention_tc_supported(int hd, int Hq, int Hkv);
 int attention_tc_tile_tokens(int Hq, int Hkv);
 int launch_attention_tc(const __half* qkv, int64_t T, const int32_t* seq_start, const int32_t* tile_seq,
                         const int32_t* tile_q0, int n_tiles_max, const int32_t* n_tiles_dev, int Hq, int Hkv, int hd,
-                        const __half* prefix_kv, int P, __half* out, int* err, int num_sms, cudaStream_t s);
+                        const PrefixKV& prefix, __half* out, int* err, int num_sms, cudaStream_t s);
 // last_idx[r] < 0 reads prefix_last (fp32 [d]) instead of a row of resid.
 void launch_label_head(const float* resid, const int32_t* last_idx, const float* prefix_last, int64_t n_rows, int d,
                        const uint16_t* g, float eps, const uint16_t* lm_head, const uint16_t* lm_bias,

@@ -69,16 +69,17 @@ __global__ void k_chunk_bounds_rows(const int64_t* cu, int64_t S, int64_t rows_p
 
 // One warp per row: the row's tokens at positions P + j (for a pair prompt the
 // first row's text, then the second's); a row with no tokens of its own gets
-// last_idx = -1 (its last position is the prefix's last).
+// last_idx = -1 (its last position is the prefix's last).  tok0 tokens (the
+// prefix, packed as a sequence before them) come first.
 __global__ void k_pack_chunk(const int64_t* cu, const int32_t* ids, const int32_t* ids2, const int64_t* offsets,
                              const int32_t* text, int32_t P, int64_t r0, int64_t r1, int32_t* tok, int32_t* pos,
-                             int32_t* seq_start, int32_t* last_idx) {
+                             int32_t* seq_start, int32_t* last_idx, int64_t tok0) {
   const int64_t w = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   const int64_t i = r0 + w;
   if (i >= r1) return;
   const int64_t base = cu[r0];
-  const int64_t dst = cu[i] - base;
+  const int64_t dst = tok0 + cu[i] - base;
   const int64_t len = cu[i + 1] - cu[i];
   const int32_t r = ids[i];
   const int32_t* src = text + offsets[r];
@@ -91,7 +92,7 @@ __global__ void k_pack_chunk(const int64_t* cu, const int32_t* ids, const int32_
   if (lane == 0) {
     seq_start[w] = static_cast<int32_t>(dst);
     last_idx[w] = len > 0 ? static_cast<int32_t>(dst + len - 1) : -1;
-    if (i == r1 - 1) seq_start[w + 1] = static_cast<int32_t>(cu[r1] - base);
+    if (i == r1 - 1) seq_start[w + 1] = static_cast<int32_t>(tok0 + cu[r1] - base);
   }
 }
 
@@ -131,8 +132,10 @@ __global__ void __launch_bounds__(1024) k_attn_tiles(const int32_t* seq_start, i
   if (threadIdx.x == 0) *n_tiles = carry;
 }
 
-// The prefix as one sequence: tokens, positions 0..P-1, seq_start = {0, P}.
-__global__ void k_pack_prefix(const int32_t* prefix, int32_t P, int32_t* tok, int32_t* pos, int32_t* seq_start) {
+// The prefix as one sequence: tokens, positions 0..P-1, seq_start = {0, P},
+// last_idx = {P - 1}.
+__global__ void k_pack_prefix(const int32_t* prefix, int32_t P, int32_t* tok, int32_t* pos, int32_t* seq_start,
+                              int32_t* last_idx) {
   for (int j = threadIdx.x; j < P; j += blockDim.x) {
     tok[j] = prefix[j];
     pos[j] = j;
@@ -140,14 +143,15 @@ __global__ void k_pack_prefix(const int32_t* prefix, int32_t P, int32_t* tok, in
   if (threadIdx.x == 0) {
     seq_start[0] = 0;
     seq_start[1] = P;
+    last_idx[0] = P - 1;
   }
 }
 
 }  // namespace
 
 void launch_pack_prefix(const int32_t* prefix, int32_t P, int32_t* tok, int32_t* pos, int32_t* seq_start,
-                        cudaStream_t s) {
-  k_pack_prefix<<<1, 256, 0, s>>>(prefix, P, tok, pos, seq_start);
+                        int32_t* last_idx, cudaStream_t s) {
+  k_pack_prefix<<<1, 256, 0, s>>>(prefix, P, tok, pos, seq_start, last_idx);
 }
 
 void launch_row_lengths(const int64_t* offsets, const int32_t* ids, int64_t S, int32_t prefix_len, int32_t* lens,
@@ -169,11 +173,11 @@ void launch_chunk_bounds_rows(const int64_t* cu, int64_t S, int64_t rows_per_chu
 
 void launch_pack_chunk(const int64_t* cu, const int32_t* ids, const int64_t* offsets, const int32_t* text,
                        int32_t prefix_len, int64_t r0, int64_t r1, int32_t* tok, int32_t* pos, int32_t* seq_start,
-                       int32_t* last_idx, cudaStream_t s, const int32_t* ids2) {
+                       int32_t* last_idx, cudaStream_t s, const int32_t* ids2, int64_t tok0) {
   if (r1 <= r0) return;
   const int64_t threads = (r1 - r0) * 32;
   k_pack_chunk<<<static_cast<unsigned>((threads + 255) / 256), 256, 0, s>>>(cu, ids, ids2, offsets, text, prefix_len,
-                                                                            r0, r1, tok, pos, seq_start, last_idx);
+                                                                            r0, r1, tok, pos, seq_start, last_idx, tok0);
 }
 
 void launch_attn_tiles(const int32_t* seq_start, int32_t n_seqs, int32_t tile_tokens, int32_t* tile_seq,

@@ -292,6 +292,39 @@ def test_rows_with_empty_text(ctx):
     ctx.free_model(mh)
 
 
+@pytest.mark.parametrize("P", [1, 63, 65, 1024, 1025])
+@pytest.mark.parametrize("gqa", [False, True])
+def test_prefix_lengths_and_chunks(ctx, P, gqa):
+    """The prefix as the first chunk's first sequence (up to 1024 tokens) and in a
+    pass of its own, for both attention kernels, rows without text included: the
+    oracle's logits, and the same bits whether the rows take one chunk or several."""
+    w = synth.C1_TINY
+    shape = replace(w.model, d_model=256, n_heads=8, n_kv_heads=2, head_dim=64, d_ffn=512) if gqa else w.model
+    rng = np.random.default_rng(P)
+    n = 40
+    lens = rng.integers(0, 90, n)
+    lens[[0, 7, 39]] = 0
+    offsets = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    table = synth.Table(n, {"rating": np.ones(n, np.int32)}, offsets,
+                        rng.integers(0, shape.vocab, int(offsets[-1])).astype(np.int32))
+    prefix = rng.integers(0, shape.vocab, P).astype(np.int32)
+    mh, W = _model(ctx, shape, w.weight_seed)
+    t = _load(ctx, table)
+    got = []
+    try:
+        for budget in (131072, max(P, 64) + 70):
+            ctx.set_option("token_budget", budget)
+            got.append(ctx.run_select(t, mh, [], prefix, w.label_ids, agg=w.agg, flags=aiq.FLAG_LOGITS))
+    finally:
+        ctx.set_option("token_budget", 131072)
+    assert got[0].n_chunks == 1 and got[1].n_chunks > 1
+    assert np.array_equal(got[0].label_logits, got[1].label_logits)
+    o = oq.run_select(table, prefix, [], w.label_ids, w.agg, tf.Model(shape, W, True))
+    compare_logits(got[0].label_logits, o.logits, f"prefix of {P}")
+    ctx.free_table(t)
+    ctx.free_model(mh)
+
+
 def test_more_rows_than_tokens():
     """A chunk whose rows are all but a few without text has more rows than
     tokens: the per-row buffers are sized for the rows."""
