@@ -140,6 +140,26 @@ def test_rmsnorm(ctx, d):
     _close(_np64(out), ref, 1.5e-3, 1e-4, f"rmsnorm d{d}")
 
 
+@pytest.mark.parametrize("d", [1024, 2048, 4096])
+def test_rmsnorm_few_rows_same_bits(ctx, d):
+    """A block per row (few rows) and a warp per row give the same bits."""
+    rng = np.random.default_rng(d)
+    T = 2433   # one row more than the block-per-row kernel takes
+    x = (rng.standard_normal((T, d)) * 3).astype(np.float32)
+    import synth
+    gb = synth.f32_to_bf16_bits((1 + 0.02 * rng.standard_normal(d)).astype(np.float32))
+    dx, dg = _h(x), _h(gb.view(np.int16))
+    outs = []
+    for n in (T, T - 1, 1):
+        out = torch.zeros((T, d), dtype=torch.float16, device="cuda")
+        ctx.op_rmsnorm(dx.data_ptr(), n, d, dg.data_ptr(), 1e-5, out.data_ptr())
+        torch.cuda.synchronize()
+        assert not out[n:].any()
+        outs.append(out)
+    assert torch.equal(outs[0][:-1], outs[1][:-1]) and torch.equal(outs[0][:1], outs[2][:1])
+    _close(_np64(outs[0]), tf.rmsnorm(x.astype(np.float64), tf.bf16_to_f64(gb), 1e-5), 1.5e-3, 1e-4, f"rmsnorm d{d}")
+
+
 @pytest.mark.parametrize("hd,Hq,Hkv", [(32, 4, 4), (64, 8, 2), (128, 4, 1), (64, 8, 8), (64, 4, 2), (128, 16, 2)])
 def test_attention_varlen(ctx, hd, Hq, Hkv):
     rng = np.random.default_rng(hd + Hq)
