@@ -77,6 +77,8 @@ __global__ void __launch_bounds__(kThreads) k_attention(const __half* __restrict
   __half* sK = sQ + BQ * LDS;     // [2][BKV][LDS]
   __half* sV = sK + 2 * BKV * LDS;
 
+  grid_launch_next();
+  grid_wait();
   const int tile = blockIdx.x;
   if (tile >= *n_tiles) return;
   const int h = blockIdx.y;
@@ -276,8 +278,8 @@ void launch_hd(const __half* qkv, const int32_t* seq_start, const int32_t* tile_
   cudaFuncSetAttribute(k_attention<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   const float scale_log2 = 1.4426950408889634f / sqrtf(static_cast<float>(HD));
   dim3 grid(n_tiles_max, Hq);
-  k_attention<HD><<<grid, kThreads, smem, s>>>(qkv, seq_start, tile_seq, tile_q0, n_tiles_dev, Hq, Hkv, prefix,
-                                               scale_log2, out);
+  launch_chained(k_attention<HD>, grid, kThreads, smem, s, 1, qkv, seq_start, tile_seq, tile_q0, n_tiles_dev, Hq, Hkv,
+                 prefix, scale_log2, out);
 }
 
 }  // namespace

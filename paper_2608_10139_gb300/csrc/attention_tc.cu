@@ -264,6 +264,8 @@ __global__ void __launch_bounds__(kThreadsTC, ACfg<HD>::CTAS)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  grid_launch_next();
+  grid_wait();
 
   const int n_work = *a.n_tiles * a.Hkv;
   // An item's bounds {start, length, first token, key/value head}; kNoPrefix is
@@ -657,8 +659,7 @@ int launch_tc(const CUtensorMap& mq, const CUtensorMap& mkv, const CUtensorMap& 
   if (e != cudaSuccess) return e;
   const int grid = n_work_max < num_sms * C::CTAS ? n_work_max : num_sms * C::CTAS;
   if (grid <= 0) return 0;
-  k_attention_tc<HD><<<grid, kThreadsTC, C::SMEM, s>>>(mq, mkv, mpre, a);
-  return cudaGetLastError();
+  return launch_chained(k_attention_tc<HD>, dim3(grid), kThreadsTC, C::SMEM, s, 1, mq, mkv, mpre, a);
 }
 
 }  // namespace

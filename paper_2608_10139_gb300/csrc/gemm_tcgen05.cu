@@ -481,6 +481,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  grid_launch_next();
+  grid_wait();
 
   const int num_n = args.N / BN;
   const int num_m = (args.M + BM - 1) / BM;
@@ -675,6 +677,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   cluster_sync();  // barriers of both CTAs initialised before any remote arrival
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  grid_launch_next();
+  grid_wait();
 
   const int num_n = args.N / BN;
   const int num_m = (args.M + 2 * BM - 1) / (2 * BM);
@@ -1031,6 +1035,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = tmem_slot;
+  grid_launch_next();
+  grid_wait();
 
   const int num_m = (args.M + MT - 1) / MT;
   const int num_tiles = num_m * (args.N / BN);
@@ -1219,8 +1225,7 @@ int launch(const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap& mc, 
   if (e != cudaSuccess) return e;
   const int tiles = ((a.M + BM - 1) / BM) * (a.N / BN);
   const int grid = tiles < num_sms ? tiles : num_sms;
-  k_gemm_tcgen05<BN, EPI><<<grid, kThreads, SM, stream>>>(ma, mb, mc, a);
-  return cudaGetLastError();
+  return launch_chained(k_gemm_tcgen05<BN, EPI>, dim3(grid), kThreads, SM, stream, 1, ma, mb, mc, a);
 }
 
 template <int EPI>
@@ -1231,21 +1236,7 @@ int launch_pair(const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap&
   if (e != cudaSuccess) return e;
   const int tiles = ((a.M + 2 * BM - 1) / (2 * BM)) * (a.N / 256);
   const int pairs = tiles < num_sms / 2 ? tiles : num_sms / 2;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(2 * pairs, 1, 1);
-  cfg.blockDim = dim3(kThreads, 1, 1);
-  cfg.dynamicSmemBytes = SM;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = 2;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  e = cudaLaunchKernelEx(&cfg, k_gemm_tcgen05_pair<EPI>, ma, mb, mc, a);
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
+  return launch_chained(k_gemm_tcgen05_pair<EPI>, dim3(2 * pairs), kThreads, SM, stream, 2, ma, mb, mc, a);
 }
 
 int dispatch_pair(const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap& mc, const KArgs& a, int num_sms,
@@ -1334,8 +1325,8 @@ int launch_few(const __half* A, int64_t lda, const __half* B, int64_t ldb, const
   cudaError_t e = cudaFuncSetAttribute(k_gemm_few<MT, BN, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, SM);
   if (e != cudaSuccess) return e;
   const int tiles = ((a.M + MT - 1) / MT) * (a.N / BN);
-  k_gemm_few<MT, BN, EPI><<<tiles < num_sms ? tiles : num_sms, kThreads, SM, stream>>>(ma, mb, a, fa);
-  return cudaGetLastError();
+  return launch_chained(k_gemm_few<MT, BN, EPI>, dim3(tiles < num_sms ? tiles : num_sms), kThreads, SM, stream, 1, ma,
+                        mb, a, fa);
 }
 
 template <int BN>

@@ -74,6 +74,8 @@ __global__ void k_chunk_bounds_rows(const int64_t* cu, int64_t S, int64_t rows_p
 __global__ void k_pack_chunk(const int64_t* cu, const int32_t* ids, const int32_t* ids2, const int64_t* offsets,
                              const int32_t* text, int32_t P, int64_t r0, int64_t r1, int32_t* tok, int32_t* pos,
                              int32_t* seq_start, int32_t* last_idx, int64_t tok0) {
+  grid_launch_next();
+  grid_wait();
   const int64_t w = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   const int64_t i = r0 + w;
@@ -101,6 +103,8 @@ __global__ void k_pack_chunk(const int64_t* cu, const int32_t* ids, const int32_
 // shuffle scan within the warps, then every warp scans the 32 warp totals.
 __global__ void __launch_bounds__(1024) k_attn_tiles(const int32_t* seq_start, int32_t n, int32_t tq,
                                                      int32_t* tile_seq, int32_t* tile_q0, int32_t* n_tiles) {
+  grid_launch_next();
+  grid_wait();
   __shared__ int32_t sh[2][32];  // alternate, so that one barrier a round is enough
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int32_t carry = 0;
@@ -136,6 +140,8 @@ __global__ void __launch_bounds__(1024) k_attn_tiles(const int32_t* seq_start, i
 // last_idx = {P - 1}.
 __global__ void k_pack_prefix(const int32_t* prefix, int32_t P, int32_t* tok, int32_t* pos, int32_t* seq_start,
                               int32_t* last_idx) {
+  grid_launch_next();
+  grid_wait();
   for (int j = threadIdx.x; j < P; j += blockDim.x) {
     tok[j] = prefix[j];
     pos[j] = j;
@@ -151,7 +157,7 @@ __global__ void k_pack_prefix(const int32_t* prefix, int32_t P, int32_t* tok, in
 
 void launch_pack_prefix(const int32_t* prefix, int32_t P, int32_t* tok, int32_t* pos, int32_t* seq_start,
                         int32_t* last_idx, cudaStream_t s) {
-  k_pack_prefix<<<1, 256, 0, s>>>(prefix, P, tok, pos, seq_start, last_idx);
+  launch_chained(k_pack_prefix, dim3(1), 256, 0, s, 1, prefix, P, tok, pos, seq_start, last_idx);
 }
 
 void launch_row_lengths(const int64_t* offsets, const int32_t* ids, int64_t S, int32_t prefix_len, int32_t* lens,
@@ -176,13 +182,13 @@ void launch_pack_chunk(const int64_t* cu, const int32_t* ids, const int64_t* off
                        int32_t* last_idx, cudaStream_t s, const int32_t* ids2, int64_t tok0) {
   if (r1 <= r0) return;
   const int64_t threads = (r1 - r0) * 32;
-  k_pack_chunk<<<static_cast<unsigned>((threads + 255) / 256), 256, 0, s>>>(cu, ids, ids2, offsets, text, prefix_len,
-                                                                            r0, r1, tok, pos, seq_start, last_idx, tok0);
+  launch_chained(k_pack_chunk, dim3(static_cast<unsigned>((threads + 255) / 256)), 256, 0, s, 1, cu, ids, ids2, offsets,
+                 text, prefix_len, r0, r1, tok, pos, seq_start, last_idx, tok0);
 }
 
 void launch_attn_tiles(const int32_t* seq_start, int32_t n_seqs, int32_t tile_tokens, int32_t* tile_seq,
                        int32_t* tile_q0, int32_t* n_tiles_dev, cudaStream_t s) {
-  k_attn_tiles<<<1, 1024, 0, s>>>(seq_start, n_seqs, tile_tokens, tile_seq, tile_q0, n_tiles_dev);
+  launch_chained(k_attn_tiles, dim3(1), 1024, 0, s, 1, seq_start, n_seqs, tile_tokens, tile_seq, tile_q0, n_tiles_dev);
 }
 
 }  // namespace aiq

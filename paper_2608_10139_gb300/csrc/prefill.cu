@@ -56,6 +56,8 @@ __global__ void k_rope_table(float* cos_t, float* sin_t, int max_pos, int hd, do
 // fixed order.
 __global__ void k_embed(const int32_t* tok, int64_t T, const uint16_t* emb, int d, float* resid, __half* xh, float* ss,
                         const uint16_t* gain, int* err) {
+  grid_launch_next();
+  grid_wait();
   const int64_t t = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (t >= T) return;
@@ -147,6 +149,8 @@ __device__ __forceinline__ bool norm_store4(const float4& v, float inv, const ui
 template <int PER_LANE>  // d / 32 / 4 float4 per lane (compile-time for register residency)
 __global__ void k_rmsnorm(const float* x, int64_t T, int d, const uint16_t* g, float eps, __half* out, int split,
                           int* err) {
+  grid_launch_next();
+  grid_wait();
   const int64_t t = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (t >= T) return;
@@ -176,6 +180,8 @@ template <int PER_LANE>
 __global__ void __launch_bounds__(256) k_rmsnorm_rows(const float* x, int d, const uint16_t* g, float eps, __half* out,
                                                       int split, int* err) {
   constexpr int PER = PER_LANE / 8;
+  grid_launch_next();
+  grid_wait();
   __shared__ float part[PER_LANE][32];
   const int64_t t = blockIdx.x;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -201,6 +207,8 @@ __global__ void __launch_bounds__(256) k_rmsnorm_rows(const float* x, int d, con
 // Generic-width fallback (d not a multiple of 128 handled elsewhere; d % 4 == 0 here).
 __global__ void k_rmsnorm_any(const float* x, int64_t T, int d, const uint16_t* g, float eps, __half* out, int split,
                               int* err) {
+  grid_launch_next();
+  grid_wait();
   const int64_t t = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (t >= T) return;
@@ -227,6 +235,8 @@ __global__ void k_rmsnorm_any(const float* x, int64_t T, int d, const uint16_t* 
 __global__ void k_label_head(const float* resid, const int32_t* last_idx, const float* prefix_last, int64_t n, int d,
                              const uint16_t* g, float eps, const uint16_t* W, const uint16_t* bias,
                              const int32_t* labels, int K, float* logits) {
+  grid_launch_next();
+  grid_wait();
   const int64_t r = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (r >= n) return;
@@ -261,6 +271,8 @@ __global__ void k_label_head(const float* resid, const int32_t* last_idx, const 
 __global__ void k_gather_last(const __half* __restrict__ att, int ld_att, const float* __restrict__ resid, int d,
                               const int32_t* last_idx, int64_t n, __half* __restrict__ att_out,
                               float* __restrict__ resid_out, int32_t* last_compact) {
+  grid_launch_next();
+  grid_wait();
   const int64_t r = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (r >= n) return;
@@ -303,7 +315,7 @@ void launch_rope_table(float* cos_t, float* sin_t, int max_pos, int head_dim, fl
 void launch_embed(const int32_t* tok, int64_t T, const uint16_t* emb, int d, float* resid, __half* xh, float* ss,
                   const uint16_t* gain, int* err, cudaStream_t s) {
   if (T <= 0) return;
-  k_embed<<<grid_for(T * 32), 256, 0, s>>>(tok, T, emb, d, resid, xh, ss, gain, err);
+  launch_chained(k_embed, dim3(grid_for(T * 32)), 256, 0, s, 1, tok, T, emb, d, resid, xh, ss, gain, err);
 }
 
 void launch_rmsnorm(const float* x, int64_t T, int d, const uint16_t* g, float eps, __half* out, int* err,
@@ -313,34 +325,35 @@ void launch_rmsnorm(const float* x, int64_t T, int d, const uint16_t* g, float e
   const int sp = split ? 1 : 0;
   if (T <= kRowBlocksMax) {
     switch (d) {
-      case 1024: k_rmsnorm_rows<8><<<static_cast<unsigned>(T), 256, 0, s>>>(x, d, g, eps, out, sp, err); return;
-      case 2048: k_rmsnorm_rows<16><<<static_cast<unsigned>(T), 256, 0, s>>>(x, d, g, eps, out, sp, err); return;
-      case 4096: k_rmsnorm_rows<32><<<static_cast<unsigned>(T), 256, 0, s>>>(x, d, g, eps, out, sp, err); return;
+      case 1024: launch_chained(k_rmsnorm_rows<8>, dim3(static_cast<unsigned>(T)), 256, 0, s, 1, x, d, g, eps, out, sp, err); return;
+      case 2048: launch_chained(k_rmsnorm_rows<16>, dim3(static_cast<unsigned>(T)), 256, 0, s, 1, x, d, g, eps, out, sp, err); return;
+      case 4096: launch_chained(k_rmsnorm_rows<32>, dim3(static_cast<unsigned>(T)), 256, 0, s, 1, x, d, g, eps, out, sp, err); return;
     }
   }
   switch (d) {
-    case 128: k_rmsnorm<1><<<grid, 256, 0, s>>>(x, T, d, g, eps, out, sp, err); break;
-    case 256: k_rmsnorm<2><<<grid, 256, 0, s>>>(x, T, d, g, eps, out, sp, err); break;
-    case 512: k_rmsnorm<4><<<grid, 256, 0, s>>>(x, T, d, g, eps, out, sp, err); break;
-    case 1024: k_rmsnorm<8><<<grid, 256, 0, s>>>(x, T, d, g, eps, out, sp, err); break;
-    case 2048: k_rmsnorm<16><<<grid, 256, 0, s>>>(x, T, d, g, eps, out, sp, err); break;
-    case 4096: k_rmsnorm<32><<<grid, 256, 0, s>>>(x, T, d, g, eps, out, sp, err); break;
-    default: k_rmsnorm_any<<<grid, 256, 0, s>>>(x, T, d, g, eps, out, sp, err); break;
+    case 128: launch_chained(k_rmsnorm<1>, dim3(grid), 256, 0, s, 1, x, T, d, g, eps, out, sp, err); break;
+    case 256: launch_chained(k_rmsnorm<2>, dim3(grid), 256, 0, s, 1, x, T, d, g, eps, out, sp, err); break;
+    case 512: launch_chained(k_rmsnorm<4>, dim3(grid), 256, 0, s, 1, x, T, d, g, eps, out, sp, err); break;
+    case 1024: launch_chained(k_rmsnorm<8>, dim3(grid), 256, 0, s, 1, x, T, d, g, eps, out, sp, err); break;
+    case 2048: launch_chained(k_rmsnorm<16>, dim3(grid), 256, 0, s, 1, x, T, d, g, eps, out, sp, err); break;
+    case 4096: launch_chained(k_rmsnorm<32>, dim3(grid), 256, 0, s, 1, x, T, d, g, eps, out, sp, err); break;
+    default: launch_chained(k_rmsnorm_any, dim3(grid), 256, 0, s, 1, x, T, d, g, eps, out, sp, err); break;
   }
 }
 
 void launch_gather_last(const __half* att, int ld_att, const float* resid, int d, const int32_t* last_idx, int64_t n,
                         __half* att_out, float* resid_out, int32_t* last_compact, cudaStream_t s) {
   if (n <= 0) return;
-  k_gather_last<<<grid_for(n * 32), 256, 0, s>>>(att, ld_att, resid, d, last_idx, n, att_out, resid_out, last_compact);
+  launch_chained(k_gather_last, dim3(grid_for(n * 32)), 256, 0, s, 1, att, ld_att, resid, d, last_idx, n, att_out,
+                 resid_out, last_compact);
 }
 
 void launch_label_head(const float* resid, const int32_t* last_idx, const float* prefix_last, int64_t n_rows, int d,
                        const uint16_t* g, float eps, const uint16_t* lm_head, const uint16_t* lm_bias,
                        const int32_t* labels, int n_labels, float* logits_out, cudaStream_t s) {
   if (n_rows <= 0) return;
-  k_label_head<<<grid_for(n_rows * 32), 256, 0, s>>>(resid, last_idx, prefix_last, n_rows, d, g, eps, lm_head,
-                                                     lm_bias, labels, n_labels, logits_out);
+  launch_chained(k_label_head, dim3(grid_for(n_rows * 32)), 256, 0, s, 1, resid, last_idx, prefix_last, n_rows, d, g, eps,
+                 lm_head, lm_bias, labels, n_labels, logits_out);
 }
 
 }  // namespace aiq
