@@ -80,6 +80,8 @@ struct DecCfg {
 // output) are merged at the end.
 template <int HD>
 __global__ void __launch_bounds__(kDecThreads, HD == 128 ? 2 : 3) k_decode_attention(DecArgs a) {
+  grid_launch_next();
+  grid_wait();
   using C = DecCfg<HD>;
   constexpr int NW = C::NW, KB = C::KB, LDS = C::LDS;
   constexpr int KS = HD / 16;  // k-steps of Q K^T
@@ -286,6 +288,8 @@ __device__ __forceinline__ void cp_async_wait() {
 template <int HD>
 __global__ void __launch_bounds__(DecStream<HD>::NW * 32, DecStream<HD>::CTAS)
     k_decode_attention_stream(DecArgs a, int n_tasks) {
+  grid_launch_next();
+  grid_wait();
   using C = DecStream<HD>;
   constexpr int KB = C::KB, LDS = C::LDS;
   constexpr int KS = HD / 16;  // k-steps of Q K^T
@@ -479,6 +483,8 @@ __global__ void __launch_bounds__(DecStream<HD>::NW * 32, DecStream<HD>::CTAS)
 __global__ void k_decode_select(unsigned long long* best, int R, int t, int max_new, int eos, int pad, int V,
                                 int32_t* done, int32_t* gen_tok, int32_t* gen_len, int32_t* next_tok, int32_t* pos,
                                 const int32_t* seq_start, int P, int* err) {
+  grid_launch_next();
+  grid_wait();
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= R) return;
   const unsigned long long key = best[r];
@@ -499,6 +505,8 @@ __global__ void k_decode_select(unsigned long long* best, int R, int t, int max_
 
 // Rows of a chunk whose text is empty take the shared prefix's last hidden state.
 __global__ void k_patch_empty_rows(float* resid, const int32_t* last_idx, const float* prefix_last, int R, int d) {
+  grid_launch_next();
+  grid_wait();
   const int r = blockIdx.x;
   if (r >= R || last_idx[r] >= 0) return;
   for (int i = threadIdx.x; i < d; i += blockDim.x) resid[static_cast<int64_t>(r) * d + i] = prefix_last[i];
@@ -544,9 +552,8 @@ int launch_dec_stream(const DecArgs& a, int R, int num_sms, cudaStream_t s) {
   if (e != cudaSuccess) return e;
   const int64_t tasks = static_cast<int64_t>(R) * a.Hkv, full = static_cast<int64_t>(num_sms) * C::CTAS;
   const int64_t need = (tasks + C::NW - 1) / C::NW;
-  k_decode_attention_stream<HD><<<static_cast<unsigned>(need < full ? need : full), C::NW * 32, C::SMEM, s>>>(
-      a, static_cast<int>(tasks));
-  return cudaGetLastError();
+  return launch_chained(k_decode_attention_stream<HD>, dim3(static_cast<unsigned>(need < full ? need : full)), C::NW * 32,
+                        C::SMEM, s, 1, a, static_cast<int>(tasks));
 }
 
 template <int HD>
@@ -559,8 +566,7 @@ int launch_dec(const DecArgs& a, int R, int num_sms, cudaStream_t s) {
   using C = DecCfg<HD>;
   cudaError_t e = cudaFuncSetAttribute(k_decode_attention<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
   if (e != cudaSuccess) return e;
-  k_decode_attention<HD><<<R * a.Hkv, kDecThreads, C::SMEM, s>>>(a);
-  return cudaGetLastError();
+  return launch_chained(k_decode_attention<HD>, dim3(R * a.Hkv), kDecThreads, C::SMEM, s, 1, a);
 }
 
 }  // namespace
@@ -586,14 +592,14 @@ void launch_decode_select(unsigned long long* best, int R, int t, int max_new, i
                           int32_t* gen_tok, int32_t* gen_len, int32_t* next_tok, int32_t* pos,
                           const int32_t* seq_start, int P, int* err, cudaStream_t s) {
   if (R <= 0) return;
-  k_decode_select<<<(R + 255) / 256, 256, 0, s>>>(best, R, t, max_new, eos, pad, V, done, gen_tok, gen_len, next_tok,
+  launch_chained(k_decode_select, dim3((R + 255) / 256), 256, 0, s, 1, best, R, t, max_new, eos, pad, V, done, gen_tok, gen_len, next_tok,
                                                   pos, seq_start, P, err);
 }
 
 void launch_patch_empty_rows(float* resid, const int32_t* last_idx, const float* prefix_last, int R, int d,
                              cudaStream_t s) {
   if (R <= 0) return;
-  k_patch_empty_rows<<<R, 128, 0, s>>>(resid, last_idx, prefix_last, R, d);
+  launch_chained(k_patch_empty_rows, dim3(R), 128, 0, s, 1, resid, last_idx, prefix_last, R, d);
 }
 
 void launch_bias_f32(const uint16_t* b, int V, int Vpad, float* out, cudaStream_t s) {

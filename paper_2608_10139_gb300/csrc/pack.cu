@@ -24,6 +24,8 @@ namespace {
 // attend, for the executed-FLOP count).
 __global__ void k_row_lengths(const int64_t* offsets, const int32_t* ids, const int32_t* ids2, int64_t S, int32_t P,
                               int32_t* lens, unsigned long long* pairs) {
+  grid_launch_next();
+  grid_wait();
   const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   unsigned long long pr = 0;
   if (i < S) {
@@ -40,6 +42,8 @@ __global__ void k_row_lengths(const int64_t* offsets, const int32_t* ids, const 
 
 // chunk_rows[2c] = first row i with cu[i] >= c * step (S if none), chunk_rows[2c+1] = cu[that row].
 __global__ void k_chunk_bounds(const int64_t* cu, int64_t S, int64_t step, int64_t n_chunks, int64_t* out) {
+  grid_launch_next();
+  grid_wait();
   const int64_t c = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (c > n_chunks) return;
   int64_t lo = 0, hi = S;  // lower bound in cu[0..S)
@@ -60,6 +64,8 @@ __global__ void k_chunk_bounds(const int64_t* cu, int64_t S, int64_t step, int64
 // chunk_rows[2c] = min(c * rows_per_chunk, S), chunk_rows[2c+1] = cu[that row].
 __global__ void k_chunk_bounds_rows(const int64_t* cu, int64_t S, int64_t rows_per_chunk, int64_t n_chunks,
                                     int64_t* out) {
+  grid_launch_next();
+  grid_wait();
   const int64_t c = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (c > n_chunks) return;
   const int64_t row = c * rows_per_chunk < S ? c * rows_per_chunk : S;
@@ -163,17 +169,17 @@ void launch_pack_prefix(const int32_t* prefix, int32_t P, int32_t* tok, int32_t*
 void launch_row_lengths(const int64_t* offsets, const int32_t* ids, int64_t S, int32_t prefix_len, int32_t* lens,
                         unsigned long long* pairs, cudaStream_t s, const int32_t* ids2) {
   if (S <= 0) return;
-  k_row_lengths<<<static_cast<unsigned>((S + 255) / 256), 256, 0, s>>>(offsets, ids, ids2, S, prefix_len, lens, pairs);
+  launch_chained(k_row_lengths, dim3(static_cast<unsigned>((S + 255) / 256)), 256, 0, s, 1, offsets, ids, ids2, S, prefix_len, lens, pairs);
 }
 
 void launch_chunk_bounds(const int64_t* cu, int64_t S, int64_t step, int64_t n_chunks, int64_t* chunk_rows,
                          cudaStream_t s) {
-  k_chunk_bounds<<<static_cast<unsigned>((n_chunks + 1 + 127) / 128), 128, 0, s>>>(cu, S, step, n_chunks, chunk_rows);
+  launch_chained(k_chunk_bounds, dim3(static_cast<unsigned>((n_chunks + 1 + 127) / 128)), 128, 0, s, 1, cu, S, step, n_chunks, chunk_rows);
 }
 
 void launch_chunk_bounds_rows(const int64_t* cu, int64_t S, int64_t rows_per_chunk, int64_t n_chunks,
                               int64_t* chunk_rows, cudaStream_t s) {
-  k_chunk_bounds_rows<<<static_cast<unsigned>((n_chunks + 1 + 127) / 128), 128, 0, s>>>(cu, S, rows_per_chunk, n_chunks,
+  launch_chained(k_chunk_bounds_rows, dim3(static_cast<unsigned>((n_chunks + 1 + 127) / 128)), 128, 0, s, 1, cu, S, rows_per_chunk, n_chunks,
                                                                                        chunk_rows);
 }
 

@@ -141,6 +141,8 @@ __device__ __forceinline__ int write_words_and_count(uint32_t byte, uint32_t* bi
 // loads of successive terms follow one after the other.
 __global__ void __launch_bounds__(kThreads) k_predicate_mask(PredSet ps, int64_t n, uint32_t* bits,
                                                              int32_t* block_counts) {
+  grid_launch_next();
+  grid_wait();
   __shared__ int red[kThreads / 32];
   const int64_t tile = blockIdx.x;
   if (threadIdx.x == 0 && (tile + 1) * kRowsPerBlock <= n) {
@@ -255,6 +257,8 @@ __device__ __forceinline__ void scan_in_last_block(const TileScan& ts) {
 template <int N8, int N4>
 __global__ void __launch_bounds__(kThreads) k_predicate_cols(PredSet ps, int64_t n, uint32_t* bits,
                                                              int32_t* block_counts, TileScan ts) {
+  grid_launch_next();
+  grid_wait();
   __shared__ int red[kThreads / 32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t ra = static_cast<int64_t>(blockIdx.x) * kRowsPerBlock + warp * 256 + lane * 4;
@@ -362,6 +366,8 @@ constexpr int kProbeThreads = 512;  // x 4 rows = kRowsPerBlock
 // that are left.
 __global__ void __launch_bounds__(kProbeThreads) k_probe_mask(PredSet ps, ProbeSpec probe, int64_t n, uint32_t* bits,
                                                               int32_t* block_counts, TileScan ts) {
+  grid_launch_next();
+  grid_wait();
   __shared__ int red[kProbeThreads / 32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t r0 = static_cast<int64_t>(blockIdx.x) * kRowsPerBlock + threadIdx.x * 4;
@@ -440,6 +446,8 @@ constexpr int kSmallThreads = 1024;
 // against 14.7 in four.
 __global__ void __launch_bounds__(kSmallThreads) k_filter_small(PredSet ps, int64_t n, int32_t* ids, int64_t* count,
                                                                 int64_t* count2) {
+  grid_launch_next();
+  grid_wait();
   __shared__ int sh[kSmallThreads / 32];
   int base = 0;
   for (int64_t p0 = 0; p0 < n; p0 += kSmallThreads * 8) {
@@ -481,6 +489,8 @@ template <bool PAYLOAD>
 __global__ void __launch_bounds__(kCompactWarps * 32) k_compact(const uint32_t* bits, const int64_t* block_offsets,
                                                                 int64_t n, int32_t* ids, const int32_t* payload,
                                                                 int32_t* payload_out, unsigned int* arrived) {
+  grid_launch_next();
+  grid_wait();
   // calls that overlap against the rules may leave the scan's counter behind: the next ones start from zero
   if (arrived && blockIdx.x == 0 && threadIdx.x == 0) *arrived = 0;
   __shared__ uint16_t s_ids[kCompactWarps][kRowsPerBlock];  // row offsets within the tile
@@ -531,6 +541,8 @@ template <bool PAYLOAD>
 __global__ void __launch_bounds__(kThreads) k_compact_wide(const uint32_t* bits, const int64_t* block_offsets,
                                                            int32_t* ids, const int32_t* payload, int32_t* payload_out,
                                                            unsigned int* arrived) {
+  grid_launch_next();
+  grid_wait();
   __shared__ int sh[kThreads / 32];
   if (arrived && blockIdx.x == 0 && threadIdx.x == 0) *arrived = 0;  // as k_compact
   const int64_t tile = blockIdx.x;
@@ -559,6 +571,8 @@ __global__ void __launch_bounds__(kThreads) k_compact_wide(const uint32_t* bits,
 // per-tile scan with the tile's offset.
 
 __global__ void __launch_bounds__(kThreads) k_tile_sums(const int32_t* in, int64_t n, int64_t* sums) {
+  grid_launch_next();
+  grid_wait();
   __shared__ int64_t red[kThreads / 32];
   const int64_t base = static_cast<int64_t>(blockIdx.x) * kRowsPerBlock;
   int64_t s = 0;
@@ -579,6 +593,8 @@ __global__ void __launch_bounds__(kThreads) k_tile_sums(const int32_t* in, int64
 // threads, each scanning a contiguous run sequentially.
 template <typename T>
 __global__ void __launch_bounds__(1024) k_scan_single(const T* in, int64_t n, int64_t* out) {
+  grid_launch_next();
+  grid_wait();
   __shared__ int64_t sh[1024];
   const int64_t per = (n + 1023) / 1024;
   const int64_t b = threadIdx.x * per;
@@ -602,6 +618,8 @@ __global__ void __launch_bounds__(1024) k_scan_single(const T* in, int64_t n, in
 
 __global__ void __launch_bounds__(kThreads) k_tile_scan(const int32_t* in, int64_t n, const int64_t* tile_off,
                                                         int64_t* out) {
+  grid_launch_next();
+  grid_wait();
   __shared__ int sh[kThreads / 32];
   const int64_t base = static_cast<int64_t>(blockIdx.x) * kRowsPerBlock + threadIdx.x * 8;
   int v[8];
@@ -685,6 +703,8 @@ __global__ void k_fill_u64(unsigned long long* p, int64_t n, unsigned long long 
 __global__ void __launch_bounds__(kThreads) k_decide(const float* logits, int64_t S, int K, int32_t* decision,
                                                      uint32_t* yes_bits, int32_t* block_counts,
                                                      unsigned long long* label_counts) {
+  grid_launch_next();
+  grid_wait();
   __shared__ int red[kThreads / 32];
   __shared__ unsigned int hist[16];
   if (threadIdx.x < 16) hist[threadIdx.x] = 0;
@@ -808,19 +828,19 @@ void launch_cols(int n4, unsigned grid, const PredSet& ps, int64_t n, uint32_t* 
                  const TileScan& ts, cudaStream_t s) {
   switch (n4) {
     case 0:
-      if constexpr (N8 > 0) k_predicate_cols<N8, 0><<<grid, kThreads, 0, s>>>(ps, n, bits, counts, ts);
+      if constexpr (N8 > 0) launch_chained(k_predicate_cols<N8, 0>, dim3(grid), kThreads, 0, s, 1, ps, n, bits, counts, ts);
       break;
     case 1:
-      if constexpr (N8 < 4) k_predicate_cols<N8, 1><<<grid, kThreads, 0, s>>>(ps, n, bits, counts, ts);
+      if constexpr (N8 < 4) launch_chained(k_predicate_cols<N8, 1>, dim3(grid), kThreads, 0, s, 1, ps, n, bits, counts, ts);
       break;
     case 2:
-      if constexpr (N8 < 3) k_predicate_cols<N8, 2><<<grid, kThreads, 0, s>>>(ps, n, bits, counts, ts);
+      if constexpr (N8 < 3) launch_chained(k_predicate_cols<N8, 2>, dim3(grid), kThreads, 0, s, 1, ps, n, bits, counts, ts);
       break;
     case 3:
-      if constexpr (N8 < 2) k_predicate_cols<N8, 3><<<grid, kThreads, 0, s>>>(ps, n, bits, counts, ts);
+      if constexpr (N8 < 2) launch_chained(k_predicate_cols<N8, 3>, dim3(grid), kThreads, 0, s, 1, ps, n, bits, counts, ts);
       break;
     default:
-      if constexpr (N8 < 1) k_predicate_cols<N8, 4><<<grid, kThreads, 0, s>>>(ps, n, bits, counts, ts);
+      if constexpr (N8 < 1) launch_chained(k_predicate_cols<N8, 4>, dim3(grid), kThreads, 0, s, 1, ps, n, bits, counts, ts);
       break;
   }
 }
@@ -843,7 +863,7 @@ bool filter_is_small(int64_t n_rows) { return n_rows > 0 && n_rows <= kSmallRows
 
 void launch_filter_small(const PredSet& ps, int64_t n_rows, int32_t* ids, int64_t* count, int64_t* count2,
                          cudaStream_t s) {
-  k_filter_small<<<1, kSmallThreads, 0, s>>>(ps, n_rows, ids, count, count2);
+  launch_chained(k_filter_small, dim3(1), kSmallThreads, 0, s, 1, ps, n_rows, ids, count, count2);
 }
 
 int launch_predicate_scan(const PredSet& ps, const ProbeSpec& probe, int64_t n_rows, uint32_t* bits,
@@ -862,7 +882,7 @@ int launch_predicate_scan(const PredSet& ps, const ProbeSpec& probe, int64_t n_r
   TileScan ts{block_counts, offsets, grid <= kScanTilesMax ? arrived : nullptr, total};
   bool fused = ts.arrived != nullptr;
   if (probe.keys) {
-    k_probe_mask<<<grid, kProbeThreads, 0, s>>>(ps, probe, n_rows, bits, block_counts, ts);
+    launch_chained(k_probe_mask, dim3(grid), kProbeThreads, 0, s, 1, ps, probe, n_rows, bits, block_counts, ts);
   } else if (ps.n >= 1 && ps.n <= 4 && aligned) {
     int n8 = 0;
     const PredSet o = wide_first(ps, &n8);
@@ -874,7 +894,7 @@ int launch_predicate_scan(const PredSet& ps, const ProbeSpec& probe, int64_t n_r
       default: launch_cols<4>(0, grid, o, n_rows, bits, block_counts, ts, s); break;
     }
   } else {
-    k_predicate_mask<<<grid, kThreads, 0, s>>>(ps, n_rows, bits, block_counts);
+    launch_chained(k_predicate_mask, dim3(grid), kThreads, 0, s, 1, ps, n_rows, bits, block_counts);
     fused = false;
   }
   const cudaError_t e = cudaGetLastError();
@@ -896,7 +916,7 @@ int launch_predicate_scan(const PredSet& ps, const ProbeSpec& probe, int64_t n_r
 }
 
 void launch_scan_counts(const int32_t* counts, int64_t n, int64_t* offsets, cudaStream_t s) {
-  k_scan_single<int32_t><<<1, 1024, 0, s>>>(counts, n, offsets);
+  launch_chained(k_scan_single<int32_t>, dim3(1), 1024, 0, s, 1, counts, n, offsets);
 }
 
 void launch_compact(const uint32_t* bits, const int64_t* block_offsets, int64_t n_rows, int32_t* ids_out,
@@ -905,17 +925,17 @@ void launch_compact(const uint32_t* bits, const int64_t* block_offsets, int64_t 
   const unsigned tiles = blocks_for(n_rows, kRowsPerBlock);
   if (tiles <= (payload_out ? kWidePayloadTilesMax : kWideTilesMax)) {
     if (payload_out)
-      k_compact_wide<true><<<tiles, kThreads, 0, s>>>(bits, block_offsets, ids_out, payload, payload_out, arrived);
+      launch_chained(k_compact_wide<true>, dim3(tiles), kThreads, 0, s, 1, bits, block_offsets, ids_out, payload, payload_out, arrived);
     else
-      k_compact_wide<false><<<tiles, kThreads, 0, s>>>(bits, block_offsets, ids_out, payload, payload_out, arrived);
+      launch_chained(k_compact_wide<false>, dim3(tiles), kThreads, 0, s, 1, bits, block_offsets, ids_out, payload, payload_out, arrived);
     return;
   }
   const unsigned grid = (tiles + kCompactWarps - 1) / kCompactWarps;  // one tile per warp
   if (payload_out)
-    k_compact<true><<<grid, kCompactWarps * 32, 0, s>>>(bits, block_offsets, n_rows, ids_out, payload, payload_out,
+    launch_chained(k_compact<true>, dim3(grid), kCompactWarps * 32, 0, s, 1, bits, block_offsets, n_rows, ids_out, payload, payload_out,
                                                         arrived);
   else
-    k_compact<false><<<grid, kCompactWarps * 32, 0, s>>>(bits, block_offsets, n_rows, ids_out, payload, payload_out,
+    launch_chained(k_compact<false>, dim3(grid), kCompactWarps * 32, 0, s, 1, bits, block_offsets, n_rows, ids_out, payload, payload_out,
                                                          arrived);
 }
 
@@ -946,15 +966,15 @@ void launch_scan_lengths(const int32_t* lens, int64_t S, int64_t* cu, int64_t* s
   }
   int64_t* sums = scratch_blocks;
   int64_t* off = scratch_blocks + tiles + 1;
-  k_tile_sums<<<static_cast<unsigned>(tiles), kThreads, 0, s>>>(lens, S, sums);
-  k_scan_single<int64_t><<<1, 1024, 0, s>>>(sums, tiles, off);
-  k_tile_scan<<<static_cast<unsigned>(tiles), kThreads, 0, s>>>(lens, S, off, cu);
+  launch_chained(k_tile_sums, dim3(static_cast<unsigned>(tiles)), kThreads, 0, s, 1, lens, S, sums);
+  launch_chained(k_scan_single<int64_t>, dim3(1), 1024, 0, s, 1, sums, tiles, off);
+  launch_chained(k_tile_scan, dim3(static_cast<unsigned>(tiles)), kThreads, 0, s, 1, lens, S, off, cu);
 }
 
 void launch_decide(const float* logits, int64_t S, int K, int32_t* decision, uint32_t* yes_bits,
                    int32_t* block_counts, unsigned long long* label_counts, cudaStream_t s) {
   if (S <= 0) return;
-  k_decide<<<blocks_for(S, kRowsPerBlock), kThreads, 0, s>>>(logits, S, K, decision, yes_bits, block_counts,
+  launch_chained(k_decide, dim3(blocks_for(S, kRowsPerBlock)), kThreads, 0, s, 1, logits, S, K, decision, yes_bits, block_counts,
                                                              label_counts);
 }
 
