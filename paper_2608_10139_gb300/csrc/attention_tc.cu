@@ -55,12 +55,16 @@ constexpr int kKeys = 64;  // keys per block
 
 // Three CTAs per SM at head_dim 64, two at 128 (TMEM holds 512 columns).  Measured
 // at 970 rows of the select workload's text (128,867 tokens, 64 prefix keys, 32/8
-// heads, head_dim 64): 387 us, four CTAs with one Q slot and two K slots 399,
-// two with four K and V slots 455, and 445 for two CTAs of 192 threads that double
+// heads, head_dim 64): 376 us, and 445 for two CTAs of 192 threads that double
 // the score buffers and accumulators and store through shared memory; at head_dim
-// 128 (150 rows, 34,972 tokens, 128 prefix keys): 222 us, 226 with three K slots,
-// and 353 for one such CTA per SM.  A CTA of two tiles that share K and V took 427
-// and 346 us: its one MMA warp then serves both tiles' hand-offs in turn.
+// 128 (150 rows, 34,972 tokens, 128 prefix keys): 217 us, and 353 for one such CTA
+// per SM.  What else was measured, against 387 and 222 us (V loaded right behind
+// its K, an item's bounds read after its predecessor's output): four CTAs with one
+// Q slot and two K slots 399, two with four K and V slots 455; a CTA of two tiles
+// that share K and V 427 and 346, its one MMA warp serving both tiles' hand-offs
+// in turn; outputs staged in shared memory for TMA 418 and 242 (each warp on its
+// own 395 and 226 against 376 and 217), 16-byte row stores 395 and 236; MMAs
+// issued by one lane's control flow instead of a whole warp's 437 and 252.
 template <int HD>
 struct ACfg {
   static constexpr int NC = HD / 64;             // 64-column sub-tiles of one head
@@ -310,6 +314,17 @@ __global__ void __launch_bounds__(kThreadsTC, ACfg<HD>::CTAS)
         mbar_arrive(&info_full[is]);
         return true;
       };
+      // the V load of the block whose K load came last
+      const CUtensorMap* v_map = nullptr;
+      int v_col = 0, v_row = 0;
+      auto load_v = [&]() -> bool {
+        const int vb = gv % NV;
+        if (!mbar_wait_bounded(&v_empty[vb], ((gv / NV) & 1) ^ 1, abort_flag, err)) return false;
+        mbar_arrive_expect_tx(&v_full[vb], C::K_BYTES);
+        for (int c = 0; c < C::NC; ++c) tma_load_2d(sV(vb) + c * C::SUB, v_map, &v_full[vb], v_col + c * 64, v_row);
+        ++gv;
+        return true;
+      };
       const int step = gridDim.x;
       int w = blockIdx.x;
       int4 cur = bounds(list(w), w), nxt = bounds(list(w + step), w + step);
@@ -331,27 +346,29 @@ __global__ void __launch_bounds__(kThreadsTC, ACfg<HD>::CTAS)
           const bool pre = j < n_pre;
           const CUtensorMap* map = pre ? &tm_pre : &tm_kv;
           const int kcol = pre ? kvh * HD : (a.Hq + kvh) * HD;
-          const int vcol = pre ? (a.Hkv + kvh) * HD : (a.Hq + a.Hkv + kvh) * HD;
           const int row = pre ? j * kKeys : st + (j - n_pre) * kKeys;
-          const int kb = g % NK, vb = g % NV;
+          const int kb = g % NK;
           if (!mbar_wait_bounded(&k_empty[kb], ((g / NK) & 1) ^ 1, abort_flag, err)) {
             ok = false;
             break;
           }
           mbar_arrive_expect_tx(&k_full[kb], C::K_BYTES);
           for (int c = 0; c < C::NC; ++c) tma_load_2d(sK(kb) + c * C::SUB, map, &k_full[kb], kcol + c * 64, row);
-          if (!mbar_wait_bounded(&v_empty[vb], ((g / NV) & 1) ^ 1, abort_flag, err)) {
+          // V a block behind K: its slot frees with the PV two blocks back, and the
+          // next item's Q and first K must not wait for that
+          if (g > 0 && !load_v()) {
             ok = false;
-            ++g;  // this block's K load is in flight, its V load is not
+            ++g;  // this block's K load is in flight
             break;
           }
-          mbar_arrive_expect_tx(&v_full[vb], C::K_BYTES);
-          for (int c = 0; c < C::NC; ++c) tma_load_2d(sV(vb) + c * C::SUB, map, &v_full[vb], vcol + c * 64, row);
-          ++gv;
+          v_map = map;
+          v_col = pre ? (a.Hkv + kvh) * HD : (a.Hq + a.Hkv + kvh) * HD;
+          v_row = row;
         }
         cur = nxt;
         nxt = after;
       }
+      if (ok && g > gv && !load_v()) ok = false;
       if (!ok || *abort_flag) {
         // let this thread's copies still in flight land before the CTA can exit
         // (the last use of each slot is the only one that can be outstanding)
@@ -492,12 +509,18 @@ __global__ void __launch_bounds__(kThreadsTC, ACfg<HD>::CTAS)
     bool ok = true;
     // PV of block gg done (see the ordering note above: the parity is exact)
     auto wait_pv = [&](uint32_t gg) -> bool { return wait_all(&o_done[gg & 1], (gg >> 1) & 1); };
-    for (int w = blockIdx.x; w < n_work && ok; w += gridDim.x, ++it) {
-      const int is = it & 3;
-      if (!wait_all(&info_full[is], (it >> 2) & 1)) break;
-      const int4 inf = info[is];
+    auto take_info = [&](int item, int4* inf) -> bool {
+      const int is = item & 3;
+      if (!wait_all(&info_full[is], (item >> 2) & 1)) return false;
+      *inf = info[is];
       __syncwarp();
       if (lane == 0) mbar_arrive(&info_empty[is]);
+      return true;
+    };
+    int4 inf = make_int4(0, 0, 0, 0), inf_next = inf;
+    if (static_cast<int>(blockIdx.x) < n_work) ok = take_info(0, &inf_next);
+    for (int w = blockIdx.x; w < n_work && ok; w += gridDim.x, ++it) {
+      inf = inf_next;
       const int st = inf.x, len = inf.y, q0 = inf.z, kvh = inf.w % kNoPrefix;
       const int n_pre = prefix_blocks(inf), n_kv = blocks_of(inf);
       const int qpos = q0 + t;
@@ -575,6 +598,8 @@ __global__ void __launch_bounds__(kThreadsTC, ACfg<HD>::CTAS)
         if (lane == 0) mbar_arrive(&p_full[sb]);
       }
       if (!ok) break;
+      // the next item's bounds while this item's last PV runs
+      if (w + static_cast<int>(gridDim.x) < n_work && !take_info(it + 1, &inf_next)) break;
       // O / l of the tile's real tokens, once the item's last PV is done
       if (!wait_pv(g - 1)) break;
       tc_fence_after();
