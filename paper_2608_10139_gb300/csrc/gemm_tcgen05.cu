@@ -810,9 +810,10 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 // ------------------------------------------------------------- few rows ---
 // Products with few rows (a generation step, the shared prefix's own pass, a
-// small chunk, the final layer's last tokens): MT x BN tiles of one CTA with
-// MT = 64 or 128 and BN = 16 .. 128, so that even N = 2048 gives every SM a slice of the weights
-// to stream.  Bound by the weights' read from DRAM; what each CTA moves per
+// small chunk, the final layer's last tokens), in narrow tiles, so that even N =
+// 2048 gives every SM a slice of the weights to stream.  Up to 64 rows a CTA by
+// itself takes all of them and BN = 16 .. 128 weight columns; more rows are shared by
+// two CTAs (k_gemm_few_pair).  Bound by the weights' read from DRAM; what each CTA moves per
 // 64-deep k-block is (rows of A + BN) x 128 bytes, so A's box holds only the
 // rows that exist (rounded up to 8; the MMA's other rows read whatever follows
 // in shared memory and are never stored).  One TMA per operand fills a stage
@@ -824,9 +825,10 @@ __global__ void __launch_bounds__(kThreads, 1)
 // Every element's products are summed in the order of the large-tile kernels
 // and every epilogue step is the same operation, so a row's results do not
 // depend on which kernel computed it.
+constexpr int kFewRows = 64;           // rows that one CTA stages
 constexpr int kFewSmem = 200 * 1024;  // operand ring
 constexpr int kFewStages = 16;
-constexpr int kFewSlack = 128 * 128;  // an A tile's MMA reads MT rows from its slot's start
+constexpr int kFewSlack = kFewRows * 128;  // an A tile's MMA reads kFewRows rows from its slot's start
 
 struct FewArgs {
   int a_rows;  // rows of A's box
@@ -974,7 +976,7 @@ __device__ __forceinline__ void epilogue_few(const KArgs& a, uint32_t trow, int 
 }
 
 // One stage's MMAs: SUB 64-deep blocks of A (a_blk bytes apart) and B.
-template <int SUB, int BN>
+template <int SUB, int BN, bool PAIR = false>
 __device__ __forceinline__ void few_issue(uint32_t d, uint64_t da, uint64_t db, uint32_t a_blk, uint32_t idesc,
                                           bool first) {
 #pragma unroll
@@ -983,14 +985,21 @@ __device__ __forceinline__ void few_issue(uint32_t d, uint64_t da, uint64_t db, 
     for (int k = 0; k < BK / UMMA_K; ++k) {
       // descriptors count 16-byte units; UMMA_K fp16 = 32 bytes
       const uint64_t a = da + sb * (a_blk >> 4) + 2 * k, b = db + sb * (BN * 128 >> 4) + 2 * k;
-      if (sb == 0 && k == 0)
-        umma_f16_ss(d, a, b, idesc, !first);
-      else
-        umma_f16_ss_acc(d, a, b, idesc);
+      if constexpr (PAIR) {
+        if (sb == 0 && k == 0)
+          umma_f16_ss_pair(d, a, b, idesc, !first);
+        else
+          umma_f16_ss_pair_acc(d, a, b, idesc);
+      } else {
+        if (sb == 0 && k == 0)
+          umma_f16_ss(d, a, b, idesc, !first);
+        else
+          umma_f16_ss_acc(d, a, b, idesc);
+      }
     }
 }
 
-template <int MT, int BN, int EPI>
+template <int BN, int EPI>
 __global__ void __launch_bounds__(kThreads, 1)
     k_gemm_few(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ CUtensorMap tma_b, KArgs args,
                FewArgs fa) {
@@ -1038,10 +1047,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   grid_launch_next();
   grid_wait();
 
-  const int num_m = (args.M + MT - 1) / MT;
-  const int num_tiles = num_m * (args.N / BN);
+  const int num_tiles = args.N / BN;
   const int kblocks = args.K / (BK * sub);
-  // row tiles fastest: the CTAs that share a weight slice run together
 
   if (warp == 0) {
     if (lane == 0) {
@@ -1049,8 +1056,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       uint32_t issued = 0, s = 0, ph = 1;
       bool ok = true;
       for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
-        const int m0 = (tile % num_m) * MT;
-        const int n0 = few_n0<BN>(tile / num_m, fa.half);
+        const int n0 = few_n0<BN>(tile, fa.half);
         for (int kb = 0; kb < kblocks; ++kb) {
           if (!mbar_wait_bounded(&empty[s], ph, abort_flag, err)) {
             ok = false;
@@ -1058,7 +1064,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
           mbar_arrive_expect_tx(&full[s], a_bytes + b_bytes);
           tma_load_4d(sB + s * b_bytes, &tma_b, &full[s], 0, n0, 0, kb * sub);
-          tma_load_3d(sA + s * a_bytes, &tma_a, &full[s], 0, m0, kb * sub);
+          tma_load_3d(sA + s * a_bytes, &tma_a, &full[s], 0, 0, kb * sub);
           ++issued;
           if (++s == stages) {
             s = 0;
@@ -1078,8 +1084,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     // The whole warp walks the stages and one elected lane issues: the
     // descriptors then stay in uniform registers.  Issue is what a short MMA
     // waits for: 90 clocks each when formed per MMA in one lane, against the
-    // tensor core's own 39 (128 x 16 x 16) or 23 (64 x 16 x 16).
-    constexpr uint32_t idesc = idesc_f16_f32(MT, BN);
+    // tensor core's own 23 (64 x 16 x 16).
+    constexpr uint32_t idesc = idesc_f16_f32(kFewRows, BN);
     const uint64_t da0 = smem_desc_k_sw128(smem_u32(sA)), db0 = smem_desc_k_sw128(smem_u32(sB));
     const uint32_t tb = __shfl_sync(0xffffffffu, tmem_base, 0);
     uint32_t s = 0, ph = 0;
@@ -1131,11 +1137,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     int acc = 0;
     uint32_t acc_ph = 0;
     for (int tile = blockIdx.x; tile < num_tiles; tile += gridDim.x) {
-      const int m0 = (tile % num_m) * MT;
-      const int n0 = few_n0<BN>(tile / num_m, fa.half);
+      const int n0 = few_n0<BN>(tile, fa.half);
       // a 64-row accumulator takes the first 16 TMEM lanes of each quarter
-      const int row = m0 + quarter * (MT / 4) + lane;
-      const bool live = (MT == 128 || lane < 16) && row < args.M;
+      const int row = quarter * 16 + lane;
+      const bool live = lane < 16 && row < args.M;
       if (EPI == EPI_RESID_F32) {
         if (live)
           prefetch_l2(static_cast<const float*>(args.ep.out) + static_cast<int64_t>(row) * args.ep.ldo + n0, BN * 4);
@@ -1143,7 +1148,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const float inv = EPI == EPI_ROPE_F16 || EPI == EPI_SWIGLU_F16 ? row_inv_rms(args.ep, row, live) : 1.f;
       if (!__all_sync(0xffffffffu, mbar_wait_bounded(&tfull[acc], acc_ph, abort_flag, err))) break;
       tc_fence_after();
-      if (m0 + quarter * (MT / 4) < args.M)  // warp-uniform: this warp holds at least one live row
+      if (quarter * 16 < args.M)  // warp-uniform: this warp holds at least one live row
         epilogue_few<BN, EPI>(args, tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + acc * BN, row, live,
                               n0, fa.half, inv);
       tc_fence_before();
@@ -1158,6 +1163,188 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem_base, TMEM_COLS);
+  }
+}
+
+// Two CTAs per tile of 128 rows x 2 BN columns (tcgen05.mma.cta_group::2, M =
+// 128): each stages 64 of the rows and the BN weight columns of one of two
+// neighbouring tiles of k_gemm_few, so that per product an SM takes in (64 + BN)
+// bytes where a CTA by itself takes (128 + BN); the arrival of the operands is what
+// bounds these products at more than 64 rows (60 to 68 bytes a clock per SM).  Each CTA's TMEM holds
+// its 64 rows: the first tile's columns on lanes 0-63, the second's on lanes
+// 64-127.  Barriers as in k_gemm_tcgen05_pair.  128 rows, 4096 x 14336: 47 -> 35 us
+// (17 at the weights' read); the four products of a 128-row block of that size
+// together 150 -> 130.
+template <int BN, int EPI>
+__global__ void __launch_bounds__(kThreads, 1)
+    k_gemm_few_pair(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ CUtensorMap tma_b, KArgs args,
+                    FewArgs fa) {
+  constexpr int TMEM_COLS = 2 * BN < 32 ? 32 : 2 * BN;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  __shared__ uint64_t full[kFewStages], empty[kFewStages], tfull[2], tempty[2], mma_done;
+  __shared__ uint32_t tmem_slot;
+  __shared__ int abort_word;
+  volatile int* abort_flag = &abort_word;
+
+  const int warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31;
+  const uint32_t rank = cluster_ctarank();
+  const bool leader = rank == 0;
+  const int pair = blockIdx.x >> 1;
+  const int n_pairs = gridDim.x >> 1;
+  int* err = args.ep.err;
+  const uint32_t stages = fa.stages, sub = fa.sub;
+  constexpr uint32_t a_blk = 64 * 128, b_blk = BN * 128;
+  const uint32_t a_bytes = sub * a_blk, b_bytes = sub * b_blk;  // a stage of this CTA
+  uint8_t* sA = smem;
+  uint8_t* sB = smem + stages * a_bytes;
+
+  if (threadIdx.x == 0) {
+    for (uint32_t s = 0; s < stages; ++s) {
+      mbar_init(&full[s], 1);   // used in the leader only
+      mbar_init(&empty[s], 1);  // per CTA, multicast by the leader's commits
+    }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&tfull[i], 1);
+      mbar_init(&tempty[i], 8);  // used in the leader only: 4 warps x 2 CTAs
+    }
+    mbar_init(&mma_done, 1);
+    *abort_flag = 0;
+    fence_mbar_init();
+    tma_prefetch_desc(&tma_a);
+    tma_prefetch_desc(&tma_b);
+  }
+  if (warp == 1) {
+    tmem_alloc_pair(&tmem_slot, TMEM_COLS);
+    tmem_relinquish_pair();
+    tc_fence_before();
+  }
+  __syncthreads();
+  cluster_sync();  // barriers of both CTAs initialised before any remote arrival
+  tc_fence_after();
+  const uint32_t tmem_base = tmem_slot;
+  grid_launch_next();
+  grid_wait();
+
+  const int num_m = (args.M + 127) / 128;
+  // row tiles fastest: the CTAs that share a weight slice run together
+  const int num_tiles = num_m * (args.N / (2 * BN));
+  const int kblocks = args.K / (BK * sub);
+
+  if (warp == 0) {
+    if (lane == 0) {
+      // ---------------------------------------------------- TMA producer
+      const uint32_t full_leader = map_to_cta(smem_u32(full), 0);
+      uint32_t issued = 0, s = 0, ph = 1;
+      bool ok = true;
+      for (int tile = pair; tile < num_tiles && ok; tile += n_pairs) {
+        const int m0 = (tile % num_m) * 128 + rank * 64;
+        const int n0 = few_n0<BN>(2 * (tile / num_m) + rank, fa.half);
+        for (int kb = 0; kb < kblocks; ++kb) {
+          if (!mbar_wait_bounded(&empty[s], ph, abort_flag, err)) {
+            ok = false;
+            break;
+          }
+          if (leader) mbar_arrive_expect_tx(&full[s], 2 * (a_bytes + b_bytes));
+          tma_load_4d_pair(sB + s * b_bytes, &tma_b, full_leader + s * 8, 0, n0, 0, kb * sub);
+          tma_load_3d_pair(sA + s * a_bytes, &tma_a, full_leader + s * 8, 0, m0, kb * sub);
+          ++issued;
+          if (++s == stages) {
+            s = 0;
+            ph ^= 1;
+          }
+        }
+      }
+      if (!ok && leader) {
+        // the leader's barrier completes only once both CTAs' bytes have landed
+        volatile int never = 0;
+        for (uint32_t i = issued > stages ? issued - stages : 0; i < issued; ++i)
+          mbar_wait_bounded(&full[i % stages], (i / stages) & 1, &never, nullptr, 200000000ull);
+      }
+    }
+  } else if (warp == 1) {
+    if (leader) {
+      // ------------------------------------------------ MMA issuer (leader)
+      constexpr uint32_t idesc = idesc_f16_f32(128, 2 * BN);
+      const uint64_t da0 = smem_desc_k_sw128(smem_u32(sA)), db0 = smem_desc_k_sw128(smem_u32(sB));
+      const uint32_t tb = __shfl_sync(0xffffffffu, tmem_base, 0);
+      uint32_t s = 0, ph = 0;
+      int acc = 0;
+      uint32_t acc_ph = 0;
+      bool ok = true;
+      for (int tile = pair; tile < num_tiles && ok; tile += n_pairs) {
+        if (!__all_sync(0xffffffffu, mbar_wait_bounded(&tempty[acc], acc_ph ^ 1, abort_flag, err))) break;
+        tc_fence_after();
+        const uint32_t d_tmem = tb + acc * BN;
+        for (int kb = 0; kb < kblocks; ++kb) {
+          if (!__all_sync(0xffffffffu, mbar_wait_bounded(&full[s], ph, abort_flag, err))) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          const uint64_t da = da0 + s * (a_bytes >> 4), db = db0 + s * (b_bytes >> 4);
+          if (elect_one()) {
+            if (sub == 4)  // four stages of eight such blocks exceed the ring
+              few_issue<4, BN, true>(d_tmem, da, db, a_blk, idesc, kb == 0);
+            else if (sub == 2)
+              few_issue<2, BN, true>(d_tmem, da, db, a_blk, idesc, kb == 0);
+            else
+              few_issue<1, BN, true>(d_tmem, da, db, a_blk, idesc, kb == 0);
+            umma_commit_pair_mc(&empty[s], 0x3);
+          }
+          __syncwarp();
+          if (++s == stages) {
+            s = 0;
+            ph ^= 1;
+          }
+        }
+        if (!ok) break;
+        if (elect_one()) umma_commit_pair_mc(&tfull[acc], 0x3);
+        __syncwarp();
+        acc ^= 1;
+        if (acc == 0) acc_ph ^= 1;
+      }
+      // every MMA issued above has completed once this arrives
+      if (elect_one()) umma_commit_pair_mc(&mma_done, 0x1);
+      __syncwarp();
+      volatile int never = 0;
+      mbar_wait_bounded(&mma_done, 0, &never, err);
+    }
+  } else {
+    // ------------------------------------------------ epilogue (both CTAs)
+    const int quarter = warp & 3;  // TMEM lanes this warp may access
+    const uint32_t tempty_leader = map_to_cta(smem_u32(tempty), 0);
+    int acc = 0;
+    uint32_t acc_ph = 0;
+    for (int tile = pair; tile < num_tiles; tile += n_pairs) {
+      const int m0 = (tile % num_m) * 128 + rank * 64 + (quarter & 1) * 32;
+      const int n0 = few_n0<BN>(2 * (tile / num_m) + (quarter >> 1), fa.half);
+      const int row = m0 + lane;
+      const bool live = row < args.M;
+      if (EPI == EPI_RESID_F32) {
+        if (live)
+          prefetch_l2(static_cast<const float*>(args.ep.out) + static_cast<int64_t>(row) * args.ep.ldo + n0, BN * 4);
+      }
+      const float inv = EPI == EPI_ROPE_F16 || EPI == EPI_SWIGLU_F16 ? row_inv_rms(args.ep, row, live) : 1.f;
+      if (!__all_sync(0xffffffffu, mbar_wait_bounded(&tfull[acc], acc_ph, abort_flag, err))) break;
+      tc_fence_after();
+      if (m0 < args.M)  // warp-uniform: this warp holds at least one live row
+        epilogue_few<BN, EPI>(args, tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + acc * BN, row, live,
+                              n0, fa.half, inv);
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive_cluster(tempty_leader + acc * 8);
+      acc ^= 1;
+      if (acc == 0) acc_ph ^= 1;
+    }
+  }
+
+  __syncthreads();
+  cluster_sync();  // no CTA leaves while its peer may still signal it
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc_pair(tmem_base, TMEM_COLS);
   }
 }
 
@@ -1300,11 +1487,11 @@ int few_half(int tile, int bn, const GemmEpilogue& ep) {
   return tile / 2;
 }
 
-template <int MT, int BN, int EPI>
+template <bool PAIR, int BN, int EPI>
 int launch_few(const __half* A, int64_t lda, const __half* B, int64_t ldb, const KArgs& a, int bn, int num_sms,
                cudaStream_t stream) {
   FewArgs fa;
-  fa.a_rows = a.M < MT ? (a.M + 7) / 8 * 8 : MT;
+  fa.a_rows = a.M < kFewRows ? (a.M + 7) / 8 * 8 : kFewRows;
   fa.half = few_half(BN, bn, a.ep);
   // the deepest stage (one TMA per operand) that leaves four of them in the ring
   const int block = (fa.a_rows + BN) * 128;
@@ -1322,28 +1509,36 @@ int launch_few(const __half* A, int64_t lda, const __half* B, int64_t ldb, const
     return cudaErrorInvalidValue;
   constexpr int SM = 1024 + kFewSmem + kFewSlack;
   static_assert(SM + 1024 <= 232448, "shared memory per block");
-  cudaError_t e = cudaFuncSetAttribute(k_gemm_few<MT, BN, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, SM);
+  void (*kernel)(const CUtensorMap, const CUtensorMap, KArgs, FewArgs);
+  int grid;
+  if constexpr (PAIR) {
+    kernel = k_gemm_few_pair<BN, EPI>;
+    grid = 2 * std::min((a.M + 127) / 128 * (a.N / (2 * BN)), num_sms / 2);
+  } else {
+    kernel = k_gemm_few<BN, EPI>;
+    grid = std::min(a.N / BN, num_sms);
+  }
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SM);
   if (e != cudaSuccess) return e;
-  const int tiles = ((a.M + MT - 1) / MT) * (a.N / BN);
-  return launch_chained(k_gemm_few<MT, BN, EPI>, dim3(tiles < num_sms ? tiles : num_sms), kThreads, SM, stream, 1, ma,
-                        mb, a, fa);
+  return launch_chained(kernel, dim3(grid), kThreads, SM, stream, PAIR ? 2 : 1, ma, mb, a, fa);
+}
+
+template <int BN, int EPI>
+int launch_few_rows(const __half* A, int64_t lda, const __half* B, int64_t ldb, const KArgs& a, int bn, int num_sms,
+                    cudaStream_t s) {
+  return a.M <= kFewRows ? launch_few<false, BN, EPI>(A, lda, B, ldb, a, bn, num_sms, s)
+                         : launch_few<true, BN, EPI>(A, lda, B, ldb, a, bn, num_sms, s);
 }
 
 template <int BN>
 int dispatch_few(const __half* A, int64_t lda, const __half* B, int64_t ldb, const KArgs& a, int bn, int num_sms,
                  cudaStream_t s) {
-  const bool m64 = a.M <= 64;
   switch (a.ep.kind) {
-    case EPI_ROPE_F16:
-      return m64 ? launch_few<64, BN, EPI_ROPE_F16>(A, lda, B, ldb, a, bn, num_sms, s)
-                 : launch_few<128, BN, EPI_ROPE_F16>(A, lda, B, ldb, a, bn, num_sms, s);
-    case EPI_SWIGLU_F16:
-      return m64 ? launch_few<64, BN, EPI_SWIGLU_F16>(A, lda, B, ldb, a, bn, num_sms, s)
-                 : launch_few<128, BN, EPI_SWIGLU_F16>(A, lda, B, ldb, a, bn, num_sms, s);
+    case EPI_ROPE_F16: return launch_few_rows<BN, EPI_ROPE_F16>(A, lda, B, ldb, a, bn, num_sms, s);
+    case EPI_SWIGLU_F16: return launch_few_rows<BN, EPI_SWIGLU_F16>(A, lda, B, ldb, a, bn, num_sms, s);
     case EPI_RESID_F32:
     case EPI_RESID_ADD:  // the same sum, added by the epilogue threads
-      return m64 ? launch_few<64, BN, EPI_RESID_F32>(A, lda, B, ldb, a, bn, num_sms, s)
-                 : launch_few<128, BN, EPI_RESID_F32>(A, lda, B, ldb, a, bn, num_sms, s);
+      return launch_few_rows<BN, EPI_RESID_F32>(A, lda, B, ldb, a, bn, num_sms, s);
   }
   return cudaErrorInvalidValue;
 }
@@ -1351,19 +1546,21 @@ int dispatch_few(const __half* A, int64_t lda, const __half* B, int64_t ldb, con
 }  // namespace
 
 // The kernels' times are estimated from what bounds them, in SM clocks, and the
-// smallest wins.  Per 64-deep k-block a CTA takes the larger of its MMAs (45
-// clocks each at 64 rows, where issue bounds them; 45 to 64 at 128 rows) and of
-// its operands' arrival (60 bytes per clock); the large tiles measure 720
+// smallest wins.  Per 64-deep k-block a CTA of the few-rows kernels takes the larger
+// of its MMAs (45 clocks each, where issue bounds them) and of its operands' arrival
+// (60 bytes per clock); the large tiles measure 720
 // (128 x 256), 540 (128 x 128) and 660 (CTA pair).  An epilogue column costs 100
 // clocks where the threads add to the residual, 50 for SwiGLU, 40 for RoPE and 22 for the
 // TMA add, and each epilogue 1200 more for its hand-offs; a tile's epilogue runs beside the next tile's main loop.  Measured
-// (us, weights from DRAM; with about 7 us of launch and event overhead):
-//   M     N      K      large   16     32     64     128
-//   24    2048   8192   55.6    18.5   21.3   23.0   32.1
-//   300   2048   8192   59.3    71.9   52.1   34.2   46.3
-//   1000  2048   8192   55.3    157    95.2   56.6   48.8
-//   24    28672  4096   53.3    67.1   48.5   44.7   48.9
-//   500   28672  4096   96.5    516    266    146    113
+// (us, weights from DRAM; with about 7 us of launch and event overhead; in brackets
+// what one CTA per 128 rows took before pairs shared them):
+//   M     N      K      large   16          32          64          128
+//   24    2048   8192   55.6    18.5        21.3        23.0        32.1
+//   128   4096   14336  96.4    41.4 (82.7) 35.0 (47.1) 39.8 (49.6) 55.2 (71.5)
+//   300   2048   8192   59.4    34.8 (72.9) 30.4 (52.4) 26.3 (33.4) 36.4 (46.5)
+//   1000  2048   8192   54.0    69.6 (157)  50.7 (95.4) 42.4 (56.5) 36.8 (48.3)
+//   24    28672  4096   53.3    67.1        48.5        44.7        48.9
+//   500   28672  4096   98.8    216 (518)   140 (266)   106 (148)   87.2 (115)
 int gemm_few_tile(int M, int N, int K, int bn, bool pair, const GemmEpilogue& ep, int num_sms) {
   if (M > kFewRowsMax) return 0;
   int epi = 0, epi_large = 0;  // clocks per column
@@ -1385,11 +1582,15 @@ int gemm_few_tile(int M, int N, int K, int bn, bool pair, const GemmEpilogue& ep
                      ? cost((M + 255) / 256 * (N / 256), num_sms / 2, 660, 256 * epi_large)
                      : cost(m128 * (N / bn), num_sms, bn == 256 ? 720 : 540, bn * epi_large);
   int tile = 0;
-  const int a_rows = M < 128 ? (M + 7) / 8 * 8 : 128;
   for (int t = 16; t <= 128; t *= 2) {
     if (t / 2 > few_half(t, bn, ep)) break;  // a tile's halves lie within a gate / up block or a head
-    const int64_t mma = M <= 64 ? std::max(180, 2 * t) : 160 + t * 3 / 4;
-    const int64_t c = cost(m128 * (N / t), num_sms, std::max<int64_t>(mma, (a_rows + t) * 128 / 60), t * epi);
+    int64_t c;
+    if (M <= 64) {
+      c = cost(N / t, num_sms, std::max(std::max(180, 2 * t), ((M + 7) / 8 * 8 + t) * 128 / 60), t * epi);
+    } else {
+      if (N % (2 * t) != 0) break;
+      c = cost(m128 * (N / (2 * t)), num_sms / 2, std::max(180, (64 + t) * 128 / 60), t * epi);
+    }
     if (c < best) best = c, tile = t;
   }
   return tile;

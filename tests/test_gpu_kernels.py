@@ -139,6 +139,39 @@ def test_rmsnorm(ctx, d):
     ref = tf.rmsnorm(x.astype(np.float64), tf.bf16_to_f64(gb), 1e-5)
     _close(_np64(out), ref, 1.5e-3, 1e-4, f"rmsnorm d{d}")
 
+@pytest.mark.parametrize("epi,N,K,bn,hd", [(1, 3072, 256, 256, 64), (1, 6144, 320, 256, 128), (2, 4096, 128, 256, 0),
+                                           (5, 2048, 512, 256, 0), (3, 4096, 192, 256, 0), (3, 1024, 128, 128, 0)])
+def test_gemm_paired_narrow_tiles_match_large_tiles(ctx, epi, N, K, bn, hd):
+    """More than 64 rows: two CTAs share a narrow tile's rows (16 to 128 columns each,
+    by the product's size).  Bit for bit the rows that large tiles give, at the
+    boundaries of the pair's 64-row halves, and nothing written past the last row."""
+    rng = np.random.default_rng(N + K + epi)
+    big = 16384 + 40
+    A = torch.randn((big, K), device="cuda").half()
+    B = (torch.randn((N, K), device="cuda") * 0.05).half()
+    width = N // 2 if epi == 3 else N
+    pos = _h(rng.integers(0, 300, big).astype(np.int32))
+    cs = torch.zeros((300, max(hd, 32) // 2), dtype=torch.float32, device="cuda")
+    sn = torch.zeros_like(cs)
+    ctx.op_rope_table(cs.data_ptr(), sn.data_ptr(), 300, max(hd, 32), 1.0e4)
+    before = torch.randn((big, width), device="cuda", dtype=torch.float32 if epi in (2, 5) else torch.float16)
+    torch.cuda.synchronize()
+
+    def run(M):
+        out = before.clone()
+        torch.cuda.synchronize()
+        ctx.op_gemm(A.data_ptr(), K, B.data_ptr(), K, M, N, K, bn, epi, out.data_ptr(), width, pos.data_ptr(),
+                    cs.data_ptr(), sn.data_ptr(), N // 2 // max(hd, 1) * hd, hd)
+        torch.cuda.synchronize()
+        return out
+
+    large = run(big)
+    for M in (65, 96, 127, 129, 192, 193, 300, 500, 1500):
+        out = run(M)
+        assert torch.equal(out[:M], large[:M]), f"epilogue {epi}, {M} rows"
+        assert torch.equal(out[M:], before[M:]), f"epilogue {epi}, {M} rows: a row past the product was written"
+
+
 
 @pytest.mark.parametrize("d", [1024, 2048, 4096])
 def test_rmsnorm_few_rows_same_bits(ctx, d):
