@@ -6,9 +6,10 @@
 // allocation-free execution loop, or a latency-bound path that cannot afford
 // cudaMalloc's implicit device-wide synchronisation or its failure under
 // memory pressure.  aiq_filter_compact_static gives them the same kernels as
-// the query path (predicate bitmask, tile-count scan, compaction), with their
-// scratch (bitmask, tile counts, tile offsets, arrival counter) held in one file-scope device
-// array instead of a context's workspace.
+// the query path (predicate bitmask with tile counts, compaction), with their
+// scratch (bitmask, tile counts) held in one file-scope device array instead of
+// a context's workspace.  No tile offsets are needed: nothing on the host waits for
+// the count before the ids are written, so the compaction adds the counts up itself.
 //
 // The array is a global of this shared library: every GPU that loads the
 // library keeps kStaticScratchBytes reserved on it until the process exits.
@@ -35,11 +36,8 @@ constexpr int64_t kStaticMaxRows = int64_t(1) << 24;                     // 16,7
 constexpr int64_t kStaticTiles = kStaticMaxRows / kRowsPerBlock;         // 8192 tiles
 constexpr size_t kBitsBytes = kStaticMaxRows / 8;                        // 2 MiB bitmask
 constexpr size_t kCountBytes = kStaticTiles * sizeof(int32_t);          // 32 KiB tile counts
-constexpr size_t kOffsetBytes = (kStaticTiles + 1) * sizeof(int64_t);   // 64 KiB + 8 tile offsets
-constexpr size_t kOffsetAt = kBitsBytes + kCountBytes;
-constexpr size_t kArrivedAt = ((kOffsetAt + kOffsetBytes + 255) / 256) * 256;  // arrival counter, zero between calls
-constexpr size_t kStaticScratchBytes = kArrivedAt + 256;
-static_assert(kStaticTiles <= kScanTilesMax, "the last block scans the tile counts");
+constexpr size_t kStaticScratchBytes = kBitsBytes + kCountBytes;
+static_assert(kStaticTiles <= kScanTilesMax, "the compaction adds up the tile counts");
 
 static __device__ __align__(256) unsigned char g_filter_scratch[kStaticScratchBytes];
 
@@ -102,19 +100,15 @@ aiq_status aiq_filter_compact_static(const aiq_term* terms, int32_t n_terms, int
   if (st != AIQ_OK) return st;
   uint32_t* bits = reinterpret_cast<uint32_t*>(scratch);
   int32_t* counts = reinterpret_cast<int32_t*>(scratch + kBitsBytes);
-  int64_t* offsets = reinterpret_cast<int64_t*>(scratch + kOffsetAt);
-  unsigned int* arrived = reinterpret_cast<unsigned int*>(scratch + kArrivedAt);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (filter_is_small(n_rows)) {
     launch_filter_small(ps, n_rows, ids_out, count_out, nullptr, s);
   } else {
     // Every scratch word the compaction reads is written earlier in this call
-    // (each tile writes its whole bitmask slice and its count; the scan writes
-    // offsets[0..tiles]), so nothing is carried over from the previous call but
-    // the arrival counter, which every scan leaves at zero.
-    launch_predicate_scan(ps, ProbeSpec{}, n_rows, bits, counts, offsets,
-                          arrived, count_out, nullptr, s);
-    launch_compact(bits, offsets, n_rows, ids_out, nullptr, nullptr, s, arrived);
+    // (each tile writes its whole bitmask slice and its count), so nothing is
+    // carried over from the previous call.
+    launch_predicate_scan(ps, ProbeSpec{}, n_rows, bits, counts, nullptr, nullptr, nullptr, nullptr, s);
+    launch_compact_counts(bits, counts, n_rows, ids_out, count_out, s);
   }
   // A failed predicate launch is recorded (and its CUDA error consumed) by its
   // launcher; take that record here so that it is reported by this call and

@@ -99,6 +99,15 @@ struct TileScan {
 constexpr int64_t kSmallRows = 16384;      // rows that one block filters on its own
 constexpr unsigned kScanTilesMax = 8192;   // tiles whose counts the last block scans
 
+// Where a compaction's tiles write: at offsets[tile], or (offsets == nullptr) at the
+// sum of the counts before them, which each block then adds up by itself; the last
+// tile's block writes *total.
+struct TileBase {
+  const int64_t* offsets;
+  const int32_t* counts;  // 16-byte aligned; read only without offsets
+  int64_t* total;
+};
+
 // Filter of 1 .. kSmallRows rows (16-byte aligned columns) in one launch: the
 // survivors' ids and their number, in *count and, when given, *count2.
 bool filter_is_small(int64_t n_rows);
@@ -107,7 +116,8 @@ void launch_filter_small(const PredSet& ps, int64_t n_rows, int32_t* ids, int64_
 // Mask bits, per-tile survivor counts and their exclusive scan offsets[tiles + 1].
 // arrived: a counter that is zero before the first call; total (optional) also
 // receives the number of survivors; scan_tmp (optional): >= 2 * (ceil(tiles /
-// 2048) + 1) int64 for the multi-block scan.  Returns the number of kernels.
+// 2048) + 1) int64 for the multi-block scan.  offsets == nullptr: no scan, the bits
+// and the counts only.  Returns the number of kernels.
 int launch_predicate_scan(const PredSet& ps, const ProbeSpec& probe, int64_t n_rows, uint32_t* bits,
                           int32_t* block_counts, int64_t* offsets, unsigned int* arrived, int64_t* total,
                           int64_t* scan_tmp, cudaStream_t s);
@@ -118,6 +128,10 @@ void launch_scan_counts(const int32_t* counts, int64_t n, int64_t* offsets, cuda
 // scan's counter) to zero.
 void launch_compact(const uint32_t* bits, const int64_t* block_offsets, int64_t n_rows, int32_t* ids_out,
                     const int32_t* payload, int32_t* payload_out, cudaStream_t s, unsigned int* arrived = nullptr);
+// The same without a scan before it, for up to kScanTilesMax tiles: the counts are
+// launch_predicate_scan's, *total receives the number of set bits.
+void launch_compact_counts(const uint32_t* bits, const int32_t* block_counts, int64_t n_rows, int32_t* ids_out,
+                           int64_t* total, cudaStream_t s);
 
 void launch_hash_build(const int64_t* keys, const int32_t* rows, int64_t n, unsigned long long* table_keys,
                        int32_t* table_vals, int64_t capacity, int* err, cudaStream_t s);

@@ -8,7 +8,8 @@
 //  * order-preserving stream compaction: tile counts -> exclusive scan ->
 //    each tile re-reads only its 256-byte bitmask slice and writes the ids of
 //    its set bits at its offset (reduce-then-scan; no inter-block waits).  Up to
-//    kScanTilesMax tiles the block that finishes last scans the counts itself;
+//    kScanTilesMax tiles the block that finishes last scans the counts itself, or,
+//    where no host waits for their sum, each compacting block adds them up;
 //    up to kSmallRows rows one block does the whole filter.
 //  * open-addressing hash table (int64 key -> build row), linear probing with
 //    a bounded probe sequence.
@@ -477,6 +478,26 @@ constexpr unsigned kWideTilesMax = 488;          // k_compact_wide without a pay
 constexpr unsigned kWidePayloadTilesMax = 2432;  // and with one: 16 blocks per SM
 constexpr int kCompactWarps = 4;  // warps (= 2048-row tiles at a time) per compaction block
 
+// Survivors before tile `end`, by all threads of a block (NT of them) together.
+template <int NT>
+__device__ __forceinline__ int sum_counts(const int32_t* counts, unsigned end, int* sh) {
+  int s = 0;
+  const unsigned quads = end / 4;
+#pragma unroll 4
+  for (unsigned i = threadIdx.x; i < quads; i += NT) {
+    const int4 v = __ldcg(reinterpret_cast<const int4*>(counts) + i);
+    s += (v.x + v.y) + (v.z + v.w);
+  }
+  if (threadIdx.x < end % 4) s += __ldcg(counts + quads * 4 + threadIdx.x);
+  s = __reduce_add_sync(0xffffffffu, s);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
+  __syncthreads();
+  s = 0;
+#pragma unroll
+  for (int w = 0; w < NT / 32; ++w) s += sh[w];
+  return s;
+}
+
 // One warp per 2048-row tile: lane l owns bitmask words l and 32 + l of the
 // tile (two coalesced loads).  In two passes (words 0..31, then 32..63) a warp
 // shuffle scan gives every lane its output position and the lane writes the
@@ -485,8 +506,14 @@ constexpr int kCompactWarps = 4;  // warps (= 2048-row tiles at a time) per comp
 // ids.  No block-wide barrier is involved.  A payload (the join's build row
 // per probe row) is gathered in that last loop (PAYLOAD): in the set-bit loop each
 // gather stalled its lane (8.5 us for 500,000 probe rows).
-template <bool PAYLOAD>
-__global__ void __launch_bounds__(kCompactWarps * 32) k_compact(const uint32_t* bits, const int64_t* block_offsets,
+//
+// DIRECT: no scan has run, a block adds up the counts before its tiles itself (all
+// of them come from L2, at 8192 tiles 32 KB for the last block), which takes the scan
+// out of the filter: 4,195,081 rows of four terms 22.0 -> 18.6 us, 16,777,211 rows of
+// one term 35.6 -> 26.0, against a scan by the predicate's last block.  For a caller
+// whose host must know the count before the ids have a place, the scan stays.
+template <bool PAYLOAD, bool DIRECT>
+__global__ void __launch_bounds__(kCompactWarps * 32) k_compact(const uint32_t* bits, TileBase tb,
                                                                 int64_t n, int32_t* ids, const int32_t* payload,
                                                                 int32_t* payload_out, unsigned int* arrived) {
   grid_launch_next();
@@ -497,10 +524,18 @@ __global__ void __launch_bounds__(kCompactWarps * 32) k_compact(const uint32_t* 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t n_tiles = (n + kRowsPerBlock - 1) / kRowsPerBlock;
   const int64_t tile = static_cast<int64_t>(blockIdx.x) * kCompactWarps + warp;
+  int64_t before = 0;
+  if (DIRECT) {
+    __shared__ int sh[kCompactWarps];
+    before = sum_counts<kCompactWarps * 32>(tb.counts, blockIdx.x * kCompactWarps, sh);
+    for (int w = 0; w < warp; ++w)
+      if (tile - warp + w < n_tiles) before += __ldcg(tb.counts + tile - warp + w);
+    if (tile == n_tiles - 1 && lane == 0) *tb.total = before + __ldcg(tb.counts + tile);
+  }
   if (tile < n_tiles) {
     const uint32_t* wt = bits + tile * (kRowsPerBlock / 32);
     const uint32_t wa = wt[lane], wb = wt[32 + lane];
-    const int64_t out = block_offsets[tile];
+    const int64_t out = DIRECT ? before : tb.offsets[tile];
     const int64_t tile0 = tile * kRowsPerBlock;
     int at0 = 0;
 #pragma unroll
@@ -537,9 +572,9 @@ __global__ void __launch_bounds__(kCompactWarps * 32) k_compact(const uint32_t* 
 // the GPU idle and walks them in turn: 500,000 rows with a payload 11.5 us, here
 // 3.8).  Without a payload the two are even at 489 tiles (3.6 us) and a warp per
 // tile is the faster above (2049 tiles: 4.4 us against 5.1).
-template <bool PAYLOAD>
-__global__ void __launch_bounds__(kThreads) k_compact_wide(const uint32_t* bits, const int64_t* block_offsets,
-                                                           int32_t* ids, const int32_t* payload, int32_t* payload_out,
+template <bool PAYLOAD, bool DIRECT>
+__global__ void __launch_bounds__(kThreads) k_compact_wide(const uint32_t* bits, TileBase tb, int32_t* ids,
+                                                           const int32_t* payload, int32_t* payload_out,
                                                            unsigned int* arrived) {
   grid_launch_next();
   grid_wait();
@@ -547,7 +582,13 @@ __global__ void __launch_bounds__(kThreads) k_compact_wide(const uint32_t* bits,
   if (arrived && blockIdx.x == 0 && threadIdx.x == 0) *arrived = 0;  // as k_compact
   const int64_t tile = blockIdx.x;
   const uint32_t byte = reinterpret_cast<const uint8_t*>(bits + tile * (kRowsPerBlock / 32))[threadIdx.x];
-  const int64_t out = block_offsets[tile];
+  int64_t out;
+  if (DIRECT) {
+    __shared__ int sums[kThreads / 32];
+    out = sum_counts<kThreads>(tb.counts, blockIdx.x, sums);
+  } else {
+    out = tb.offsets[tile];
+  }
   const int64_t r0 = tile * kRowsPerBlock + threadIdx.x * 8;
   int m[8];
   if (PAYLOAD) {
@@ -556,6 +597,7 @@ __global__ void __launch_bounds__(kThreads) k_compact_wide(const uint32_t* bits,
   }
   int total;
   int64_t at = out + block_excl_scan<kThreads>(__popc(byte), sh, &total);
+  if (DIRECT && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *tb.total = out + total;
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
     if ((byte >> j) & 1u) {
@@ -870,6 +912,7 @@ int launch_predicate_scan(const PredSet& ps, const ProbeSpec& probe, int64_t n_r
                           int32_t* block_counts, int64_t* offsets, unsigned int* arrived, int64_t* total,
                           int64_t* scan_tmp, cudaStream_t s) {
   if (n_rows <= 0) {
+    if (!offsets) return 0;
     cudaMemsetAsync(offsets, 0, sizeof(int64_t), s);
     if (total) cudaMemcpyAsync(total, offsets, sizeof(int64_t), cudaMemcpyDefault, s);
     return 0;
@@ -879,7 +922,7 @@ int launch_predicate_scan(const PredSet& ps, const ProbeSpec& probe, int64_t n_r
   for (int i = 0; i < ps.n; ++i) aligned = aligned && (reinterpret_cast<uintptr_t>(ps.p[i].col) & 15) == 0;
   // One block scans 2048 counts a microsecond: past kScanTilesMax tiles the
   // three-kernel scan, whose blocks share the counts, is the faster.
-  TileScan ts{block_counts, offsets, grid <= kScanTilesMax ? arrived : nullptr, total};
+  TileScan ts{block_counts, offsets, offsets && grid <= kScanTilesMax ? arrived : nullptr, total};
   bool fused = ts.arrived != nullptr;
   if (probe.keys) {
     launch_chained(k_probe_mask, dim3(grid), kProbeThreads, 0, s, 1, ps, probe, n_rows, bits, block_counts, ts);
@@ -903,7 +946,7 @@ int launch_predicate_scan(const PredSet& ps, const ProbeSpec& probe, int64_t n_r
     snprintf(buf, sizeof(buf), "predicate mask launch (grid %u, terms %d)", grid, ps.n);
     set_launch_error(buf, e);
   }
-  if (fused) return 1;
+  if (fused || !offsets) return 1;
   int launches = 4;
   if (scan_tmp) {
     launch_scan_lengths(block_counts, grid, offsets, scan_tmp, s);
@@ -923,20 +966,32 @@ void launch_compact(const uint32_t* bits, const int64_t* block_offsets, int64_t 
                     const int32_t* payload, int32_t* payload_out, cudaStream_t s, unsigned int* arrived) {
   if (n_rows <= 0) return;
   const unsigned tiles = blocks_for(n_rows, kRowsPerBlock);
+  const TileBase tb{block_offsets, nullptr, nullptr};
   if (tiles <= (payload_out ? kWidePayloadTilesMax : kWideTilesMax)) {
-    if (payload_out)
-      launch_chained(k_compact_wide<true>, dim3(tiles), kThreads, 0, s, 1, bits, block_offsets, ids_out, payload, payload_out, arrived);
-    else
-      launch_chained(k_compact_wide<false>, dim3(tiles), kThreads, 0, s, 1, bits, block_offsets, ids_out, payload, payload_out, arrived);
+    const auto kernel = payload_out ? k_compact_wide<true, false> : k_compact_wide<false, false>;
+    launch_chained(kernel, dim3(tiles), kThreads, 0, s, 1, bits, tb, ids_out, payload, payload_out, arrived);
     return;
   }
   const unsigned grid = (tiles + kCompactWarps - 1) / kCompactWarps;  // one tile per warp
-  if (payload_out)
-    launch_chained(k_compact<true>, dim3(grid), kCompactWarps * 32, 0, s, 1, bits, block_offsets, n_rows, ids_out, payload, payload_out,
-                                                        arrived);
+  const auto kernel = payload_out ? k_compact<true, false> : k_compact<false, false>;
+  launch_chained(kernel, dim3(grid), kCompactWarps * 32, 0, s, 1, bits, tb, n_rows, ids_out, payload, payload_out,
+                 arrived);
+}
+
+void launch_compact_counts(const uint32_t* bits, const int32_t* block_counts, int64_t n_rows, int32_t* ids_out,
+                           int64_t* total, cudaStream_t s) {
+  if (n_rows <= 0) {
+    cudaMemsetAsync(total, 0, sizeof(int64_t), s);
+    return;
+  }
+  const unsigned tiles = blocks_for(n_rows, kRowsPerBlock);
+  const TileBase tb{nullptr, block_counts, total};
+  if (tiles <= kWideTilesMax)
+    launch_chained(k_compact_wide<false, true>, dim3(tiles), kThreads, 0, s, 1, bits, tb, ids_out, nullptr, nullptr,
+                   nullptr);
   else
-    launch_chained(k_compact<false>, dim3(grid), kCompactWarps * 32, 0, s, 1, bits, block_offsets, n_rows, ids_out, payload, payload_out,
-                                                         arrived);
+    launch_chained(k_compact<false, true>, dim3((tiles + kCompactWarps - 1) / kCompactWarps), kCompactWarps * 32, 0, s,
+                   1, bits, tb, n_rows, ids_out, nullptr, nullptr, nullptr);
 }
 
 void launch_hash_build(const int64_t* keys, const int32_t* rows, int64_t n, unsigned long long* table_keys,

@@ -99,6 +99,30 @@ def test_filter_term_mixes(ctx, n):
         ctx.free_table(ref_t)
 
 
+@pytest.mark.parametrize("n", [16385, 2048 * 9, 2048 * 488, 2048 * 488 + 1, 2048 * 490 + 5, 2048 * 491, 2048 * 3000 - 1,
+                               (1 << 24) - 3, 1 << 24])
+def test_static_filter_tile_groups(n):
+    """The allocation-free filter's compaction adds up the tile counts itself: sizes
+    around its switch from a block to a warp per tile (488 tiles), groups of four
+    tiles with 1 .. 4 of them present, and the largest table, with all, some and no
+    rows kept."""
+    torch = pytest.importorskip("torch")
+    g = torch.Generator(device="cuda").manual_seed(n)
+    col = torch.randint(0, 10, (n,), dtype=torch.int32, device="cuda", generator=g)
+    ids = torch.empty(n, dtype=torch.int32, device="cuda")
+    count = torch.empty(1, dtype=torch.int64, device="cuda")
+    for terms in ([], [(rel.GE, 9)], [(rel.GE, 3)] * 5, [(rel.LT, 0)]):
+        keep = torch.ones(n, dtype=torch.bool, device="cuda")
+        for op, v in terms:
+            keep &= col >= v if op == rel.GE else col < v
+        want = keep.nonzero().flatten().int()
+        torch.cuda.synchronize()
+        aiq.filter_compact_static([(col.data_ptr(), aiq.INT32, op, v) for op, v in terms], n, ids.data_ptr(),
+                                  count.data_ptr(), 0)
+        torch.cuda.synchronize()
+        assert int(count) == len(want) and torch.equal(ids[:len(want)], want), terms
+
+
 @pytest.mark.parametrize("m,n", [(1, 3), (40, 2047), (3000, 70_001), ((1 << 22) + 3, 20_000)])
 def test_join_probe_sizes(ctx, m, n):
     """Build sides hashed straight from their columns and (the largest) compacted
