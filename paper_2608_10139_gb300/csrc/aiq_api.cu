@@ -336,7 +336,7 @@ bool pair_tiles(const aiq_ctx* c, int M, int bn) { return c->gemm_pair && bn == 
 
 // Slots per 128 columns that the product's epilogue writes its sums of squares in.
 int gemm_ss_split(const aiq_ctx* c, int M, int N, int K, int bn, const GemmEpilogue& ep) {
-  return gemm_few_tile(M, N, K, bn, pair_tiles(c, M, bn), ep, c->num_sms) ? 8 : 1;
+  return gemm_few_tile(M, N, K, bn, pair_tiles(c, M, bn), ep, c->num_sms).bn ? 8 : 1;
 }
 
 // k_algo: the product's own depth when the GEMM runs over a two-term operand

@@ -811,9 +811,9 @@ __global__ void __launch_bounds__(kThreads, 1)
 // ------------------------------------------------------------- few rows ---
 // Products with few rows (a generation step, the shared prefix's own pass, a
 // small chunk, the final layer's last tokens), in narrow tiles, so that even N =
-// 2048 gives every SM a slice of the weights to stream.  Up to 64 rows a CTA by
-// itself takes all of them and BN = 16 .. 128 weight columns; more rows are shared by
-// two CTAs (k_gemm_few_pair).  Bound by the weights' read from DRAM; what each CTA moves per
+// 2048 gives every SM a slice of the weights to stream: tiles of up to 64 rows and BN
+// = 16 .. 128 weight columns, by one CTA (k_gemm_few) or, with more rows, by two that
+// share 128 rows and 2 BN columns (k_gemm_few_pair).  Bound by the weights' read from DRAM; what each CTA moves per
 // 64-deep k-block is (rows of A + BN) x 128 bytes, so A's box holds only the
 // rows that exist (rounded up to 8; the MMA's other rows read whatever follows
 // in shared memory and are never stored).  One TMA per operand fills a stage
@@ -828,6 +828,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 constexpr int kFewRows = 64;           // rows that one CTA stages
 constexpr int kFewSmem = 200 * 1024;  // operand ring
 constexpr int kFewStages = 16;
+constexpr int kFewEpiWarps = 8;
+constexpr int kFewThreads = 64 + 32 * kFewEpiWarps;
 constexpr int kFewSlack = kFewRows * 128;  // an A tile's MMA reads kFewRows rows from its slot's start
 
 struct FewArgs {
@@ -857,120 +859,118 @@ __device__ __forceinline__ int few_n0(int nt, int half) {
   return (nt / per) * 2 * half + (nt % per) * (BN / 2);
 }
 
+// The accumulator's columns are shared by the two warps of a TMEM quarter (`part`
+// 0 and 1): 16-column steps in turn where the threads add to the residual, else a
+// half each of the tile's column pairs (tiles of 16 columns go to part 0).
 template <int BN, int EPI>
 __device__ __forceinline__ void epilogue_few(const KArgs& a, uint32_t trow, int row, bool live, int n0, int half,
-                                             float inv) {
+                                             float inv, int part) {
   const GemmEpilogue& ep = a.ep;
-  constexpr int HB = BN / 2;
-  constexpr int W = HB < 16 ? HB : 16;  // columns of each half per step
   bool bad = false;
   const int64_t r = row;
+  if constexpr (EPI == EPI_RESID_F32) {
 #pragma unroll 1
-  for (int c = 0; c < HB; c += W) {
-    uint32_t ru[W], rv[W];
+    for (int c = part * 16; c < BN; c += 32) {
+      uint32_t rv[16];
+      tmem_ld_32x32b_x8(trow + c, rv);
+      tmem_ld_32x32b_x8(trow + c + 8, rv + 8);
+      tmem_ld_wait();
+      if (live) {
+        float v[16];
+        float4* o4 = reinterpret_cast<float4*>(static_cast<float*>(ep.out) + r * ep.ldo + n0 + c);
 #pragma unroll
-    for (int j = 0; j < W; j += 8) {
-      tmem_ld_32x32b_x8(trow + c + j, ru + j);
-      tmem_ld_32x32b_x8(trow + HB + c + j, rv + j);
-    }
-    tmem_ld_wait();
-    if (live) {
-      float x[W], y[W];
-#pragma unroll
-      for (int j = 0; j < W; ++j) {
-        x[j] = u2f(ru[j]) * inv;
-        y[j] = u2f(rv[j]) * inv;
-      }
-      if constexpr (EPI == EPI_SWIGLU_F16) {
-        __half* o = static_cast<__half*>(ep.out) + r * ep.ldo + (n0 / (2 * half)) * half + n0 % (2 * half) + c;
-#pragma unroll
-        for (int j = 0; j < W; ++j) x[j] = x[j] / (1.0f + expf(-x[j])) * y[j];
-#pragma unroll
-        for (int j = 0; j < W; j += 8) store_f16x8(o + j, x + j, bad);
-        if (ep.lo_off > 0) {
-#pragma unroll
-          for (int j = 0; j < W; ++j) y[j] = x[j] - __half2float(__float2half_rn(x[j]));
-#pragma unroll
-          for (int j = 0; j < W; j += 8) store_f16x8(o + ep.lo_off + j, y + j, bad);
-        }
-      } else if constexpr (EPI == EPI_RESID_F32) {
-        float* o = static_cast<float*>(ep.out) + r * ep.ldo + n0 + c;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          float* v = h ? y : x;
-          float4* o4 = reinterpret_cast<float4*>(o + h * HB);
-#pragma unroll
-          for (int j = 0; j < W / 4; ++j) {
-            float4 t = o4[j];
-            t.x += v[4 * j];
-            t.y += v[4 * j + 1];
-            t.z += v[4 * j + 2];
-            t.w += v[4 * j + 3];
-            o4[j] = t;
-            v[4 * j] = t.x;
-            v[4 * j + 1] = t.y;
-            v[4 * j + 2] = t.z;
-            v[4 * j + 3] = t.w;
-          }
+        for (int j = 0; j < 4; ++j) {
+          float4 t = o4[j];
+          t.x += u2f(rv[4 * j]);
+          t.y += u2f(rv[4 * j + 1]);
+          t.z += u2f(rv[4 * j + 2]);
+          t.w += u2f(rv[4 * j + 3]);
+          o4[j] = t;
+          v[4 * j] = t.x;
+          v[4 * j + 1] = t.y;
+          v[4 * j + 2] = t.z;
+          v[4 * j + 3] = t.w;
         }
         if (ep.xh_out) {
-          float* ss = ep.ss_out + r * ep.ss_parts + (n0 + c) / 16;  // ss_split == 8: one slot per 16 columns
-          if constexpr (BN == 16) {
-            float s = 0.f;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) s = __fmaf_rn(x[j], x[j], s);
-#pragma unroll
-            for (int j = 0; j < 8; ++j) s = __fmaf_rn(y[j], y[j], s);
-            ss[0] = s;
-          } else {
-            ss[0] = sum_sq16(x);
-            ss[HB / 16] = sum_sq16(y);
-          }
+          ep.ss_out[r * ep.ss_parts + (n0 + c) / 16] = sum_sq16(v);  // ss_split == 8: one slot per 16 columns
           __half* xh = ep.xh_out + r * ep.ldo + n0 + c;
 #pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            float* v = h ? y : x;
+          for (int j = 0; j < 16; j += 8) {
+            if (ep.xh_gain) {
+              const uint4 gv = __ldg(reinterpret_cast<const uint4*>(ep.xh_gain + n0 + c + j));
+              const uint32_t gw[4] = {gv.x, gv.y, gv.z, gv.w};
 #pragma unroll
-            for (int j = 0; j < W; j += 8) {
-              if (ep.xh_gain) {
-                const uint4 gv = __ldg(reinterpret_cast<const uint4*>(ep.xh_gain + n0 + c + h * HB + j));
-                const uint32_t gw[4] = {gv.x, gv.y, gv.z, gv.w};
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                  v[j + 2 * i] *= __uint_as_float(gw[i] << 16);
-                  v[j + 2 * i + 1] *= __uint_as_float(gw[i] & 0xFFFF0000u);
-                }
+              for (int i = 0; i < 4; ++i) {
+                v[j + 2 * i] *= __uint_as_float(gw[i] << 16);
+                v[j + 2 * i + 1] *= __uint_as_float(gw[i] & 0xFFFF0000u);
               }
-              store_f16x8(xh + h * HB + j, v + j, bad);
             }
+            store_f16x8(xh + j, v + j, bad);
           }
-        }
-      } else {
-        __half* o = static_cast<__half*>(ep.out) + r * ep.ldo + n0 + c;
-        if (EPI == EPI_ROPE_F16 && n0 < ep.rope_cols) {
-          // column n0 + c + j of the head's first half and its partner `half` columns on
-          const int64_t toff = static_cast<int64_t>(ep.positions[row]) * half + n0 % (2 * half) + c;
-#pragma unroll
-          for (int j = 0; j < W; j += 4) {
-            const float4 cs4 = __ldg(reinterpret_cast<const float4*>(ep.rope_cos + toff + j));
-            const float4 sn4 = __ldg(reinterpret_cast<const float4*>(ep.rope_sin + toff + j));
-            const float cs[4] = {cs4.x, cs4.y, cs4.z, cs4.w}, sn[4] = {sn4.x, sn4.y, sn4.z, sn4.w};
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              const float a1 = x[j + i], a2 = y[j + i];
-              x[j + i] = a1 * cs[i] - a2 * sn[i];
-              y[j + i] = a2 * cs[i] + a1 * sn[i];
-            }
-          }
-        }
-#pragma unroll
-        for (int j = 0; j < W; j += 8) {
-          store_f16x8(o + j, x + j, bad);
-          store_f16x8(o + half + j, y + j, bad);
         }
       }
+      __syncwarp();
     }
-    __syncwarp();
+  } else {
+    constexpr int HB = BN / 2;
+    constexpr int PER = HB < 16 ? HB : HB / 2;  // columns of each half per warp
+    constexpr int W = PER < 16 ? PER : 16;      // and per step
+    const int c1 = HB < 16 && part ? 0 : (part + 1) * PER;
+#pragma unroll 1
+    for (int c = part * PER; c < c1; c += W) {
+      uint32_t ru[W], rv[W];
+#pragma unroll
+      for (int j = 0; j < W; j += 8) {
+        tmem_ld_32x32b_x8(trow + c + j, ru + j);
+        tmem_ld_32x32b_x8(trow + HB + c + j, rv + j);
+      }
+      tmem_ld_wait();
+      if (live) {
+        float x[W], y[W];
+#pragma unroll
+        for (int j = 0; j < W; ++j) {
+          x[j] = u2f(ru[j]) * inv;
+          y[j] = u2f(rv[j]) * inv;
+        }
+        if constexpr (EPI == EPI_SWIGLU_F16) {
+          __half* o = static_cast<__half*>(ep.out) + r * ep.ldo + (n0 / (2 * half)) * half + n0 % (2 * half) + c;
+#pragma unroll
+          for (int j = 0; j < W; ++j) x[j] = x[j] / (1.0f + expf(-x[j])) * y[j];
+#pragma unroll
+          for (int j = 0; j < W; j += 8) store_f16x8(o + j, x + j, bad);
+          if (ep.lo_off > 0) {
+#pragma unroll
+            for (int j = 0; j < W; ++j) y[j] = x[j] - __half2float(__float2half_rn(x[j]));
+#pragma unroll
+            for (int j = 0; j < W; j += 8) store_f16x8(o + ep.lo_off + j, y + j, bad);
+          }
+        } else {
+          __half* o = static_cast<__half*>(ep.out) + r * ep.ldo + n0 + c;
+          if (n0 < ep.rope_cols) {
+            // column n0 + c + j of the head's first half and its partner `half` columns on
+            const int64_t toff = static_cast<int64_t>(ep.positions[row]) * half + n0 % (2 * half) + c;
+#pragma unroll
+            for (int j = 0; j < W; j += 4) {
+              const float4 cs4 = __ldg(reinterpret_cast<const float4*>(ep.rope_cos + toff + j));
+              const float4 sn4 = __ldg(reinterpret_cast<const float4*>(ep.rope_sin + toff + j));
+              const float cs[4] = {cs4.x, cs4.y, cs4.z, cs4.w}, sn[4] = {sn4.x, sn4.y, sn4.z, sn4.w};
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                const float a1 = x[j + i], a2 = y[j + i];
+                x[j + i] = a1 * cs[i] - a2 * sn[i];
+                y[j + i] = a2 * cs[i] + a1 * sn[i];
+              }
+            }
+          }
+#pragma unroll
+          for (int j = 0; j < W; j += 8) {
+            store_f16x8(o + j, x + j, bad);
+            store_f16x8(o + half + j, y + j, bad);
+          }
+        }
+      }
+      __syncwarp();
+    }
   }
   if (bad) set_dev_error(ep.err, DEVERR_FP16_RANGE);
 }
@@ -1000,7 +1000,7 @@ __device__ __forceinline__ void few_issue(uint32_t d, uint64_t da, uint64_t db, 
 }
 
 template <int BN, int EPI>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kFewThreads, 1)
     k_gemm_few(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ CUtensorMap tma_b, KArgs args,
                FewArgs fa) {
   constexpr int TMEM_COLS = 2 * BN < 32 ? 32 : 2 * BN;
@@ -1028,7 +1028,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(&tfull[i], 1);
-      mbar_init(&tempty[i], 4);
+      mbar_init(&tempty[i], kFewEpiWarps);
     }
     mbar_init(&mma_done, 1);
     *abort_flag = 0;
@@ -1047,7 +1047,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   grid_launch_next();
   grid_wait();
 
-  const int num_tiles = args.N / BN;
+  const int num_m = (args.M + kFewRows - 1) / kFewRows;
+  const int num_tiles = num_m * (args.N / BN);
   const int kblocks = args.K / (BK * sub);
 
   if (warp == 0) {
@@ -1056,7 +1057,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       uint32_t issued = 0, s = 0, ph = 1;
       bool ok = true;
       for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
-        const int n0 = few_n0<BN>(tile, fa.half);
+        const int m0 = (tile % num_m) * kFewRows;
+        const int n0 = few_n0<BN>(tile / num_m, fa.half);
         for (int kb = 0; kb < kblocks; ++kb) {
           if (!mbar_wait_bounded(&empty[s], ph, abort_flag, err)) {
             ok = false;
@@ -1064,7 +1066,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
           mbar_arrive_expect_tx(&full[s], a_bytes + b_bytes);
           tma_load_4d(sB + s * b_bytes, &tma_b, &full[s], 0, n0, 0, kb * sub);
-          tma_load_3d(sA + s * a_bytes, &tma_a, &full[s], 0, 0, kb * sub);
+          tma_load_3d(sA + s * a_bytes, &tma_a, &full[s], 0, m0, kb * sub);
           ++issued;
           if (++s == stages) {
             s = 0;
@@ -1134,23 +1136,25 @@ __global__ void __launch_bounds__(kThreads, 1)
   } else {
     // ------------------------------------------------------------ epilogue
     const int quarter = warp & 3;  // TMEM lanes this warp may access
+    const int part = (warp - 2) >> 2;
     int acc = 0;
     uint32_t acc_ph = 0;
     for (int tile = blockIdx.x; tile < num_tiles; tile += gridDim.x) {
-      const int n0 = few_n0<BN>(tile, fa.half);
+      const int m0 = (tile % num_m) * kFewRows + quarter * 16;
+      const int n0 = few_n0<BN>(tile / num_m, fa.half);
       // a 64-row accumulator takes the first 16 TMEM lanes of each quarter
-      const int row = quarter * 16 + lane;
+      const int row = m0 + lane;
       const bool live = lane < 16 && row < args.M;
       if (EPI == EPI_RESID_F32) {
-        if (live)
+        if (live && part == 0)
           prefetch_l2(static_cast<const float*>(args.ep.out) + static_cast<int64_t>(row) * args.ep.ldo + n0, BN * 4);
       }
       const float inv = EPI == EPI_ROPE_F16 || EPI == EPI_SWIGLU_F16 ? row_inv_rms(args.ep, row, live) : 1.f;
       if (!__all_sync(0xffffffffu, mbar_wait_bounded(&tfull[acc], acc_ph, abort_flag, err))) break;
       tc_fence_after();
-      if (quarter * 16 < args.M)  // warp-uniform: this warp holds at least one live row
+      if (m0 < args.M)  // warp-uniform: this warp holds at least one live row
         epilogue_few<BN, EPI>(args, tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + acc * BN, row, live,
-                              n0, fa.half, inv);
+                              n0, fa.half, inv, part);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&tempty[acc]);
@@ -1174,9 +1178,9 @@ __global__ void __launch_bounds__(kThreads, 1)
 // its 64 rows: the first tile's columns on lanes 0-63, the second's on lanes
 // 64-127.  Barriers as in k_gemm_tcgen05_pair.  128 rows, 4096 x 14336: 47 -> 35 us
 // (17 at the weights' read); the four products of a 128-row block of that size
-// together 150 -> 130.
+// together 150 -> 130, one CTA taking 128 rows before.
 template <int BN, int EPI>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kFewThreads, 1)
     k_gemm_few_pair(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ CUtensorMap tma_b, KArgs args,
                     FewArgs fa) {
   constexpr int TMEM_COLS = 2 * BN < 32 ? 32 : 2 * BN;
@@ -1207,7 +1211,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(&tfull[i], 1);
-      mbar_init(&tempty[i], 8);  // used in the leader only: 4 warps x 2 CTAs
+      mbar_init(&tempty[i], 2 * kFewEpiWarps);  // used in the leader only
     }
     mbar_init(&mma_done, 1);
     *abort_flag = 0;
@@ -1314,6 +1318,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   } else {
     // ------------------------------------------------ epilogue (both CTAs)
     const int quarter = warp & 3;  // TMEM lanes this warp may access
+    const int part = (warp - 2) >> 2;
     const uint32_t tempty_leader = map_to_cta(smem_u32(tempty), 0);
     int acc = 0;
     uint32_t acc_ph = 0;
@@ -1323,7 +1328,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int row = m0 + lane;
       const bool live = row < args.M;
       if (EPI == EPI_RESID_F32) {
-        if (live)
+        if (live && part == 0)
           prefetch_l2(static_cast<const float*>(args.ep.out) + static_cast<int64_t>(row) * args.ep.ldo + n0, BN * 4);
       }
       const float inv = EPI == EPI_ROPE_F16 || EPI == EPI_SWIGLU_F16 ? row_inv_rms(args.ep, row, live) : 1.f;
@@ -1331,7 +1336,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       tc_fence_after();
       if (m0 < args.M)  // warp-uniform: this warp holds at least one live row
         epilogue_few<BN, EPI>(args, tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + acc * BN, row, live,
-                              n0, fa.half, inv);
+                              n0, fa.half, inv, part);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive_cluster(tempty_leader + acc * 8);
@@ -1516,29 +1521,29 @@ int launch_few(const __half* A, int64_t lda, const __half* B, int64_t ldb, const
     grid = 2 * std::min((a.M + 127) / 128 * (a.N / (2 * BN)), num_sms / 2);
   } else {
     kernel = k_gemm_few<BN, EPI>;
-    grid = std::min(a.N / BN, num_sms);
+    grid = std::min((a.M + kFewRows - 1) / kFewRows * (a.N / BN), num_sms);
   }
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SM);
   if (e != cudaSuccess) return e;
-  return launch_chained(kernel, dim3(grid), kThreads, SM, stream, PAIR ? 2 : 1, ma, mb, a, fa);
+  return launch_chained(kernel, dim3(grid), kFewThreads, SM, stream, PAIR ? 2 : 1, ma, mb, a, fa);
 }
 
 template <int BN, int EPI>
-int launch_few_rows(const __half* A, int64_t lda, const __half* B, int64_t ldb, const KArgs& a, int bn, int num_sms,
-                    cudaStream_t s) {
-  return a.M <= kFewRows ? launch_few<false, BN, EPI>(A, lda, B, ldb, a, bn, num_sms, s)
-                         : launch_few<true, BN, EPI>(A, lda, B, ldb, a, bn, num_sms, s);
+int launch_few_rows(const __half* A, int64_t lda, const __half* B, int64_t ldb, const KArgs& a, int bn, bool two,
+                    int num_sms, cudaStream_t s) {
+  return two ? launch_few<true, BN, EPI>(A, lda, B, ldb, a, bn, num_sms, s)
+             : launch_few<false, BN, EPI>(A, lda, B, ldb, a, bn, num_sms, s);
 }
 
 template <int BN>
-int dispatch_few(const __half* A, int64_t lda, const __half* B, int64_t ldb, const KArgs& a, int bn, int num_sms,
-                 cudaStream_t s) {
+int dispatch_few(const __half* A, int64_t lda, const __half* B, int64_t ldb, const KArgs& a, int bn, bool two,
+                 int num_sms, cudaStream_t s) {
   switch (a.ep.kind) {
-    case EPI_ROPE_F16: return launch_few_rows<BN, EPI_ROPE_F16>(A, lda, B, ldb, a, bn, num_sms, s);
-    case EPI_SWIGLU_F16: return launch_few_rows<BN, EPI_SWIGLU_F16>(A, lda, B, ldb, a, bn, num_sms, s);
+    case EPI_ROPE_F16: return launch_few_rows<BN, EPI_ROPE_F16>(A, lda, B, ldb, a, bn, two, num_sms, s);
+    case EPI_SWIGLU_F16: return launch_few_rows<BN, EPI_SWIGLU_F16>(A, lda, B, ldb, a, bn, two, num_sms, s);
     case EPI_RESID_F32:
     case EPI_RESID_ADD:  // the same sum, added by the epilogue threads
-      return launch_few_rows<BN, EPI_RESID_F32>(A, lda, B, ldb, a, bn, num_sms, s);
+      return launch_few_rows<BN, EPI_RESID_F32>(A, lda, B, ldb, a, bn, two, num_sms, s);
   }
   return cudaErrorInvalidValue;
 }
@@ -1551,9 +1556,12 @@ int dispatch_few(const __half* A, int64_t lda, const __half* B, int64_t ldb, con
 // (60 bytes per clock); the large tiles measure 720
 // (128 x 256), 540 (128 x 128) and 660 (CTA pair).  An epilogue column costs 100
 // clocks where the threads add to the residual, 50 for SwiGLU, 40 for RoPE and 22 for the
-// TMA add, and each epilogue 1200 more for its hand-offs; a tile's epilogue runs beside the next tile's main loop.  Measured
-// (us, weights from DRAM; with about 7 us of launch and event overhead; in brackets
-// what one CTA per 128 rows took before pairs shared them):
+// TMA add with four epilogue warps, 70, 25 and 25 with the few-rows kernels' eight, and
+// each epilogue 1200 more for its hand-offs (1800 in a pair, whose launch takes 1400
+// longer: products of 64 to 3000 rows and N, K <= 512 take 10.5 us in pairs and 8.8
+// without); a tile's epilogue runs beside the next tile's main loop.  Measured
+// (us, weights from DRAM; with about 7 us of launch and event overhead; from 128 rows
+// on by pairs, and in brackets what one CTA per 128 rows took):
 //   M     N      K      large   16          32          64          128
 //   24    2048   8192   55.6    18.5        21.3        23.0        32.1
 //   128   4096   14336  96.4    41.4 (82.7) 35.0 (47.1) 39.8 (49.6) 55.2 (71.5)
@@ -1561,37 +1569,39 @@ int dispatch_few(const __half* A, int64_t lda, const __half* B, int64_t ldb, con
 //   1000  2048   8192   54.0    69.6 (157)  50.7 (95.4) 42.4 (56.5) 36.8 (48.3)
 //   24    28672  4096   53.3    67.1        48.5        44.7        48.9
 //   500   28672  4096   98.8    216 (518)   140 (266)   106 (148)   87.2 (115)
-int gemm_few_tile(int M, int N, int K, int bn, bool pair, const GemmEpilogue& ep, int num_sms) {
-  if (M > kFewRowsMax) return 0;
+// Eight epilogue warps against four: 16384 x 2048 SwiGLU, 500 rows 37.8 -> 35.6, 1000
+// rows 57.2 -> 52.1; 1024 x 128, 10184 rows 33.1 -> 25.2.
+FewTile gemm_few_tile(int M, int N, int K, int bn, bool pair, const GemmEpilogue& ep, int num_sms) {
+  if (M > kFewRowsMax) return {};
   int epi = 0, epi_large = 0;  // clocks per column
   switch (ep.kind) {
-    case EPI_ROPE_F16: epi = epi_large = 40; break;
-    case EPI_SWIGLU_F16: epi = epi_large = 50; break;
-    case EPI_RESID_F32: epi = epi_large = 100; break;
-    case EPI_RESID_ADD: epi = 100, epi_large = 22; break;
-    default: return 0;  // the plain and argmax epilogues
+    case EPI_ROPE_F16: epi = 25, epi_large = 40; break;
+    case EPI_SWIGLU_F16: epi = 25, epi_large = 50; break;
+    case EPI_RESID_F32: epi = 70, epi_large = 100; break;
+    case EPI_RESID_ADD: epi = 70, epi_large = 22; break;
+    default: return {};  // the plain and argmax epilogues
   }
   const int64_t kblocks = K / BK;
-  auto cost = [&](int64_t tiles, int64_t units, int64_t per_kblock, int64_t epilogue) {
+  auto cost = [&](int64_t tiles, int64_t units, int64_t per_kblock, int64_t epilogue, int64_t hand_off = 1200) {
     const int64_t waves = (tiles + units - 1) / units, main = kblocks * per_kblock;
-    epilogue += 1200;
+    epilogue += hand_off;
     return main + (waves - 1) * std::max(main, epilogue) + epilogue;
   };
   const int64_t m128 = (M + 127) / 128;
   int64_t best = pair && K % (BK * CfgPair::SUB) == 0
                      ? cost((M + 255) / 256 * (N / 256), num_sms / 2, 660, 256 * epi_large)
                      : cost(m128 * (N / bn), num_sms, bn == 256 ? 720 : 540, bn * epi_large);
-  int tile = 0;
+  FewTile tile;
+  const int rows = M < kFewRows ? (M + 7) / 8 * 8 : kFewRows;
+  const int64_t m64 = (M + 63) / 64;
   for (int t = 16; t <= 128; t *= 2) {
     if (t / 2 > few_half(t, bn, ep)) break;  // a tile's halves lie within a gate / up block or a head
-    int64_t c;
-    if (M <= 64) {
-      c = cost(N / t, num_sms, std::max(std::max(180, 2 * t), ((M + 7) / 8 * 8 + t) * 128 / 60), t * epi);
-    } else {
-      if (N % (2 * t) != 0) break;
-      c = cost(m128 * (N / (2 * t)), num_sms / 2, std::max(180, (64 + t) * 128 / 60), t * epi);
-    }
-    if (c < best) best = c, tile = t;
+    const int64_t load = (rows + t) * 128 / 60;
+    int64_t c = cost(m64 * (N / t), num_sms, std::max<int64_t>({180, 2 * t, load}), t * epi);
+    if (c < best) best = c, tile = {t, false};
+    if (M <= kFewRows || N % (2 * t) != 0) continue;
+    c = 1400 + cost(m128 * (N / (2 * t)), num_sms / 2, std::max<int64_t>(180, load), t * epi, 1800);
+    if (c < best) best = c, tile = {t, true};
   }
   return tile;
 }
@@ -1613,11 +1623,12 @@ int gemm_f16_tcgen05(const __half* A, int64_t lda, const __half* B, int64_t ldb,
       (!ep.out || (reinterpret_cast<uintptr_t>(ep.out) & 15) || (ep.ldo * 4) % 16 != 0 || ep.xh_out))
     return cudaErrorInvalidValue;
   KArgs a{M, N, K, ep};
-  switch (gemm_few_tile(M, N, K, bn, pair, ep, num_sms)) {
-    case 16: return dispatch_few<16>(A, lda, B, ldb, a, bn, num_sms, stream);
-    case 32: return dispatch_few<32>(A, lda, B, ldb, a, bn, num_sms, stream);
-    case 64: return dispatch_few<64>(A, lda, B, ldb, a, bn, num_sms, stream);
-    case 128: return dispatch_few<128>(A, lda, B, ldb, a, bn, num_sms, stream);
+  const FewTile few = gemm_few_tile(M, N, K, bn, pair, ep, num_sms);
+  switch (few.bn) {
+    case 16: return dispatch_few<16>(A, lda, B, ldb, a, bn, few.two_ctas, num_sms, stream);
+    case 32: return dispatch_few<32>(A, lda, B, ldb, a, bn, few.two_ctas, num_sms, stream);
+    case 64: return dispatch_few<64>(A, lda, B, ldb, a, bn, few.two_ctas, num_sms, stream);
+    case 128: return dispatch_few<128>(A, lda, B, ldb, a, bn, few.two_ctas, num_sms, stream);
   }
   CUtensorMap ma, mb, mc;
   if (!make_map(&ma, A, M, K, lda, BM) || !make_map(&mb, B, N, K, ldb, pair ? 128 : bn)) return cudaErrorInvalidValue;

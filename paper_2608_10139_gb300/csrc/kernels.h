@@ -57,10 +57,15 @@ struct GemmEpilogue {
 // pair: 256 x 256 tiles on clusters of two CTAs (cta_group::2); needs bn == 256.
 // Returns 0 or a cudaError_t value.
 constexpr int kFewRowsMax = 16384;  // rows that the few-rows kernel takes at most
-// Tile width of the few-rows kernel that gemm_f16_tcgen05 takes for this product
-// (16, 32, 64 or 128), or 0 for the large-tile kernels.  A product with ss_out
-// needs ss_split = 8 where this is not 0, and 1 where it is.
-int gemm_few_tile(int M, int N, int K, int bn, bool pair, const GemmEpilogue& ep, int num_sms);
+// Columns of a CTA's tile (16, 32, 64 or 128) of the few-rows kernel that
+// gemm_f16_tcgen05 takes for this product, and whether two CTAs share its rows;
+// bn = 0: the large-tile kernels.  A product with ss_out needs ss_split = 8 where
+// bn is not 0, and 1 where it is.
+struct FewTile {
+  int bn = 0;
+  bool two_ctas = false;
+};
+FewTile gemm_few_tile(int M, int N, int K, int bn, bool pair, const GemmEpilogue& ep, int num_sms);
 int gemm_f16_tcgen05(const __half* A, int64_t lda, const __half* B, int64_t ldb, int M, int N, int K, int bn,
                      bool pair, const GemmEpilogue& ep, int num_sms, cudaStream_t stream);
 

@@ -140,10 +140,11 @@ def test_rmsnorm(ctx, d):
     _close(_np64(out), ref, 1.5e-3, 1e-4, f"rmsnorm d{d}")
 
 @pytest.mark.parametrize("epi,N,K,bn,hd", [(1, 3072, 256, 256, 64), (1, 6144, 320, 256, 128), (2, 4096, 128, 256, 0),
-                                           (5, 2048, 512, 256, 0), (3, 4096, 192, 256, 0), (3, 1024, 128, 128, 0)])
+                                           (5, 2048, 512, 256, 0), (3, 4096, 192, 256, 0), (3, 1024, 128, 128, 0),
+                                           (2, 2048, 6144, 256, 0)])
 def test_gemm_paired_narrow_tiles_match_large_tiles(ctx, epi, N, K, bn, hd):
-    """More than 64 rows: two CTAs share a narrow tile's rows (16 to 128 columns each,
-    by the product's size).  Bit for bit the rows that large tiles give, at the
+    """More than 64 rows: one CTA per 64 rows or two that share 128, with 16 to 128
+    columns each, by the product's size.  Bit for bit the rows that large tiles give, at the
     boundaries of the pair's 64-row halves, and nothing written past the last row."""
     rng = np.random.default_rng(N + K + epi)
     big = 16384 + 40
