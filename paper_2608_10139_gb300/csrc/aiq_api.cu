@@ -841,25 +841,34 @@ aiq_status prefill_phase(aiq_ctx* c, const TableD& t, ModelD& m, const aiq_selec
   int32_t *lens, *prefix_d, *labels_d = nullptr;
   int64_t *cu, *scan_scratch;
   unsigned long long* pairs_d;
-  AIQ_TRY(ws(c, "q.lens", S, &lens));
   AIQ_TRY(ws(c, "q.cu", S + 1, &cu));
-  AIQ_TRY(ws(c, "q.scan", 2 * (S / kRowsPerBlock + 2), &scan_scratch));
-  AIQ_TRY(ws(c, "q.pairs", 1, &pairs_d));
   AIQ_TRY(ws(c, "q.prefix", std::max<int32_t>(P, 1), &prefix_d));
   if (P > 0) CUDA_TRY(cudaMemcpyAsync(prefix_d, q->prefix, P * sizeof(int32_t), cudaMemcpyHostToDevice, c->stream));
   if (K > 0) {
     AIQ_TRY(ws(c, "q.labels", K, &labels_d));
     CUDA_TRY(cudaMemcpyAsync(labels_d, q->label_ids, K * sizeof(int32_t), cudaMemcpyHostToDevice, c->stream));
   }
-  CUDA_TRY(cudaMemsetAsync(pairs_d, 0, sizeof(unsigned long long), c->stream));
-  {
-    ProfScope p(c, "pack_plan", 0, 0);
-    launch_row_lengths(col.offsets, st->ids, S, P, lens, pairs_d, c->stream, st->ids2);
-    launch_scan_lengths(lens, S, cu, scan_scratch, c->stream);
-    counted(c, 4);
+  if (plan_is_small(S)) {
+    {
+      ProfScope p(c, "pack_plan", 0, 0);
+      launch_plan_rows(col.offsets, st->ids, st->ids2, S, P, cu, c->d_pin, c->d_pin + 1, c->stream);
+      counted(c, 1);
+    }
+    AIQ_TRY(sync_and_check(c));
+  } else {
+    AIQ_TRY(ws(c, "q.lens", S, &lens));
+    AIQ_TRY(ws(c, "q.scan", 2 * (S / kRowsPerBlock + 2), &scan_scratch));
+    AIQ_TRY(ws(c, "q.pairs", 1, &pairs_d));
+    CUDA_TRY(cudaMemsetAsync(pairs_d, 0, sizeof(unsigned long long), c->stream));
+    {
+      ProfScope p(c, "pack_plan", 0, 0);
+      launch_row_lengths(col.offsets, st->ids, S, P, lens, pairs_d, c->stream, st->ids2);
+      launch_scan_lengths(lens, S, cu, scan_scratch, c->stream);
+      counted(c, 4);
+    }
+    CUDA_TRY(cudaMemcpyAsync(c->h_pin + 1, pairs_d, sizeof(int64_t), cudaMemcpyDeviceToHost, c->stream));
+    AIQ_TRY(read_i64(c, cu + S, 1, c->h_pin));
   }
-  CUDA_TRY(cudaMemcpyAsync(c->h_pin + 1, pairs_d, sizeof(int64_t), cudaMemcpyDeviceToHost, c->stream));
-  AIQ_TRY(read_i64(c, cu + S, 1, c->h_pin));
   const int64_t T = c->h_pin[0];
   st->T = T;
   st->pairs = c->h_pin[1];
@@ -886,16 +895,21 @@ aiq_status prefill_phase(aiq_ctx* c, const TableD& t, ModelD& m, const aiq_selec
     n_chunks = std::max<int64_t>(1, (T + step - 1) / step);
   }
   st->n_chunks = n_chunks;
-  int64_t* chunk_d;
-  AIQ_TRY(ws(c, "q.chunks", 2 * (n_chunks + 1), &chunk_d));
-  if (gp)
-    launch_chunk_bounds_rows(cu, S, rows_per_chunk, n_chunks, chunk_d, c->stream);
-  else
-    launch_chunk_bounds(cu, S, step, n_chunks, chunk_d, c->stream);
-  counted(c, 1);
   std::vector<int64_t> chunks(2 * (n_chunks + 1));
-  CUDA_TRY(cudaMemcpyAsync(chunks.data(), chunk_d, chunks.size() * sizeof(int64_t), cudaMemcpyDeviceToHost, c->stream));
-  AIQ_TRY(sync_and_check(c));
+  if (n_chunks == 1) {
+    chunks = {0, 0, S, T};  // every row: no launch and no wait needed
+  } else {
+    int64_t* chunk_d;
+    AIQ_TRY(ws(c, "q.chunks", 2 * (n_chunks + 1), &chunk_d));
+    if (gp)
+      launch_chunk_bounds_rows(cu, S, rows_per_chunk, n_chunks, chunk_d, c->stream);
+    else
+      launch_chunk_bounds(cu, S, step, n_chunks, chunk_d, c->stream);
+    counted(c, 1);
+    CUDA_TRY(
+        cudaMemcpyAsync(chunks.data(), chunk_d, chunks.size() * sizeof(int64_t), cudaMemcpyDeviceToHost, c->stream));
+    AIQ_TRY(sync_and_check(c));
+  }
   AIQ_TRY(ensure_rope(c, m, static_cast<int>(P + max_len + (gp ? gp->max_new : 0))));
   // The shared prefix runs through the decoder once.  As the first sequence of the
   // first chunk it costs no pass over the weights and no launches of its own (the

@@ -151,6 +151,12 @@ void launch_fill_u64(unsigned long long* p, int64_t n, unsigned long long v, cud
 // ids2 (optional): a second row per sequence whose text follows the first's (Q4 pairs).
 void launch_row_lengths(const int64_t* offsets, const int32_t* ids, int64_t S, int32_t prefix_len, int32_t* lens,
                         unsigned long long* pairs, cudaStream_t s, const int32_t* ids2 = nullptr);
+// The lengths' exclusive scan cu[S+1], their total and the pairs in one launch, for
+// 1 .. kPlanRows rows; total and pairs may be host memory that the device maps.
+constexpr int64_t kPlanRows = 8192;
+bool plan_is_small(int64_t S);
+void launch_plan_rows(const int64_t* offsets, const int32_t* ids, const int32_t* ids2, int64_t S, int32_t prefix_len,
+                      int64_t* cu, int64_t* total, int64_t* pairs, cudaStream_t s);
 // Exclusive scan of int32 lengths into int64 cu[S+1] (multi-block).
 void launch_scan_lengths(const int32_t* lens, int64_t S, int64_t* cu, int64_t* scratch_blocks, cudaStream_t s);
 // chunk_rows[c] = first row whose start offset >= c * budget_step, c = 0..n_chunks.

@@ -40,6 +40,79 @@ __global__ void k_row_lengths(const int64_t* offsets, const int32_t* ids, const 
   if ((threadIdx.x & 31) == 0 && pr) atomicAdd(pairs, pr);
 }
 
+// Few rows: what k_row_lengths and the three kernels of the lengths' scan do, in one
+// block, with the totals straight into host memory that the device maps.  The chain
+// is launches and little else at these sizes: a query over 319 rows took 322 us, with
+// this kernel and no launch for the bounds of a single chunk 293.
+__global__ void __launch_bounds__(1024) k_plan_rows(const int64_t* offsets, const int32_t* ids, const int32_t* ids2,
+                                                    int32_t S, int32_t P, int64_t* cu, int64_t* total,
+                                                    int64_t* pairs) {
+  grid_launch_next();
+  grid_wait();
+  constexpr int PER = 4;  // consecutive rows a thread
+  __shared__ int64_t sh[2][32];  // alternate, so that one barrier a round is enough
+  __shared__ unsigned long long shp[32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  int64_t carry = 0;
+  unsigned long long pr = 0;
+  for (int32_t b = 0, k = 0; b < S; b += 1024 * PER, k ^= 1) {
+    const int32_t i0 = b + threadIdx.x * PER;
+    int32_t r[PER], r2[PER];
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+      r[j] = i0 + j < S ? ids[i0 + j] : -1;
+      r2[j] = ids2 && i0 + j < S ? ids2[i0 + j] : -1;
+    }
+    int64_t len[PER], sum = 0;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+      len[j] = r[j] >= 0 ? offsets[r[j] + 1] - offsets[r[j]] : 0;
+      if (r2[j] >= 0) len[j] += offsets[r2[j] + 1] - offsets[r2[j]];
+    }
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+      pr += static_cast<unsigned long long>(len[j] * P + len[j] * (len[j] + 1) / 2);
+      sum += len[j];
+    }
+    int64_t incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int64_t y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += y;
+    }
+    if (lane == 31) sh[k][warp] = incl;
+    __syncthreads();
+    int64_t tot = sh[k][lane];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int64_t y = __shfl_up_sync(0xffffffffu, tot, o);
+      if (lane >= o) tot += y;
+    }
+    const int64_t before = __shfl_sync(0xffffffffu, tot, (warp - 1) & 31);
+    int64_t at = carry + (warp ? before : 0) + incl - sum;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+      if (i0 + j < S) cu[i0 + j] = at;
+      at += len[j];
+    }
+    carry += __shfl_sync(0xffffffffu, tot, 31);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) pr += __shfl_xor_sync(0xffffffffu, pr, o);
+  if (lane == 0) shp[warp] = pr;
+  __syncthreads();
+  if (warp == 0) {
+    pr = shp[lane];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) pr += __shfl_xor_sync(0xffffffffu, pr, o);
+    if (lane == 0) {
+      cu[S] = carry;
+      *total = carry;
+      *pairs = static_cast<int64_t>(pr);
+    }
+  }
+}
+
 // chunk_rows[2c] = first row i with cu[i] >= c * step (S if none), chunk_rows[2c+1] = cu[that row].
 __global__ void k_chunk_bounds(const int64_t* cu, int64_t S, int64_t step, int64_t n_chunks, int64_t* out) {
   grid_launch_next();
@@ -170,6 +243,14 @@ void launch_row_lengths(const int64_t* offsets, const int32_t* ids, int64_t S, i
                         unsigned long long* pairs, cudaStream_t s, const int32_t* ids2) {
   if (S <= 0) return;
   launch_chained(k_row_lengths, dim3(static_cast<unsigned>((S + 255) / 256)), 256, 0, s, 1, offsets, ids, ids2, S, prefix_len, lens, pairs);
+}
+
+bool plan_is_small(int64_t S) { return S > 0 && S <= kPlanRows; }
+
+void launch_plan_rows(const int64_t* offsets, const int32_t* ids, const int32_t* ids2, int64_t S, int32_t prefix_len,
+                      int64_t* cu, int64_t* total, int64_t* pairs, cudaStream_t s) {
+  launch_chained(k_plan_rows, dim3(1), 1024, 0, s, 1, offsets, ids, ids2, static_cast<int32_t>(S), prefix_len, cu,
+                 total, pairs);
 }
 
 void launch_chunk_bounds(const int64_t* cu, int64_t S, int64_t step, int64_t n_chunks, int64_t* chunk_rows,

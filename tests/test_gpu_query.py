@@ -349,6 +349,35 @@ def test_prefix_lengths_and_chunks(ctx, P, gqa):
     ctx.free_model(mh)
 
 
+def test_row_plan_sizes(ctx):
+    """Up to 8192 rows one block measures and places the rows' texts, above that a
+    chain of kernels: token counts, work counts and logits agree on both sides, at
+    the edges of a thread's four rows and of a block's 4096."""
+    w = synth.C1_TINY
+    rng = np.random.default_rng(8)
+    n = 8193
+    lens = rng.integers(0, 10, n)
+    lens[[0, 1, n - 1]] = [0, 3, 0]
+    offsets = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    table = synth.Table(n, {"rating": np.arange(n, dtype=np.int32)}, offsets,
+                        rng.integers(0, w.model.vocab, int(offsets[-1])).astype(np.int32))
+    prefix = rng.integers(0, w.model.vocab, 17).astype(np.int32)
+    mh, _ = _model(ctx, w.model, w.weight_seed)
+    t = _load(ctx, table)
+    run = lambda k: ctx.run_select(t, mh, [("rating", rel.LT, k)], prefix, w.label_ids, flags=aiq.FLAG_LOGITS)
+    all_rows = run(n)
+    for k in (1, 2, 4, 5, 4095, 4096, 4097, 8192):
+        r = run(k)
+        assert r.n_candidates == k and r.n_tokens == 17 * k + offsets[k]
+        assert np.array_equal(r.label_logits, all_rows.label_logits[:k]), k
+    # the last row has no text: the same tokens and attention pairs, and one row more in what
+    # runs on last tokens alone (the final layer's output projection and MLP, the label scores)
+    d, f = w.model.d_model, w.model.d_ffn
+    assert all_rows.prefill_flops - r.prefill_flops == 2 * (d * d + 3 * d * f) + 2 * d * len(w.label_ids)
+    ctx.free_table(t)
+    ctx.free_model(mh)
+
+
 def test_more_rows_than_tokens():
     """A chunk whose rows are all but a few without text has more rows than
     tokens: the per-row buffers are sized for the rows."""
