@@ -177,6 +177,7 @@ struct aiq_ctx {
   int* d_err = nullptr;           // its device address
   int64_t* h_pin = nullptr;  // pinned staging for control scalars
   int64_t* d_pin = nullptr;  // its device address
+  bool join_table_live = false;      // a join is building or probing its table
   unsigned int* d_arrived = nullptr;  // arrival counter of the tile-count scans (zero between launches)
   size_t bytes_max = SIZE_MAX;
   size_t bytes_used = 0;
@@ -226,6 +227,15 @@ void dfree(aiq_ctx* c, void* p, size_t bytes) {
   c->bytes_used -= std::max<size_t>(bytes, 256);
 }
 
+void release_join_table(aiq_ctx* c) {
+  cudaStreamSynchronize(c->stream);
+  for (const char* name : {"j.keys", "j.vals"}) {
+    DevBuf& b = c->ws[name];
+    if (b.p) dfree(c, b.p, b.bytes);
+    b = DevBuf{};
+  }
+}
+
 // Grow-only named workspace buffer.
 template <typename T>
 aiq_status ws(aiq_ctx* c, const char* name, size_t count, T** out) {
@@ -240,7 +250,14 @@ aiq_status ws(aiq_ctx* c, const char* name, size_t count, T** out) {
     }
     size_t want = bytes + bytes / 4;
     void* p = nullptr;
-    if (dalloc(c, &p, want) != AIQ_OK) AIQ_TRY(dalloc(c, &p, want = bytes));
+    aiq_status st = dalloc(c, &p, want);
+    if (st != AIQ_OK) st = dalloc(c, &p, want = bytes);
+    if (st != AIQ_OK && !c->join_table_live) {
+      // a join's table is of no use once it has been probed: its room may be what is missing
+      release_join_table(c);
+      st = dalloc(c, &p, want);
+    }
+    AIQ_TRY(st);
     b.p = p;
     b.bytes = want;
   }
@@ -451,9 +468,17 @@ aiq_status filter_compact(aiq_ctx* c, const TableD& t, const PredSet& ps, const 
   if (pr.keys) {
     AIQ_TRY(ws(c, (b + ".match").c_str(), std::max<int64_t>(n, 1), &pr.match_out));
   }
+  const bool own_scan = nb > kScanTilesMax;
   {
     ProfScope p(c, "predicate_mask", 0, 0);
-    counted(c, launch_predicate_scan(ps, pr, n, bits, bcnt, boff, c->d_arrived, c->d_pin, scan_tmp, c->stream));
+    counted(c, launch_predicate_scan(ps, pr, n, bits, bcnt, own_scan ? nullptr : boff, c->d_arrived, c->d_pin,
+                                     c->stream));
+  }
+  if (own_scan) {
+    ProfScope p(c, "scan_tiles", 0, 0);
+    launch_scan_lengths(bcnt, nb, boff, scan_tmp, c->stream);
+    CUDA_TRY(cudaMemcpyAsync(c->h_pin, boff + nb, sizeof(int64_t), cudaMemcpyDeviceToHost, c->stream));
+    counted(c, 3);
   }
   AIQ_TRY(sync_and_check(c));
   const int64_t S = c->h_pin[0];
@@ -1198,42 +1223,50 @@ aiq_status run_query(aiq_ctx* c, const TableD* build, int32_t build_key, const a
   CUDA_TRY(cudaEventRecord(ev[0], c->stream));
   QueryState st;
   ProbeSpec pr;
+  c->join_table_live = build != nullptr;
   if (build) {
     PredSet bps{};
     AIQ_TRY(make_pred_set(*build, build_preds, n_bp, &bps));
     const int64_t* bkeys = static_cast<const int64_t*>(build->cols[build_key].data);
-    int64_t cap = 64;
-    while (cap < 2 * build->n_rows) cap <<= 1;
-    unsigned long long* tk = nullptr;
-    int32_t* tv = nullptr;
     // Up to kDirectBuildRows build rows (100 MB of table) the rows that pass the
     // terms go straight into a table sized for all rows; above, and where that
-    // table does not fit, they are compacted first and the table sized for them.
-    if (build->n_rows <= kDirectBuildRows && ws(c, "j.keys", cap, &tk) == AIQ_OK &&
-        ws(c, "j.vals", cap, &tv) == AIQ_OK) {
-      ProfScope p(c, "hash_build", 0, 0);
-      launch_fill_u64(tk, cap, 0x8000000000000000ull, c->stream);
-      launch_hash_build_where(bkeys, bps, build->n_rows, tk, tv, cap, c->d_err, c->stream);
-      counted(c, 1 + (build->n_rows > 0));
-    } else {
-      int64_t Sb = 0;
-      int32_t* bids;
-      AIQ_TRY(filter_compact(c, *build, bps, ProbeSpec{}, "jb", &Sb, &bids, nullptr));
-      cap = 64;
+    // table leaves no room, they are compacted first and the table sized for them.
+    auto build_table = [&](bool direct) -> aiq_status {
+      unsigned long long* tk;
+      int32_t *tv, *bids = nullptr;
+      int64_t Sb = build->n_rows, cap = 64;
+      if (!direct) AIQ_TRY(filter_compact(c, *build, bps, ProbeSpec{}, "jb", &Sb, &bids, nullptr));
       while (cap < 2 * Sb) cap <<= 1;
       AIQ_TRY(ws(c, "j.keys", cap, &tk));
       AIQ_TRY(ws(c, "j.vals", cap, &tv));
       ProfScope p(c, "hash_build", 0, 0);
       launch_fill_u64(tk, cap, 0x8000000000000000ull, c->stream);
-      launch_hash_build(bkeys, bids, Sb, tk, tv, cap, c->d_err, c->stream);
+      if (direct)
+        launch_hash_build_where(bkeys, bps, Sb, tk, tv, cap, c->d_err, c->stream);
+      else
+        launch_hash_build(bkeys, bids, Sb, tk, tv, cap, c->d_err, c->stream);
       counted(c, 1 + (Sb > 0));
+      pr.keys = static_cast<const int64_t*>(probe.cols[probe_key].data);
+      pr.table_keys = tk;
+      pr.table_vals = tv;
+      pr.capacity = cap;
+      return AIQ_OK;
+    };
+    aiq_status s = AIQ_ERR_OOM;
+    if (build->n_rows <= kDirectBuildRows) {
+      s = build_table(true);
+      if (s == AIQ_OK) s = filter_compact(c, probe, ps, pr, "sel", &st.S, &st.ids, &st.build_rows);
+      if (s == AIQ_ERR_OOM) release_join_table(c);
     }
-    pr.keys = static_cast<const int64_t*>(probe.cols[probe_key].data);
-    pr.table_keys = tk;
-    pr.table_vals = tv;
-    pr.capacity = cap;
+    if (s == AIQ_ERR_OOM) {
+      s = build_table(false);
+      if (s == AIQ_OK) s = filter_compact(c, probe, ps, pr, "sel", &st.S, &st.ids, &st.build_rows);
+    }
+    AIQ_TRY(s);
+  } else {
+    AIQ_TRY(filter_compact(c, probe, ps, pr, "sel", &st.S, &st.ids, nullptr));
   }
-  AIQ_TRY(filter_compact(c, probe, ps, pr, "sel", &st.S, &st.ids, build ? &st.build_rows : nullptr));
+  c->join_table_live = false;
   CUDA_TRY(cudaEventRecord(ev[1], c->stream));
 
   ResultH R;

@@ -107,7 +107,7 @@ aiq_status aiq_filter_compact_static(const aiq_term* terms, int32_t n_terms, int
     // Every scratch word the compaction reads is written earlier in this call
     // (each tile writes its whole bitmask slice and its count), so nothing is
     // carried over from the previous call.
-    launch_predicate_scan(ps, ProbeSpec{}, n_rows, bits, counts, nullptr, nullptr, nullptr, nullptr, s);
+    launch_predicate_scan(ps, ProbeSpec{}, n_rows, bits, counts, nullptr, nullptr, nullptr, s);
     launch_compact_counts(bits, counts, n_rows, ids_out, count_out, s);
   }
   // A failed predicate launch is recorded (and its CUDA error consumed) by its

@@ -120,12 +120,12 @@ void launch_filter_small(const PredSet& ps, int64_t n_rows, int32_t* ids, int64_
                          cudaStream_t s);
 // Mask bits, per-tile survivor counts and their exclusive scan offsets[tiles + 1].
 // arrived: a counter that is zero before the first call; total (optional) also
-// receives the number of survivors; scan_tmp (optional): >= 2 * (ceil(tiles /
-// 2048) + 1) int64 for the multi-block scan.  offsets == nullptr: no scan, the bits
-// and the counts only.  Returns the number of kernels.
+// receives the number of survivors.  offsets == nullptr: no scan, the bits and the
+// counts only (above kScanTilesMax tiles launch_scan_lengths scans them faster).
+// Returns the number of kernels.
 int launch_predicate_scan(const PredSet& ps, const ProbeSpec& probe, int64_t n_rows, uint32_t* bits,
                           int32_t* block_counts, int64_t* offsets, unsigned int* arrived, int64_t* total,
-                          int64_t* scan_tmp, cudaStream_t s);
+                          cudaStream_t s);
 // Exclusive scan of n int32 counts into int64 offsets[n+1] (one block).
 void launch_scan_counts(const int32_t* counts, int64_t n, int64_t* offsets, cudaStream_t s);
 // Order-preserving compaction of set bits: ids_out[k] = row of the k-th set bit;

@@ -910,7 +910,7 @@ void launch_filter_small(const PredSet& ps, int64_t n_rows, int32_t* ids, int64_
 
 int launch_predicate_scan(const PredSet& ps, const ProbeSpec& probe, int64_t n_rows, uint32_t* bits,
                           int32_t* block_counts, int64_t* offsets, unsigned int* arrived, int64_t* total,
-                          int64_t* scan_tmp, cudaStream_t s) {
+                          cudaStream_t s) {
   if (n_rows <= 0) {
     if (!offsets) return 0;
     cudaMemsetAsync(offsets, 0, sizeof(int64_t), s);
@@ -920,8 +920,8 @@ int launch_predicate_scan(const PredSet& ps, const ProbeSpec& probe, int64_t n_r
   const unsigned grid = blocks_for(n_rows, kRowsPerBlock);
   bool aligned = true;
   for (int i = 0; i < ps.n; ++i) aligned = aligned && (reinterpret_cast<uintptr_t>(ps.p[i].col) & 15) == 0;
-  // One block scans 2048 counts a microsecond: past kScanTilesMax tiles the
-  // three-kernel scan, whose blocks share the counts, is the faster.
+  // One block scans 2048 counts a microsecond: past kScanTilesMax tiles the caller
+  // runs the three-kernel scan, whose blocks share the counts.
   TileScan ts{block_counts, offsets, offsets && grid <= kScanTilesMax ? arrived : nullptr, total};
   bool fused = ts.arrived != nullptr;
   if (probe.keys) {
@@ -947,15 +947,9 @@ int launch_predicate_scan(const PredSet& ps, const ProbeSpec& probe, int64_t n_r
     set_launch_error(buf, e);
   }
   if (fused || !offsets) return 1;
-  int launches = 4;
-  if (scan_tmp) {
-    launch_scan_lengths(block_counts, grid, offsets, scan_tmp, s);
-  } else {
-    launch_scan_counts(block_counts, grid, offsets, s);
-    launches = 2;
-  }
+  launch_scan_counts(block_counts, grid, offsets, s);
   if (total) cudaMemcpyAsync(total, offsets + grid, sizeof(int64_t), cudaMemcpyDefault, s);
-  return launches;
+  return 2;
 }
 
 void launch_scan_counts(const int32_t* counts, int64_t n, int64_t* offsets, cudaStream_t s) {

@@ -123,6 +123,60 @@ def test_static_filter_tile_groups(n):
         assert int(count) == len(want) and torch.equal(ids[:len(want)], want), terms
 
 
+def test_static_filter_under_capture():
+    """The allocation-free filter recorded into a graph between the caller's own kernels,
+    in its one-launch and two-launch forms: every replay filters what the column then holds."""
+    torch = pytest.importorskip("torch")
+    for n in (9000, 70_001):
+        col = torch.zeros(n, dtype=torch.int32, device="cuda")
+        base = torch.arange(n, dtype=torch.int32, device="cuda")
+        ids = torch.empty(n, dtype=torch.int32, device="cuda")
+        count = torch.zeros(1, dtype=torch.int64, device="cuda")
+        twice = torch.zeros(1, dtype=torch.int64, device="cuda")
+        call = lambda: aiq.filter_compact_static([(col.data_ptr(), aiq.INT32, rel.GE, 6)], n, ids.data_ptr(),
+                                                 count.data_ptr(), torch.cuda.current_stream().cuda_stream)
+        torch.cuda.synchronize()
+        call()   # the device address is looked up before any capture
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            torch.remainder(base, 10, out=col)
+            call()
+            torch.add(count, count, out=twice)
+        for step in range(3):
+            base += 3
+            ids.fill_(-1)
+            g.replay()
+            torch.cuda.synchronize()
+            want = (base % 10 >= 6).nonzero().flatten().int()
+            assert int(count) == len(want) and int(twice) == 2 * len(want)
+            assert torch.equal(ids[:len(want)], want)
+
+
+@pytest.mark.parametrize("room", [64 << 20, 14 << 20, 10 << 20, 3 << 20])
+def test_join_table_without_room(room):
+    """A join whose table for all build rows (15.7 MB) does not fit under the byte cap,
+    or only half of it, is sized for the rows that pass their term instead."""
+    from helpers import gpu_ctx
+    rng = np.random.default_rng(2)
+    m, n = 300_000, 20_000
+    build = {"k": rng.permutation(m).astype(np.int64), "y": rng.integers(0, 100, m).astype(np.int32)}
+    probe = {"k": rng.integers(0, m, n).astype(np.int64)}
+    c = gpu_ctx()   # a context of its own: no workspace left by larger queries
+    try:
+        tb, tp = c.load_table(build), c.load_table(probe)
+        c.set_option("device_bytes_max", m * 12 + n * 8 + 65536 + room)
+        r = c.run_join_select(tb, "k", [("y", rel.EQ, 7)], tp, "k", 0, [], [], [0, 1], agg=aiq.AGG_COUNT,
+                              flags=aiq.FLAG_RELATIONAL_ONLY)
+        row_of = np.full(m, -1)
+        row_of[build["k"]] = np.arange(m)
+        b = row_of[probe["k"]]
+        want = np.flatnonzero(build["y"][b] == 7)
+        assert np.array_equal(r.cand_row_ids, want) and np.array_equal(r.cand_build_rows, b[want])
+    finally:
+        c.close()
+
+
 @pytest.mark.parametrize("m,n", [(1, 3), (40, 2047), (3000, 70_001), ((1 << 22) + 3, 20_000)])
 def test_join_probe_sizes(ctx, m, n):
     """Build sides hashed straight from their columns and (the largest) compacted
