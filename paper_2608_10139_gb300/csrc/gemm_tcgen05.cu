@@ -18,6 +18,8 @@
 //             reads 32-column slices with tcgen05.ld and applies the fused
 //             epilogue (RoPE, SwiGLU, fp32 residual add) while the MMA warp
 //             already fills the other accumulator.
+// Pairs of CTAs on 256 x 256 tiles, and narrow tiles for few rows, follow the
+// same structure and say where they differ.
 #include <cudaTypedefs.h>
 
 #include <algorithm>

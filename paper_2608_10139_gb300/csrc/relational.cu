@@ -509,7 +509,7 @@ __device__ __forceinline__ int sum_counts(const int32_t* counts, unsigned end, i
 //
 // DIRECT: no scan has run, a block adds up the counts before its tiles itself (all
 // of them come from L2, at 8192 tiles 32 KB for the last block), which takes the scan
-// out of the filter: 4,195,081 rows of four terms 22.0 -> 18.6 us, 16,777,211 rows of
+// out of the filter: 4,195,081 rows of three terms (67 MB) 22.0 -> 18.6 us, 16,777,211 rows of
 // one term 35.6 -> 26.0, against a scan by the predicate's last block.  For a caller
 // whose host must know the count before the ids have a place, the scan stays.
 template <bool PAYLOAD, bool DIRECT>
