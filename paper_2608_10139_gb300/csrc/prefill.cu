@@ -113,9 +113,11 @@ __global__ void k_embed(const int32_t* tok, int64_t T, const uint16_t* emb, int 
 }
 
 // Sum of four squares, in a fixed order: a row's statistics are the same bits
-// whichever of the two kernels below forms them.
+// whichever of the two kernels below forms them.  It is the order in which the
+// expression x * x + y * y + z * z + w * w is contracted (y's square rounded, the
+// others joining it by fused steps), which gave these rows before.
 __device__ __forceinline__ float sq4(const float4& v) {
-  return __fmaf_rn(v.w, v.w, __fmaf_rn(v.z, v.z, __fmaf_rn(v.y, v.y, __fmul_rn(v.x, v.x))));
+  return __fmaf_rn(v.w, v.w, __fmaf_rn(v.z, v.z, __fmaf_rn(v.x, v.x, __fmul_rn(v.y, v.y))));
 }
 
 // Four normalised values of a row (columns c .. c + 3), stored as fp16 and, with
