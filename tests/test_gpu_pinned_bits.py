@@ -6,12 +6,14 @@ with yesterday's sees all of them differ.  The checksums below are of the
 outputs that the first kernels of this library gave on the same inputs; every
 kernel that took their place since keeps their order of summation."""
 import zlib
+from dataclasses import replace
 
 import numpy as np
 import pytest
 
 import synth
-from helpers import gpu_ctx
+from helpers import gpu_ctx, weights_list
+from paper_2608_10139_gb300 import aiq
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -55,3 +57,35 @@ RMSNORM = {128: (3904390063, 2493164157), 256: (3067552901, 692534954), 512: (10
 @pytest.mark.parametrize("d", [128, 256, 512, 768, 1024, 2048, 4096])
 def test_rmsnorm_bits(ctx, d):
     assert rmsnorm_crc(ctx, d) == RMSNORM[d]
+
+
+SHAPES = {"one layer": replace(synth.C1_TINY.model, n_layers=1),
+          "one wide layer": replace(synth.C1_TINY.model, n_layers=1, d_model=1152, d_ffn=256)}
+BUDGETS = (131072, 4000, 300)   # tokens: one chunk of some 16,000, several, chunks of a few rows
+
+
+def logits_crc(ctx, shape, budget, k):
+    w = synth.C1_TINY
+    q = synth.make_inputs(w)
+    W = synth.make_weights(SHAPES[shape], w.weight_seed)
+    m = ctx.load_model(SHAPES[shape], weights_list(SHAPES[shape], W))
+    t = ctx.load_table(q.table.cols, (q.table.offsets, q.table.tokens))
+    try:
+        ctx.set_option("token_budget", budget)
+        return _crc(ctx.run_select(t, m, [], q.prefix, [100, 101, 77][:k], agg=aiq.AGG_GROUP_LABEL,
+                                   flags=aiq.FLAG_LOGITS).label_logits)
+    finally:
+        ctx.set_option("token_budget", 131072)
+        ctx.free_table(t)
+        ctx.free_model(m)
+
+
+LOGITS = {("one layer", 2): 903127134, ("one layer", 3): 2015117514,
+          ("one wide layer", 2): 878337199, ("one wide layer", 3): 1545911119}
+
+
+@pytest.mark.parametrize("budget", BUDGETS)
+@pytest.mark.parametrize("shape", SHAPES)
+def test_query_logits_bits(ctx, shape, budget):
+    for k in (2, 3):   # labels
+        assert logits_crc(ctx, shape, budget, k) == LOGITS[shape, k]
