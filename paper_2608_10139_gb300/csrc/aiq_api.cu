@@ -351,11 +351,6 @@ inline void counted(aiq_ctx* c, int n) { c->launches += n; }
 
 bool pair_tiles(const aiq_ctx* c, int M, int bn) { return c->gemm_pair && bn == 256 && M >= 512; }
 
-// Slots per 128 columns that the product's epilogue writes its sums of squares in.
-int gemm_ss_split(const aiq_ctx* c, int M, int N, int K, int bn, const GemmEpilogue& ep) {
-  return gemm_few_tile(M, N, K, bn, pair_tiles(c, M, bn), ep, c->num_sms).bn ? 8 : 1;
-}
-
 // k_algo: the product's own depth when the GEMM runs over a two-term operand
 // (K = 2 k_algo); the statistics count the algorithmic FLOPs and bytes.
 aiq_status gemm(aiq_ctx* c, const char* name, const __half* A, int64_t lda, const __half* B, int64_t ldb, int M, int N,
@@ -370,6 +365,15 @@ aiq_status gemm(aiq_ctx* c, const char* name, const __half* A, int64_t lda, cons
   if (e != 0)
     return fail(AIQ_ERR_CUDA, std::string("tcgen05 GEMM launch: ") + cudaGetErrorString(static_cast<cudaError_t>(e)));
   return AIQ_OK;
+}
+
+// The sums of squares that the next layer's norm takes from this product's new
+// residual, where its kernel does not write them itself.
+void resid_sums(aiq_ctx* c, int M, int N, int K, int bn, const GemmEpilogue& ep) {
+  if (M <= 0 || !gemm_few_tile(M, N, K, bn, pair_tiles(c, M, bn), ep, c->num_sms).bn) return;
+  ProfScope p(c, "row_ss", 0, 4.0 * M * N);
+  launch_row_ss(static_cast<const float*>(ep.out), M, N, ep.ss_out, c->stream);
+  counted(c, 1);
 }
 
 // Query tokens per attention work item: the tcgen05 kernel's (head_dim 64/128)
@@ -525,7 +529,7 @@ constexpr int32_t kMergedPrefixMax = 1024;  // prefix tokens that run with the f
 struct PrefillBufs {
   int32_t *tok, *pos, *seq_start, *last_idx, *tile_seq, *tile_q0, *n_tiles, *last_compact;
   float *resid, *resid_last;
-  float* ss_attn;  // sums of squares of the residual, [T][d / 128] (few rows: [T][d / 16])
+  float* ss_attn;  // per-128-column sums of squares of the residual, [T][d / 128]
   __half *xn, *qkv, *att, *act;
 };
 
@@ -545,8 +549,7 @@ aiq_status prefill_bufs(aiq_ctx* c, const ModelD& m, int64_t B, int64_t max_rows
   AIQ_TRY(ws(c, "pf.att", B * g.n_heads * g.head_dim, &pb->att));
   AIQ_TRY(ws(c, "pf.act", std::max(B, max_rows) * g.d_ffn * (m.mlp_split ? 2 : 1), &pb->act));
   AIQ_TRY(ws(c, "pf.resid_last", max_rows * g.d_model, &pb->resid_last));
-  // few-row products write eight slots per 128 columns
-  AIQ_TRY(ws(c, "pf.ss_attn", std::max(B, 8 * std::min<int64_t>(B, kFewRowsMax)) * (g.d_model / 128), &pb->ss_attn));
+  AIQ_TRY(ws(c, "pf.ss_attn", B * (g.d_model / 128), &pb->ss_attn));
   AIQ_TRY(ws(c, "pf.last_compact", max_rows, &pb->last_compact));
   return AIQ_OK;
 }
@@ -576,7 +579,6 @@ aiq_status run_layers(aiq_ctx* c, ModelD& m, const PrefillBufs& b, int64_t T, in
   // standalone kernel: fusing it into the O-projection epilogue cost more
   // there than the kernel it removed.
   const int parts = d / 128;
-  int ss_split = 1;  // slots of ss_attn per 128 columns, as the last producer wrote them
   {
     // bf16 row in; fp32 residual, fp16 copy and the partial sums of squares out
     ProfScope p(c, "embed", 0, double(T) * d * 8.0 + double(T) * parts * 4.0);
@@ -597,8 +599,7 @@ aiq_status run_layers(aiq_ctx* c, ModelD& m, const PrefillBufs& b, int64_t T, in
     e1.head_dim = hd;
     e1.err = c->d_err;
     e1.row_ss = b.ss_attn;
-    e1.ss_parts = parts * ss_split;
-    e1.ss_split = ss_split;
+    e1.ss_parts = parts;
     e1.d_norm = static_cast<float>(d);
     e1.eps = g.rms_eps;
     AIQ_TRY(gemm(c, "gemm_qkv_rope", b.xn, d, L.wqkv, d, M, nqkv, d, m.bn_qkv, e1));
@@ -644,9 +645,9 @@ aiq_status run_layers(aiq_ctx* c, ModelD& m, const PrefillBufs& b, int64_t T, in
       e2.xh_out = b.xn;
       e2.xh_gain = l + 1 < g.n_layers ? m.layers[l + 1].attn_norm : nullptr;
       e2.ss_out = b.ss_attn;
-      e2.ss_split = ss_split = gemm_ss_split(c, M, d, ks * f, m.bn_d, e2);
-      e2.ss_parts = parts * ss_split;
+      e2.ss_parts = parts;
       AIQ_TRY(gemm(c, "gemm_down_resid", b.act, ks * f, L.wd, ks * f, M, d, ks * f, m.bn_d, e2, f));
+      if (l + 1 < g.n_layers) resid_sums(c, M, d, ks * f, m.bn_d, e2);
     } else {
       // final layer, rows only: gather each sequence's last token (the
       // attention output is dead afterwards, so its rows are packed into
@@ -752,7 +753,6 @@ aiq_status decode_layers(aiq_ctx* c, ModelD& m, const PrefillBufs& b, const Deco
   const int nqkv = (Hq + 2 * Hkv) * hd;
   const int64_t ldkv = 2 * static_cast<int64_t>(Hkv) * hd;
   const int parts = dm / 128;
-  int ss_split = 1;
   {
     ProfScope p(c, "embed", 0, double(R) * dm * 8.0 + double(R) * parts * 4.0);
     launch_embed(d.next, R, m.embed, dm, b.resid, b.xn, b.ss_attn, m.layers[0].attn_norm, c->d_err, c->stream);
@@ -771,8 +771,7 @@ aiq_status decode_layers(aiq_ctx* c, ModelD& m, const PrefillBufs& b, const Deco
     e1.head_dim = hd;
     e1.err = c->d_err;
     e1.row_ss = b.ss_attn;
-    e1.ss_parts = parts * ss_split;
-    e1.ss_split = ss_split;
+    e1.ss_parts = parts;
     e1.d_norm = static_cast<float>(dm);
     e1.eps = g.rms_eps;
     AIQ_TRY(gemm(c, "dec_gemm_qkv_rope", b.xn, dm, L.wqkv, dm, R, nqkv, dm, m.bn_qkv, e1));
@@ -813,9 +812,9 @@ aiq_status decode_layers(aiq_ctx* c, ModelD& m, const PrefillBufs& b, const Deco
     e2.xh_out = b.xn;
     e2.xh_gain = l + 1 < g.n_layers ? m.layers[l + 1].attn_norm : nullptr;
     e2.ss_out = b.ss_attn;
-    e2.ss_split = ss_split = gemm_ss_split(c, R, dm, ks * f, m.bn_d, e2);
-    e2.ss_parts = parts * ss_split;
+    e2.ss_parts = parts;
     AIQ_TRY(gemm(c, "dec_gemm_down_resid", b.act, ks * f, L.wd, ks * f, R, dm, ks * f, m.bn_d, e2, f));
+    if (l + 1 < g.n_layers) resid_sums(c, R, dm, ks * f, m.bn_d, e2);
   }
   return AIQ_OK;
 }

@@ -154,29 +154,13 @@ __device__ __forceinline__ void add_store_f32x32(float* dst, const float* v, flo
   }
 }
 
-// Sum of squares of 16 consecutive columns.  A row's sum over 128 columns is
-// always these eight sums added in order, whichever tile width formed them, so
-// that a row's norm does not depend on how many rows its GEMM had.
-__device__ __forceinline__ float sum_sq16(const float* v) {
-  float s = 0.f;
-#pragma unroll
-  for (int j = 0; j < 16; ++j) s = __fmaf_rn(v[j], v[j], s);
-  return s;
-}
-
 // 1 / RMS of an accumulator row from its partial sums of squares (fixed
 // summation order), or 1 when the GEMM's input is already normalised.
 __device__ __forceinline__ float row_inv_rms(const GemmEpilogue& ep, int row, bool live) {
   if (!ep.row_ss || !live) return 1.f;
   const float* p = ep.row_ss + static_cast<int64_t>(row) * ep.ss_parts;
   float s = 0.f;
-  if (ep.ss_split == 8) {  // eight 16-column sums per 128 columns (ss_parts is a multiple of 8)
-    const float4* p4 = reinterpret_cast<const float4*>(p);
-    for (int i = 0; i < ep.ss_parts / 8; ++i) {
-      const float4 a = __ldg(p4 + 2 * i), b = __ldg(p4 + 2 * i + 1);
-      s += ((((((a.x + a.y) + a.z) + a.w) + b.x) + b.y) + b.z) + b.w;
-    }
-  } else if ((ep.ss_parts & 3) == 0) {
+  if ((ep.ss_parts & 3) == 0) {
     const float4* p4 = reinterpret_cast<const float4*>(p);
     for (int i = 0; i < ep.ss_parts / 4; ++i) {
       const float4 v = __ldg(p4 + i);
@@ -222,7 +206,7 @@ __device__ __forceinline__ void epilogue_tile(const KArgs& a, uint32_t trow, int
   bool bad = false;
   if constexpr (EPI == EPI_RESID_F32) {
     float* o = static_cast<float*>(ep.out) + static_cast<int64_t>(row) * ep.ldo + n0;
-    float part = 0.f;  // sum of squares of the new residual over 128 columns (sum_sq16 groups, in order)
+    float part = 0.f;  // sum of squares of the new residual over 128 columns (k_row_ss keeps its order)
 #pragma unroll 1
     for (int c = 0; c < BN; c += 64) {
       float v0[32], v1[32];
@@ -232,9 +216,8 @@ __device__ __forceinline__ void epilogue_tile(const KArgs& a, uint32_t trow, int
         add_store_f32x32(o + c + 32, v1, v1);
         if (ep.xh_out) {
           __half* xh = ep.xh_out + static_cast<int64_t>(row) * ep.ldo + n0 + c;
-          const float s0 = sum_sq16(v0), s1 = sum_sq16(v0 + 16), s2 = sum_sq16(v1), s3 = sum_sq16(v1 + 16);
-          part = (c & 64) ? part + s0 : s0;
-          part = ((part + s1) + s2) + s3;
+#pragma unroll
+          for (int j = 0; j < 32; ++j) part = __fadd_rn(part, __fmaf_rn(v0[j], v0[j], __fmul_rn(v1[j], v1[j])));
           if (ep.xh_gain) {
             // the next attention norm's gain goes on the activation (the QKV
             // weights stay exact): one fp16 rounding of x * g per element
@@ -253,7 +236,10 @@ __device__ __forceinline__ void epilogue_tile(const KArgs& a, uint32_t trow, int
           }
           store_f16x32(xh, v0, bad);
           store_f16x32(xh + 32, v1, bad);
-          if ((c & 127) == 64) ep.ss_out[static_cast<int64_t>(row) * ep.ss_parts + (n0 + c) / 128] = part;
+          if ((c & 127) == 64) {
+            ep.ss_out[static_cast<int64_t>(row) * ep.ss_parts + (n0 + c) / 128] = part;
+            part = 0.f;
+          }
         }
       }
     }
@@ -894,7 +880,6 @@ __device__ __forceinline__ void epilogue_few(const KArgs& a, uint32_t trow, int 
           v[4 * j + 3] = t.w;
         }
         if (ep.xh_out) {
-          ep.ss_out[r * ep.ss_parts + (n0 + c) / 16] = sum_sq16(v);  // ss_split == 8: one slot per 16 columns
           __half* xh = ep.xh_out + r * ep.ldo + n0 + c;
 #pragma unroll
           for (int j = 0; j < 16; j += 8) {

@@ -34,11 +34,11 @@ struct GemmEpilogue {
   //    rsqrt(sum(row_ss[row][0..ss_parts)) / d_norm + eps) before the epilogue;
   //  - producer (RESID): also write the new residual as fp16 (xh_out), times
   //    the next norm's gain (xh_gain, bf16 [N]) when given, and the unscaled
-  //    residual's per-128-column sums of squares (ss_out [row][n / 128]), or
-  //    with ss_split == 8 their eight 16-column terms (ss_out [row][n / 16]).
+  //    residual's per-128-column sums of squares (ss_out [row][n / 128]).  The
+  //    few-rows kernels' tiles are narrower than that and leave ss_out to
+  //    launch_row_ss.
   const float* row_ss = nullptr;
-  int ss_parts = 0;                    // slots per row
-  int ss_split = 1;                    // slots per 128 columns: 1, or 8 where gemm_few_tile says so
+  int ss_parts = 0;
   float d_norm = 1.f;
   float eps = 0.f;
   __half* xh_out = nullptr;
@@ -59,8 +59,8 @@ struct GemmEpilogue {
 constexpr int kFewRowsMax = 16384;  // rows that the few-rows kernel takes at most
 // Columns of a CTA's tile (16, 32, 64 or 128) of the few-rows kernel that
 // gemm_f16_tcgen05 takes for this product, and whether two CTAs share its rows;
-// bn = 0: the large-tile kernels.  A product with ss_out needs ss_split = 8 where
-// bn is not 0, and 1 where it is.
+// bn = 0: the large-tile kernels.  Where bn is not 0 a product's ss_out is not
+// written: launch_row_ss follows.
 struct FewTile {
   int bn = 0;
   bool two_ctas = false;
@@ -193,6 +193,9 @@ void launch_embed(const int32_t* tok, int64_t T, const uint16_t* emb, int d, flo
 // fp16(v - fp16(v)) (a two-term operand for a K-doubled GEMM).
 void launch_rmsnorm(const float* x, int64_t T, int d, const uint16_t* g, float eps, __half* out, int* err,
                     cudaStream_t s, bool split = false);
+// Sums of squares of every 128 columns of a dense fp32 [T, d] (d a multiple of
+// 128) into ss[T][d / 128], the same bits as the large-tile RESID epilogue's.
+void launch_row_ss(const float* x, int64_t T, int d, float* ss, cudaStream_t s);
 // prefix.kv (optional): [P, 2 Hkv hd] fp16 keys then values of a shared prefix that
 // every sequence's queries also attend (prefix positions precede the sequence).
 struct PrefixKV {

@@ -206,6 +206,40 @@ __global__ void __launch_bounds__(256) k_rmsnorm_rows(const float* x, int d, con
   if (bad) set_dev_error(err, DEVERR_FP16_RANGE);
 }
 
+// Sums of squares of 128-column groups for the fused attention norm, after a
+// product whose tiles are narrower than a group.  A group's 64 terms (a column's
+// square and that of the column 32 on) are added one after the other, as the
+// thread that holds a whole row does it in the large tiles, so that a row's norm
+// does not depend on how many rows its product had.  A warp forms the terms of
+// eight groups (its 32 loads all in flight) and eight lanes walk them; what
+// bounds it is that walk and a launch: 6.3 us between events for 5,000 rows of 128,
+// where an empty pair of events measures 4.
+constexpr int kSsWarps = 8, kSsGroups = 8;  // warps per block, groups per warp
+__global__ void __launch_bounds__(kSsWarps * 32) k_row_ss(const float* x, int64_t groups, float* ss) {
+  grid_launch_next();
+  grid_wait();
+  __shared__ float term[kSsWarps][kSsGroups][65];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t g0 = (static_cast<int64_t>(blockIdx.x) * kSsWarps + warp) * kSsGroups;
+  float v[kSsGroups][4];
+#pragma unroll
+  for (int i = 0; i < kSsGroups; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v[i][j] = g0 + i < groups ? x[(g0 + i) * 128 + j * 32 + lane] : 0.f;
+#pragma unroll
+  for (int i = 0; i < kSsGroups; ++i) {
+    term[warp][i][lane] = __fmaf_rn(v[i][0], v[i][0], __fmul_rn(v[i][1], v[i][1]));
+    term[warp][i][32 + lane] = __fmaf_rn(v[i][2], v[i][2], __fmul_rn(v[i][3], v[i][3]));
+  }
+  __syncwarp();
+  if (lane < kSsGroups && g0 + lane < groups) {
+    float part = 0.f;
+#pragma unroll
+    for (int j = 0; j < 64; ++j) part = __fadd_rn(part, term[warp][lane][j]);
+    ss[g0 + lane] = part;
+  }
+}
+
 // Generic-width fallback (d not a multiple of 128 handled elsewhere; d % 4 == 0 here).
 __global__ void k_rmsnorm_any(const float* x, int64_t T, int d, const uint16_t* g, float eps, __half* out, int split,
                               int* err) {
@@ -361,6 +395,13 @@ void launch_rmsnorm(const float* x, int64_t T, int d, const uint16_t* g, float e
     case 4096: launch_chained(k_rmsnorm<32>, dim3(grid), 256, 0, s, 1, x, T, d, g, eps, out, sp, err); break;
     default: launch_chained(k_rmsnorm_any, dim3(grid), 256, 0, s, 1, x, T, d, g, eps, out, sp, err); break;
   }
+}
+
+void launch_row_ss(const float* x, int64_t T, int d, float* ss, cudaStream_t s) {
+  if (T <= 0) return;
+  const int64_t groups = T * (d / 128);
+  constexpr int64_t per = kSsWarps * kSsGroups;
+  launch_chained(k_row_ss, dim3(static_cast<unsigned>((groups + per - 1) / per)), kSsWarps * 32, 0, s, 1, x, groups, ss);
 }
 
 void launch_gather_last(const __half* att, int ld_att, const float* resid, int d, const int32_t* last_idx, int64_t n,

@@ -60,7 +60,9 @@ def test_rmsnorm_bits(ctx, d):
 
 
 SHAPES = {"one layer": replace(synth.C1_TINY.model, n_layers=1),
-          "one wide layer": replace(synth.C1_TINY.model, n_layers=1, d_model=1152, d_ffn=256)}
+          "one wide layer": replace(synth.C1_TINY.model, n_layers=1, d_model=1152, d_ffn=256),
+          "tiny": synth.C1_TINY.model,
+          "grouped": replace(synth.C1_TINY.model, n_layers=3, d_model=512, n_heads=8, n_kv_heads=2, head_dim=64, d_ffn=1024)}
 BUDGETS = (131072, 4000, 300)   # tokens: one chunk of some 16,000, several, chunks of a few rows
 
 
@@ -81,7 +83,9 @@ def logits_crc(ctx, shape, budget, k):
 
 
 LOGITS = {("one layer", 2): 903127134, ("one layer", 3): 2015117514,
-          ("one wide layer", 2): 878337199, ("one wide layer", 3): 1545911119}
+          ("one wide layer", 2): 878337199, ("one wide layer", 3): 1545911119,
+          ("tiny", 2): 4004519680, ("tiny", 3): 843533209,
+          ("grouped", 2): 665073265, ("grouped", 3): 355354920}
 
 
 @pytest.mark.parametrize("budget", BUDGETS)
