@@ -64,11 +64,11 @@ __device__ __forceinline__ void load_rows(__half* dst, const __half* src, int ro
 }
 
 template <int HD>
-__global__ void __launch_bounds__(kThreads) k_attention(const __half* __restrict__ qkv, const int32_t* seq_start,
+__global__ void __launch_bounds__(kThreads) k_attention(const __half* qkv, const int32_t* seq_start,
                                                         const int32_t* tile_seq, const int32_t* tile_q0,
                                                         const int32_t* n_tiles, int Hq, int Hkv,
                                                         PrefixKV prefix, float scale_log2,
-                                                        __half* __restrict__ out) {
+                                                        __half* out) {
   constexpr int LDS = HD + 8;
   constexpr int KS = HD / 16;  // k-steps of QK^T
   constexpr int DN = HD / 8;   // 8-wide output column tiles

@@ -300,11 +300,11 @@ __global__ void __launch_bounds__(kThreadsTC, ACfg<HD>::CTAS)
       auto list = [&](int w) -> int2 {
         if (w >= n_work) return make_int2(0, 0);
         const int i = w / a.Hkv;
-        return make_int2(__ldg(a.tile_seq + i), __ldg(a.tile_q0 + i));
+        return make_int2(a.tile_seq[i], a.tile_q0[i]);
       };
       auto bounds = [&](int2 l, int w) -> int4 {
-        const int st = __ldg(a.seq_start + l.x);
-        return make_int4(st, __ldg(a.seq_start + l.x + 1) - st, l.y,
+        const int st = a.seq_start[l.x];
+        return make_int4(st, a.seq_start[l.x + 1] - st, l.y,
                          w % a.Hkv + (a.prefix_is_seq0 && l.x == 0 ? kNoPrefix : 0));
       };
       auto publish = [&](int item, const int4& inf) -> bool {

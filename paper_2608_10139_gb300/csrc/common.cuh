@@ -41,8 +41,11 @@ __device__ __forceinline__ uint64_t global_timer_ns() {
 // Kernels of a query follow one another on one stream, each reading what the one
 // before wrote.  Launched through launch_chained a kernel may start while the one
 // before still runs: its set-up overlaps, and grid_wait() holds every access to
-// global memory (but to weights) until that kernel has finished and its writes are
-// visible.  grid_launch_next() allows the next kernel to start in the same way.
+// global memory until that kernel has finished and its writes are visible.  Such a
+// kernel is resident while others write, so ld.global.nc (__ldg, or a pointer that is
+// const and __restrict__), which asks for memory that nobody writes as long as the
+// kernel lives, is for data that no kernel of the chain writes alone: weights, gains,
+// biases and RoPE tables.  All else, the caller's columns too, is read by plain loads.  grid_launch_next() allows the next kernel to start in the same way.
 // Both do nothing in a kernel that was launched in the ordinary way.
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

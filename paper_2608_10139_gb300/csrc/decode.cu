@@ -313,8 +313,8 @@ __global__ void __launch_bounds__(DecStream<HD>::NW * 32, DecStream<HD>::CTAS)
     if (i < n_tasks) {
       t.r = i / a.Hkv;
       t.h = i % a.Hkv;
-      t.st = __ldg(a.seq_start + t.r);
-      t.len = __ldg(a.seq_start + t.r + 1) - t.st;
+      t.st = a.seq_start[t.r];
+      t.len = a.seq_start[t.r + 1] - t.st;
     }
     return t;
   };

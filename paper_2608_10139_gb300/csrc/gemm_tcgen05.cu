@@ -163,7 +163,7 @@ __device__ __forceinline__ float row_inv_rms(const GemmEpilogue& ep, int row, bo
   if ((ep.ss_parts & 3) == 0) {
     const float4* p4 = reinterpret_cast<const float4*>(p);
     for (int i = 0; i < ep.ss_parts / 4; ++i) {
-      const float4 v = __ldg(p4 + i);
+      const float4 v = p4[i];
       s += v.x;
       s += v.y;
       s += v.z;

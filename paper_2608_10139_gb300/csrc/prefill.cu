@@ -321,12 +321,24 @@ __global__ void __launch_bounds__(256) k_label_head(const float* resid, const in
   }
 }
 
+// One warp copies n 16-byte words, eight a lane in flight.
+__device__ __forceinline__ void copy_row(const uint4* src, uint4* dst, int n, int lane) {
+  for (int c0 = lane; c0 < n; c0 += 32 * 8) {
+    uint4 v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      if (c0 + 32 * i < n) v[i] = src[c0 + 32 * i];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      if (c0 + 32 * i < n) dst[c0 + 32 * i] = v[i];
+  }
+}
+
 // Final layer, rows only: gather each row's last token (attention output and
 // residual) into dense [n, .] buffers; last_compact[r] = r, or -1 for a row
 // without tokens of its own (its logits come from the prefix's last state).
-__global__ void k_gather_last(const __half* __restrict__ att, int ld_att, const float* __restrict__ resid, int d,
-                              const int32_t* last_idx, int64_t n, __half* __restrict__ att_out,
-                              float* __restrict__ resid_out, int32_t* last_compact) {
+__global__ void k_gather_last(const __half* att, int ld_att, const float* resid, int d, const int32_t* last_idx,
+                              int64_t n, __half* att_out, float* resid_out, int32_t* last_compact) {
   grid_launch_next();
   grid_wait();
   const int64_t r = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
@@ -335,14 +347,9 @@ __global__ void k_gather_last(const __half* __restrict__ att, int ld_att, const 
   const int32_t li = last_idx[r];
   if (lane == 0) last_compact[r] = li >= 0 ? static_cast<int32_t>(r) : -1;
   const int64_t src = li >= 0 ? li : 0;
-  const uint4* a = reinterpret_cast<const uint4*>(att + src * ld_att);
-  uint4* ao = reinterpret_cast<uint4*>(att_out + r * ld_att);
-#pragma unroll 8
-  for (int c = lane; c < ld_att / 8; c += 32) ao[c] = a[c];
-  const float4* x = reinterpret_cast<const float4*>(resid + src * d);
-  float4* xo = reinterpret_cast<float4*>(resid_out + r * d);
-#pragma unroll 8
-  for (int c = lane; c < d / 4; c += 32) xo[c] = x[c];
+  copy_row(reinterpret_cast<const uint4*>(att + src * ld_att), reinterpret_cast<uint4*>(att_out + r * ld_att), ld_att / 8,
+           lane);
+  copy_row(reinterpret_cast<const uint4*>(resid + src * d), reinterpret_cast<uint4*>(resid_out + r * d), d / 4, lane);
 }
 
 constexpr int64_t kRowBlocksMax = 2432;  // rows that take a block each: two waves of eight blocks per SM

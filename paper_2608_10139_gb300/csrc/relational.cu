@@ -42,7 +42,7 @@ __device__ __forceinline__ void load_term(const PredDev& p, int64_t r0, int64_t 
     if (full) {
       const int4* q = reinterpret_cast<const int4*>(c);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) t.w[j] = __ldg(q + j);
+      for (int j = 0; j < 4; ++j) t.w[j] = q[j];
     } else {
       int64_t* v = reinterpret_cast<int64_t*>(t.w);
 #pragma unroll
@@ -52,8 +52,8 @@ __device__ __forceinline__ void load_term(const PredDev& p, int64_t r0, int64_t 
     const int32_t* c = static_cast<const int32_t*>(p.col) + r0;
     if (full) {
       const int4* q = reinterpret_cast<const int4*>(c);
-      t.w[0] = __ldg(q);
-      t.w[1] = __ldg(q + 1);
+      t.w[0] = q[0];
+      t.w[1] = q[1];
     } else {
       int32_t* v = reinterpret_cast<int32_t*>(t.w);
 #pragma unroll
@@ -271,10 +271,10 @@ __global__ void __launch_bounds__(kThreads) k_predicate_cols(PredSet ps, int64_t
     if (i < N8) {
       const int64_t* c = static_cast<const int64_t*>(ps.p[i].col);
       if (full) {
-        t[i].w[0] = __ldg(reinterpret_cast<const int4*>(c + ra));
-        t[i].w[1] = __ldg(reinterpret_cast<const int4*>(c + ra) + 1);
-        t[i].w[2] = __ldg(reinterpret_cast<const int4*>(c + rb));
-        t[i].w[3] = __ldg(reinterpret_cast<const int4*>(c + rb) + 1);
+        t[i].w[0] = *reinterpret_cast<const int4*>(c + ra);
+        t[i].w[1] = reinterpret_cast<const int4*>(c + ra)[1];
+        t[i].w[2] = *reinterpret_cast<const int4*>(c + rb);
+        t[i].w[3] = reinterpret_cast<const int4*>(c + rb)[1];
       } else {
         int64_t* v = reinterpret_cast<int64_t*>(t[i].w);
 #pragma unroll
@@ -286,8 +286,8 @@ __global__ void __launch_bounds__(kThreads) k_predicate_cols(PredSet ps, int64_t
     } else {
       const int32_t* c = static_cast<const int32_t*>(ps.p[i].col);
       if (full) {
-        t[i].w[0] = __ldg(reinterpret_cast<const int4*>(c + ra));
-        t[i].w[1] = __ldg(reinterpret_cast<const int4*>(c + rb));
+        t[i].w[0] = *reinterpret_cast<const int4*>(c + ra);
+        t[i].w[1] = *reinterpret_cast<const int4*>(c + rb);
       } else {
         int32_t* v = reinterpret_cast<int32_t*>(t[i].w);
 #pragma unroll
@@ -335,8 +335,8 @@ __device__ __forceinline__ uint32_t eval_rows4(const PredDev& p, int64_t r0, int
     const int64_t* c = static_cast<const int64_t*>(p.col) + r0;
     int64_t* v = reinterpret_cast<int64_t*>(t.w);
     if (full) {
-      t.w[0] = __ldg(reinterpret_cast<const int4*>(c));
-      t.w[1] = __ldg(reinterpret_cast<const int4*>(c) + 1);
+      t.w[0] = *reinterpret_cast<const int4*>(c);
+      t.w[1] = reinterpret_cast<const int4*>(c)[1];
     } else {
 #pragma unroll
       for (int j = 0; j < 4; ++j) v[j] = r0 + j < n ? c[j] : 0;
@@ -348,7 +348,7 @@ __device__ __forceinline__ uint32_t eval_rows4(const PredDev& p, int64_t r0, int
   const int32_t* c = static_cast<const int32_t*>(p.col) + r0;
   int32_t* v = reinterpret_cast<int32_t*>(t.w);
   if (full) {
-    t.w[0] = __ldg(reinterpret_cast<const int4*>(c));
+    t.w[0] = *reinterpret_cast<const int4*>(c);
   } else {
 #pragma unroll
     for (int j = 0; j < 4; ++j) v[j] = r0 + j < n ? c[j] : 0;
@@ -377,8 +377,8 @@ __global__ void __launch_bounds__(kProbeThreads) k_probe_mask(PredSet ps, ProbeS
     nib = r0 + 4 <= n ? 0xFu : ((1u << (n - r0)) - 1u);
     unsigned long long key[4];
     if (r0 + 4 <= n) {
-      const ulonglong2 a = __ldg(reinterpret_cast<const ulonglong2*>(probe.keys + r0));
-      const ulonglong2 b = __ldg(reinterpret_cast<const ulonglong2*>(probe.keys + r0) + 1);
+      const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(probe.keys + r0);
+      const ulonglong2 b = reinterpret_cast<const ulonglong2*>(probe.keys + r0)[1];
       key[0] = a.x, key[1] = a.y, key[2] = b.x, key[3] = b.y;
     } else {
 #pragma unroll
@@ -593,7 +593,7 @@ __global__ void __launch_bounds__(kThreads) k_compact_wide(const uint32_t* bits,
   int m[8];
   if (PAYLOAD) {
 #pragma unroll
-    for (int j = 0; j < 8; ++j) m[j] = (byte >> j) & 1u ? __ldg(payload + r0 + j) : 0;
+    for (int j = 0; j < 8; ++j) m[j] = (byte >> j) & 1u ? payload[r0 + j] : 0;
   }
   int total;
   int64_t at = out + block_excl_scan<kThreads>(__popc(byte), sh, &total);
