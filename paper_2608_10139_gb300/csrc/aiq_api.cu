@@ -382,6 +382,12 @@ int attention_tile_tokens(const aiq_ctx* c, int Hq, int Hkv, int hd) {
   return c->attention_tc && attention_tc_supported(hd, Hq, Hkv) ? attention_tc_tile_tokens(Hq, Hkv) : 64;
 }
 
+// Entries of a packed chunk's work list: every sequence's blocks of that many
+// tokens, the last of each as short as one token.
+int64_t attention_items(const aiq_ctx* c, int64_t T, int64_t n_seqs, int Hq, int Hkv, int hd) {
+  return T / attention_tile_tokens(c, Hq, Hkv, hd) + n_seqs;
+}
+
 // The work list of a packed chunk, the same for each of its layers.
 void attention_tiles(aiq_ctx* c, int64_t n_seqs, const int32_t* seq_start, int32_t* tile_seq, int32_t* tile_q0,
                      int32_t* n_tiles, int Hq, int Hkv, int hd) {
@@ -395,8 +401,7 @@ aiq_status attention(aiq_ctx* c, const __half* qkv, int64_t T, int64_t n_seqs, c
                      const int32_t* tile_seq, const int32_t* tile_q0, const int32_t* n_tiles, int Hq, int Hkv, int hd,
                      const PrefixKV& prefix, __half* out) {
   const bool tc = c->attention_tc && attention_tc_supported(hd, Hq, Hkv);
-  const int tq = attention_tile_tokens(c, Hq, Hkv, hd);
-  const int n_tiles_max = static_cast<int>((T + tq - 1) / tq + n_seqs);
+  const int n_tiles_max = static_cast<int>(attention_items(c, T, n_seqs, Hq, Hkv, hd));
   ProfScope p(c, "attention", 0, 0);
   if (tc) {
     const int e = launch_attention_tc(qkv, T, seq_start, tile_seq, tile_q0, n_tiles_max, n_tiles, Hq, Hkv, hd, prefix,
@@ -540,8 +545,9 @@ aiq_status prefill_bufs(aiq_ctx* c, const ModelD& m, int64_t B, int64_t max_rows
   AIQ_TRY(ws(c, "pf.pos", B, &pb->pos));
   AIQ_TRY(ws(c, "pf.seq_start", B + 1, &pb->seq_start));
   AIQ_TRY(ws(c, "pf.last", B, &pb->last_idx));
-  AIQ_TRY(ws(c, "pf.tile_seq", B / 8 + B + 1, &pb->tile_seq));
-  AIQ_TRY(ws(c, "pf.tile_q0", B / 8 + B + 1, &pb->tile_q0));
+  const int64_t items = attention_items(c, B, max_rows, g.n_heads, g.n_kv_heads, g.head_dim);
+  AIQ_TRY(ws(c, "pf.tile_seq", items, &pb->tile_seq));
+  AIQ_TRY(ws(c, "pf.tile_q0", items, &pb->tile_q0));
   AIQ_TRY(ws(c, "pf.n_tiles", 1, &pb->n_tiles));
   AIQ_TRY(ws(c, "pf.resid", B * g.d_model, &pb->resid));
   AIQ_TRY(ws(c, "pf.xn", B * g.d_model * (m.mlp_split ? 2 : 1), &pb->xn));
@@ -2077,7 +2083,7 @@ aiq_status aiq_op_attention(aiq_ctx* c, const void* qkv, int64_t T, const int32_
   if (n_seqs == 0 || T == 0) return AIQ_OK;
   CUDA_TRY(cudaSetDevice(c->device));
   int32_t *tile_seq, *tile_q0, *n_tiles;
-  const int64_t cap = T / 8 + n_seqs + 1;
+  const int64_t cap = attention_items(c, T, n_seqs, Hq, Hkv, hd);
   AIQ_TRY(ws(c, "op.tile_seq", cap, &tile_seq));
   AIQ_TRY(ws(c, "op.tile_q0", cap, &tile_q0));
   AIQ_TRY(ws(c, "op.n_tiles", 1, &n_tiles));

@@ -217,6 +217,30 @@ def test_attention_varlen(ctx, hd, Hq, Hkv):
         _close(got[s:s + n], ref, 4e-3, 4e-3, f"attention seq {i} len {n} hd {hd}")
 
 
+@pytest.mark.parametrize("hd,Hq,Hkv", [(64, 32, 1), (128, 64, 1), (64, 128, 1), (128, 256, 2)])
+def test_attention_many_heads_per_key_head(ctx, hd, Hq, Hkv):
+    """32 to 128 query heads per key/value head: 4 tokens a work item down to one, so
+    that a chunk has up to as many items as tokens and sequences (the list is sized
+    for them), rows of one token included."""
+    lens = [1] * 40 + [700, 3, 641, 2, 900]
+    T, W = sum(lens), (Hq + 2 * Hkv) * hd
+    g = torch.Generator(device="cuda").manual_seed(hd + Hq)
+    qkv = torch.randn((T, W), generator=g, device="cuda").half()
+    starts = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    out = torch.zeros((T, Hq * hd), dtype=torch.float16, device="cuda")
+    ds = _h(starts)
+    torch.cuda.synchronize()
+    ctx.op_attention(qkv.data_ptr(), T, ds.data_ptr(), len(lens), Hq, Hkv, hd, out.data_ptr())
+    torch.cuda.synchronize()
+    for s, n in zip(starts, lens):
+        q, k, v = qkv[s:s + n].double().split([Hq * hd, Hkv * hd, Hkv * hd], 1)
+        q = q.view(n, Hkv, Hq // Hkv, hd)
+        z = torch.einsum("mkgd,nkd->kgmn", q, k.view(n, Hkv, hd)) / hd ** 0.5
+        z = z.masked_fill(torch.ones((n, n), dtype=torch.bool, device="cuda").triu(1), -torch.inf).softmax(-1)
+        ref = torch.einsum("kgmn,nkd->mkgd", z, v.view(n, Hkv, hd)).reshape(n, Hq * hd)
+        _close(_np64(out[s:s + n]), ref.cpu().numpy(), 4e-3, 4e-3, f"{Hq // Hkv} heads per key head, {n} tokens")
+
+
 @pytest.mark.parametrize("hd,Hq,Hkv,P", [(32, 4, 4, 16), (64, 8, 2, 64), (64, 8, 2, 70), (128, 4, 1, 130),
                                          (64, 32, 8, 64), (128, 32, 8, 128)])
 def test_attention_with_shared_prefix(ctx, hd, Hq, Hkv, P):
