@@ -1601,15 +1601,19 @@ int gemm_f16_tcgen05(const __half* A, int64_t lda, const __half* B, int64_t ldb,
   if (K % (BK * CfgPair::SUB) != 0) pair = false;  // CTA-pair stages hold 128-deep k-blocks
   if ((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(B)) & 15) return cudaErrorMisalignedAddress;
   if ((lda * 2) % 16 != 0 || (ldb * 2) % 16 != 0) return cudaErrorInvalidValue;
+  KArgs a{M, N, K, ep};
   if (ep.kind == EPI_ROPE_F16) {
     const int hd = ep.head_dim;
     if (!(hd == 32 || hd == 64 || hd == 128) || bn % hd != 0 || !ep.positions || !ep.rope_cos) return cudaErrorInvalidValue;
+    // a head that starts below rope_cols is rotated whole: past this point the
+    // kernels see multiples of a head only
+    const int cols = std::min(std::max(ep.rope_cols, 0), N);
+    a.ep.rope_cols = (cols + hd - 1) / hd * hd;
   }
   if (ep.kind == EPI_ARGMAX && (!ep.bias || !ep.best)) return cudaErrorInvalidValue;
   if (ep.kind == EPI_RESID_ADD &&
       (!ep.out || (reinterpret_cast<uintptr_t>(ep.out) & 15) || (ep.ldo * 4) % 16 != 0 || ep.xh_out))
     return cudaErrorInvalidValue;
-  KArgs a{M, N, K, ep};
   const FewTile few = gemm_few_tile(M, N, K, bn, pair, ep, num_sms);
   switch (few.bn) {
     case 16: return dispatch_few<16>(A, lda, B, ldb, a, bn, few.two_ctas, num_sms, stream);

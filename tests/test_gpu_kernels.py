@@ -126,6 +126,37 @@ def test_gemm_qkv_rope(ctx, hd, Hq, Hkv, bn):
     _close(_np64(out), ref, 2e-3, 2e-3 * np.sqrt(K) * 0.05, f"rope hd{hd}")
 
 
+@pytest.mark.parametrize("M", [40, 16384 + 40])
+@pytest.mark.parametrize("rope_cols", [-5, 0, 1, 10, 96, 250, 1 << 30])
+def test_gemm_rope_columns_inside_a_head(ctx, M, rope_cols):
+    """A head that starts below rope_cols is rotated whole, wherever in it rope_cols
+    lies, in narrow tiles (few rows) and wide ones: the bits of the next head boundary."""
+    hd, N, K = 64, 256, 128
+    g = torch.Generator(device="cuda").manual_seed(M)
+    A = torch.randn((M, K), generator=g, device="cuda").half()
+    B = (torch.randn((N, K), generator=g, device="cuda") * 0.05).half()
+    pos = torch.arange(M, dtype=torch.int32, device="cuda") % 300
+    cs = torch.zeros((300, hd // 2), dtype=torch.float32, device="cuda")
+    sn = torch.zeros_like(cs)
+    ctx.op_rope_table(cs.data_ptr(), sn.data_ptr(), 300, hd, 1.0e4)
+
+    def run(cols):
+        out = torch.zeros((M, N), dtype=torch.float16, device="cuda")
+        torch.cuda.synchronize()
+        ctx.op_gemm(A.data_ptr(), K, B.data_ptr(), K, M, N, K, 256, 1, out.data_ptr(), N, pos.data_ptr(), cs.data_ptr(),
+                    sn.data_ptr(), cols, hd)
+        torch.cuda.synchronize()
+        return out
+
+    whole = -(-min(max(rope_cols, 0), N) // hd) * hd
+    out = run(rope_cols)
+    assert torch.equal(out, run(whole))
+    y = A.double() @ B.double().t()
+    qk = tf.rope(y[:, :whole].cpu().numpy().reshape(M, -1, hd), pos.cpu().numpy(), 1.0e4).reshape(M, whole)
+    ref = np.concatenate([qk, y[:, whole:].cpu().numpy()], axis=1)
+    _close(_np64(out), ref, 2e-3, 2e-3 * np.sqrt(K) * 0.05, f"rope_cols {rope_cols}")
+
+
 @pytest.mark.parametrize("d", [128, 2048, 4096])
 def test_rmsnorm(ctx, d):
     rng = np.random.default_rng(d)
