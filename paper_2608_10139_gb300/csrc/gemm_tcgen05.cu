@@ -1604,7 +1604,8 @@ int gemm_f16_tcgen05(const __half* A, int64_t lda, const __half* B, int64_t ldb,
   KArgs a{M, N, K, ep};
   if (ep.kind == EPI_ROPE_F16) {
     const int hd = ep.head_dim;
-    if (!(hd == 32 || hd == 64 || hd == 128) || bn % hd != 0 || !ep.positions || !ep.rope_cos) return cudaErrorInvalidValue;
+    if (!(hd == 32 || hd == 64 || hd == 128) || bn % hd != 0 || !ep.positions || !ep.rope_cos || !ep.rope_sin)
+      return cudaErrorInvalidValue;
     // a head that starts below rope_cols is rotated whole: past this point the
     // kernels see multiples of a head only
     const int cols = std::min(std::max(ep.rope_cols, 0), N);

@@ -6,6 +6,7 @@ import pytest
 
 from helpers import gpu_ctx
 from oracle import transformer as tf
+from paper_2608_10139_gb300 import aiq
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -155,6 +156,15 @@ def test_gemm_rope_columns_inside_a_head(ctx, M, rope_cols):
     qk = tf.rope(y[:, :whole].cpu().numpy().reshape(M, -1, hd), pos.cpu().numpy(), 1.0e4).reshape(M, whole)
     ref = np.concatenate([qk, y[:, whole:].cpu().numpy()], axis=1)
     _close(_np64(out), ref, 2e-3, 2e-3 * np.sqrt(K) * 0.05, f"rope_cols {rope_cols}")
+
+
+@pytest.mark.parametrize("missing", ["positions", "cos", "sin"])
+def test_gemm_rope_needs_its_tables(ctx, missing):
+    """Refused on the host, before anything is launched."""
+    t = {k: torch.zeros(64 * 256, dtype=torch.float32, device="cuda") for k in ("a", "b", "out", "positions", "cos", "sin")}
+    p = {k: 0 if k == missing else v.data_ptr() for k, v in t.items()}
+    with pytest.raises(aiq.AiqError):
+        ctx.op_gemm(p["a"], 64, p["b"], 64, 8, 128, 64, 128, 1, p["out"], 128, p["positions"], p["cos"], p["sin"], 128, 64)
 
 
 @pytest.mark.parametrize("d", [128, 2048, 4096])
