@@ -707,22 +707,28 @@ aiq_status ensure_lm_f16(aiq_ctx* c, ModelD& m) {
   if (m.lm_f16) return AIQ_OK;
   const aiq_model_config& g = m.cfg;
   const int vpad = (g.vocab + 255) / 256 * 256;
-  __half* w = nullptr;
-  float* b = nullptr;
-  void* p = nullptr;
-  AIQ_TRY(dalloc(c, &p, static_cast<size_t>(vpad) * g.d_model * sizeof(__half)));
-  w = static_cast<__half*>(p);
-  m.allocs.push_back(DevBuf{p, std::max<size_t>(static_cast<size_t>(vpad) * g.d_model * sizeof(__half), 256)});
-  AIQ_TRY(dalloc(c, &p, static_cast<size_t>(vpad) * sizeof(float)));
-  b = static_cast<float*>(p);
-  m.allocs.push_back(DevBuf{p, std::max<size_t>(static_cast<size_t>(vpad) * sizeof(float), 256)});
-  CUDA_TRY(cudaMemsetAsync(w, 0, static_cast<size_t>(vpad) * g.d_model * sizeof(__half), c->stream));
-  launch_bf16_to_f16(m.lm_head, w, g.vocab, g.d_model, 0, 0, c->d_err, c->stream);
-  launch_bias_f32(m.lm_bias, g.vocab, vpad, b, c->stream);
-  counted(c, 2);
-  AIQ_TRY(sync_and_check(c));
-  m.lm_f16 = w;
-  m.lm_bias_f32 = b;
+  DevBuf w, b;
+  w.bytes = static_cast<size_t>(vpad) * g.d_model * sizeof(__half);
+  b.bytes = static_cast<size_t>(vpad) * sizeof(float);
+  auto make = [&]() -> aiq_status {
+    AIQ_TRY(dalloc(c, &w.p, w.bytes));
+    AIQ_TRY(dalloc(c, &b.p, b.bytes));
+    CUDA_TRY(cudaMemsetAsync(w.p, 0, w.bytes, c->stream));
+    launch_bf16_to_f16(m.lm_head, static_cast<__half*>(w.p), g.vocab, g.d_model, 0, 0, c->d_err, c->stream);
+    launch_bias_f32(m.lm_bias, g.vocab, vpad, static_cast<float*>(b.p), c->stream);
+    counted(c, 2);
+    return sync_and_check(c);
+  };
+  const aiq_status st = make();
+  if (st != AIQ_OK) {
+    dfree(c, w.p, w.bytes);
+    dfree(c, b.p, b.bytes);
+    return st;
+  }
+  m.allocs.push_back(w);
+  m.allocs.push_back(b);
+  m.lm_f16 = static_cast<__half*>(w.p);
+  m.lm_bias_f32 = static_cast<float*>(b.p);
   m.vpad = vpad;
   return AIQ_OK;
 }

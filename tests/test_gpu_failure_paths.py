@@ -134,3 +134,25 @@ def test_activation_overflow_is_reported_then_the_context_recovers(inputs, fresh
         _same(_query(ctx, q, W), fresh)
     finally:
         ctx.close()
+
+
+def test_refused_transforms_hold_no_more_memory(inputs):
+    """A transform refused for want of room keeps nothing that it made half of: under a
+    cap that rises by 8 KB a try (less than any buffer of the full-vocabulary head, so
+    that some tries get its first and not its second), it runs once the cap reaches
+    what it needs."""
+    q, W = inputs
+    c = gpu_ctx()
+    try:
+        t = c.load_table(q.table.cols, (q.table.offsets, q.table.tokens))
+        m = c.load_model(W_TINY.model, weights_list(W_TINY.model, W))
+        for cap in range(1 << 20, 64 << 20, 8 << 10):
+            c.set_option("device_bytes_max", cap)
+            try:
+                c.run_transform(t, m, [("rating", aiq.GE, 5)], q.prefix, 2)
+                return
+            except aiq.AiqError as e:
+                assert e.status == aiq.ERR_OOM
+        pytest.fail("64 MB were not enough for a transform of 15 MB")
+    finally:
+        c.close()
