@@ -236,6 +236,14 @@ void release_join_table(aiq_ctx* c) {
   }
 }
 
+// A join's table is in use while one of these lives: until it has been probed, or
+// the query has failed.
+struct JoinTableInUse {
+  aiq_ctx* c;
+  explicit JoinTableInUse(aiq_ctx* c_) : c(c_) { c->join_table_live = true; }
+  ~JoinTableInUse() { c->join_table_live = false; }
+};
+
 // Grow-only named workspace buffer.
 template <typename T>
 aiq_status ws(aiq_ctx* c, const char* name, size_t count, T** out) {
@@ -1234,8 +1242,8 @@ aiq_status run_query(aiq_ctx* c, const TableD* build, int32_t build_key, const a
   CUDA_TRY(cudaEventRecord(ev[0], c->stream));
   QueryState st;
   ProbeSpec pr;
-  c->join_table_live = build != nullptr;
   if (build) {
+    const JoinTableInUse in_use(c);
     PredSet bps{};
     AIQ_TRY(make_pred_set(*build, build_preds, n_bp, &bps));
     const int64_t* bkeys = static_cast<const int64_t*>(build->cols[build_key].data);
@@ -1277,7 +1285,6 @@ aiq_status run_query(aiq_ctx* c, const TableD* build, int32_t build_key, const a
   } else {
     AIQ_TRY(filter_compact(c, probe, ps, pr, "sel", &st.S, &st.ids, nullptr));
   }
-  c->join_table_live = false;
   CUDA_TRY(cudaEventRecord(ev[1], c->stream));
 
   ResultH R;

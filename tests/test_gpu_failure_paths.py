@@ -156,3 +156,44 @@ def test_refused_transforms_hold_no_more_memory(inputs):
         pytest.fail("64 MB were not enough for a transform of 15 MB")
     finally:
         c.close()
+
+
+def test_room_of_a_failed_joins_table(inputs):
+    """A join that fails (a repeated build key) leaves its table (15.7 MB) behind; a
+    transform under a cap that needs the table's room takes it back."""
+    q, W = inputs
+    m = 300_000
+    keys = np.arange(m, dtype=np.int64)
+    keys[-1] = 0
+
+    def context():
+        c = gpu_ctx()
+        text = c.load_table(q.table.cols, (q.table.offsets, q.table.tokens))
+        build, probe = c.load_table({"k": keys}), c.load_table({"k": keys[:1000]})
+        return c, text, build, probe, c.load_model(W_TINY.model, weights_list(W_TINY.model, W))
+
+    def transform(c, text, model, cap):
+        c.set_option("device_bytes_max", cap)
+        return c.run_transform(text, model, [("rating", aiq.GE, 5)], q.prefix, 2)
+
+    c, text, _, _, model = context()
+    try:
+        loaded = sum(v.nbytes for v in (*q.table.cols.values(), q.table.offsets, q.table.tokens, keys, *weights_list(W_TINY.model, W)))
+        for cap in range(loaded, loaded + (1 << 30), 1 << 20):   # the least room it runs in, to 1 MB
+            try:
+                want = transform(c, text, model, cap)
+                break
+            except aiq.AiqError as e:
+                assert e.status == aiq.ERR_OOM
+    finally:
+        c.close()
+    c, text, build, probe, model = context()
+    try:
+        with pytest.raises(aiq.AiqError) as e:
+            c.run_join_select(build, "k", [], probe, "k", 0, [], [], [0, 1], agg=aiq.AGG_COUNT,
+                              flags=aiq.FLAG_RELATIONAL_ONLY)
+        assert e.value.status == aiq.ERR_INVALID_ARG
+        got = transform(c, text, model, cap + (1 << 20))
+        assert np.array_equal(got.gen_tokens, want.gen_tokens)
+    finally:
+        c.close()
