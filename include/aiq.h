@@ -273,8 +273,10 @@ aiq_status aiq_result_free(aiq_ctx* ctx, aiq_result_h result);
 /* Thread-local description of the last failure on this thread ("" if none). */
 const char* aiq_last_error(void);
 
-/* Options: "token_budget" (max packed tokens per prefill chunk, default
- * 131072), "profile" (0/1: time every GEMM launch with CUDA events),
+/* Options: "token_budget" (max packed tokens per prefill chunk, the shared
+ * prefix's included where it runs with the first one; a longer row or prefix
+ * raises it; default 131072), "profile" (0/1: time every GEMM launch with CUDA
+ * events),
  * "gemm_pair" (0/1, default 1: 256 x 256 GEMM tiles on CTA pairs where
  * N % 256 == 0 and M >= 512; also selects them for aiq_op_gemm with bn = 256),
  * "attention_tc" (0/1, default 1: tcgen05 attention where the head shape

@@ -919,6 +919,12 @@ aiq_status prefill_phase(aiq_ctx* c, const TableD& t, ModelD& m, const aiq_selec
   st->P = P;
   const int64_t max_len = col.max_len * (st->ids2 ? 2 : 1);  // longest row text; the prefix runs on its own
   int64_t n_chunks = 1, step = 0, rows_per_chunk = 0;
+  // The shared prefix runs through the decoder once.  As the first sequence of the
+  // first chunk it costs no pass over the weights and no launches of its own (the
+  // 1B shape, 58 rows behind 64 tokens: 11.5 -> 10.9 ms; the tiny query 467 -> 376
+  // us); a pass of its own, before the chunks, is left for generation, for a prefix
+  // that is long or fills a chunk, and where the larger chunk's buffers do not fit.
+  bool merged = false;
   if (gp) {
     // a chunk's rows decode together, one token each per step: as few chunks
     // of equal row counts as fit at most decode_rows rows, 2^20 tokens and
@@ -936,7 +942,10 @@ aiq_status prefill_phase(aiq_ctx* c, const TableD& t, ModelD& m, const aiq_selec
   } else {
     const int64_t B = std::max<int64_t>(std::max<int64_t>(c->token_budget, max_len), P);
     step = B - max_len + 1;
-    n_chunks = std::max<int64_t>(1, (T + step - 1) / step);
+    // the first chunk's tokens, the prefix among them, stay within B as every chunk's do
+    merged = P > 0 && P <= kMergedPrefixMax && P < step;
+    const int64_t before = merged ? P : 0;
+    n_chunks = T <= step && T + before <= B ? 1 : (T + before + step - 1) / step;
   }
   st->n_chunks = n_chunks;
   std::vector<int64_t> chunks(2 * (n_chunks + 1));
@@ -948,19 +957,13 @@ aiq_status prefill_phase(aiq_ctx* c, const TableD& t, ModelD& m, const aiq_selec
     if (gp)
       launch_chunk_bounds_rows(cu, S, rows_per_chunk, n_chunks, chunk_d, c->stream);
     else
-      launch_chunk_bounds(cu, S, step, n_chunks, chunk_d, c->stream);
+      launch_chunk_bounds(cu, S, merged ? P : 0, step, n_chunks, chunk_d, c->stream);
     counted(c, 1);
     CUDA_TRY(
         cudaMemcpyAsync(chunks.data(), chunk_d, chunks.size() * sizeof(int64_t), cudaMemcpyDeviceToHost, c->stream));
     AIQ_TRY(sync_and_check(c));
   }
   AIQ_TRY(ensure_rope(c, m, static_cast<int>(P + max_len + (gp ? gp->max_new : 0))));
-  // The shared prefix runs through the decoder once.  As the first sequence of the
-  // first chunk it costs no pass over the weights and no launches of its own (the
-  // 1B shape, 58 rows behind 64 tokens: 11.5 -> 10.9 ms; the tiny query 467 -> 376
-  // us); a pass of its own, before the chunks, is left for generation, for a long
-  // prefix and where the larger chunk's buffers do not fit.
-  bool merged = P > 0 && P <= kMergedPrefixMax && !gp;
   int64_t Bmax, Rmax;
   PrefillBufs pb;
   for (;;) {

@@ -159,9 +159,10 @@ void launch_plan_rows(const int64_t* offsets, const int32_t* ids, const int32_t*
                       int64_t* cu, int64_t* total, int64_t* pairs, cudaStream_t s);
 // Exclusive scan of int32 lengths into int64 cu[S+1] (multi-block).
 void launch_scan_lengths(const int32_t* lens, int64_t S, int64_t* cu, int64_t* scratch_blocks, cudaStream_t s);
-// chunk_rows[c] = first row whose start offset >= c * budget_step, c = 0..n_chunks.
-void launch_chunk_bounds(const int64_t* cu, int64_t S, int64_t step, int64_t n_chunks, int64_t* chunk_rows,
-                         cudaStream_t s);
+// chunk_rows[c] = first row that starts at or past token c * step, c = 0..n_chunks, `before`
+// tokens preceding the first row (the prefix, where it runs with the first chunk).
+void launch_chunk_bounds(const int64_t* cu, int64_t S, int64_t before, int64_t step, int64_t n_chunks,
+                         int64_t* chunk_rows, cudaStream_t s);
 // Chunks of equal row counts: chunk_rows[2c] = min(c * rows_per_chunk, S), [2c+1] = cu[that row].
 void launch_chunk_bounds_rows(const int64_t* cu, int64_t S, int64_t rows_per_chunk, int64_t n_chunks,
                               int64_t* chunk_rows, cudaStream_t s);

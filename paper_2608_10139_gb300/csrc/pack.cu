@@ -113,8 +113,9 @@ __global__ void __launch_bounds__(1024) k_plan_rows(const int64_t* offsets, cons
   }
 }
 
-// chunk_rows[2c] = first row i with cu[i] >= c * step (S if none), chunk_rows[2c+1] = cu[that row].
-__global__ void k_chunk_bounds(const int64_t* cu, int64_t S, int64_t step, int64_t n_chunks, int64_t* out) {
+// chunk_rows[2c] = first row i with before + cu[i] >= c * step (S if none), chunk_rows[2c+1] = cu[that row].
+__global__ void k_chunk_bounds(const int64_t* cu, int64_t S, int64_t before, int64_t step, int64_t n_chunks,
+                               int64_t* out) {
   grid_launch_next();
   grid_wait();
   const int64_t c = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -123,7 +124,7 @@ __global__ void k_chunk_bounds(const int64_t* cu, int64_t S, int64_t step, int64
   if (c == n_chunks) {
     lo = S;
   } else {
-    const int64_t target = c * step;
+    const int64_t target = c * step - before;
     while (lo < hi) {
       const int64_t mid = (lo + hi) >> 1;
       if (cu[mid] < target) lo = mid + 1;
@@ -253,9 +254,10 @@ void launch_plan_rows(const int64_t* offsets, const int32_t* ids, const int32_t*
                  total, pairs);
 }
 
-void launch_chunk_bounds(const int64_t* cu, int64_t S, int64_t step, int64_t n_chunks, int64_t* chunk_rows,
-                         cudaStream_t s) {
-  launch_chained(k_chunk_bounds, dim3(static_cast<unsigned>((n_chunks + 1 + 127) / 128)), 128, 0, s, 1, cu, S, step, n_chunks, chunk_rows);
+void launch_chunk_bounds(const int64_t* cu, int64_t S, int64_t before, int64_t step, int64_t n_chunks,
+                         int64_t* chunk_rows, cudaStream_t s) {
+  launch_chained(k_chunk_bounds, dim3(static_cast<unsigned>((n_chunks + 1 + 127) / 128)), 128, 0, s, 1, cu, S, before,
+                 step, n_chunks, chunk_rows);
 }
 
 void launch_chunk_bounds_rows(const int64_t* cu, int64_t S, int64_t rows_per_chunk, int64_t n_chunks,

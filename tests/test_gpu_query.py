@@ -403,6 +403,37 @@ def test_prefix_lengths_and_chunks(ctx, P, gqa):
     ctx.free_model(mh)
 
 
+@pytest.mark.parametrize("P,budget,chunks", [(0, 1024, 1), (63, 1024, 1), (64, 1024, 1), (65, 1024, 2), (960, 1024, 2),
+                                             (961, 1024, 1), (64, 200, 8), (150, 200, 8)])
+def test_prefix_counts_in_the_token_budget(ctx, P, budget, chunks):
+    """The first chunk's tokens are within the budget, the prefix's among them: 15 rows
+    of 64 tokens behind prefixes that just fit with them and just do not; a prefix
+    that would fill a chunk takes a pass of its own.  The same logits as in one chunk."""
+    w = synth.C1_TINY
+    rng = np.random.default_rng(P)
+    offsets = np.arange(16, dtype=np.int64) * 64
+    table = synth.Table(15, {"rating": np.ones(15, np.int32)}, offsets,
+                        rng.integers(0, w.model.vocab, 960).astype(np.int32))
+    prefix = rng.integers(0, w.model.vocab, P).astype(np.int32)
+    mh, _ = _model(ctx, w.model, w.weight_seed)
+    t = _load(ctx, table)
+    got = []
+    try:
+        for b in (131072, budget):
+            ctx.set_option("token_budget", b)
+            got.append(ctx.run_select(t, mh, [], prefix, w.label_ids, agg=w.agg, flags=aiq.FLAG_LOGITS))
+    finally:
+        ctx.set_option("token_budget", 131072)
+    assert [r.n_chunks for r in got] == [1, chunks]
+    assert np.array_equal(got[0].label_logits, got[1].label_logits)
+    # with the rows, the prefix's final layer runs its output projection and MLP for one token only
+    d, f, step = w.model.d_model, w.model.d_ffn, budget - 63
+    alone = max(P - 1, 0) * 2 * (d * d + 3 * d * f)
+    assert got[1].prefill_flops - got[0].prefill_flops == (alone if P >= step else 0)
+    ctx.free_table(t)
+    ctx.free_model(mh)
+
+
 def test_row_plan_sizes(ctx):
     """Up to 8192 rows one block measures and places the rows' texts, above that a
     chain of kernels: token counts, work counts and logits agree on both sides, at
