@@ -177,7 +177,7 @@ struct aiq_ctx {
   int* d_err = nullptr;           // its device address
   int64_t* h_pin = nullptr;  // pinned staging for control scalars
   int64_t* d_pin = nullptr;  // its device address
-  bool join_table_live = false;      // a join is building or probing its table
+  bool tight = false;        // a call's second try: the routes that need the least device memory
   unsigned int* d_arrived = nullptr;  // arrival counter of the tile-count scans (zero between launches)
   size_t bytes_max = SIZE_MAX;
   size_t bytes_used = 0;
@@ -227,22 +227,35 @@ void dfree(aiq_ctx* c, void* p, size_t bytes) {
   c->bytes_used -= std::max<size_t>(bytes, 256);
 }
 
-void release_join_table(aiq_ctx* c) {
+// Gives workspace buffers back: those whose names start with `prefix`.
+void release_workspace(aiq_ctx* c, const std::string& prefix = "") {
   cudaStreamSynchronize(c->stream);
-  for (const char* name : {"j.keys", "j.vals"}) {
-    DevBuf& b = c->ws[name];
-    if (b.p) dfree(c, b.p, b.bytes);
-    b = DevBuf{};
-  }
+  for (auto& kv : c->ws)
+    if (kv.first.compare(0, prefix.size(), prefix) == 0) {
+      dfree(c, kv.second.p, kv.second.bytes);
+      kv.second = DevBuf{};
+    }
 }
 
-// A join's table is in use while one of these lives: until it has been probed, or
-// the query has failed.
-struct JoinTableInUse {
-  aiq_ctx* c;
-  explicit JoinTableInUse(aiq_ctx* c_) : c(c_) { c->join_table_live = true; }
-  ~JoinTableInUse() { c->join_table_live = false; }
-};
+// Runs a call and, where it finds no room for a buffer, runs it again from an empty
+// workspace (no buffer's content outlives a call) by the routes that need the least:
+// buffers as large as they must be, the prefix in a pass of its own, a join's table
+// for the rows that pass their terms, given back once it has been probed.
+template <typename F>
+aiq_status with_room(aiq_ctx* c, F run) {
+  aiq_status st = run();
+  if (st != AIQ_ERR_OOM) return st;
+  const auto abandon = [&] {
+    release_workspace(c);
+    *c->h_err = 0;  // what the abandoned kernels found is no other call's
+  };
+  abandon();
+  c->tight = true;
+  st = run();
+  c->tight = false;
+  if (st == AIQ_ERR_OOM) abandon();
+  return st;
+}
 
 // Grow-only named workspace buffer.
 template <typename T>
@@ -256,16 +269,9 @@ aiq_status ws(aiq_ctx* c, const char* name, size_t count, T** out) {
       b.p = nullptr;
       b.bytes = 0;
     }
-    size_t want = bytes + bytes / 4;
+    size_t want = c->tight ? bytes : bytes + bytes / 4;
     void* p = nullptr;
-    aiq_status st = dalloc(c, &p, want);
-    if (st != AIQ_OK) st = dalloc(c, &p, want = bytes);
-    if (st != AIQ_OK && !c->join_table_live) {
-      // a join's table is of no use once it has been probed: its room may be what is missing
-      release_join_table(c);
-      st = dalloc(c, &p, want);
-    }
-    AIQ_TRY(st);
+    if (dalloc(c, &p, want) != AIQ_OK) AIQ_TRY(dalloc(c, &p, want = bytes));
     b.p = p;
     b.bytes = want;
   }
@@ -461,8 +467,9 @@ aiq_status filter_compact(aiq_ctx* c, const TableD& t, const PredSet& ps, const 
   std::string b = tag;
   ProbeSpec pr = probe;
   int32_t* ids;
-  // a small table: one launch, where there is room for every row's id
-  if (!pr.keys && filter_is_small(n) && ws(c, (b + ".ids").c_str(), n, &ids) == AIQ_OK) {
+  // a small table: one launch, with room for every row's id
+  if (!pr.keys && filter_is_small(n) && !c->tight) {
+    AIQ_TRY(ws(c, (b + ".ids").c_str(), n, &ids));
     {
       ProfScope p(c, "predicate_mask", 0, 0);
       launch_filter_small(ps, n, ids, c->d_pin, nullptr, c->stream);
@@ -923,7 +930,7 @@ aiq_status prefill_phase(aiq_ctx* c, const TableD& t, ModelD& m, const aiq_selec
   // first chunk it costs no pass over the weights and no launches of its own (the
   // 1B shape, 58 rows behind 64 tokens: 11.5 -> 10.9 ms; the tiny query 467 -> 376
   // us); a pass of its own, before the chunks, is left for generation, for a prefix
-  // that is long or fills a chunk, and where the larger chunk's buffers do not fit.
+  // that is long or fills a chunk, and where device memory is short.
   bool merged = false;
   if (gp) {
     // a chunk's rows decode together, one token each per step: as few chunks
@@ -943,7 +950,7 @@ aiq_status prefill_phase(aiq_ctx* c, const TableD& t, ModelD& m, const aiq_selec
     const int64_t B = std::max<int64_t>(std::max<int64_t>(c->token_budget, max_len), P);
     step = B - max_len + 1;
     // the first chunk's tokens, the prefix among them, stay within B as every chunk's do
-    merged = P > 0 && P <= kMergedPrefixMax && P < step;
+    merged = P > 0 && P <= kMergedPrefixMax && P < step && !c->tight;
     const int64_t before = merged ? P : 0;
     n_chunks = T <= step && T + before <= B ? 1 : (T + before + step - 1) / step;
   }
@@ -964,22 +971,15 @@ aiq_status prefill_phase(aiq_ctx* c, const TableD& t, ModelD& m, const aiq_selec
     AIQ_TRY(sync_and_check(c));
   }
   AIQ_TRY(ensure_rope(c, m, static_cast<int>(P + max_len + (gp ? gp->max_new : 0))));
-  int64_t Bmax, Rmax;
-  PrefillBufs pb;
-  for (;;) {
-    Bmax = P;
-    Rmax = 1;
-    for (int64_t i = 0; i < n_chunks; ++i) {
-      const bool with_prefix = merged && i == 0;
-      Bmax = std::max(Bmax, chunks[2 * (i + 1) + 1] - chunks[2 * i + 1] + (with_prefix ? P : 0));
-      Rmax = std::max(Rmax, chunks[2 * (i + 1)] - chunks[2 * i] + (with_prefix ? 1 : 0));
-    }
-    // a chunk of rows with empty text has more rows than tokens
-    const aiq_status s = prefill_bufs(c, m, std::max<int64_t>({Bmax, Rmax, 64}), Rmax, &pb);
-    if (s == AIQ_OK) break;
-    if (!merged) return s;
-    merged = false;
+  int64_t Bmax = P, Rmax = 1;
+  for (int64_t i = 0; i < n_chunks; ++i) {
+    const bool with_prefix = merged && i == 0;
+    Bmax = std::max(Bmax, chunks[2 * (i + 1) + 1] - chunks[2 * i + 1] + (with_prefix ? P : 0));
+    Rmax = std::max(Rmax, chunks[2 * (i + 1)] - chunks[2 * i] + (with_prefix ? 1 : 0));
   }
+  PrefillBufs pb;
+  // a chunk of rows with empty text has more rows than tokens
+  AIQ_TRY(prefill_bufs(c, m, std::max<int64_t>({Bmax, Rmax, 64}), Rmax, &pb));
   st->merged_prefix = merged;
   const aiq_model_config& g = m.cfg;
   const int64_t ldkv = 2 * static_cast<int64_t>(g.n_kv_heads) * g.head_dim;
@@ -1246,14 +1246,13 @@ aiq_status run_query(aiq_ctx* c, const TableD* build, int32_t build_key, const a
   QueryState st;
   ProbeSpec pr;
   if (build) {
-    const JoinTableInUse in_use(c);
     PredSet bps{};
     AIQ_TRY(make_pred_set(*build, build_preds, n_bp, &bps));
     const int64_t* bkeys = static_cast<const int64_t*>(build->cols[build_key].data);
     // Up to kDirectBuildRows build rows (100 MB of table) the rows that pass the
-    // terms go straight into a table sized for all rows; above, and where that
-    // table leaves no room, they are compacted first and the table sized for them.
-    auto build_table = [&](bool direct) -> aiq_status {
+    // terms go straight into a table sized for all rows; above, and where device
+    // memory is short, they are compacted first and the table sized for them.
+    auto build_and_probe = [&](bool direct) -> aiq_status {
       unsigned long long* tk;
       int32_t *tv, *bids = nullptr;
       int64_t Sb = build->n_rows, cap = 64;
@@ -1272,19 +1271,17 @@ aiq_status run_query(aiq_ctx* c, const TableD* build, int32_t build_key, const a
       pr.table_keys = tk;
       pr.table_vals = tv;
       pr.capacity = cap;
-      return AIQ_OK;
+      return filter_compact(c, probe, ps, pr, "sel", &st.S, &st.ids, &st.build_rows);
     };
-    aiq_status s = AIQ_ERR_OOM;
-    if (build->n_rows <= kDirectBuildRows) {
-      s = build_table(true);
-      if (s == AIQ_OK) s = filter_compact(c, probe, ps, pr, "sel", &st.S, &st.ids, &st.build_rows);
-      if (s == AIQ_ERR_OOM) release_join_table(c);
-    }
-    if (s == AIQ_ERR_OOM) {
-      s = build_table(false);
-      if (s == AIQ_OK) s = filter_compact(c, probe, ps, pr, "sel", &st.S, &st.ids, &st.build_rows);
+    const bool few = build->n_rows <= kDirectBuildRows;
+    aiq_status s = build_and_probe(few && !c->tight);
+    if (s == AIQ_ERR_OOM && few && c->tight) {  // with most rows passing, their ids may be what does not fit
+      release_workspace(c);
+      s = build_and_probe(true);
     }
     AIQ_TRY(s);
+    if (c->tight)
+      for (const char* done : {"j.", "jb."}) release_workspace(c, done);
   } else {
     AIQ_TRY(filter_compact(c, probe, ps, pr, "sel", &st.S, &st.ids, nullptr));
   }
@@ -1924,7 +1921,7 @@ aiq_status aiq_run_select(aiq_ctx* c, aiq_table table, aiq_model model, const ai
   if (q->agg == AIQ_AGG_GROUP_BUILD_KEY && !(q->flags & AIQ_FLAG_RELATIONAL_ONLY))
     return fail(AIQ_ERR_INVALID_ARG, "GROUP_BUILD_KEY needs aiq_run_join_select");
   CUDA_TRY(cudaSetDevice(c->device));
-  return run_query(c, nullptr, -1, nullptr, 0, t->second, -1, m, q, out);
+  return with_room(c, [&] { return run_query(c, nullptr, -1, nullptr, 0, t->second, -1, m, q, out); });
 }
 
 aiq_status aiq_run_join_select(aiq_ctx* c, aiq_table build, int32_t build_key, const aiq_pred* build_preds,
@@ -1944,7 +1941,9 @@ aiq_status aiq_run_join_select(aiq_ctx* c, aiq_table build, int32_t build_key, c
   auto mi = c->models.find(model);
   if (mi != c->models.end()) m = &mi->second;
   CUDA_TRY(cudaSetDevice(c->device));
-  return run_query(c, &b->second, build_key, build_preds, n_build_preds, p->second, probe_key, m, q, out);
+  return with_room(c, [&] {
+    return run_query(c, &b->second, build_key, build_preds, n_build_preds, p->second, probe_key, m, q, out);
+  });
 }
 
 aiq_status aiq_run_transform(aiq_ctx* c, aiq_table table, aiq_model model, const aiq_select* q,
@@ -1955,7 +1954,7 @@ aiq_status aiq_run_transform(aiq_ctx* c, aiq_table table, aiq_model model, const
   auto mi = c->models.find(model);
   if (mi == c->models.end()) return fail(AIQ_ERR_NOT_FOUND, "unknown model handle");
   CUDA_TRY(cudaSetDevice(c->device));
-  return run_transform(c, t->second, &mi->second, q, gen, out);
+  return with_room(c, [&] { return run_transform(c, t->second, &mi->second, q, gen, out); });
 }
 
 aiq_status aiq_run_pair_select(aiq_ctx* c, aiq_table table, int32_t key_column, aiq_model model,
@@ -1969,7 +1968,7 @@ aiq_status aiq_run_pair_select(aiq_ctx* c, aiq_table table, int32_t key_column, 
   auto mi = c->models.find(model);
   if (mi == c->models.end()) return fail(AIQ_ERR_NOT_FOUND, "unknown model handle");
   CUDA_TRY(cudaSetDevice(c->device));
-  return run_pair_select(c, t->second, key_column, &mi->second, q, out);
+  return with_room(c, [&] { return run_pair_select(c, t->second, key_column, &mi->second, q, out); });
 }
 
 aiq_status aiq_result(aiq_ctx* c, aiq_result_h h, aiq_result_view* out) {
@@ -2100,9 +2099,11 @@ aiq_status aiq_op_attention(aiq_ctx* c, const void* qkv, int64_t T, const int32_
   CUDA_TRY(cudaSetDevice(c->device));
   int32_t *tile_seq, *tile_q0, *n_tiles;
   const int64_t cap = attention_items(c, T, n_seqs, Hq, Hkv, hd);
-  AIQ_TRY(ws(c, "op.tile_seq", cap, &tile_seq));
-  AIQ_TRY(ws(c, "op.tile_q0", cap, &tile_q0));
-  AIQ_TRY(ws(c, "op.n_tiles", 1, &n_tiles));
+  AIQ_TRY(with_room(c, [&]() -> aiq_status {
+    AIQ_TRY(ws(c, "op.tile_seq", cap, &tile_seq));
+    AIQ_TRY(ws(c, "op.tile_q0", cap, &tile_q0));
+    return ws(c, "op.n_tiles", 1, &n_tiles);
+  }));
   if (P < 0 || (P > 0 && !prefix_kv)) return fail(AIQ_ERR_INVALID_ARG, "bad prefix");
   attention_tiles(c, n_seqs, seq_start, tile_seq, tile_q0, n_tiles, Hq, Hkv, hd);
   const PrefixKV prefix{static_cast<const __half*>(prefix_kv), 2 * static_cast<int64_t>(Hkv) * hd, P, false};

@@ -197,3 +197,43 @@ def test_room_of_a_failed_joins_table(inputs):
         assert np.array_equal(got.gen_tokens, want.gen_tokens)
     finally:
         c.close()
+
+
+def test_query_runs_in_the_room_that_it_needs(inputs):
+    """A query whose prefix would run with the first chunk (2,088 tokens of 2,216) fits
+    where it does with a pass of its own (1,216 tokens at a time): the sum of that
+    route's buffers, whatever smaller caps were tried before."""
+    _, W = inputs
+    g, P, n, L = W_TINY.model, 1000, 19, 64
+    rng = np.random.default_rng(4)
+    T, offsets = n * L, np.arange(n + 1, dtype=np.int64) * L
+    tokens = rng.integers(0, g.vocab, T).astype(np.int32)
+    prefix = rng.integers(0, g.vocab, P).astype(np.int32)
+    d, qd, kd, f = g.d_model, g.n_heads * g.head_dim, g.n_kv_heads * g.head_dim, g.d_ffn
+    per_token = 4 * 4 + 4 * d + 2 * d + 2 * (qd + 2 * kd) + 2 * qd + 2 * f + 4 * (d // 128)
+    need = T * per_token + g.n_layers * P * 2 * kd * 2 + 2 * 4 * 2048 * (g.head_dim // 2)   # with the RoPE tables
+    small = 64 << 10   # per-row buffers, work lists, 256 bytes at least for each
+    want = None
+    for tries in ([], [2.0, 0.5], [0.3, 0.6, 0.9, 0.95]):   # of the room, before
+        c = gpu_ctx()
+        try:
+            t = c.load_table({"rating": np.ones(n, np.int32)}, (offsets, tokens))
+            m = c.load_model(g, weights_list(g, W))
+            c.set_option("token_budget", 2100)
+            run = lambda: c.run_select(t, m, [], prefix, W_TINY.label_ids, flags=aiq.FLAG_LOGITS)  # noqa: E731
+            c.set_option("device_bytes_max", 1)
+            with pytest.raises(aiq.AiqError) as e:
+                run()
+            held = int(str(e.value).split("(")[1].split()[0]) - 256   # "(held + asked for > cap)"
+            for part in tries:
+                c.set_option("device_bytes_max", held + int(part * need))
+                try:
+                    run()
+                except aiq.AiqError as e:
+                    assert e.status == aiq.ERR_OOM and part < 1
+            c.set_option("device_bytes_max", held + need + small)
+            r = run()
+            assert want is None or np.array_equal(r.label_logits, want)
+            want = r.label_logits
+        finally:
+            c.close()
