@@ -237,6 +237,15 @@ void release_workspace(aiq_ctx* c, const std::string& prefix = "") {
     }
 }
 
+// As dalloc, for what outlives a call (tables, weights): no workspace is in use
+// between calls, so it gives way.
+aiq_status dalloc_kept(aiq_ctx* c, void** p, size_t bytes) {
+  const aiq_status st = dalloc(c, p, bytes);
+  if (st != AIQ_ERR_OOM) return st;
+  release_workspace(c);
+  return dalloc(c, p, bytes);
+}
+
 // Runs a call and, where it finds no room for a buffer, runs it again from an empty
 // workspace (no buffer's content outlives a call) by the routes that need the least:
 // buffers as large as they must be, the prefix in a pass of its own, a join's table
@@ -1608,7 +1617,7 @@ void free_table(aiq_ctx* c, TableD& t) {
 template <typename T>
 aiq_status model_alloc(aiq_ctx* c, ModelD& m, size_t count, T** out) {
   void* p = nullptr;
-  AIQ_TRY(dalloc(c, &p, count * sizeof(T)));
+  AIQ_TRY(dalloc_kept(c, &p, count * sizeof(T)));
   m.allocs.push_back(DevBuf{p, std::max<size_t>(count * sizeof(T), 256)});
   *out = static_cast<T*>(p);
   return AIQ_OK;
@@ -1737,7 +1746,7 @@ aiq_status aiq_load_table(aiq_ctx* c, const aiq_column* cols, int32_t n_cols, in
         col.max_id = std::max<int64_t>(col.max_id, ids[k]);
       }
       bytes = static_cast<size_t>(ntok) * sizeof(int32_t);
-      aiq_status st = dalloc(c, reinterpret_cast<void**>(&col.offsets), (n_rows + 1) * sizeof(int64_t));
+      aiq_status st = dalloc_kept(c, reinterpret_cast<void**>(&col.offsets), (n_rows + 1) * sizeof(int64_t));
       if (st != AIQ_OK) {
         free_table(c, t);
         return st;
@@ -1755,7 +1764,7 @@ aiq_status aiq_load_table(aiq_ctx* c, const aiq_column* cols, int32_t n_cols, in
       bytes = static_cast<size_t>(n_rows) * (a.type == AIQ_INT64 ? 8 : 4);
     }
     col.bytes = bytes;
-    aiq_status st = dalloc(c, &col.data, bytes);
+    aiq_status st = dalloc_kept(c, &col.data, bytes);
     if (st != AIQ_OK) {
       cudaStreamSynchronize(c->stream);
       if (col.offsets) dfree(c, col.offsets, (n_rows + 1) * sizeof(int64_t));
@@ -1836,7 +1845,7 @@ aiq_status aiq_load_model(aiq_ctx* c, const aiq_model_config* cfg, const void* c
   uint16_t* stage = nullptr;
   const size_t stage_elems = std::max<size_t>(2 * f * d, (size_t)(qd + 2 * kd) * d);
   void* sp = nullptr;
-  aiq_status st = dalloc(c, &sp, stage_elems * 2);
+  aiq_status st = dalloc_kept(c, &sp, stage_elems * 2);
   if (st != AIQ_OK) return st;
   stage = static_cast<uint16_t*>(sp);
   auto fail_model = [&](aiq_status s2) {

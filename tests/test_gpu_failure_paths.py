@@ -237,3 +237,27 @@ def test_query_runs_in_the_room_that_it_needs(inputs):
             want = r.label_logits
         finally:
             c.close()
+
+
+def test_loads_take_back_a_joins_room(inputs):
+    """After a join (a table of 15.7 MB for 300,000 build rows) a table and a model load
+    under a cap that has room for them and not for what the join left behind."""
+    _, W = inputs
+    c = gpu_ctx()
+    try:
+        keys = np.arange(300_000, dtype=np.int64)
+        build, probe = c.load_table({"k": keys}), c.load_table({"k": keys[:1000]})
+        c.run_join_select(build, "k", [], probe, "k", 0, [], [], [0, 1], agg=aiq.AGG_COUNT, flags=aiq.FLAG_RELATIONAL_ONLY)
+        held = keys.nbytes + 8000
+        c.set_option("device_bytes_max", held + keys.nbytes + (64 << 10))
+        t = c.load_table({"k": keys})
+        c.free_table(t)
+        r = c.run_join_select(build, "k", [("k", aiq.LT, 10)], probe, "k", 0, [], [], [0, 1], agg=aiq.AGG_COUNT,
+                              flags=aiq.FLAG_RELATIONAL_ONLY)
+        assert np.array_equal(r.cand_row_ids, np.arange(10))
+        c.set_option("device_bytes_max", 0)
+        c.run_join_select(build, "k", [], probe, "k", 0, [], [], [0, 1], agg=aiq.AGG_COUNT, flags=aiq.FLAG_RELATIONAL_ONLY)
+        c.set_option("device_bytes_max", held + (12 << 20))
+        c.free_model(c.load_model(W_TINY.model, weights_list(W_TINY.model, W)))
+    finally:
+        c.close()
