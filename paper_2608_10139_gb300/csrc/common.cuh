@@ -51,10 +51,16 @@ __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;
 __device__ __forceinline__ void grid_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 #ifdef __CUDACC__
-// cluster: CTAs per cluster along x (1: none).
-template <typename... P, typename... A>
+template <typename T>
+struct AsIs {
+  using type = T;  // not deduced from an argument
+};
+
+// cluster: CTAs per cluster along x (1: none).  The arguments convert to the
+// kernel's parameters implicitly or not at all, as between <<< >>> and ( ).
+template <typename... P>
 cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t stream, int cluster,
-                           A&&... args) {
+                           typename AsIs<P>::type... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = dim3(static_cast<unsigned>(threads), 1, 1);
@@ -69,7 +75,7 @@ cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, int threads, size_t 
   attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = cluster > 1 ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 #endif
 
