@@ -481,7 +481,7 @@ aiq_status filter_compact(aiq_ctx* c, const TableD& t, const PredSet& ps, const 
     AIQ_TRY(ws(c, (b + ".ids").c_str(), n, &ids));
     {
       ProfScope p(c, "predicate_mask", 0, 0);
-      launch_filter_small(ps, n, ids, c->d_pin, nullptr, c->stream);
+      launch_filter_small(ps, n, ids, c->d_pin, c->stream);
       counted(c, 1);
     }
     AIQ_TRY(sync_and_check(c));
@@ -520,7 +520,7 @@ aiq_status filter_compact(aiq_ctx* c, const TableD& t, const PredSet& ps, const 
   if (pr.keys) AIQ_TRY(ws(c, (b + ".payload").c_str(), std::max<int64_t>(S, 1), &pay));
   {
     ProfScope p(c, "compact", 0, 0);
-    launch_compact(bits, boff, n, ids, pr.match_out, pay, c->stream, c->d_arrived);
+    launch_compact(bits, boff, n, ids, pr.match_out, pay, c->stream);
     counted(c, n > 0);
   }
   *S_out = S;

@@ -102,7 +102,7 @@ aiq_status aiq_filter_compact_static(const aiq_term* terms, int32_t n_terms, int
   int32_t* counts = reinterpret_cast<int32_t*>(scratch + kBitsBytes);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (filter_is_small(n_rows)) {
-    launch_filter_small(ps, n_rows, ids_out, count_out, nullptr, s);
+    launch_filter_small(ps, n_rows, ids_out, count_out, s);
   } else {
     // Every scratch word the compaction reads is written earlier in this call
     // (each tile writes its whole bitmask slice and its count), so nothing is

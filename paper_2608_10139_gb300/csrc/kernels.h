@@ -114,10 +114,9 @@ struct TileBase {
 };
 
 // Filter of 1 .. kSmallRows rows (16-byte aligned columns) in one launch: the
-// survivors' ids and their number, in *count and, when given, *count2.
+// survivors' ids and their number in *count.
 bool filter_is_small(int64_t n_rows);
-void launch_filter_small(const PredSet& ps, int64_t n_rows, int32_t* ids, int64_t* count, int64_t* count2,
-                         cudaStream_t s);
+void launch_filter_small(const PredSet& ps, int64_t n_rows, int32_t* ids, int64_t* count, cudaStream_t s);
 // Mask bits, per-tile survivor counts and their exclusive scan offsets[tiles + 1].
 // arrived: a counter that is zero before the first call; total (optional) also
 // receives the number of survivors.  offsets == nullptr: no scan, the bits and the
@@ -129,10 +128,9 @@ int launch_predicate_scan(const PredSet& ps, const ProbeSpec& probe, int64_t n_r
 // Exclusive scan of n int32 counts into int64 offsets[n+1] (one block).
 void launch_scan_counts(const int32_t* counts, int64_t n, int64_t* offsets, cudaStream_t s);
 // Order-preserving compaction of set bits: ids_out[k] = row of the k-th set bit;
-// optionally gathers `payload[row]` into payload_out[k], and sets *arrived (a
-// scan's counter) to zero.
+// optionally gathers `payload[row]` into payload_out[k].
 void launch_compact(const uint32_t* bits, const int64_t* block_offsets, int64_t n_rows, int32_t* ids_out,
-                    const int32_t* payload, int32_t* payload_out, cudaStream_t s, unsigned int* arrived = nullptr);
+                    const int32_t* payload, int32_t* payload_out, cudaStream_t s);
 // The same without a scan before it, for up to kScanTilesMax tiles: the counts are
 // launch_predicate_scan's, *total receives the number of set bits.
 void launch_compact_counts(const uint32_t* bits, const int32_t* block_counts, int64_t n_rows, int32_t* ids_out,

@@ -445,8 +445,7 @@ constexpr int kSmallThreads = 1024;
 // thread, scans the survivor counts and writes the ids.  At these sizes a launch
 // costs more than the rows: a call on 10,007 rows takes 8.0 us in one launch,
 // against 14.7 in four.
-__global__ void __launch_bounds__(kSmallThreads) k_filter_small(PredSet ps, int64_t n, int32_t* ids, int64_t* count,
-                                                                int64_t* count2) {
+__global__ void __launch_bounds__(kSmallThreads) k_filter_small(PredSet ps, int64_t n, int32_t* ids, int64_t* count) {
   grid_launch_next();
   grid_wait();
   __shared__ int sh[kSmallThreads / 32];
@@ -468,10 +467,7 @@ __global__ void __launch_bounds__(kSmallThreads) k_filter_small(PredSet ps, int6
     base += total;
     __syncthreads();  // sh is reused
   }
-  if (threadIdx.x == 0) {
-    *count = base;
-    if (count2) *count2 = base;
-  }
+  if (threadIdx.x == 0) *count = base;
 }
 
 constexpr unsigned kWideTilesMax = 488;          // k_compact_wide without a payload
@@ -515,11 +511,9 @@ __device__ __forceinline__ int sum_counts(const int32_t* counts, unsigned end, i
 template <bool PAYLOAD, bool DIRECT>
 __global__ void __launch_bounds__(kCompactWarps * 32) k_compact(const uint32_t* bits, TileBase tb,
                                                                 int64_t n, int32_t* ids, const int32_t* payload,
-                                                                int32_t* payload_out, unsigned int* arrived) {
+                                                                int32_t* payload_out) {
   grid_launch_next();
   grid_wait();
-  // calls that overlap against the rules may leave the scan's counter behind: the next ones start from zero
-  if (arrived && blockIdx.x == 0 && threadIdx.x == 0) *arrived = 0;
   __shared__ uint16_t s_ids[kCompactWarps][kRowsPerBlock];  // row offsets within the tile
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t n_tiles = (n + kRowsPerBlock - 1) / kRowsPerBlock;
@@ -574,12 +568,10 @@ __global__ void __launch_bounds__(kCompactWarps * 32) k_compact(const uint32_t* 
 // tile is the faster above (2049 tiles: 4.4 us against 5.1).
 template <bool PAYLOAD, bool DIRECT>
 __global__ void __launch_bounds__(kThreads) k_compact_wide(const uint32_t* bits, TileBase tb, int32_t* ids,
-                                                           const int32_t* payload, int32_t* payload_out,
-                                                           unsigned int* arrived) {
+                                                           const int32_t* payload, int32_t* payload_out) {
   grid_launch_next();
   grid_wait();
   __shared__ int sh[kThreads / 32];
-  if (arrived && blockIdx.x == 0 && threadIdx.x == 0) *arrived = 0;  // as k_compact
   const int64_t tile = blockIdx.x;
   const uint32_t byte = reinterpret_cast<const uint8_t*>(bits + tile * (kRowsPerBlock / 32))[threadIdx.x];
   int64_t out;
@@ -903,9 +895,8 @@ PredSet wide_first(const PredSet& ps, int* n8) {
 
 bool filter_is_small(int64_t n_rows) { return n_rows > 0 && n_rows <= kSmallRows; }
 
-void launch_filter_small(const PredSet& ps, int64_t n_rows, int32_t* ids, int64_t* count, int64_t* count2,
-                         cudaStream_t s) {
-  launch_chained(k_filter_small, dim3(1), kSmallThreads, 0, s, 1, ps, n_rows, ids, count, count2);
+void launch_filter_small(const PredSet& ps, int64_t n_rows, int32_t* ids, int64_t* count, cudaStream_t s) {
+  launch_chained(k_filter_small, dim3(1), kSmallThreads, 0, s, 1, ps, n_rows, ids, count);
 }
 
 int launch_predicate_scan(const PredSet& ps, const ProbeSpec& probe, int64_t n_rows, uint32_t* bits,
@@ -957,19 +948,18 @@ void launch_scan_counts(const int32_t* counts, int64_t n, int64_t* offsets, cuda
 }
 
 void launch_compact(const uint32_t* bits, const int64_t* block_offsets, int64_t n_rows, int32_t* ids_out,
-                    const int32_t* payload, int32_t* payload_out, cudaStream_t s, unsigned int* arrived) {
+                    const int32_t* payload, int32_t* payload_out, cudaStream_t s) {
   if (n_rows <= 0) return;
   const unsigned tiles = blocks_for(n_rows, kRowsPerBlock);
   const TileBase tb{block_offsets, nullptr, nullptr};
   if (tiles <= (payload_out ? kWidePayloadTilesMax : kWideTilesMax)) {
     const auto kernel = payload_out ? k_compact_wide<true, false> : k_compact_wide<false, false>;
-    launch_chained(kernel, dim3(tiles), kThreads, 0, s, 1, bits, tb, ids_out, payload, payload_out, arrived);
+    launch_chained(kernel, dim3(tiles), kThreads, 0, s, 1, bits, tb, ids_out, payload, payload_out);
     return;
   }
   const unsigned grid = (tiles + kCompactWarps - 1) / kCompactWarps;  // one tile per warp
   const auto kernel = payload_out ? k_compact<true, false> : k_compact<false, false>;
-  launch_chained(kernel, dim3(grid), kCompactWarps * 32, 0, s, 1, bits, tb, n_rows, ids_out, payload, payload_out,
-                 arrived);
+  launch_chained(kernel, dim3(grid), kCompactWarps * 32, 0, s, 1, bits, tb, n_rows, ids_out, payload, payload_out);
 }
 
 void launch_compact_counts(const uint32_t* bits, const int32_t* block_counts, int64_t n_rows, int32_t* ids_out,
@@ -981,11 +971,10 @@ void launch_compact_counts(const uint32_t* bits, const int32_t* block_counts, in
   const unsigned tiles = blocks_for(n_rows, kRowsPerBlock);
   const TileBase tb{nullptr, block_counts, total};
   if (tiles <= kWideTilesMax)
-    launch_chained(k_compact_wide<false, true>, dim3(tiles), kThreads, 0, s, 1, bits, tb, ids_out, nullptr, nullptr,
-                   nullptr);
+    launch_chained(k_compact_wide<false, true>, dim3(tiles), kThreads, 0, s, 1, bits, tb, ids_out, nullptr, nullptr);
   else
     launch_chained(k_compact<false, true>, dim3((tiles + kCompactWarps - 1) / kCompactWarps), kCompactWarps * 32, 0, s,
-                   1, bits, tb, n_rows, ids_out, nullptr, nullptr, nullptr);
+                   1, bits, tb, n_rows, ids_out, nullptr, nullptr);
 }
 
 void launch_hash_build(const int64_t* keys, const int32_t* rows, int64_t n, unsigned long long* table_keys,
