@@ -224,6 +224,7 @@ __global__ void __launch_bounds__(kThreadsTC, ACfg<HD>::CTAS)
   auto sK = [&](int b) { return smem + C::OFF_K + b * C::K_BYTES; };
   auto sV = [&](int b) { return smem + C::OFF_V + b * C::K_BYTES; };
   if (smem_u32(smem) & 1023) {  // no tile is touched then
+    grid_wait();  // not done before the kernel ahead is
     if (threadIdx.x == 0) set_dev_error(a.err, DEVERR_BOUNDS);
     return;
   }

@@ -1,8 +1,11 @@
-"""Kernels that may be resident while the one before still writes (those that
+"""What a kernel of a programmatic chain must keep to, read in the sources.
+
+Kernels that may be resident while the one before still writes (those that
 call grid_wait) read what the chain writes by plain loads: ld.global.nc, which
 __ldg and a const __restrict__ parameter stand for, promises memory that nobody
-writes during the kernel's whole life.  No run shows a breach reliably, so the
-sources are read."""
+writes during the kernel's whole life.  A thread that returns before grid_wait
+lets its kernel end before the one ahead of it has, and the one behind start on
+unfinished data.  No run shows a breach of either reliably."""
 import glob
 import os
 import re
@@ -37,3 +40,11 @@ def test_read_only_loads_take_constant_data():
             assert inside or READ_ONLY.search(m.group(1)), f"{os.path.basename(path)}: __ldg({m.group(1)}"
         for arg in re.findall(r"\bload_f32x32\(([^)]*)\)", src):
             assert arg.startswith(("const float* src", "ep.bias", "ep.rope_cos", "ep.rope_sin")), arg
+
+
+def test_no_thread_leaves_before_the_wait():
+    for path in SOURCES:
+        for head, body in re.findall(r"__global__(.*?)\{(.*?)\n\}", _code(path), flags=re.S):
+            if "grid_wait()" in body:
+                before = body[:body.index("grid_wait()")]
+                assert not re.search(r"\breturn\b(?! ?\w)", before), f"{os.path.basename(path)}: {head.strip()[:120]}"
