@@ -53,9 +53,12 @@ __global__ void k_rope_table(float* cos_t, float* sin_t, int max_pos, int hd, do
 // row is also written as fp16, times the first layer's attention-norm gain
 // when `gain` is given (the fused RMSNorm's input), and its sums of squares
 // per 128 columns (16 lanes x 8 values, of the unscaled row) are stored, in a
-// fixed order.
-__global__ void k_embed(const int32_t* tok, int64_t T, const uint16_t* emb, int d, float* resid, __half* xh, float* ss,
-                        const uint16_t* gain, int* err) {
+// fixed order.  Bound by the copy bandwidth as long as the SMs are full of warps:
+// eight blocks each need the 32 registers asked for here (the system-scope error
+// word alone took it to 38 and six blocks: 92,000 rows of 2048 362 -> 402 us).
+__global__ void __launch_bounds__(256, 8)
+    k_embed(const int32_t* tok, int64_t T, const uint16_t* emb, int d, float* resid, __half* xh, float* ss,
+            const uint16_t* gain, int* err) {
   grid_launch_next();
   grid_wait();
   const int64_t t = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
