@@ -21,7 +21,12 @@ def _registers(source):
     return {name: int(n) for name, n in found}
 
 
-@pytest.mark.parametrize("source,kernel", [("prefill.cu", "k_embed")])
-def test_streaming_kernels_fill_an_sm(source, kernel):
-    of = {k: n for k, n in _registers(source).items() if kernel in k}
-    assert of and all(n <= 32 for n in of.values()), of
+@pytest.mark.parametrize("source,kernels", [
+    ("prefill.cu", ["k_embed"]),
+    ("relational.cu", ["k_predicate_colsILi0ELi1E", "k_predicate_colsILi0ELi2E", "k_predicate_colsILi1ELi0E"]),
+])
+def test_streaming_kernels_fill_an_sm(source, kernels):
+    registers = _registers(source)
+    for kernel in kernels:
+        of = {k: n for k, n in registers.items() if kernel in k}
+        assert of and all(n <= 32 for n in of.values()), of
