@@ -153,6 +153,47 @@ def test_static_filter_under_capture():
             assert torch.equal(ids[:len(want)], want)
 
 
+@pytest.mark.parametrize("n", [9000, 70_001])
+@pytest.mark.parametrize("before", ["nothing", "copy", "memset", "join of two streams", "a call"])
+def test_static_filter_captured_after(n, before):
+    """Recorded behind each kind of graph node: none, copies and memsets (which let no
+    kernel start early), two branches, and a call of its own."""
+    torch = pytest.importorskip("torch")
+    src = torch.arange(n, dtype=torch.int32, device="cuda")
+    col = torch.full((n,), 9, dtype=torch.int32, device="cuda")
+    other = torch.zeros(n, dtype=torch.int32, device="cuda")
+    ids = torch.empty(n, dtype=torch.int32, device="cuda")
+    count = torch.zeros(1, dtype=torch.int64, device="cuda")
+    call = lambda: aiq.filter_compact_static([(col.data_ptr(), aiq.INT32, rel.GE, 6)], n, ids.data_ptr(),  # noqa: E731
+                                             count.data_ptr(), torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    call()
+    torch.cuda.synchronize()
+    g, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    with torch.cuda.graph(g):
+        if before == "copy":
+            col.copy_(src)
+        elif before == "memset":
+            col.zero_()
+        elif before == "join of two streams":
+            side.wait_stream(torch.cuda.current_stream())
+            with torch.cuda.stream(side):
+                torch.add(src, 1, out=other)
+            torch.remainder(src, 10, out=col)
+            torch.cuda.current_stream().wait_stream(side)
+        elif before == "a call":
+            call()
+        call()
+    for _ in range(2):
+        col.fill_(9)
+        ids.fill_(-1)
+        g.replay()
+        torch.cuda.synchronize()
+        want = {"copy": src >= 6, "memset": src < 0, "join of two streams": src % 10 >= 6}.get(before, src >= 0)
+        want = want.nonzero().flatten().int()
+        assert int(count) == len(want) and torch.equal(ids[:len(want)], want)
+
+
 @pytest.mark.parametrize("room", [64 << 20, 14 << 20, 10 << 20, 3 << 20])
 def test_join_table_without_room(room):
     """A join whose table for all build rows (15.7 MB) does not fit under the byte cap,
