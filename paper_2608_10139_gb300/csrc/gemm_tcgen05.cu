@@ -1546,7 +1546,9 @@ int dispatch_few(const __half* A, int64_t lda, const __half* B, int64_t ldb, con
 // TMA add with four epilogue warps, 70, 25 and 25 with the few-rows kernels' eight, and
 // each epilogue 1200 more for its hand-offs (1800 in a pair, whose launch takes 1400
 // longer: products of 64 to 3000 rows and N, K <= 512 take 10.5 us in pairs and 8.8
-// without); a tile's epilogue runs beside the next tile's main loop.  Measured
+// without); a tile's epilogue runs beside the next tile's main loop.  A product that
+// feeds a norm costs 4000 more in narrow tiles, the launch of k_row_ss behind it (a tiny
+// decoder's query over 319 rows 300 us without this term, 288 with).  Measured
 // (us, weights from DRAM; with about 7 us of launch and event overhead; from 128 rows
 // on by pairs, and in brackets what one CTA per 128 rows took):
 //   M     N      K      large   16          32          64          128
@@ -1579,15 +1581,16 @@ FewTile gemm_few_tile(int M, int N, int K, int bn, bool pair, const GemmEpilogue
                      ? cost((M + 255) / 256 * (N / 256), num_sms / 2, 660, 256 * epi_large)
                      : cost(m128 * (N / bn), num_sms, bn == 256 ? 720 : 540, bn * epi_large);
   FewTile tile;
+  const int64_t sums = ep.ss_out ? 4000 : 0;
   const int rows = M < kFewRows ? (M + 7) / 8 * 8 : kFewRows;
   const int64_t m64 = (M + 63) / 64;
   for (int t = 16; t <= 128; t *= 2) {
     if (t / 2 > few_half(t, bn, ep)) break;  // a tile's halves lie within a gate / up block or a head
     const int64_t load = (rows + t) * 128 / 60;
-    int64_t c = cost(m64 * (N / t), num_sms, std::max<int64_t>({180, 2 * t, load}), t * epi);
+    int64_t c = sums + cost(m64 * (N / t), num_sms, std::max<int64_t>({180, 2 * t, load}), t * epi);
     if (c < best) best = c, tile = {t, false};
     if (M <= kFewRows || N % (2 * t) != 0) continue;
-    c = 1400 + cost(m128 * (N / (2 * t)), num_sms / 2, std::max<int64_t>(180, load), t * epi, 1800);
+    c = sums + 1400 + cost(m128 * (N / (2 * t)), num_sms / 2, std::max<int64_t>(180, load), t * epi, 1800);
     if (c < best) best = c, tile = {t, true};
   }
   return tile;
