@@ -45,7 +45,7 @@ L2_BYTES = 129 * 1024 * 1024
 # DRAM traffic of one tcgen05 GEMM launch from an ncu capture, valid only for the
 # GEMM source it was measured on (sha256 prefix of csrc/gemm_tcgen05.cu followed
 # by csrc/common.cuh, the device helpers it includes).
-GEMM_TRAFFIC = {"source_sha": "be5614b48d6d1e0d", "bytes_per_launch": 3.680e9}
+GEMM_TRAFFIC = {"source_sha": "b5a856459a28cacf", "bytes_per_launch": 3.919e9}
 
 
 def parse():

@@ -278,7 +278,9 @@ const char* aiq_last_error(void);
  * raises it; default 131072), "profile" (0/1: time every GEMM launch with CUDA
  * events),
  * "gemm_pair" (0/1, default 1: 256 x 256 GEMM tiles on CTA pairs where
- * N % 256 == 0 and M >= 512; also selects them for aiq_op_gemm with bn = 256),
+ * N % 256 == 0 and M >= 512, except where narrower tiles are estimated to be
+ * faster, which up to 16,384 rows may be taken whatever this option says; also
+ * selects them for aiq_op_gemm with bn = 256),
  * "attention_tc" (0/1, default 1: tcgen05 attention where the head shape
  * allows), "mlp_split" (read by aiq_load_model; 1: the model's MLP GEMMs
  * take their activations as two fp16 terms, fp16(v) and fp16(v - fp16(v)),
@@ -290,8 +292,9 @@ const char* aiq_last_error(void);
  * decode together, default 4096; the chunk's token budget grows to fit them,
  * up to 2^20 tokens and 32 GB of cached prompt keys/values), "device_bytes_max"
  * (the context's device byte cap, as AIQ_DEVICE_BYTES_MAX at aiq_init; <= 0
- * lifts it; memory already held stays, only further growth is refused with
- * AIQ_ERR_OOM). */
+ * lifts it; tables and models already held stay; a load or a query that finds no
+ * room takes back the context's workspace, and a query runs again in the least
+ * that it needs, before it is refused with AIQ_ERR_OOM). */
 aiq_status aiq_set_option(aiq_ctx* ctx, const char* name, int64_t value);
 
 /* The context's CUDA stream (a cudaStream_t), for callers that time the

@@ -53,18 +53,19 @@ namespace {
 constexpr int kThreadsTC = 192;
 constexpr int kKeys = 64;  // keys per block
 
-// Three CTAs per SM at head_dim 64, two at 128 (TMEM holds 512 columns).  Measured
-// at 970 rows of the select workload's text (128,867 tokens, 64 prefix keys, 32/8
-// heads, head_dim 64): 376 us, and 445 for two CTAs of 192 threads that double
-// the score buffers and accumulators and store through shared memory; at head_dim
-// 128 (150 rows, 34,972 tokens, 128 prefix keys): 217 us, and 353 for one such CTA
-// per SM.  What else was measured, against 387 and 222 us (V loaded right behind
-// its K, an item's bounds read after its predecessor's output): four CTAs with one
-// Q slot and two K slots 399, two with four K and V slots 455; a CTA of two tiles
-// that share K and V 427 and 346, its one MMA warp serving both tiles' hand-offs
-// in turn; outputs staged in shared memory for TMA 418 and 242 (each warp on its
-// own 395 and 226 against 376 and 217), 16-byte row stores 395 and 236; MMAs
-// issued by one lane's control flow instead of a whole warp's 437 and 252.
+// Three CTAs per SM at head_dim 64, two at 128 (TMEM holds 512 columns).  The launch
+// measures, for 970 rows of the select workload's text (128,867 tokens, 64 prefix
+// keys, 32/8 heads, head_dim 64), 360 us, and 418 for two CTAs of 192 threads that
+// double the score buffers and accumulators and store through shared memory; at
+// head_dim 128 (150 rows, 34,972 tokens, 128 prefix keys) 202 us, and 326 for one such
+// CTA per SM.  A whole call adds some 15 to 25 us.  What else was measured, each
+// against the kernel it changed and with what the timing added: four CTAs with one Q
+// slot and two K slots 399, two with four K and V slots 455, a CTA of two tiles that
+// share K and V 427 and 346, its one MMA warp serving both tiles' hand-offs in turn,
+// outputs staged in shared memory for TMA 418 and 242, 16-byte row stores 395 and 236,
+// MMAs issued by one lane's control flow instead of a whole warp's 437 and 252, all
+// against 387 and 222; outputs staged by each warp on its own 395 and 226 against 376
+// and 217.
 template <int HD>
 struct ACfg {
   static constexpr int NC = HD / 64;             // 64-column sub-tiles of one head
