@@ -215,8 +215,8 @@ __global__ void __launch_bounds__(256) k_rmsnorm_rows(const float* x, int d, con
 // thread that holds a whole row does it in the large tiles, so that a row's norm
 // does not depend on how many rows its product had.  A warp forms the terms of
 // eight groups (its 32 loads all in flight) and eight lanes walk them; what
-// bounds it is that walk and a launch: 6.3 us between events for 5,000 rows of 128,
-// where an empty pair of events measures 4.
+// bounds it is that walk behind one trip to memory: 590 rows of 2048 take 4.2 us from a
+// cold cache.
 constexpr int kSsWarps = 8, kSsGroups = 8;  // warps per block, groups per warp
 __global__ void __launch_bounds__(kSsWarps * 32) k_row_ss(const float* x, int64_t groups, float* ss) {
   grid_launch_next();
@@ -271,8 +271,8 @@ __global__ void k_rmsnorm_any(const float* x, int64_t T, int d, const uint16_t* 
 // then K dot products with the label rows of the LM head plus its bias.  A lane
 // takes columns lane, lane + 32, ... in turn, the order that its sums have always
 // had, 32 of them and two labels' rows in flight: one column at a time each walk of
-// the row was a chain of 64 loads (46 rows of 2048, 2 labels, between events: 33.5 ->
-// 12.2 us).  PER: columns in flight.
+// the row was a chain of 64 loads (46 rows of 2048, 2 labels: 28 -> 8.8 us from a cold
+// cache).  PER: columns in flight.
 template <int PER>
 __global__ void __launch_bounds__(256) k_label_head(const float* resid, const int32_t* last_idx,
                                                     const float* prefix_last, int64_t n, int d, const uint16_t* g,
